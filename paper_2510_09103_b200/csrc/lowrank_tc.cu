@@ -664,7 +664,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
       const TcBlock& t = P->blk[bi];
       const adapm_block& b = c->blocks[t.id];
       const int mb = (int)bi * kMapsPerBlock;
-      const bool stream = t.half != t.rp;
+      const bool stream = 2 * t.rp > 256;
       const int nbc1 = (2 * t.rp + 63) / 64, nbc2 = (4 * t.rp + 63) / 64;
       if (!stream) nbc_max = std::max(nbc_max, nbc2);
       if (b.v_mode == ADAPM_V_ELEMENT) any_element_v = true;
