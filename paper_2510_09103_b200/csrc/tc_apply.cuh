@@ -39,6 +39,7 @@ namespace tc {
 constexpr int kApplyThreads = 352;         // producer warp, MMA warp, eight epilogue warps, mover warp
 constexpr int kApplyNT = 128;              // columns per tile
 constexpr int kApplyQC = 32;               // columns per quarter tile
+constexpr int kApplyAcc = 4;               // accumulators
 constexpr int kApplyMaxStages = 8;         // R ring depth limit
 constexpr int kApplyMaxBufs = 6;           // g / W ring depth limit
 constexpr int kWBoxBytes = 128 * kApplyQC * 4;   // a quarter tile of W: 128 rows of 128 bytes
@@ -81,7 +82,7 @@ struct ApplyArgs {
 };
 
 struct __align__(8) ApplyShared {
-  uint64_t lfull, lempty, rfull[kApplyMaxStages], rempty[kApplyMaxStages], tfull[2], tempty[2];
+  uint64_t lfull, lempty, rfull[kApplyMaxStages], rempty[kApplyMaxStages], tfull[kApplyAcc], tempty[kApplyAcc];
   uint64_t wfull[kApplyMaxBufs];   // a quarter's g and W have landed
   uint64_t wdone[kApplyMaxBufs];   // all eight epilogue warps have put their new W back
   uint32_t tmem_base;
@@ -107,13 +108,13 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   if (threadIdx.x == 0) {
     mbar_init(&sh.lfull, 1); mbar_init(&sh.lempty, 1);
     for (int i = 0; i < kApplyMaxStages; ++i) { mbar_init(&sh.rfull[i], 1); mbar_init(&sh.rempty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 8); }
+    for (int i = 0; i < kApplyAcc; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 8); }
     for (int i = 0; i < kApplyMaxBufs; ++i) { mbar_init(&sh.wfull[i], 1); mbar_init(&sh.wdone[i], 8); }
     sh.abort = 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&sh.tmem_base, 256);
+    tmem_alloc(&sh.tmem_base, kApplyAcc * kApplyNT);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -122,155 +123,170 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   const uint32_t tmem_base = sh.tmem_base;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      uint32_t item_phase = 0, rphase = 0;
-      int rs = 0;
-      bool ok = true;
-      int l_loads = 0, r_loads = 0;
-      for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
-        const ApplyItem I = a.items[it];
-        if (kStream) {
-          // a stage = 64 columns of [L hi, L lo, R^T hi, R^T lo] of one set; previous set first
-          const int nbh = (I.rp + 63) >> 6;
-          for (int t = 0; t < I.n_tiles && ok; ++t) {
-            const int col0 = (I.tile0 + t) * kApplyNT;
-            for (int si = 0; si < n_sets && ok; ++si) {
-              const int xs = (si == 0 ? a.parity : 1 - a.parity) * 2 * I.half;
-              for (int jb = 0; jb < nbh; ++jb) {
-                if (!mbar_wait(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-                uint8_t* st = smem_r + (size_t)rs * (4 * kBoxBytes);
+    // ------------------------------------------------------------------ producer (all lanes run, one issues)
+    const bool leader = elect_one();
+    uint32_t item_phase = 0, rphase = 0;
+    int rs = 0;
+    bool ok = true;
+    int l_loads = 0, r_loads = 0;
+    for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
+      const ApplyItem& I = a.items[it];
+      const CUtensorMap* const ml = a.maps + I.map_l;
+      const CUtensorMap* const mr = a.maps + I.map_r;
+      const int n_tiles = I.n_tiles, row0 = I.row0;
+      int col0 = I.tile0 * kApplyNT;
+      if (kStream) {
+        // a stage = 64 columns of [L hi, L lo, R^T hi, R^T lo] of one set; previous set first
+        const int nbh = (I.rp + 63) >> 6, half = I.half;
+        for (int t = 0; t < n_tiles && ok; ++t, col0 += kApplyNT) {
+          for (int si = 0; si < n_sets && ok; ++si) {
+            const int xs = (si == 0 ? a.parity : 1 - a.parity) * 2 * half;
+            for (int jb = 0; jb < nbh; ++jb) {
+              if (!mbar_wait_warp(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
+              uint8_t* st = smem_r + rs * (4 * kBoxBytes);
+              if (leader) {
                 mbar_arrive_expect_tx(&sh.rfull[rs], 4u * kBoxBytes);
-                tma_load_box(st, a.maps + I.map_l, xs + 64 * jb, I.row0, &sh.rfull[rs]);
-                tma_load_box(st + kBoxBytes, a.maps + I.map_l, xs + I.half + 64 * jb, I.row0, &sh.rfull[rs]);
-                tma_load_box(st + 2 * kBoxBytes, a.maps + I.map_r, xs + 64 * jb, col0, &sh.rfull[rs]);
-                tma_load_box(st + 3 * kBoxBytes, a.maps + I.map_r, xs + I.half + 64 * jb, col0, &sh.rfull[rs]);
-                ++r_loads;
-                if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
+                tma_load_box(st, ml, xs + 64 * jb, row0, &sh.rfull[rs]);
+                tma_load_box(st + kBoxBytes, ml, xs + half + 64 * jb, row0, &sh.rfull[rs]);
+                tma_load_box(st + 2 * kBoxBytes, mr, xs + 64 * jb, col0, &sh.rfull[rs]);
+                tma_load_box(st + 3 * kBoxBytes, mr, xs + half + 64 * jb, col0, &sh.rfull[rs]);
               }
+              __syncwarp();
+              ++r_loads;
+              if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
             }
           }
-          continue;
         }
-        if (!mbar_wait(&sh.lempty, item_phase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-        const int nb = n_sets == 2 ? I.nbc2 : I.nbc1;
-        // with only the previous set in use, and that set in the right half, the boxes start there
-        const int x0 = (n_sets == 1 && a.parity) ? 2 * I.rp : 0;
-        mbar_arrive_expect_tx(&sh.lfull, (uint32_t)nb * kBoxBytes);
-        for (int bc = 0; bc < nb; ++bc)
-          tma_load_box(smem_l + (size_t)bc * kBoxBytes, a.maps + I.map_l, x0 + 64 * bc, I.row0, &sh.lfull);
-        ++l_loads;
-        for (int t = 0; t < I.n_tiles && ok; ++t) {
-          const int col0 = (I.tile0 + t) * kApplyNT;
-          for (int bc = 0; bc < nb; ++bc) {
-            if (!mbar_wait(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-            mbar_arrive_expect_tx(&sh.rfull[rs], (uint32_t)kBoxBytes);
-            tma_load_box(smem_r + (size_t)rs * kBoxBytes, a.maps + I.map_r, x0 + 64 * bc, col0, &sh.rfull[rs]);
-            ++r_loads;
-            if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
-          }
-        }
-        item_phase ^= 1u;
+        continue;
       }
-      if (!ok) {   // let the copies already issued land before the CTA exits
-        if (l_loads)
-          for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.lfull, (uint32_t)(l_loads - 1) & 1u); ++spin)
-            __nanosleep(64);
-        const int back = r_loads < a.n_rstages ? r_loads : a.n_rstages;
-        for (int q = 0; q < back; ++q) {
-          int st = rs - 1 - q;
-          uint32_t ph = rphase;
-          if (st < 0) { st += a.n_rstages; ph ^= 1u; }
-          for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.rfull[st], ph); ++spin) __nanosleep(64);
+      if (!mbar_wait_warp(&sh.lempty, item_phase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
+      const int nb = n_sets == 2 ? I.nbc2 : I.nbc1;
+      // with only the previous set in use, and that set in the right half, the boxes start there
+      const int x0 = (n_sets == 1 && a.parity) ? 2 * I.rp : 0;
+      if (leader) {
+        mbar_arrive_expect_tx(&sh.lfull, (uint32_t)nb * kBoxBytes);
+        for (int bc = 0; bc < nb; ++bc) tma_load_box(smem_l + bc * kBoxBytes, ml, x0 + 64 * bc, row0, &sh.lfull);
+      }
+      __syncwarp();
+      ++l_loads;
+      for (int t = 0; t < n_tiles && ok; ++t, col0 += kApplyNT) {
+        for (int bc = 0; bc < nb; ++bc) {
+          if (!mbar_wait_warp(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
+          if (leader) {
+            mbar_arrive_expect_tx(&sh.rfull[rs], (uint32_t)kBoxBytes);
+            tma_load_box(smem_r + rs * kBoxBytes, mr, x0 + 64 * bc, col0, &sh.rfull[rs]);
+          }
+          __syncwarp();
+          ++r_loads;
+          if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
         }
+      }
+      item_phase ^= 1u;
+    }
+    if (!ok) {   // let the copies already issued land before the CTA exits
+      if (l_loads)
+        for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.lfull, (uint32_t)(l_loads - 1) & 1u); ++spin)
+          __nanosleep(64);
+      const int back = r_loads < a.n_rstages ? r_loads : a.n_rstages;
+      for (int q = 0; q < back; ++q) {
+        int st = rs - 1 - q;
+        uint32_t ph = rphase;
+        if (st < 0) { st += a.n_rstages; ph ^= 1u; }
+        for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.rfull[st], ph); ++spin) __nanosleep(64);
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      uint32_t item_phase = 0, rphase = 0;
-      int rs = 0;
-      int j = 0;   // running tile count of this CTA
-      bool ok = true;
-      const uint32_t l_base = smem_u32(smem_l), r_base = smem_u32(smem_r);
-      const uint32_t dhi = desc_hi();
-      for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
-        const ApplyItem I = a.items[it];
-        const int ks = I.rp >> 4;     // 16-wide K steps per part (hi or lo of one set)
-        const int ktot = n_sets * 2 * ks;
-        const int nb = n_sets == 2 ? I.nbc2 : I.nbc1;
-        const uint32_t idesc_pos = make_idesc(kApplyNT, false, false, false);
-        const uint32_t idesc_neg = make_idesc(kApplyNT, false, false, true);
-        const uint32_t la = desc_lo(l_base, 16);
-        if (kStream) {
-          const int nbh = (I.rp + 63) >> 6;
-          for (int t = 0; t < I.n_tiles && ok; ++t, ++j) {
-            const int acc = j & 1;
-            const uint32_t acc_phase = (uint32_t)(j >> 1) & 1u;
-            if (!mbar_wait(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
-            const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
-            uint32_t accumulate = 0;
-            for (int si = 0; si < n_sets && ok; ++si) {
-              const uint32_t idesc = si ? idesc_neg : idesc_pos;      // the refitted set enters negated
-              for (int jb = 0; jb < nbh; ++jb) {
-                if (!mbar_wait(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t st = r_base + (uint32_t)rs * (4u * kBoxBytes);
-                const uint32_t ahi = desc_lo(st, 16), alo = desc_lo(st + kBoxBytes, 16);
-                const uint32_t bhi = desc_lo(st + 2 * kBoxBytes, 16), blo = desc_lo(st + 3 * kBoxBytes, 16);
+    // ------------------------------------------------------------------ MMA issuer (all lanes run, one issues)
+    const bool leader = elect_one();
+    uint32_t item_phase = 0, rphase = 0;
+    int rs = 0;
+    int j = 0;   // running tile count of this CTA
+    bool ok = true;
+    const uint32_t l_base = smem_u32(smem_l), r_base = smem_u32(smem_r);
+    const uint32_t dhi = desc_hi();
+    const uint32_t idesc_pos = make_idesc(kApplyNT, false, false, false);
+    const uint32_t idesc_neg = make_idesc(kApplyNT, false, false, true);
+    for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
+      const int n_tiles = a.items[it].n_tiles;
+      const int ks = a.items[it].rp >> 4;     // 16-wide K steps per part (hi or lo of one set)
+      if (kStream) {
+        const int nbh = (ks + 3) >> 2;
+        for (int t = 0; t < n_tiles && ok; ++t, ++j) {
+          const int acc = j % kApplyAcc;
+          const uint32_t acc_phase = (uint32_t)(j / kApplyAcc) & 1u;
+          if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
+          for (int si = 0; si < n_sets && ok; ++si) {
+            const uint32_t idesc = si ? idesc_neg : idesc_pos;      // the refitted set enters negated
+            for (int jb = 0; jb < nbh; ++jb) {
+              if (!mbar_wait_warp(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
+              tc_fence_after();
+              const uint32_t st = r_base + (uint32_t)rs * (4u * kBoxBytes);
+              const uint32_t ahi = desc_lo(st, 16), alo = desc_lo(st + kBoxBytes, 16);
+              const uint32_t bhi = desc_lo(st + 2 * kBoxBytes, 16), blo = desc_lo(st + 3 * kBoxBytes, 16);
+              if (leader) {
+#pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
-                  if (4 * jb + kk >= ks) break;
-                  const uint32_t o = (uint32_t)(kk * 2);
-                  mma_bf16(d, desc_join(ahi + o, dhi), desc_join(bhi + o, dhi), idesc, accumulate);
-                  mma_bf16(d, desc_join(alo + o, dhi), desc_join(bhi + o, dhi), idesc, 1u);
-                  mma_bf16(d, desc_join(ahi + o, dhi), desc_join(blo + o, dhi), idesc, 1u);
-                  accumulate = 1;
+                  if (4 * jb + kk < ks) {
+                    const uint32_t o = (uint32_t)(kk * 2);
+                    mma_bf16(d, desc_join(ahi + o, dhi), desc_join(bhi + o, dhi), idesc, (si | jb | kk) != 0);
+                    mma_bf16(d, desc_join(alo + o, dhi), desc_join(bhi + o, dhi), idesc, 1u);
+                    mma_bf16(d, desc_join(ahi + o, dhi), desc_join(blo + o, dhi), idesc, 1u);
+                  }
                 }
                 mma_commit(&sh.rempty[rs]);
-                if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
               }
+              __syncwarp();
+              if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
             }
-            if (ok) mma_commit(&sh.tfull[acc]);
           }
-          continue;
+          if (ok && leader) mma_commit(&sh.tfull[acc]);
+          __syncwarp();
         }
-        if (!mbar_wait(&sh.lfull, item_phase, abort, a.status, ST_WAIT_FULL)) break;
-        for (int t = 0; t < I.n_tiles && ok; ++t, ++j) {
-          const int acc = j & 1;
-          const uint32_t acc_phase = (uint32_t)(j >> 1) & 1u;
-          if (!mbar_wait(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
-          const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
-          uint32_t accumulate = 0;
-          // K step k of the [.., 4rp] operands: box k / 4 (16 KB apart), 32 bytes per step inside it
-          auto kstep = [](int k) { return (uint32_t)((k >> 2) * (kBoxBytes >> 4) + (k & 3) * 2); };
-          for (int bc = 0; bc < nb; ++bc) {
-            if (!mbar_wait(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t rb = desc_lo(r_base + (uint32_t)rs * kBoxBytes, 16);
+        continue;
+      }
+      const int nb = n_sets == 2 ? a.items[it].nbc2 : a.items[it].nbc1;
+      if (!mbar_wait_warp(&sh.lfull, item_phase, abort, a.status, ST_WAIT_FULL)) break;
+      for (int t = 0; t < n_tiles && ok; ++t, ++j) {
+        const int acc = j % kApplyAcc;
+        const uint32_t acc_phase = (uint32_t)(j / kApplyAcc) & 1u;
+        if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
+        const uint32_t la = desc_lo(l_base, 16);
+        // K step k of the [.., 4rp] operands: box k / 4 (16 KB apart), 32 bytes per step inside it
+        auto kstep = [](int k) { return (uint32_t)((k >> 2) * (kBoxBytes >> 4) + (k & 3) * 2); };
+        for (int bc = 0; bc < nb; ++bc) {
+          if (!mbar_wait_warp(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t rb = desc_lo(r_base + (uint32_t)rs * kBoxBytes, 16);
+          if (leader) {
+#pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               const int kb = 4 * bc + kk;              // K step of [R0 hi | R0 lo | R hi | R lo] held by this box
-              if (kb >= ktot) break;
-              const int set = kb >= 2 * ks ? 1 : 0;
-              const int w = kb - set * 2 * ks;         // K step inside the set: hi part, then lo part
-              // the set that holds the refitted factors enters with a negated A operand
-              const uint32_t idesc = (n_sets == 2 && (set ^ a.parity)) ? idesc_neg : idesc_pos;
-              const uint64_t b = desc_join(rb + (uint32_t)(kk * 2), dhi);
-              if (w < ks) {                            // hi * hi, lo * hi
-                mma_bf16(d, desc_join(la + kstep(kb), dhi), b, idesc, accumulate);
-                mma_bf16(d, desc_join(la + kstep(kb + ks), dhi), b, idesc, 1u);
-              } else {                                 // hi * lo
-                mma_bf16(d, desc_join(la + kstep(kb - ks), dhi), b, idesc, accumulate);
+              if (kb < n_sets * 2 * ks) {
+                const int set = kb >= 2 * ks ? 1 : 0;
+                const int w = kb - set * 2 * ks;       // K step inside the set: hi part, then lo part
+                // the set that holds the refitted factors enters with a negated A operand
+                const uint32_t idesc = (n_sets == 2 && (set ^ a.parity)) ? idesc_neg : idesc_pos;
+                const uint64_t b = desc_join(rb + (uint32_t)(kk * 2), dhi);
+                // hi * hi and lo * hi, or hi * lo
+                mma_bf16(d, desc_join(la + kstep(w < ks ? kb : kb - ks), dhi), b, idesc, kb != 0);
+                if (w < ks) mma_bf16(d, desc_join(la + kstep(kb + ks), dhi), b, idesc, 1u);
               }
-              accumulate = 1;
             }
             mma_commit(&sh.rempty[rs]);
-            if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
           }
-          if (ok) mma_commit(&sh.tfull[acc]);
+          __syncwarp();
+          if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
         }
-        if (ok) mma_commit(&sh.lempty);
-        item_phase ^= 1u;
+        if (ok && leader) mma_commit(&sh.tfull[acc]);
+        __syncwarp();
       }
+      if (ok && leader) mma_commit(&sh.lempty);
+      __syncwarp();
+      item_phase ^= 1u;
     }
   } else if (warp == 10) {
     // ------------------------------------------------------------------ g / W mover
@@ -362,12 +378,12 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
       const int n_q = 4 * I.n_tiles;
       for (int q = 0; q < n_q; ++q, ++k) {
         const int jt = j + (q >> 2), sub = q & 3;
-        const int acc = jt & 1;
+        const int acc = jt % kApplyAcc;
         const int b = k % a.n_bufs;
         if (sub == 0) {
           // one lane per warp polls, then the warp agrees: the tensor-memory loads need all 32 lanes
           bool got = true;
-          if (lane == 0) got = mbar_wait(&sh.tfull[acc], (uint32_t)(jt >> 1) & 1u, abort, a.status, ST_WAIT_TMEM_FULL);
+          if (lane == 0) got = mbar_wait(&sh.tfull[acc], (uint32_t)(jt / kApplyAcc) & 1u, abort, a.status, ST_WAIT_TMEM_FULL);
           got = __shfl_sync(0xffffffffu, got, 0);
           if (!got) { ok = false; break; }
           tc_fence_after();
@@ -443,7 +459,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 256);
+    tmem_dealloc(tmem_base, kApplyAcc * kApplyNT);
   }
 }
 

@@ -69,6 +69,33 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// One lane of a fully active warp, always the same.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
+}
+
+// mbar_wait for a whole warp.  The issuing warps run their loops with all lanes and let one lane issue: what the loops
+// compute is then uniform across the warp for the compiler too, so that descriptors and addresses live in the uniform
+// registers that the MMA and TMA instructions read.  In code of a single lane every operand of every MMA is moved there
+// first, and those moves, not the MMAs, set the pace (measured on the refit engine, four panel launches of a step:
+// 858 -> 752 us at rank 8, 159 -> 140 us on the 60M shapes; on the apply kernel without its memory traffic, 1.5B
+// shapes: 2.1 -> 1.4 ms).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* status,
+                                               int32_t code, uint32_t limit = kSpinLimit) {
+  for (uint32_t it = 0; it < limit; ++it) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (it > 32) {
+      __nanosleep(it > 4096 ? 256 : 32);
+      if ((it & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0)) return false;
+    }
+  }
+  *abort = 1;
+  atomicOr(status, code);
+  return false;
+}
+
 // ---- 256-bit global accesses (32-byte aligned addresses) -------------------------------------------
 // Eight floats past the L1 (they are used once).
 __device__ __forceinline__ void ldcg_f32x8(const float* p, float* v) {

@@ -29,9 +29,9 @@
 // its MMAs, warps 4-7 add up g^2 per row from the gradient tiles of the first segment when the
 // launch asks for it (the second-moment statistic of the block-mean form then needs no pass of its
 // own over g), warps 8-15 drain the accumulators (two groups of four warps that take the 16-column
-// pieces of an item alternately); warps 2 and 3 have no work.  The two issuing threads run dependent
+// pieces of an item alternately); warps 2 and 3 have no work.  The two issuing warps run dependent
 // scalar code, so their per-stage instruction count is what bounds the rate; both loops are kept
-// short.  With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
+// short, and all lanes run them so that their operands stay in uniform registers (mbar_wait_warp).  With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
 // Every wait is bounded; when one runs out the CTA records a status bit, stops taking work and
 // leaves through the common exit (which frees its tensor memory).  A launch that finds the status
 // word set on entry does nothing.
@@ -145,17 +145,12 @@ __device__ __forceinline__ void load_stage(uint8_t* sa, int a_tile, int box_byte
 
 // The MMAs of one stage: nk K steps, NA operands, NM MMAs per operand and step.
 template <int NA, int NM, bool MN_MAJOR_A>
-__device__ __forceinline__ void mma_stage(uint32_t d_base, const Seg& S, uint32_t sa, int a_tile, uint32_t a_lbo,
-                                          uint32_t blo, uint32_t b2, uint32_t dhi, uint32_t idesc, int nk,
-                                          uint32_t& accumulate) {
-  uint32_t alo[NA], dcol[NA];
+__device__ __forceinline__ void mma_stage(const uint32_t* dcol, uint32_t d_part, uint32_t same, uint32_t sa, int a_tile,
+                                          uint32_t a_lbo, uint32_t blo, uint32_t b2, uint32_t dhi, uint32_t idesc, int nk,
+                                          uint32_t accumulate) {
+  uint32_t alo[NA];
 #pragma unroll
-  for (int p = 0; p < NA; ++p) {
-    alo[p] = desc_lo(sa + (uint32_t)(p * a_tile), a_lbo);
-    dcol[p] = d_base + (uint32_t)S.d_col[p];
-  }
-  const uint32_t d_part = (uint32_t)S.d_part;
-  const bool same = S.same_acc != 0;
+  for (int p = 0; p < NA; ++p) alo[p] = desc_lo(sa + (uint32_t)(p * a_tile), a_lbo);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     if (q < nk) {
@@ -164,11 +159,10 @@ __device__ __forceinline__ void mma_stage(uint32_t d_base, const Seg& S, uint32_
 #pragma unroll
       for (int p = 0; p < NA; ++p) {
         const uint64_t ad = desc_join(alo[p] + astep, dhi);
-        const uint32_t acc_p = (p > 0 && same) ? 1u : accumulate;
+        const uint32_t acc_p = q > 0 ? 1u : ((p > 0 && same) ? 1u : accumulate);
         mma_bf16(dcol[p], ad, bd, idesc, acc_p);
         if (NM == 2) mma_bf16(dcol[p] + d_part, ad, desc_join(blo + b2 + (uint32_t)(q * 128), dhi), idesc, acc_p);
       }
-      accumulate = 1u;
     }
   }
 }
@@ -205,133 +199,148 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
   const int ksteps = stage_k >> 4;                  // MMA K steps per full stage
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t issued = 0;
-      bool ok = true;
-      for (int it = it_begin; it < it_end && ok; ++it) {
-        const Item& I = a.items[it];
-        if (I.wait_count > 0) {
-          // Bounded like every wait here: a team member that never arrives ends this CTA with a status, not a
-          // hang.  The bound is generous (about a second), because a member may start late when other work
-          // holds SMs; the consumers' own bounds are longer still, so this is the wait that reports.
-          volatile int32_t* cnt = a.team_counters + I.team;
-          uint32_t spin = 0;
-          while (*cnt < I.wait_count) {
-            if (++spin >= a.team_spin_limit || ((spin & 255u) == 0 && *abort)) { ok = false; break; }
-            __nanosleep(256);
-          }
-          if (!ok) {
-            *abort = 1;
-            atomicOr(a.status, ST_WAIT_TEAM);
-            break;
-          }
+    // ------------------------------------------------------------------ producer (all lanes run, one issues)
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t issued = 0;
+    bool ok = true;
+    for (int it = it_begin; it < it_end && ok; ++it) {
+      const Item& I = a.items[it];
+      const int wait_count = I.wait_count, signal = I.signal, n_seg = I.n_seg;
+      int32_t* const team = a.team_counters + I.team;
+      if (wait_count > 0) {
+        // Bounded like every wait here: a team member that never arrives ends this CTA with a status, not a
+        // hang.  The bound is generous (about a second), because a member may start late when other work
+        // holds SMs; the consumers' own bounds are longer still, so this is the wait that reports.
+        volatile int32_t* cnt = team;
+        uint32_t spin = 0;
+        while (__any_sync(0xffffffffu, *cnt < wait_count)) {
+          if (++spin >= a.team_spin_limit || ((spin & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0))) { ok = false; break; }
+          __nanosleep(256);
         }
-        for (int s = 0; s < I.n_seg && ok; ++s) {
-          const Seg S = I.seg[s];
-          const CUtensorMap* ma = a.maps + S.map_a;
-          const CUtensorMap* mb = a.maps + S.map_b;
-          const int nst = (S.k + stage_k - 1) / stage_k;
-          int x[kMaxA], y[kMaxA];
+        if (!ok) {
+          *abort = 1;
+          if (leader) atomicOr(a.status, ST_WAIT_TEAM);
+          break;
+        }
+      }
+      for (int s = 0; s < n_seg && ok; ++s) {
+        const Seg& S = I.seg[s];
+        const CUtensorMap* ma = a.maps + S.map_a;
+        const CUtensorMap* mb = a.maps + S.map_b;
+        const int nst = (S.k + stage_k - 1) / stage_k, a_mode = S.a_mode, n_a = S.n_a;
+        const uint32_t tx_bytes = S.tx_bytes;
+        int x[kMaxA], y[kMaxA];
 #pragma unroll
-          for (int p = 0; p < kMaxA; ++p) { x[p] = S.ax[p]; y[p] = S.ay[p]; }
-          int yb = 0;
-          const int dx = S.a_mode ? 0 : stage_k, dy = S.a_mode ? stage_k : 0;
-          // K along x: stage_k / 64 boxes of 64 x 128, 16 KB apart; K along y: two boxes of 64 x stage_k
-          const int n_box = S.a_mode ? 2 : (stage_k >> 6);
-          const int box_bytes = S.a_mode ? stage_k * 128 : kBoxBytes;
-          for (int c = 0; c < nst; ++c) {
-            if (!mbar_wait(&sh.empty[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
-            uint8_t* sa = stages + stage * a.stage_bytes;
-            uint64_t* bar = &sh.full[stage];
-            mbar_arrive_expect_tx(bar, S.tx_bytes);
+        for (int p = 0; p < kMaxA; ++p) { x[p] = S.ax[p]; y[p] = S.ay[p]; }
+        int yb = 0;
+        const int dx = a_mode ? 0 : stage_k, dy = a_mode ? stage_k : 0;
+        // K along x: stage_k / 64 boxes of 64 x 128, 16 KB apart; K along y: two boxes of 64 x stage_k
+        const int n_box = a_mode ? 2 : (stage_k >> 6);
+        const int box_bytes = a_mode ? stage_k * 128 : kBoxBytes;
+        for (int c = 0; c < nst; ++c) {
+          if (!mbar_wait_warp(&sh.empty[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
+          uint8_t* sa = stages + stage * a.stage_bytes;
+          uint64_t* bar = &sh.full[stage];
+          if (leader) {
+            mbar_arrive_expect_tx(bar, tx_bytes);
             if (n_box == 2) {
-              if (S.n_a == 2) load_stage<2, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else if (S.n_a == 3) load_stage<3, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+              if (n_a == 2) load_stage<2, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+              else if (n_a == 3) load_stage<3, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
               else load_stage<1, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
             } else {
-              if (S.n_a == 2) load_stage<2, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else if (S.n_a == 3) load_stage<3, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+              if (n_a == 2) load_stage<2, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+              else if (n_a == 3) load_stage<3, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
               else load_stage<1, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
             }
-#pragma unroll
-            for (int p = 0; p < kMaxA; ++p) { x[p] += dx; y[p] += dy; }
-            yb += stage_k;
-            ++issued;
-            if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
           }
+          __syncwarp();
+#pragma unroll
+          for (int p = 0; p < kMaxA; ++p) { x[p] += dx; y[p] += dy; }
+          yb += stage_k;
+          ++issued;
+          if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
         }
-        if (ok && I.signal) atomicAdd(a.team_counters + I.team, (int)I.signal);
       }
-      if (!ok) {
-        // leave no copy in flight: every stage that was filled must have landed before the CTA exits
-        const int back = issued < (uint32_t)a.n_stages ? (int)issued : a.n_stages;
-        for (int q = 0; q < back; ++q) {
-          int st = stage - 1 - q;
-          uint32_t ph = phase;
-          if (st < 0) { st += a.n_stages; ph ^= 1u; }
-          for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.full[st], ph); ++spin) __nanosleep(64);
-        }
+      if (ok && signal && leader) atomicAdd(team, signal);
+    }
+    if (!ok) {
+      // leave no copy in flight: every stage that was filled must have landed before the CTA exits
+      const int back = issued < (uint32_t)a.n_stages ? (int)issued : a.n_stages;
+      for (int q = 0; q < back; ++q) {
+        int st = stage - 1 - q;
+        uint32_t ph = phase;
+        if (st < 0) { st += a.n_stages; ph ^= 1u; }
+        for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.full[st], ph); ++spin) __nanosleep(64);
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int j = 0;
-      const uint32_t stages_u32 = smem_u32(stages);
-      const uint32_t dhi = desc_hi();
-      const uint32_t b_lbo = (uint32_t)stage_k * 128u;      // bytes between the 64-column chunks of B
-      for (int it = it_begin; it < it_end && ok; ++it, ++j) {
-        const Item& I = a.items[it];
-        const int acc = j % a.n_acc;
-        const uint32_t acc_phase = (uint32_t)(j / a.n_acc) & 1u;
-        if (!mbar_wait(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY, wlim)) break;
-        tc_fence_after();
-        const uint32_t d_base = tmem_base + (uint32_t)(acc * a.acc_cols);
-        for (int s = 0; s < I.n_seg && ok; ++s) {
-          const Seg S = I.seg[s];
-          const uint32_t idesc = make_idesc(S.n, S.a_mode != 0, true, false);
-          const int nst = (S.k + stage_k - 1) / stage_k;
-          // per K step of 16, in 16-byte units: K along x walks 32 B inside a box and 16 KB to the
-          // next box; K along y walks 16 rows of 128 B
-          const uint32_t a_lbo = S.a_mode ? b_lbo : 16u;
-          const uint32_t b2 = ((uint32_t)S.b2_chunk * b_lbo) >> 4;
-          uint32_t accumulate = S.first ? 0u : 1u;
-          int k_left = S.k;
-          for (int c = 0; c < nst; ++c, k_left -= stage_k) {
-            if (!mbar_wait(&sh.full[stage], phase, abort, a.status, ST_WAIT_FULL, wlim)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t sa = stages_u32 + (uint32_t)(stage * a.stage_bytes);
-            const uint32_t blo = desc_lo(sa + (uint32_t)a.a_bytes, b_lbo);
-            const int nk = k_left >= stage_k ? ksteps : (k_left + 15) >> 4;
-            if (S.n_mma == 2) {
-              if (S.a_mode) {
-                if (S.n_a == 2) mma_stage<2, 2, true>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-                else mma_stage<1, 2, true>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+    // ------------------------------------------------------------------ MMA issuer (all lanes run, one issues)
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int j = 0;
+    const uint32_t stages_u32 = smem_u32(stages);
+    const uint32_t dhi = desc_hi();
+    const uint32_t b_lbo = (uint32_t)stage_k * 128u;      // bytes between the 64-column chunks of B
+    for (int it = it_begin; it < it_end && ok; ++it, ++j) {
+      const Item& I = a.items[it];
+      const int acc = j % a.n_acc;
+      const uint32_t acc_phase = (uint32_t)(j / a.n_acc) & 1u;
+      if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY, wlim)) break;
+      tc_fence_after();
+      const uint32_t d_base = tmem_base + (uint32_t)(acc * a.acc_cols);
+      const int n_seg = I.n_seg;
+      for (int s = 0; s < n_seg && ok; ++s) {
+        const Seg& S = I.seg[s];
+        const int k = S.k, n_a = S.n_a, n_mma = S.n_mma, a_mode = S.a_mode;
+        const uint32_t idesc = make_idesc(S.n, a_mode != 0, true, false);
+        const int nst = (k + stage_k - 1) / stage_k;
+        // per K step of 16, in 16-byte units: K along x walks 32 B inside a box and 16 KB to the
+        // next box; K along y walks 16 rows of 128 B
+        const uint32_t a_lbo = a_mode ? b_lbo : 16u;
+        const uint32_t b2 = ((uint32_t)S.b2_chunk * b_lbo) >> 4;
+        uint32_t accumulate = S.first ? 0u : 1u;
+        const uint32_t d_part = (uint32_t)S.d_part, same = (uint32_t)S.same_acc;
+        uint32_t dcol[kMaxA];
+#pragma unroll
+        for (int p = 0; p < kMaxA; ++p) dcol[p] = d_base + (uint32_t)S.d_col[p];
+        int k_left = k;
+        for (int c = 0; c < nst; ++c, k_left -= stage_k) {
+          if (!mbar_wait_warp(&sh.full[stage], phase, abort, a.status, ST_WAIT_FULL, wlim)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t sa = stages_u32 + (uint32_t)(stage * a.stage_bytes);
+          const uint32_t blo = desc_lo(sa + (uint32_t)a.a_bytes, b_lbo);
+          const int nk = k_left >= stage_k ? ksteps : (k_left + 15) >> 4;
+          if (leader) {
+            if (n_mma == 2) {
+              if (a_mode) {
+                if (n_a == 2) mma_stage<2, 2, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+                else mma_stage<1, 2, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
               } else {
-                if (S.n_a == 2) mma_stage<2, 2, false>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-                else mma_stage<1, 2, false>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+                if (n_a == 2) mma_stage<2, 2, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+                else mma_stage<1, 2, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
               }
-            } else if (S.a_mode) {
-              if (S.n_a == 2) mma_stage<2, 1, true>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else if (S.n_a == 3) mma_stage<3, 1, true>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else mma_stage<1, 1, true>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+            } else if (a_mode) {
+              if (n_a == 2) mma_stage<2, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+              else if (n_a == 3) mma_stage<3, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+              else mma_stage<1, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
             } else {
-              if (S.n_a == 2) mma_stage<2, 1, false>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else if (S.n_a == 3) mma_stage<3, 1, false>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else mma_stage<1, 1, false>(d_base, S, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+              if (n_a == 2) mma_stage<2, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+              else if (n_a == 3) mma_stage<3, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
+              else mma_stage<1, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
             }
             mma_commit(&sh.empty[stage]);
-            if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
           }
+          __syncwarp();
+          accumulate = 1u;
+          if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
         }
-        if (ok) mma_commit(&sh.tfull[acc]);
       }
+      if (ok && leader) mma_commit(&sh.tfull[acc]);
+      __syncwarp();
     }
   } else if (warp < 4) {
     // no work
