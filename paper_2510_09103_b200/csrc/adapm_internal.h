@@ -101,14 +101,47 @@ struct GemmProb {
 };
 
 // ---------------------------------------------------------------------------------------------
+// exact-fp32 refit (lowrank_fp32.cu)
+// ---------------------------------------------------------------------------------------------
+// One r x r matrix: out[c][k] = sum_x X[x][k] Y[x][c].  Units are (row tile, column tile, K chunk), chunks innermost.
+struct Fp32Gram {
+  int64_t x_off, y_off, ld;
+  int64_t part_off, out_off;      // workspace floats: partial products, the matrix
+  int32_t x_base, y_base;         // Base
+  int32_t r, K, k_chunk, splits;  // k_chunk: multiple of 16
+  int32_t along_k;                // 1: X and Y are stored [r, K], 0: [K, r]
+  int32_t tn;                     // tiles of 8 tn columns and 16 ceil(tn / 2) rows
+  int32_t tiles_n;
+  int32_t counter;                // first of the tiles' arrival counters
+  int32_t first_unit;             // prefix sum of units
+  int32_t pad_;
+};
+// out = cur - eta ( cur Ga - b1 prev Gb - (1 - b1) s Q ), Q = g Y, owner by owner (rows of L, columns of R).
+// gb_off < 0: prev is cur and Gb is Ga (the first pass of a step).
+struct Fp32Refit {
+  int64_t g_off, ldg;             // element offset and pitch of the gradient
+  int64_t y_off, cur_off, prev_off, out_off;
+  int64_t save_off;               // workspace floats: where the current factors are copied to, or -1
+  int64_t ga_off, gb_off, part_off;   // workspace floats
+  int32_t y_base, cur_base, prev_base, out_base;
+  int32_t owners, r, K, k_chunk, splits;
+  int32_t along_k;                // 1: rows of L (g and Y with K contiguous, L [owners, r]); 0: columns of R
+  int32_t tn, tiles_n;            // tiles of 128 owners x 8 tn
+  int32_t counter, first_unit;
+  float eta, b1;
+};
+
+// ---------------------------------------------------------------------------------------------
 // low-rank apply: m^c = cg g + c0 L0 R0 - c1 L R, then line 9 of Algorithm 1
 // ---------------------------------------------------------------------------------------------
+constexpr int kApplyTile = 64;
+
 struct ApplyBlk {
   int64_t off;                    // params / grads element offset
-  int64_t l0_off, r0_off;         // previous factors (state), floats
+  int64_t l0_off, r0_off;         // previous factors, floats
   int64_t l1_off, r1_off;         // refitted factors, floats
   int64_t v_off;                  // state
-  int32_t l1_base, pad0_;         // where the refitted factors live (state when K_eff == 0, else workspace)
+  int32_t l0_base, r0_base, l1_base, r1_base;   // where they live (state or workspace)
   int32_t rows, cols, rank;
   int32_t v_mode;                 // ADAPM_V_ELEMENT | ADAPM_V_BLOCKMEAN (group scalars already updated)
   int32_t v_group_rows;           // rows per group (>= 1)
@@ -143,6 +176,8 @@ enum LaunchKind : int32_t {
   LK_GRADNORM,          // global gradient norm and the clip factor
   LK_TC_COPY,           // previous split copy of L -> final set (steps that hold L)
   LK_SPD_INVERSE,       // damped inverses of the r x r Gram matrices (preconditioned passes)
+  LK_FP32_GRAM,         // the r x r matrices of an exact-fp32 refit pass
+  LK_FP32_REFIT,        // its products with the gradient and the factor update
   LK_TC_CONVERT_WORK    // split copy of fp32 arrays that live in the workspace (the transformed factors)
 };
 // when a launch of the program runs
@@ -178,8 +213,13 @@ int launch_gradnorm(const NormRange* d_tab, const int32_t* d_cta_range, int64_t 
                     float* partials, float max_norm, int check_finite, float* gscale, int32_t* status, cudaStream_t s);
 int launch_gemm(const GemmProb* d_tab, int64_t n_prob, int64_t n_tiles, const Bases& b, int grad_dtype,
                 cudaStream_t s);
-int launch_apply_simt(const ApplyBlk* d_tab, int64_t n_blk, int64_t n_tiles, const Bases& b, const StepScalars& sc,
-                      int grad_dtype, cudaStream_t s);
+// `counters`: arrival counters of the tiles that are cut along K, zero between launches
+int launch_fp32_gram(const Fp32Gram* d_tab, const int32_t* d_unit_job, int64_t n_units, const Bases& b, int32_t* counters,
+                     cudaStream_t s);
+int launch_fp32_refit(const Fp32Refit* d_tab, const int32_t* d_unit_job, int64_t n_units, const Bases& b, int grad_dtype,
+                      int32_t* counters, cudaStream_t s);
+int launch_apply_simt(const ApplyBlk* d_tab, const int32_t* d_tile_blk, int64_t n_tiles, const Bases& b,
+                      const StepScalars& sc, int grad_dtype, cudaStream_t s);
 int launch_spd_inverse(const InverseJob* d_tab, int64_t n_jobs, float* work, float damping, const int32_t* status,
                        cudaStream_t s);
 int launch_copy_ranges(const NormRange* d_tab, const int32_t* d_cta_range, int64_t n_ctas, float* dst, const float* src,
@@ -208,7 +248,7 @@ struct adapm_ctx {
 
   // workspace layout (floats)
   int64_t work_floats = 0;
-  int64_t ws_lr[2] = {0, 0};           // two copies of the L,R section (ping-pong iterates)
+  int64_t ws_lr[3] = {0, 0, 0};        // copies of the L,R section: two ping-pong iterates, the step's previous factors
   void* workspace = nullptr;
   size_t workspace_bytes = 0;
 
@@ -235,6 +275,8 @@ struct adapm_ctx {
   float* d_gscale = nullptr;           // device scalars {s, s^2}: the step's clip factor (global norm clipping), or null
   void* shadow = nullptr;              // caller's bf16 copy of the parameters (adapm_set_shadow_params), or null
   int use_gscale = 0;                  // the program starts with the gradient-norm pass
+  int32_t* d_counters = nullptr;       // n_counters zeros: arrivals at the K-split tiles of the exact-fp32 refit
+  int64_t n_counters = 0;
   unsigned char* d_probe = nullptr;    // item table of the expired-wait probe
 
   size_t step_bytes = 0;

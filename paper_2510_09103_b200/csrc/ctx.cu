@@ -70,6 +70,304 @@ int validate(const adapm_block* blocks, int64_t n, const adapm_hparams& hp) {
   return ADAPM_OK;
 }
 
+
+// The apply launch of the CUDA-core blocks; previous L and R and the refitted pair at the given bases (floats).
+void add_simt_apply(adapm_ctx* c, const std::vector<int64_t>& ids, int phase, int l0_base, int64_t l0_shift, int r0_base,
+                    int64_t r0_shift, int l1_base, int64_t l1_shift, int r1_base, int64_t r1_shift) {
+  std::vector<ApplyBlk> ab;
+  std::vector<int32_t> tile_blk;
+  for (int64_t i : ids) {
+    const adapm_block& b = c->blocks[i];
+    ApplyBlk a;
+    std::memset(&a, 0, sizeof(a));
+    a.off = b.offset;
+    a.l0_base = l0_base; a.l0_off = l0_shift + c->l_off[i];
+    a.r0_base = r0_base; a.r0_off = r0_shift + c->r_off[i];
+    a.l1_base = l1_base; a.l1_off = l1_shift + c->l_off[i];
+    a.r1_base = r1_base; a.r1_off = r1_shift + c->r_off[i];
+    a.v_off = c->v_off[i]; a.rows = b.rows; a.cols = b.cols; a.rank = b.rank; a.v_mode = b.v_mode;
+    a.v_group_rows = b.v_group_rows == 0 ? b.rows : b.v_group_rows;
+    a.lr_scale = b.lr_scale; a.wd = b.weight_decay;
+    a.tiles_n = (b.cols + kApplyTile - 1) / kApplyTile; a.first_tile = (int64_t)tile_blk.size();
+    tile_blk.insert(tile_blk.end(), (size_t)((b.rows + kApplyTile - 1) / kApplyTile) * a.tiles_n, (int32_t)ab.size());
+    ab.push_back(a);
+  }
+  Launch L{LK_APPLY_SIMT, append_table(c->h_tables, ab), (int64_t)ab.size(), (int64_t)tile_blk.size()};
+  L.aux0 = append_table(c->h_tables, tile_blk);
+  L.phase = phase;
+  c->program.push_back(L);
+}
+
+// The refitted factors go back to the state, sub-buffer by sub-buffer (the padding between them is not touched).
+void add_commit(adapm_ctx* c, const std::vector<int64_t>& ids, int phase) {
+  std::vector<NormRange> ranges;
+  std::vector<int32_t> cta_range;
+  for (int64_t i : ids) {
+    const adapm_block& b = c->blocks[i];
+    for (int which = phase == 2 ? 1 : 0; which < 2; ++which) {      // (a step that holds L has only R to bring back)
+      NormRange r{which ? c->r_off[i] : c->l_off[i], (int64_t)b.rank * (which ? b.cols : b.rows), (int64_t)cta_range.size()};
+      for (int64_t q = 0; q < (r.numel + kNormChunk - 1) / kNormChunk; ++q) cta_range.push_back((int32_t)ranges.size());
+      ranges.push_back(r);
+    }
+  }
+  Launch CM{LK_COMMIT, append_table(c->h_tables, ranges), (int64_t)ranges.size(), (int64_t)cta_range.size()};
+  CM.aux0 = append_table(c->h_tables, cta_range);
+  CM.phase = phase;
+  c->program.push_back(CM);
+}
+
+// The preconditioned passes (scaled gradient descent) of the CUDA-core blocks, on the batched GEMM.
+// Workspace: two copies of the [L,R] section (ping-pong iterates), A/B with the same layout, Gram matrices and inverses.
+void build_precond_program(adapm_ctx* c, const std::vector<int64_t>& lowrank_ids, const std::vector<double>& etas,
+                           int64_t& work_cursor) {
+  const adapm_hparams* hp = &c->hp;
+  auto& prog = c->program;
+  const int n = (int)c->blocks.size(), K_eff = (int)etas.size();
+  const bool with_hold = hp->refresh_period > 1 && K_eff > 0;
+  {
+    c->ws_lr[0] = work_cursor; work_cursor += c->lr_section_floats;
+    c->ws_lr[1] = work_cursor; work_cursor += c->lr_section_floats;
+    const int64_t ws_ab = work_cursor; work_cursor += c->lr_section_floats;
+    std::vector<int64_t> gram_off(n, 0);
+    for (int64_t i : lowrank_ids) {
+      gram_off[i] = work_cursor;
+      work_cursor += round_up(6LL * c->blocks[i].rank * c->blocks[i].rank, kStateAlign);
+    }
+    const float b1 = hp->beta1, a1 = 1.f - hp->beta1;
+    int src_base = BASE_STATE; int64_t src_shift = 0;   // where the current iterate lives
+    int dst_buf = 0;
+    // with a refresh period the passes exist twice: refitting both factors (phase 1) and holding L (phase 2)
+    for (int phase = (with_hold ? 1 : 0); phase <= (with_hold ? 2 : 0); ++phase) {
+    const bool hold = phase == 2;
+    src_base = BASE_STATE; src_shift = 0; dst_buf = 0;
+    for (int it = 0; it < K_eff; ++it) {
+      const float se = (float)etas[it];
+      const int64_t dst_shift = c->ws_lr[dst_buf];
+      std::vector<GemmProb> pAB, pG, pU1, pU2, pU3;
+      std::vector<InverseJob> inv;
+      int64_t tAB = 0, tG = 0, tU1 = 0, tU2 = 0, tU3 = 0;
+      auto push = [](std::vector<GemmProb>& v, GemmProb p, int64_t& tiles) {
+        p.tiles_n = (p.N + 63) / 64;
+        p.first_tile = tiles;
+        tiles += (int64_t)((p.M + 63) / 64) * p.tiles_n;
+        v.push_back(p);
+      };
+      for (int64_t i : lowrank_ids) {
+        const adapm_block& b = c->blocks[i];
+        const int m = b.rows, nn = b.cols, r = b.rank;
+        const int64_t Lc = src_shift + c->l_off[i], Rc = src_shift + c->r_off[i];   // current iterate
+        const int64_t L0 = c->l_off[i], R0 = c->r_off[i];                             // previous factors (state)
+        const int64_t Ld = dst_shift + c->l_off[i], Rd = dst_shift + c->r_off[i];
+        const int64_t Aw = ws_ab + c->l_off[i], Bw = ws_ab + c->r_off[i];
+        const int64_t G1 = gram_off[i], G2 = G1 + (int64_t)r * r, G3 = G2 + (int64_t)r * r, G4 = G3 + (int64_t)r * r;
+        GemmProb p;
+        auto reset = [&]() {
+          std::memset(&p, 0, sizeof(p));
+          p.z1_base = p.z2_base = BASE_NONE;
+          p.alpha = 1.f;
+        };
+        // A = g R^T  (m x r), contraction over n
+        reset(); p.x_base = BASE_GRADS; p.x_off = b.offset; p.sxi = nn; p.sxk = 1;
+        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = 1; p.syj = nn;
+        p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = nn; p.ldc = r; if (!hold) push(pAB, p, tAB);
+        // B = L^T g  (r x n), contraction over m
+        reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = 1; p.sxk = r;
+        p.y_base = BASE_GRADS; p.y_off = b.offset; p.syk = nn; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = m; p.ldc = nn; push(pAB, p, tAB);
+        // G1 = R R^T, G2 = R0 R^T  (contraction over n)
+        reset(); p.x_base = (int8_t)src_base; p.x_off = Rc; p.sxi = nn; p.sxk = 1;
+        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = 1; p.syj = nn;
+        p.c_base = BASE_WORK; p.c_off = G1; p.M = r; p.N = r; p.K = nn; p.ldc = r; if (!hold) push(pG, p, tG);
+        p.x_base = BASE_STATE; p.x_off = R0; p.c_off = G2; if (!hold) push(pG, p, tG);
+        // G3 = L^T L, G4 = L^T L0  (contraction over m)
+        reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = 1; p.sxk = r;
+        p.y_base = (int8_t)src_base; p.y_off = Lc; p.syk = r; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = G3; p.M = r; p.N = r; p.K = m; p.ldc = r; push(pG, p, tG);
+        p.y_base = BASE_STATE; p.y_off = L0; p.c_off = G4; push(pG, p, tG);
+        // Preconditioned pass: A <- L G1 - a1 A, A <- A - b1 L0 G2 (= dl/dL), L' = L - se A S1 with
+        // S1 = (G1 + d I)^-1; B <- G3 R - a1 B, B <- B - b1 G4 R0 (= dl/dR), R' = R - se S3 B, S3 = (G3 + d I)^-1.
+        const int64_t S1 = G4 + (int64_t)r * r, S3 = S1 + (int64_t)r * r;
+        if (!hold) inv.push_back({G1, S1, r, 0});
+        inv.push_back({G3, S3, r, 0});
+        if (!hold) {
+          reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = r; p.sxk = 1;
+          p.y_base = BASE_WORK; p.y_off = G1; p.syk = r; p.syj = 1;
+          p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = r; p.ldc = r;
+          p.z1_base = BASE_WORK; p.z1_off = Aw; p.c1 = -a1; push(pU1, p, tU1);
+          reset(); p.x_base = BASE_STATE; p.x_off = L0; p.sxi = r; p.sxk = 1;
+          p.y_base = BASE_WORK; p.y_off = G2; p.syk = r; p.syj = 1;
+          p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = r; p.ldc = r;
+          p.alpha = -b1; p.beta = 1.f; push(pU2, p, tU2);
+        }
+        reset(); p.x_base = BASE_WORK; p.x_off = Aw; p.sxi = r; p.sxk = 1;
+        p.y_base = BASE_WORK; p.y_off = S1; p.syk = r; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = Ld; p.M = m; p.N = r; p.K = r; p.ldc = r;
+        p.alpha = -se; p.z1_base = (int8_t)src_base; p.z1_off = Lc; p.c1 = 1.f;
+        if (hold) { p.K = 0; p.alpha = 0.f; }                                            // L' = L
+        push(pU3, p, tU3);
+        reset(); p.x_base = BASE_WORK; p.x_off = G3; p.sxi = r; p.sxk = 1;
+        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = nn; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
+        p.z1_base = BASE_WORK; p.z1_off = Bw; p.c1 = -a1; push(pU1, p, tU1);
+        reset(); p.x_base = BASE_WORK; p.x_off = G4; p.sxi = r; p.sxk = 1;
+        p.y_base = BASE_STATE; p.y_off = R0; p.syk = nn; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
+        p.alpha = -b1; p.beta = 1.f; push(pU2, p, tU2);
+        reset(); p.x_base = BASE_WORK; p.x_off = S3; p.sxi = r; p.sxk = 1;
+        p.y_base = BASE_WORK; p.y_off = Bw; p.syk = nn; p.syj = 1;
+        p.c_base = BASE_WORK; p.c_off = Rd; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
+        p.alpha = -se; p.z1_base = (int8_t)src_base; p.z1_off = Rc; p.c1 = 1.f; push(pU3, p, tU3);
+      }
+      for (auto* pv : {&pAB, &pG, &pU1, &pU2, &pU3}) {
+        if (pv == &pU1 && !inv.empty()) {       // the inverses need the Gram matrices and feed the last update
+          Launch IL{LK_SPD_INVERSE, append_table(c->h_tables, inv), (int64_t)inv.size(), (int64_t)inv.size()};
+          IL.phase = phase;
+          prog.push_back(IL);
+        }
+        if (pv->empty()) continue;
+        const int64_t tiles = pv == &pAB ? tAB : (pv == &pG ? tG : (pv == &pU1 ? tU1 : (pv == &pU2 ? tU2 : tU3)));
+        Launch GL{LK_GEMM, append_table(c->h_tables, *pv), (int64_t)pv->size(), tiles};
+        GL.phase = phase;
+        prog.push_back(GL);
+      }
+      src_base = BASE_WORK; src_shift = dst_shift;
+      c->final_lr_buf = dst_buf;
+      dst_buf ^= 1;
+    }
+    }
+    add_simt_apply(c, lowrank_ids, 0, BASE_STATE, 0, BASE_STATE, 0, src_base, src_shift, src_base, src_shift);
+    if (c->final_lr_buf >= 0) add_commit(c, lowrank_ids, 0);
+  }
+}
+
+// Algorithm 2 for the CUDA-core blocks: per pass one launch for the r x r matrices and one for the products with the
+// gradient and the factor update.  The iterates alternate between two workspace copies of the [L,R] section; the first
+// pass copies the step's previous factors to a third and the last pass writes the state, so that nothing is copied back.
+// (A step with a single pass ends in the workspace and is committed after the apply.)
+void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std::vector<double>& etas, int64_t& work_cursor) {
+  const adapm_hparams& hp = c->hp;
+  const int K_eff = (int)etas.size();
+  const bool with_hold = hp.refresh_period > 1 && K_eff > 0;
+  for (int64_t& w : c->ws_lr) { w = work_cursor; work_cursor += K_eff > 0 ? c->lr_section_floats : 0; }
+  const int64_t ws_prev = c->ws_lr[2];
+  const int64_t scratch = work_cursor;           // matrices and partial products, every pass anew
+  int64_t scratch_end = work_cursor;
+  // columns per thread of a rank's tiles (8 tn columns each): as few tiles of up to 40 columns as cover it, all of one width
+  auto tiles_of = [](int r) { return (r + 39) / 40; };
+  auto tn_of = [&](int r) { return ((r + tiles_of(r) - 1) / tiles_of(r) + 7) / 8; };
+  // K loops are cut so that a launch has about `waves` CTAs per SM and none is much longer than the rest; a chunk is
+  // never below 128, where its partial products would cost as much as its share of the gradient.
+  struct Cut { int32_t k_chunk, splits; };
+  auto cut = [](int K, int64_t chunk) {
+    const int64_t n = std::max<int64_t>(1, (K + chunk / 2) / chunk);
+    Cut q;
+    q.k_chunk = (int32_t)round_up((K + n - 1) / n, 16);
+    q.splits = (K + q.k_chunk - 1) / q.k_chunk;
+    return q;
+  };
+  constexpr int64_t kSms = 148, kWavesRefit = 9, kWavesGram = 4;
+
+  for (int phase = (with_hold ? 1 : 0); phase <= (with_hold ? 2 : 0); ++phase) {
+    const bool hold = phase == 2;
+    for (int it = 0; it < K_eff; ++it) {
+      const bool first = it == 0, last = it == K_eff - 1 && K_eff > 1;
+      const int cur_base = first ? BASE_STATE : BASE_WORK;
+      const int64_t cur = first ? 0 : c->ws_lr[(it - 1) & 1], prev = first ? 0 : ws_prev;
+      const int out_base = last ? BASE_STATE : BASE_WORK;
+      const int64_t out = last ? 0 : c->ws_lr[it & 1];
+      int64_t k_refit = 0, k_gram = 0;            // K summed over the tiles
+      for (int64_t i : ids) {
+        const adapm_block& b = c->blocks[i];
+        const int64_t tr = tiles_of(b.rank), tg = tr * tr * (first ? 1 : 2);
+        k_refit += tr * ((hold ? 0 : (int64_t)(b.rows + 127) / 128 * b.cols) + (int64_t)(b.cols + 127) / 128 * b.rows);
+        k_gram += tg * ((hold ? 0 : (int64_t)b.cols) + b.rows);
+      }
+      const int64_t chunk_refit = std::max<int64_t>(128, k_refit / (kSms * kWavesRefit));
+      const int64_t chunk_gram = std::max<int64_t>(128, k_gram / (kSms * kWavesGram));
+      std::vector<Fp32Gram> grams;
+      std::vector<Fp32Refit> refits;
+      int64_t at = scratch, counters = 0;
+      for (int64_t i : ids) {
+        const adapm_block& b = c->blocks[i];
+        const int m = b.rows, n = b.cols, r = b.rank;
+        for (int side = hold ? 1 : 0; side < 2; ++side) {          // 0: L, by rows; 1: R, by columns
+          // the side's factor F (owners x r) and the other one Y (K x r): Q = g Y, Ga = Y^T Y, Gb = Y0^T Y
+          const int64_t f_off = side ? c->r_off[i] : c->l_off[i], y_off = side ? c->l_off[i] : c->r_off[i];
+          const int owners = side ? n : m, K = side ? m : n, along_k = side ? 0 : 1;
+          // a held L stays where it is, in the state
+          const int y_base = hold ? BASE_STATE : cur_base;
+          const int64_t yc = (hold ? 0 : cur) + y_off, yp = (hold ? 0 : prev) + y_off;
+          auto gram = [&](int64_t x_off) {
+            Fp32Gram g;
+            std::memset(&g, 0, sizeof(g));
+            g.x_base = g.y_base = y_base; g.x_off = x_off; g.y_off = yc; g.ld = side ? r : n;
+            g.r = r; g.K = K; g.along_k = along_k;
+            const Cut q = cut(K, chunk_gram);
+            g.k_chunk = q.k_chunk; g.splits = q.splits;
+            g.tn = tn_of(r); g.tiles_n = tiles_of(r);
+            const int tile_rows = 16 * ((g.tn + 1) / 2), tiles = g.tiles_n * ((r + tile_rows - 1) / tile_rows);
+            g.out_off = at; at += round_up((int64_t)r * r, kStateAlign);
+            g.part_off = at; if (q.splits > 1) at += (int64_t)tiles * q.splits * tile_rows * 8 * g.tn;
+            at = round_up(at, kStateAlign);
+            g.counter = (int32_t)counters; counters += tiles;
+            grams.push_back(g);
+            return g.out_off;
+          };
+          Fp32Refit u;
+          std::memset(&u, 0, sizeof(u));
+          u.g_off = b.offset; u.ldg = n; u.y_base = y_base; u.y_off = yc;
+          u.cur_base = u.prev_base = cur_base; u.cur_off = cur + f_off; u.prev_off = prev + f_off;
+          u.out_base = out_base; u.out_off = out + f_off;
+          u.save_off = first && K_eff > 1 ? ws_prev + f_off : -1;
+          u.owners = owners; u.r = r; u.K = K; u.along_k = along_k; u.eta = (float)etas[it]; u.b1 = hp.beta1;
+          u.tn = tn_of(r); u.tiles_n = tiles_of(r);
+          u.ga_off = gram(yc);
+          u.gb_off = first ? -1 : (hold ? u.ga_off : gram(yp));
+          if (!first && !hold) grams.back().x_base = prev == 0 ? BASE_STATE : BASE_WORK;
+          const Cut q = cut(K, chunk_refit);
+          u.k_chunk = q.k_chunk; u.splits = q.splits;
+          const int tiles = u.tiles_n * ((owners + 127) / 128);
+          u.part_off = at; if (q.splits > 1) at += (int64_t)tiles * q.splits * 128 * 8 * u.tn;
+          at = round_up(at, kStateAlign);
+          u.counter = (int32_t)counters; counters += tiles;
+          refits.push_back(u);
+        }
+      }
+      scratch_end = std::max(scratch_end, at);
+      c->n_counters = std::max(c->n_counters, counters);
+      // longest chunks first
+      std::stable_sort(grams.begin(), grams.end(), [](const Fp32Gram& a, const Fp32Gram& b) { return a.k_chunk > b.k_chunk; });
+      std::stable_sort(refits.begin(), refits.end(),
+                       [](const Fp32Refit& a, const Fp32Refit& b) { return a.k_chunk * a.tn > b.k_chunk * b.tn; });
+      std::vector<int32_t> unit_gram, unit_refit;
+      for (size_t q = 0; q < grams.size(); ++q) {
+        Fp32Gram& g = grams[q];
+        const int tile_rows = 16 * ((g.tn + 1) / 2);
+        g.first_unit = (int32_t)unit_gram.size();
+        unit_gram.insert(unit_gram.end(), (size_t)g.tiles_n * ((g.r + tile_rows - 1) / tile_rows) * g.splits, (int32_t)q);
+      }
+      for (size_t q = 0; q < refits.size(); ++q) {
+        Fp32Refit& u = refits[q];
+        u.first_unit = (int32_t)unit_refit.size();
+        unit_refit.insert(unit_refit.end(), (size_t)u.tiles_n * ((u.owners + 127) / 128) * u.splits, (int32_t)q);
+      }
+      Launch GL{LK_FP32_GRAM, append_table(c->h_tables, grams), (int64_t)grams.size(), (int64_t)unit_gram.size()};
+      GL.aux0 = append_table(c->h_tables, unit_gram); GL.phase = phase;
+      c->program.push_back(GL);
+      Launch UL{LK_FP32_REFIT, append_table(c->h_tables, refits), (int64_t)refits.size(), (int64_t)unit_refit.size()};
+      UL.aux0 = append_table(c->h_tables, unit_refit); UL.phase = phase;
+      c->program.push_back(UL);
+    }
+    // where the step's previous factors and the refitted ones are when the passes are over
+    const int old_base = K_eff > 1 ? BASE_WORK : BASE_STATE, new_base = K_eff == 1 ? BASE_WORK : BASE_STATE;
+    const int64_t old_at = K_eff > 1 ? ws_prev : 0, new_at = K_eff == 1 ? c->ws_lr[0] : 0;
+    add_simt_apply(c, ids, phase, hold ? BASE_STATE : old_base, hold ? 0 : old_at, old_base, old_at,
+                   hold ? BASE_STATE : new_base, hold ? 0 : new_at, new_base, new_at);
+    if (K_eff == 1) { c->final_lr_buf = 0; add_commit(c, ids, phase); }
+  }
+  work_cursor = scratch_end;
+}
+
 }  // namespace
 
 // the tensor-core program of the low-rank blocks; defined in lowrank_tc.cu
@@ -332,176 +630,8 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     }
   }
   if (!lowrank_ids.empty()) {
-    // workspace: two copies of the [L,R] section (ping-pong iterates), A/B with the same layout, Gram matrices
-    c->ws_lr[0] = work_cursor; work_cursor += c->lr_section_floats;
-    c->ws_lr[1] = work_cursor; work_cursor += c->lr_section_floats;
-    const int64_t ws_ab = work_cursor; work_cursor += c->lr_section_floats;
-    std::vector<int64_t> gram_off(n, 0);
-    for (int64_t i : lowrank_ids) {
-      gram_off[i] = work_cursor;
-      work_cursor += round_up((hp->inner_precond ? 6LL : 4LL) * c->blocks[i].rank * c->blocks[i].rank, kStateAlign);
-    }
-    const float b1 = hp->beta1, a1 = 1.f - hp->beta1;
-    int src_base = BASE_STATE; int64_t src_shift = 0;   // where the current iterate lives
-    int dst_buf = 0;
-    // with a refresh period the passes exist twice: refitting both factors (phase 1) and holding L (phase 2)
-    for (int phase = (with_hold ? 1 : 0); phase <= (with_hold ? 2 : 0); ++phase) {
-    const bool hold = phase == 2;
-    src_base = BASE_STATE; src_shift = 0; dst_buf = 0;
-    for (int it = 0; it < K_eff; ++it) {
-      const float se = (float)etas[it];
-      const int64_t dst_shift = c->ws_lr[dst_buf];
-      std::vector<GemmProb> pAB, pG, pU1, pU2, pU3;
-      std::vector<InverseJob> inv;
-      int64_t tAB = 0, tG = 0, tU1 = 0, tU2 = 0, tU3 = 0;
-      const bool precond = hp->inner_precond != 0;
-      auto push = [](std::vector<GemmProb>& v, GemmProb p, int64_t& tiles) {
-        p.tiles_n = (p.N + 63) / 64;
-        p.first_tile = tiles;
-        tiles += (int64_t)((p.M + 63) / 64) * p.tiles_n;
-        v.push_back(p);
-      };
-      for (int64_t i : lowrank_ids) {
-        const adapm_block& b = c->blocks[i];
-        const int m = b.rows, nn = b.cols, r = b.rank;
-        const int64_t Lc = src_shift + c->l_off[i], Rc = src_shift + c->r_off[i];   // current iterate
-        const int64_t L0 = c->l_off[i], R0 = c->r_off[i];                             // previous factors (state)
-        const int64_t Ld = dst_shift + c->l_off[i], Rd = dst_shift + c->r_off[i];
-        const int64_t Aw = ws_ab + c->l_off[i], Bw = ws_ab + c->r_off[i];
-        const int64_t G1 = gram_off[i], G2 = G1 + (int64_t)r * r, G3 = G2 + (int64_t)r * r, G4 = G3 + (int64_t)r * r;
-        GemmProb p;
-        auto reset = [&]() {
-          std::memset(&p, 0, sizeof(p));
-          p.z1_base = p.z2_base = BASE_NONE;
-          p.alpha = 1.f;
-        };
-        // A = g R^T  (m x r), contraction over n
-        reset(); p.x_base = BASE_GRADS; p.x_off = b.offset; p.sxi = nn; p.sxk = 1;
-        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = 1; p.syj = nn;
-        p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = nn; p.ldc = r; if (!hold) push(pAB, p, tAB);
-        // B = L^T g  (r x n), contraction over m
-        reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = 1; p.sxk = r;
-        p.y_base = BASE_GRADS; p.y_off = b.offset; p.syk = nn; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = m; p.ldc = nn; push(pAB, p, tAB);
-        // G1 = R R^T, G2 = R0 R^T  (contraction over n)
-        reset(); p.x_base = (int8_t)src_base; p.x_off = Rc; p.sxi = nn; p.sxk = 1;
-        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = 1; p.syj = nn;
-        p.c_base = BASE_WORK; p.c_off = G1; p.M = r; p.N = r; p.K = nn; p.ldc = r; if (!hold) push(pG, p, tG);
-        p.x_base = BASE_STATE; p.x_off = R0; p.c_off = G2; if (!hold) push(pG, p, tG);
-        // G3 = L^T L, G4 = L^T L0  (contraction over m)
-        reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = 1; p.sxk = r;
-        p.y_base = (int8_t)src_base; p.y_off = Lc; p.syk = r; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = G3; p.M = r; p.N = r; p.K = m; p.ldc = r; push(pG, p, tG);
-        p.y_base = BASE_STATE; p.y_off = L0; p.c_off = G4; push(pG, p, tG);
-        if (precond) {
-          // Preconditioned pass: A <- L G1 - a1 A, A <- A - b1 L0 G2 (= dl/dL), L' = L - se A S1 with
-          // S1 = (G1 + d I)^-1; B <- G3 R - a1 B, B <- B - b1 G4 R0 (= dl/dR), R' = R - se S3 B, S3 = (G3 + d I)^-1.
-          const int64_t S1 = G4 + (int64_t)r * r, S3 = S1 + (int64_t)r * r;
-          if (!hold) inv.push_back({G1, S1, r, 0});
-          inv.push_back({G3, S3, r, 0});
-          if (!hold) {
-            reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = r; p.sxk = 1;
-            p.y_base = BASE_WORK; p.y_off = G1; p.syk = r; p.syj = 1;
-            p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = r; p.ldc = r;
-            p.z1_base = BASE_WORK; p.z1_off = Aw; p.c1 = -a1; push(pU1, p, tU1);
-            reset(); p.x_base = BASE_STATE; p.x_off = L0; p.sxi = r; p.sxk = 1;
-            p.y_base = BASE_WORK; p.y_off = G2; p.syk = r; p.syj = 1;
-            p.c_base = BASE_WORK; p.c_off = Aw; p.M = m; p.N = r; p.K = r; p.ldc = r;
-            p.alpha = -b1; p.beta = 1.f; push(pU2, p, tU2);
-          }
-          reset(); p.x_base = BASE_WORK; p.x_off = Aw; p.sxi = r; p.sxk = 1;
-          p.y_base = BASE_WORK; p.y_off = S1; p.syk = r; p.syj = 1;
-          p.c_base = BASE_WORK; p.c_off = Ld; p.M = m; p.N = r; p.K = r; p.ldc = r;
-          p.alpha = -se; p.z1_base = (int8_t)src_base; p.z1_off = Lc; p.c1 = 1.f;
-          if (hold) { p.K = 0; p.alpha = 0.f; }                                            // L' = L
-          push(pU3, p, tU3);
-          reset(); p.x_base = BASE_WORK; p.x_off = G3; p.sxi = r; p.sxk = 1;
-          p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = nn; p.syj = 1;
-          p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
-          p.z1_base = BASE_WORK; p.z1_off = Bw; p.c1 = -a1; push(pU1, p, tU1);
-          reset(); p.x_base = BASE_WORK; p.x_off = G4; p.sxi = r; p.sxk = 1;
-          p.y_base = BASE_STATE; p.y_off = R0; p.syk = nn; p.syj = 1;
-          p.c_base = BASE_WORK; p.c_off = Bw; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
-          p.alpha = -b1; p.beta = 1.f; push(pU2, p, tU2);
-          reset(); p.x_base = BASE_WORK; p.x_off = S3; p.sxi = r; p.sxk = 1;
-          p.y_base = BASE_WORK; p.y_off = Bw; p.syk = nn; p.syj = 1;
-          p.c_base = BASE_WORK; p.c_off = Rd; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
-          p.alpha = -se; p.z1_base = (int8_t)src_base; p.z1_off = Rc; p.c1 = 1.f; push(pU3, p, tU3);
-          continue;
-        }
-        // L' = L - se ( L G1 - b1 L0 G2 - a1 A )
-        reset(); p.x_base = (int8_t)src_base; p.x_off = Lc; p.sxi = r; p.sxk = 1;
-        p.y_base = BASE_WORK; p.y_off = G1; p.syk = r; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = Ld; p.M = m; p.N = r; p.K = r; p.ldc = r;
-        p.alpha = -se; p.beta = 0.f; p.z1_base = (int8_t)src_base; p.z1_off = Lc; p.c1 = 1.f;
-        p.z2_base = BASE_WORK; p.z2_off = Aw; p.c2 = se * a1;
-        if (hold) { p.K = 0; p.alpha = 0.f; p.z2_base = BASE_NONE; p.c2 = 0.f; }      // L' = L
-        push(pU1, p, tU1);
-        reset(); p.x_base = BASE_STATE; p.x_off = L0; p.sxi = r; p.sxk = 1;
-        p.y_base = BASE_WORK; p.y_off = G2; p.syk = r; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = Ld; p.M = m; p.N = r; p.K = r; p.ldc = r;
-        p.alpha = se * b1; p.beta = 1.f; if (!hold) push(pU2, p, tU2);
-        // R' = R - se ( G3 R - b1 G4 R0 - a1 B )
-        reset(); p.x_base = BASE_WORK; p.x_off = G3; p.sxi = r; p.sxk = 1;
-        p.y_base = (int8_t)src_base; p.y_off = Rc; p.syk = nn; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = Rd; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
-        p.alpha = -se; p.beta = 0.f; p.z1_base = (int8_t)src_base; p.z1_off = Rc; p.c1 = 1.f;
-        p.z2_base = BASE_WORK; p.z2_off = Bw; p.c2 = se * a1; push(pU1, p, tU1);
-        reset(); p.x_base = BASE_WORK; p.x_off = G4; p.sxi = r; p.sxk = 1;
-        p.y_base = BASE_STATE; p.y_off = R0; p.syk = nn; p.syj = 1;
-        p.c_base = BASE_WORK; p.c_off = Rd; p.M = r; p.N = nn; p.K = r; p.ldc = nn;
-        p.alpha = se * b1; p.beta = 1.f; push(pU2, p, tU2);
-      }
-      for (auto* pv : {&pAB, &pG, &pU1, &pU2, &pU3}) {
-        if (pv == &pU1 && !inv.empty()) {       // the inverses need the Gram matrices and feed the last update
-          Launch IL{LK_SPD_INVERSE, append_table(c->h_tables, inv), (int64_t)inv.size(), (int64_t)inv.size()};
-          IL.phase = phase;
-          prog.push_back(IL);
-        }
-        if (pv->empty()) continue;
-        const int64_t tiles = pv == &pAB ? tAB : (pv == &pG ? tG : (pv == &pU1 ? tU1 : (pv == &pU2 ? tU2 : tU3)));
-        Launch GL{LK_GEMM, append_table(c->h_tables, *pv), (int64_t)pv->size(), tiles};
-        GL.phase = phase;
-        prog.push_back(GL);
-      }
-      src_base = BASE_WORK; src_shift = dst_shift;
-      c->final_lr_buf = dst_buf;
-      dst_buf ^= 1;
-    }
-    }
-    // apply
-    std::vector<ApplyBlk> ab;
-    int64_t tiles = 0;
-    for (int64_t i : lowrank_ids) {
-      const adapm_block& b = c->blocks[i];
-      ApplyBlk a;
-      std::memset(&a, 0, sizeof(a));
-      a.off = b.offset; a.l0_off = c->l_off[i]; a.r0_off = c->r_off[i];
-      a.l1_base = src_base; a.l1_off = src_shift + c->l_off[i]; a.r1_off = src_shift + c->r_off[i];
-      a.v_off = c->v_off[i]; a.rows = b.rows; a.cols = b.cols; a.rank = b.rank; a.v_mode = b.v_mode;
-      a.v_group_rows = b.v_group_rows == 0 ? b.rows : b.v_group_rows;
-      a.lr_scale = b.lr_scale; a.wd = b.weight_decay;
-      a.tiles_n = (b.cols + 63) / 64; a.first_tile = tiles;
-      tiles += (int64_t)((b.rows + 63) / 64) * a.tiles_n;
-      ab.push_back(a);
-    }
-    prog.push_back({LK_APPLY_SIMT, append_table(c->h_tables, ab), (int64_t)ab.size(), tiles});
-    if (c->final_lr_buf >= 0) {
-      // the refitted factors go back to the state, sub-buffer by sub-buffer (the padding between them is not touched)
-      std::vector<NormRange> ranges;
-      std::vector<int32_t> cta_range;
-      for (int64_t i : lowrank_ids) {
-        const adapm_block& b = c->blocks[i];
-        for (int which = 0; which < 2; ++which) {
-          NormRange r{which ? c->r_off[i] : c->l_off[i], (int64_t)b.rank * (which ? b.cols : b.rows), (int64_t)cta_range.size()};
-          for (int64_t q = 0; q < (r.numel + kNormChunk - 1) / kNormChunk; ++q) cta_range.push_back((int32_t)ranges.size());
-          ranges.push_back(r);
-        }
-      }
-      Launch CM{LK_COMMIT, append_table(c->h_tables, ranges), (int64_t)ranges.size(), (int64_t)cta_range.size()};
-      CM.aux0 = append_table(c->h_tables, cta_range);
-      prog.push_back(CM);
-    }
+    if (hp->inner_precond) build_precond_program(c, lowrank_ids, etas, work_cursor);
+    else build_fp32_program(c, lowrank_ids, etas, work_cursor);
   }
   c->work_floats = work_cursor;
 
@@ -516,6 +646,10 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     const float ones[2] = {1.f, 1.f};
     e = cudaMalloc((void**)&c->d_gscale, 256);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_gscale, ones, sizeof(ones), cudaMemcpyHostToDevice);
+  }
+  if (e == cudaSuccess && c->n_counters > 0) {
+    e = cudaMalloc((void**)&c->d_counters, (size_t)c->n_counters * 4);
+    if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, (size_t)c->n_counters * 4);
   }
   {
     std::vector<unsigned char> probe;
@@ -540,6 +674,7 @@ extern "C" void adapm_destroy(adapm_ctx* c) {
   if (c->d_status) cudaFree(c->d_status);
   if (c->d_probe) cudaFree(c->d_probe);
   if (c->d_gscale) cudaFree(c->d_gscale);
+  if (c->d_counters) cudaFree(c->d_counters);
   delete c;
 }
 
@@ -731,8 +866,15 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
         rc = launch_spd_inverse((const InverseJob*)tab, L.n_items, work, hp.precond_damping, c->d_status, s); break;
       case LK_GEMM:
         rc = launch_gemm((const GemmProb*)tab, L.n_items, L.grid, b, hp.grad_dtype, s); break;
+      case LK_FP32_GRAM:
+        rc = launch_fp32_gram((const Fp32Gram*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, b, c->d_counters, s); break;
+      case LK_FP32_REFIT:
+        rc = launch_fp32_refit((const Fp32Refit*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, b, hp.grad_dtype,
+                               c->d_counters, s);
+        break;
       case LK_APPLY_SIMT:
-        rc = launch_apply_simt((const ApplyBlk*)tab, L.n_items, L.grid, b, sc, hp.grad_dtype, s); break;
+        rc = launch_apply_simt((const ApplyBlk*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, b, sc, hp.grad_dtype, s);
+        break;
       case LK_COMMIT:
         rc = launch_copy_ranges((const NormRange*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, (float*)state,
                                 work + c->ws_lr[c->final_lr_buf], c->d_status, s);
@@ -789,6 +931,8 @@ extern "C" const char* adapm_launch_kind_name(int32_t kind) {
     case LK_TC_COPY: return "tc_copy";
     case LK_STREAM: return "stream_update";
     case LK_GEMM: return "gemm_simt";
+    case LK_FP32_GRAM: return "fp32_gram";
+    case LK_FP32_REFIT: return "fp32_refit";
     case LK_SPD_INVERSE: return "spd_inverse";
     case LK_APPLY_SIMT: return "apply_simt";
     case LK_COMMIT: return "commit_copy";

@@ -1,7 +1,7 @@
-// CUDA-core (FFMA) kernels of the low-rank path: a batched strided GEMM that carries every product
-// of Algorithm 2, the fused "apply" kernel that rebuilds m^c = cg g + c0 L0 R0 - c1 L R tile by tile
-// and writes the parameters, and the L_0 initialiser.  This path is exact fp32 and handles every
-// shape and gradient dtype; the tensor-core path replaces it where its layout rules are met.
+// CUDA-core (FFMA) kernels around the low-rank path: a batched strided GEMM (the preconditioned passes
+// and the data-driven start), the damped inverses of the Gram matrices, and the L_0 initialisers.
+// Exact fp32, every shape and gradient dtype.  The ordinary refit without tensor cores is in
+// lowrank_fp32.cu.
 #include "adapm_internal.h"
 #include "device_math.cuh"
 
@@ -124,66 +124,6 @@ __global__ void __launch_bounds__(256, 3) gemm_kernel(const GemmProb* __restrict
       if (Z1) x += P.c1 * Z1[o];
       if (Z2) x += P.c2 * Z2[o];
       C[o] = x;
-    }
-  }
-}
-
-template <bool BF16G>
-__global__ void __launch_bounds__(256) apply_simt_kernel(const ApplyBlk* __restrict__ tab, int n_blk, Bases b,
-                                                         StepScalars sc) {
-  __shared__ __align__(16) float Xs[TK][TM + 4];
-  __shared__ __align__(16) float Ys[TK][TN + 4];
-  __shared__ ApplyBlk sA;
-  __shared__ int skip;
-  if (threadIdx.x == 0) {
-    sA = find_by_first_tile(tab, n_blk, (int64_t)blockIdx.x);
-    skip = *b.status != 0;
-  }
-  __syncthreads();
-  if (skip) return;
-  const ApplyBlk& A = sA;
-  const float gs = b.gscale ? __ldg(b.gscale) : 1.f;
-  uint16_t* shadow = b.shadow ? b.shadow + A.off : nullptr;
-  const int64_t tile = (int64_t)blockIdx.x - A.first_tile;
-  const int i0 = (int)(tile / A.tiles_n) * TM, j0 = (int)(tile % A.tiles_n) * TN;
-  const int m = A.rows, n = A.cols, r = A.rank;
-
-  float* state = static_cast<float*>(b.p[BASE_STATE]);
-  const float* L0 = state + A.l0_off;
-  const float* R0 = state + A.r0_off;
-  const float* L1 = static_cast<const float*>(b.p[A.l1_base]) + A.l1_off;
-  const float* R1 = static_cast<const float*>(b.p[A.l1_base]) + A.r1_off;
-
-  float p0[4][4] = {}, p1[4][4] = {};
-  tile_mainloop<BF16G>(p0, L0, false, r, 1, R0, false, n, 1, m, n, r, i0, j0, Xs, Ys);   // P_{t-1} tile
-  tile_mainloop<BF16G>(p1, L1, false, r, 1, R1, false, n, 1, m, n, r, i0, j0, Xs, Ys);   // P_t tile
-
-  float* W = static_cast<float*>(b.p[BASE_PARAMS]) + A.off;
-  const void* G = static_cast<const char*>(b.p[BASE_GRADS]) + (size_t)A.off * (BF16G ? 2 : 4);
-  float* V = state + A.v_off;
-  const float lr_s = sc.lr * A.lr_scale;
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-#pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int i = i0 + ty * 4 + rr;
-    if (i >= m) continue;
-    float v_row = 0.f;
-    if (A.v_mode == ADAPM_V_BLOCKMEAN) v_row = V[i / A.v_group_rows];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int j = j0 + tx * 4 + c;
-      if (j >= n) continue;
-      const int64_t o = (int64_t)i * n + j;
-      const float g = gs * load_operand<BF16G>(G, true, o);
-      const float mc = sc.cg * g + sc.c0 * p0[rr][c] - sc.c1 * p1[rr][c];
-      float v = v_row;
-      if (A.v_mode == ADAPM_V_ELEMENT) {
-        v = sc.beta2 * V[o] + (1.f - sc.beta2) * (g * g);
-        V[o] = v;
-      }
-      const float w_new = adapm_param_update(W[o], mc, v, sc, lr_s, A.wd);
-      W[o] = w_new;
-      if (shadow) shadow[o] = (uint16_t)(pack_bf16x2(w_new, 0.f) & 0xffffu);
     }
   }
 }
@@ -325,17 +265,6 @@ int launch_gemm(const GemmProb* d_tab, int64_t n_prob, int64_t n_tiles, const Ba
     gemm_kernel<true><<<(unsigned)n_tiles, 256, 0, s>>>(d_tab, (int)n_prob, b);
   else
     gemm_kernel<false><<<(unsigned)n_tiles, 256, 0, s>>>(d_tab, (int)n_prob, b);
-  ADAPM_LAUNCH_CHECK();
-  return ADAPM_OK;
-}
-
-int launch_apply_simt(const ApplyBlk* d_tab, int64_t n_blk, int64_t n_tiles, const Bases& b, const StepScalars& sc,
-                      int grad_dtype, cudaStream_t s) {
-  if (n_tiles <= 0) return ADAPM_OK;
-  if (grad_dtype == ADAPM_GRAD_BF16)
-    apply_simt_kernel<true><<<(unsigned)n_tiles, 256, 0, s>>>(d_tab, (int)n_blk, b, sc);
-  else
-    apply_simt_kernel<false><<<(unsigned)n_tiles, 256, 0, s>>>(d_tab, (int)n_blk, b, sc);
   ADAPM_LAUNCH_CHECK();
   return ADAPM_OK;
 }

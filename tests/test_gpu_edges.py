@@ -34,3 +34,21 @@ def _follow(specs, dtype="bf16", steps=4, path=A.PATH_AUTO, **hp):
 def test_ranks_at_the_edges_of_the_apply_kernels_forms(rank):
     _follow([(264, 328, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 1), (300, 264, A.MOM_LOWRANK, rank, A.V_ELEMENT, 0)],
             path=A.PATH_TENSOR)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rank", [1, 8, 9, 24, 40, 41, 81, 300])
+def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
+    """Column tiles of every width, one to eight of them, K loops that are cut and that are not, aligned and
+    unaligned rows."""
+    big = rank > 64
+    _follow([(130, 1030 if not big else 330, A.MOM_LOWRANK, min(rank, 130), A.V_BLOCKMEAN, 1),
+             (400, 517 if not big else 380, A.MOM_LOWRANK, rank, A.V_ELEMENT, 0),
+             (304, 304, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 0)], dtype=dtype, path=A.PATH_SIMT)
+
+
+@pytest.mark.parametrize("iters,period", [(1, 0), (2, 0), (3, 0), (2, 3), (3, 3), (5, 3)])
+def test_exact_fp32_refit_by_number_of_passes(iters, period):
+    """K = 1 has no effective pass, K = 2 a single one that ends in the workspace, K = 3 two."""
+    _follow([(150, 77, A.MOM_LOWRANK, 12, A.V_BLOCKMEAN, 1), (64, 264, A.MOM_LOWRANK, 5, A.V_BLOCKMEAN, 0)], dtype="f32",
+            steps=5, inner_iters=iters, refresh_period=period)
