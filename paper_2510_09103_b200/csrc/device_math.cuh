@@ -87,4 +87,46 @@ __device__ __forceinline__ float adapm_param_update(float w, float mc, float v, 
   return w - lr_s * (ratio + wd * w);
 }
 
+// x limited to [-c, c]; a NaN stays NaN.
+__device__ __forceinline__ float clamp_keep_nan(float x, float c) {
+  float y;
+  asm("{\n.reg .f32 t;\nmin.NaN.f32 t, %1, %2;\nmax.NaN.f32 %0, t, %3;\n}" : "=f"(y) : "f"(x), "f"(c), "f"(-c));
+  return y;
+}
+
+// The update of N elements with a second moment of their own.  The square root and the quotient are taken from the
+// hardware's approximations with one step of Newton's iteration each (for the root: s += (v - s^2) y / 2, y ~ 1/sqrt(v);
+// for the quotient: q += (m - q d) r, r ~ 1/d), which leaves both within an ulp or so and
+// needs half the instructions of sqrtf and the division, and no branch per element.  What lies outside the range where
+// the iteration holds (zero and near-zero v, overflow) takes the functions themselves.
+template <int N>
+__device__ __forceinline__ void adapm_param_update_n(float* w, const float* mc, const float* v, const StepScalars& sc,
+                                                     float lr_s, float wd) {
+  float vs[N], lo = 1.f, hi = 1.f;
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    vs[e] = v[e] * sc.inv_bc2;
+    lo = fminf(lo, vs[e]);
+    hi = fmaxf(hi, vs[e]);
+  }
+  bool usual = lo >= 1e-30f && hi <= 1e30f && sc.eps <= 1e30f;
+#pragma unroll
+  for (int e = 0; e < N; ++e) usual = usual && fabsf(mc[e]) <= 1e30f && vs[e] == vs[e];      // (false for a NaN)
+  if (usual) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const float y = rsqrtf(vs[e]);
+      float s = vs[e] * y;
+      s = fmaf(fmaf(-s, s, vs[e]), 0.5f * y, s);
+      const float d = s + sc.eps, r = __fdividef(1.f, d), m = mc[e] * sc.inv_bc1;
+      float q = m * r;
+      q = fmaf(fmaf(-q, d, m), r, q);
+      w[e] = w[e] - lr_s * (clamp_keep_nan(q, sc.clip) + wd * w[e]);
+    }
+  } else {
+#pragma unroll 1
+    for (int e = 0; e < N; ++e) w[e] = adapm_param_update(w[e], mc[e], v[e], sc, lr_s, wd);
+  }
+}
+
 }  // namespace adapm

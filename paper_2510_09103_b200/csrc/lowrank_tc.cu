@@ -146,7 +146,7 @@ struct MapSet {                     // tensor maps for one combination of caller
 struct TcProgram {
   std::vector<TcBlock> blk;
   int64_t n_convert_owners = 0;
-  int smem_engine = 0, smem_apply = 0;
+  int smem_engine = 0;
   int nb_max = 1, stage_k = 128, rp_max = 16, half_max = 16;
   int64_t work_begin = 0, work_end = 0;   // the tensor path's part of the workspace, in floats
   // shared-memory plan of an engine launch whose segments have up to n_a A operands
@@ -159,8 +159,18 @@ struct TcProgram {
     e.smem = std::max(e.n_stages, 1) * e.stage_bytes + 1024;
     return e;
   }
-  int apply_r_region = 0, apply_r_stages = 3, apply_w_region = 0, apply_bufs = 2, apply_buf_bytes = 0;
-  int apply_s_w_region = 0, apply_s_bufs = 2, smem_apply_s = 0;   // the streaming form of the apply kernel
+  int apply_buf_bytes = 0;
+  // shared-memory plan of an apply launch
+  struct ApplyConfig { int n_rstages, w_region, n_bufs, smem; };
+  ApplyConfig apply_config(bool stream, bool tma) const {
+    ApplyConfig e;
+    e.n_rstages = stream ? 2 : 4;
+    e.w_region = e.n_rstages * (stream ? 4 : 1) * tc::kBoxBytes;
+    // (an even number: see the kernel's epilogue)
+    e.n_bufs = tma ? std::min(tc::kApplyMaxBufs, (226 * 1024 - e.w_region) / apply_buf_bytes) & ~1 : 0;
+    e.smem = e.w_region + (tma ? e.n_bufs * apply_buf_bytes : tc::kPatchesBytes) + 1024;
+    return e;
+  }
   int n_sms = 148;
   bool rotate = false;             // sets swap roles from step to step (there is at least one refit pass)
   int32_t* d_team_counters = nullptr;   // pacing counters of the panel launches (see schedule_panels)
@@ -201,6 +211,12 @@ void tensor_state_changed(adapm_ctx* c) {
 // program construction
 // ---------------------------------------------------------------------------------------------------
 namespace {
+
+using ApplyKernel = void (*)(tc::ApplyArgs);
+ApplyKernel apply_kernel(bool stream, bool tma) {
+  if (stream) return tma ? tc::tc_apply_kernel<true, true> : tc::tc_apply_kernel<true, false>;
+  return tma ? tc::tc_apply_kernel<false, true> : tc::tc_apply_kernel<false, false>;
+}
 
 int round16(int x) { return (x + 15) / 16 * 16; }
 int round64(int x) { return (x + 63) / 64 * 64; }
@@ -657,68 +673,51 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   // ---- apply ---------------------------------------------------------------------------------------------------
   // Blocks up to rank 128 keep the L panel of an item resident; above that L is streamed like R (second launch).
   {
-    std::vector<tc::ApplyItem> items, items_s;
-    int nbc_max = 1;
+    std::vector<tc::ApplyItem> lists[2][2];      // [L streamed][rows of the parameters start on 16 bytes]
     bool any_element_v = false;
+    int64_t all_tiles = 0;
+    for (const TcBlock& t : P->blk) {
+      const adapm_block& b = c->blocks[t.id];
+      all_tiles += (int64_t)((b.rows + 127) / 128) * ((b.cols + tc::kApplyNT - 1) / tc::kApplyNT);
+    }
+    // Column tiles per item: 16 where the set is large (the L panel is loaded once per item), fewer where that would
+    // leave CTAs without work.
+    const int run_len = (int)std::min<int64_t>(16, std::max<int64_t>(1, all_tiles / (4 * P->n_sms)));
     for (size_t bi = 0; bi < P->blk.size(); ++bi) {
       const TcBlock& t = P->blk[bi];
       const adapm_block& b = c->blocks[t.id];
       const int mb = (int)bi * kMapsPerBlock;
-      const bool stream = 2 * t.rp > 256;
-      const int nbc1 = (2 * t.rp + 63) / 64, nbc2 = (4 * t.rp + 63) / 64;
-      if (!stream) nbc_max = std::max(nbc_max, nbc2);
       if (b.v_mode == ADAPM_V_ELEMENT) any_element_v = true;
       const int tiles = (b.cols + tc::kApplyNT - 1) / tc::kApplyNT;
-      const int runs = (tiles + 15) / 16;
+      const int runs = (tiles + run_len - 1) / run_len;
       for (int p0 = 0; p0 < b.rows; p0 += 128) {
         for (int q = 0; q < runs; ++q) {
           tc::ApplyItem a;
           std::memset(&a, 0, sizeof(a));
           a.off = b.offset; a.v_off = c->v_off[t.id]; a.rows = b.rows; a.cols = b.cols; a.r = b.rank; a.rp = t.rp;
-          a.half = t.half;
+          a.half = t.half; a.l_off = t.lc[0];
           a.map_l = mb + MAP_LCAT; a.map_r = mb + MAP_RCAT;
           a.map_w = mb + MAP_W; a.map_g = mb + MAP_G32; a.map_v = mb + MAP_V; a.map_sh = mb + MAP_SH;
           a.row0 = p0;
           a.tile0 = (int)((int64_t)tiles * q / runs);
           a.n_tiles = (int)((int64_t)tiles * (q + 1) / runs) - a.tile0;
-          a.nbc1 = nbc1; a.nbc2 = nbc2; a.v_mode = b.v_mode;
+          a.v_mode = b.v_mode;
           a.v_group_rows = b.v_group_rows == 0 ? b.rows : b.v_group_rows;
           a.lr_scale = b.lr_scale; a.wd = b.weight_decay;
-          (stream ? items_s : items).push_back(a);
+          lists[2 * t.rp > 256 ? 1 : 0][b.cols % 8 == 0 ? 1 : 0].push_back(a);
         }
       }
     }
-    // shared memory: the L panel (both factor sets side by side), a ring of R^T boxes, a ring of g / W quarter
-    // tiles.  Three R stages, and whatever is left for g / W: measured, the g / W ring pays more per KB than a
-    // deeper R ring, but two R stages leave the MMA warp waiting on every box.
-    const int l_region = nbc_max * tc::kBoxBytes;
-    P->apply_r_stages = 3;
-    P->apply_r_region = l_region;
     P->apply_buf_bytes = tc::kApplyBufBytes + (any_element_v ? tc::kWBoxBytes : 0);
-    auto bufs_with = [&](int r_stages) { return (226 * 1024 - l_region - r_stages * tc::kBoxBytes) / P->apply_buf_bytes; };
-    if (any_element_v && bufs_with(3) < 3 && bufs_with(1) >= 3) {
-      // the larger buffers of a per-element v: a third buffer is worth more than the second and third R stage
-      // (measured on the 1.5B shapes: 9.6 ms with three R stages and two buffers, 8.0 ms with one and three)
-      P->apply_r_stages = 1;
-    } else if (bufs_with(3) < 2) {   // two buffers at least: give up an R stage
-      P->apply_r_stages = 2;
-    }
-    P->apply_w_region = l_region + P->apply_r_stages * tc::kBoxBytes;
-    P->apply_bufs = std::max(1, std::min(tc::kApplyMaxBufs, (226 * 1024 - P->apply_w_region) / P->apply_buf_bytes));
-    P->smem_apply = P->apply_w_region + P->apply_bufs * P->apply_buf_bytes + 1024;
-    // the streaming form: two stages of four boxes, the rest for g / W
-    P->apply_s_w_region = 2 * 4 * tc::kBoxBytes;
-    P->apply_s_bufs = std::max(1, std::min(tc::kApplyMaxBufs, (226 * 1024 - P->apply_s_w_region) / P->apply_buf_bytes));
-    P->smem_apply_s = P->apply_s_w_region + P->apply_s_bufs * P->apply_buf_bytes + 1024;
-    if (!items.empty()) {
+    for (int form = 0; form < 4; ++form) {
+      std::vector<tc::ApplyItem>& items = lists[form >> 1][form & 1];
+      if (items.empty()) continue;
+      // longest first, so that the last round of items is the shortest
+      std::stable_sort(items.begin(), items.end(),
+                       [](const tc::ApplyItem& x, const tc::ApplyItem& y) { return x.n_tiles > y.n_tiles; });
       Launch A{LK_TC_APPLY, append_items(c->h_tables, items), (int64_t)items.size(),
                std::min<int64_t>((int64_t)items.size(), P->n_sms)};
-      prog.push_back(A);
-    }
-    if (!items_s.empty()) {
-      Launch A{LK_TC_APPLY, append_items(c->h_tables, items_s), (int64_t)items_s.size(),
-               std::min<int64_t>((int64_t)items_s.size(), P->n_sms)};
-      A.aux0 = 1;
+      A.aux0 = form >> 1; A.aux1 = form & 1;
       prog.push_back(A);
     }
   }
@@ -733,10 +732,10 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   if (e == cudaSuccess && P->n_teams > 0) e = cudaMalloc((void**)&P->d_team_counters, P->n_teams * sizeof(int32_t));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(tc::tc_items_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P->smem_engine);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::tc_apply_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P->smem_apply);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::tc_apply_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, P->smem_apply_s);
+  for (int form = 0; form < 4; ++form)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(apply_kernel(form >> 1, form & 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               P->apply_config(form >> 1, form & 1).smem);
   if (e != cudaSuccess) {
     set_cuda_error(e, "build_tensor_program");
     return ADAPM_ECUDA;
@@ -888,18 +887,14 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       a.state = (float*)b.p[BASE_STATE]; a.status = c->d_status; a.sc = sc;
       a.use_new = sc.c1 != 0.f ? 1 : 0;
       a.parity = parity;
+      const TcProgram::ApplyConfig e = P->apply_config(L.aux0 != 0, L.aux1 != 0);
+      a.work = (const uint16_t*)b.p[BASE_WORK]; a.params = (float*)b.p[BASE_PARAMS];
+      a.grads = (const uint16_t*)b.p[BASE_GRADS]; a.shadow_out = b.shadow;
+      a.n_rstages = e.n_rstages; a.w_region_off = e.w_region; a.n_bufs = e.n_bufs;
       a.buf_bytes = P->apply_buf_bytes;
       a.gscale = b.gscale;
       a.shadow = b.shadow != nullptr;
-      if (L.aux0 == 0) {
-        a.r_region_off = P->apply_r_region; a.n_rstages = P->apply_r_stages;
-        a.w_region_off = P->apply_w_region; a.n_bufs = P->apply_bufs;
-        tc::tc_apply_kernel<false><<<(unsigned)L.grid, tc::kApplyThreads, P->smem_apply, s>>>(a);
-      } else {
-        a.r_region_off = 0; a.n_rstages = 2;
-        a.w_region_off = P->apply_s_w_region; a.n_bufs = P->apply_s_bufs;
-        tc::tc_apply_kernel<true><<<(unsigned)L.grid, tc::kApplyThreads, P->smem_apply_s, s>>>(a);
-      }
+      apply_kernel(L.aux0 != 0, L.aux1 != 0)<<<(unsigned)L.grid, tc::kApplyThreads, e.smem, s>>>(a);
       break;
     }
     default:

@@ -4,27 +4,35 @@
 //   m^c = cg g + c0 L0 R0 - c1 L R          (= g + c (P_{t-1} - P_t) with the correction on)
 //   W  <- W - lr s_b ( clamp( m^c / (sqrt(v) + eps) ) + lambda_b W )
 //
-// An item is a 128-row panel of one block times a run of column tiles.  The split-bf16 rows
-// [L0 hi | L0 lo | L hi | L lo] of the panel stay in shared memory for the whole run; per column tile
-// the matching rows of [R0^T hi | R0^T lo | R^T hi | R^T lo] arrive one 64-column box at a time
-// through a ring of 16 KB stages, and every 16 columns of a box are multiplied at once with the
-// resident L columns they pair with (hi*hi and lo*hi for columns of a hi part, hi*lo for columns of
-// a lo part; the new set with a negated A operand), so the accumulator ends up holding
-// D = L0 R0 - L R.
+// An item is a 128-row panel of one block times a run of column tiles.  Up to rank 128 the split-bf16 rows
+// [L0 hi | L0 lo | L hi | L lo] of the panel are the A operand and stay in tensor memory for the whole run
+// (two bf16 per column, the refitted set with its sign turned: 2 rp + two accumulators of 128 <= 512
+// columns); per column tile the matching rows of [R0^T hi | R0^T lo | R^T hi | R^T lo] arrive one 64-column
+// box at a time through a ring of 16 KB stages, and every 16 columns of a box are multiplied at once with
+// the L columns they pair with (hi*hi and lo*hi for columns of a hi part, hi*lo for columns of a lo part),
+// so the accumulator ends up holding D = L0 R0 - L R.  Four warps load the L panel of the next item when
+// the last MMA of the present one is through.  With L in shared memory instead (4 rp columns x 128 rows: 80
+// KB at rank 80, 128 KB at rank 128) the operand reads of A share the shared memory's bandwidth and the ring
+// below has room for two or three buffers: 2.42 -> 1.4 ms at rank 128, 8.3 -> 6.8 ms on the 1.5B shapes with
+// a per-element v.
 //
-// g and W never pass through registers on their way in or out: a mover thread brings them in
-// quarter tiles (128 rows x 32 columns: 16 KB of W, 8 KB of g) by TMA into a small ring of
-// shared-memory buffers, several quarters ahead of their use, and writes the updated W back from
-// the same buffer by TMA.  Each of the 256 epilogue threads owns one row of the panel: it reads its
-// accumulator row from tensor memory, its 16 columns of g and W from the (swizzled) buffer, and
-// puts the new W back in place.  A per-element v, where a block has one, travels like W.
+// Ranks above 128 leave no room for L in tensor memory.  The kernel's second form (kStream) streams L as
+// well: a stage of its ring holds four boxes - 64 columns of L hi, L lo, R^T hi and R^T lo of one factor
+// set - and feeds hi*hi, lo*hi and hi*lo for those columns; the previous set is always taken first, the
+// refitted set second.  (Tiles of 96 columns would fit L up to rank 208 beside one accumulator; measured,
+// that was slower, 8.3 against 6.3 ms on eight layers of the 8B shapes.)
+//
+// kTma (parameter rows start on 16 bytes: cols a multiple of 8): g and W never pass through registers on
+// their way in or out.  A mover thread brings them in quarters (128 rows x 32 columns: 16 KB of W, 8 KB of
+// g) by TMA into a ring of shared-memory buffers, several quarters ahead of their use, and writes the
+// updated W back from the same buffer by TMA.  The two groups of 128 epilogue threads take the quarters in
+// turn; a thread owns one row of the panel: it reads its accumulator row from tensor memory, its columns of g
+// and W from the (swizzled) buffer, and puts the new W back in place.  A per-element v, where a block has
+// one, travels like W.
+// (Quarters of 32 rows x 128 columns take four times as many boxes: 4.4 ms instead of 3.0 on the 1.5B shapes.)
+// Otherwise an epilogue warp turns a 32 x 32 chunk of the accumulator through a patch of shared memory and
+// works along the rows of the parameters, one column per lane, whatever the alignment of the rows.
 // The m x n matrices m_t, r_t and m^c are never stored.
-//
-// Ranks above 128 do not leave room for a resident L panel (4 rp columns of 128 rows).  The kernel's
-// second form (kStream) streams L as well: a stage of its ring holds four boxes - 64 columns of
-// L hi, L lo, R^T hi and R^T lo of one factor set - and feeds hi*hi, lo*hi and hi*lo for those
-// columns; the previous set is always taken first, the refitted set second.  Everything after the
-// accumulator (the g / W ring, the epilogue) is the same code.
 #pragma once
 
 #include <cuda.h>
@@ -36,29 +44,30 @@
 namespace adapm {
 namespace tc {
 
-constexpr int kApplyThreads = 352;         // producer warp, MMA warp, eight epilogue warps, mover warp
+constexpr int kApplyThreads = 480;         // producer, MMA, eight epilogue warps, mover, four warps that load L
 constexpr int kApplyNT = 128;              // columns per tile
 constexpr int kApplyQC = 32;               // columns per quarter tile
-constexpr int kApplyAcc = 4;               // accumulators
 constexpr int kApplyMaxStages = 8;         // R ring depth limit
-constexpr int kApplyMaxBufs = 6;           // g / W ring depth limit
+constexpr int kApplyMaxBufs = 8;           // g / W ring depth limit
 constexpr int kWBoxBytes = 128 * kApplyQC * 4;   // a quarter tile of W: 128 rows of 128 bytes
 constexpr int kGBoxBytes = 128 * kApplyQC * 2;   // and of g: 128 rows of 64 bytes
 constexpr int kApplyBufBytes = kWBoxBytes + kGBoxBytes;    // + kWBoxBytes where a block has a per-element v
+constexpr int kPatchPitch = 33;            // floats per row of an epilogue warp's patch
+constexpr int kPatchesBytes = 8 * 32 * kPatchPitch * 4;
 
 struct ApplyItem {
   int64_t off;               // element offset of the block in params / grads
   int64_t v_off;             // float offset of v in state
+  int64_t l_off;             // bf16 element offset of the L array in the workspace (row pitch 4 half)
   int32_t rows, cols, r, rp;
   int32_t half;              // column at which the lo part of a factor set starts (a set is 2 half columns wide)
-  int32_t map_l, map_r;      // split factors, previous and final set side by side: [rows, 4rp] and [cols, 4rp]
+  int32_t map_l, map_r;      // split factors, previous and final set side by side: [rows, 4 half] and [cols, 4 half]
                              // = [hi0 | lo0 | hi1 | lo1], boxes of 64 x 128
   int32_t map_w, map_g;      // params and grads of the block, boxes of 32 x 128
   int32_t map_v;             // per-element v of the block (same boxes as params); unused with a group v
   int32_t map_sh;            // bf16 copy of the params (same boxes as grads); used when the launch has a shadow
   int32_t row0;              // first row of the panel
   int32_t tile0, n_tiles;    // column tiles [tile0, tile0 + n_tiles) of 128 columns
-  int32_t nbc1, nbc2;        // 64-wide boxes across the 2rp columns of the previous set / the 4rp of both
   int32_t v_mode, v_group_rows;
   float lr_scale, wd;
 };
@@ -67,126 +76,193 @@ struct ApplyArgs {
   const ApplyItem* items;
   int32_t n_items;
   const CUtensorMap* maps;
+  const uint16_t* work;      // workspace viewed as bf16
+  float* params;             // params, grads and shadow by address (!kTma; kTma goes through the maps)
+  const uint16_t* grads;
+  uint16_t* shadow_out;
   float* state;
   int32_t* status;
   StepScalars sc;
   int32_t use_new;           // 0: c1 == 0, the refitted factors are not needed
   int32_t parity;            // 0: the left half of the operands holds the previous factors, 1: the right half
   const float* gscale;       // device scalar: every gradient counts as gscale[0] * g (nullptr: 1)
-  int32_t shadow;            // 1: the bf16 copy of the parameters is written with W (ApplyItem::map_sh)
-  int32_t r_region_off;      // byte offset of the R ring inside the dynamic shared memory
-  int32_t n_rstages;         // R ring depth (1..kApplyMaxStages); a stage is one 64 x 128 box of R^T
-  int32_t w_region_off;      // byte offset of the g / W ring
-  int32_t n_bufs;            // g / W ring depth (1..kApplyMaxBufs)
+  int32_t shadow;            // 1: the bf16 copy of the parameters is written with W
+  int32_t n_rstages;         // R ring depth (1..kApplyMaxStages); a stage is one 64 x 128 box of R^T (kStream: four boxes)
+  int32_t w_region_off;      // byte offset of the g / W ring (kTma) or of the patches inside the dynamic shared memory
+  int32_t n_bufs;            // g / W ring depth (2..kApplyMaxBufs, even: see the epilogue)
   int32_t buf_bytes;         // one buffer: W, g and, if any block of the launch has a per-element v, v
 };
 
 struct __align__(8) ApplyShared {
-  uint64_t lfull, lempty, rfull[kApplyMaxStages], rempty[kApplyMaxStages], tfull[kApplyAcc], tempty[kApplyAcc];
+  uint64_t lfull, lempty, rfull[kApplyMaxStages], rempty[kApplyMaxStages], tfull[2], tempty[2];
   uint64_t wfull[kApplyMaxBufs];   // a quarter's g and W have landed
-  uint64_t wdone[kApplyMaxBufs];   // all eight epilogue warps have put their new W back
+  uint64_t wdone[kApplyMaxBufs];   // a group of four epilogue warps has put its new W back
   uint32_t tmem_base;
   int abort;
 };
 
-template <bool kStream>
+// The epilogue of one warp without TMA: 32 x 32 chunks of the accumulator, one column per lane.
+__device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplyShared& sh, float* patch, uint32_t tmem_acc) {
+  constexpr int kChunks = kApplyNT / 32, kBatch = 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sub = warp & 3, grp = (warp - 2) >> 2;           // which 32 accumulator rows; chunks grp, grp + 2, ...
+  const uint32_t lane_addr = (uint32_t)(32 * sub) << 16;
+  const StepScalars& sc = a.sc;
+  const float gs = a.gscale ? *a.gscale : 1.f;
+  int j = 0;
+  for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
+    const ApplyItem I = a.items[it];
+    const bool grouped = I.v_mode == ADAPM_V_BLOCKMEAN;
+    const float lr_s = sc.lr * I.lr_scale;
+    const int row0 = I.row0 + 32 * sub, rows = I.rows - row0;
+    // one denominator per row when v is a group scalar (lane = row of the chunk): m^c / (sqrt(v) + eps) is a product
+    float kr = 0.f;
+    if (grouped && lane < rows) {
+      const float v_row = a.state[I.v_off + (row0 + lane) / I.v_group_rows];
+      kr = sc.inv_bc1 / (sqrtf(v_row * sc.inv_bc2) + sc.eps);
+    }
+    for (int t = 0; t < I.n_tiles; ++t, ++j) {
+      const int acc = j & 1;
+      for (int c = grp; c < kChunks; c += 2) {
+        const int col = (I.tile0 + t) * kApplyNT + 32 * c + lane;
+        const bool cok = col < I.cols;
+        const int64_t o = (int64_t)row0 * I.cols + col;
+        float* W = a.params + I.off + o;
+        const uint16_t* G = a.grads + I.off + o;
+        float* V = a.state + I.v_off + o;
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += kBatch) {
+          float w[kBatch], v[kBatch];
+          uint16_t g[kBatch];
+#pragma unroll
+          for (int r = 0; r < kBatch; ++r) {
+            const int64_t at = (int64_t)(r0 + r) * I.cols;
+            w[r] = 0.f; v[r] = 0.f; g[r] = 0;
+            if (cok && r0 + r < rows) {
+              w[r] = W[at];
+              g[r] = G[at];
+              if (!grouped) v[r] = V[at];
+            }
+          }
+          if (r0 == 0) {
+            // one lane polls, then the warp agrees: the tensor-memory loads need all 32 lanes
+            bool got = true;
+            if (lane == 0) got = mbar_wait(&sh.tfull[acc], (uint32_t)(j >> 1) & 1u, &sh.abort, a.status, ST_WAIT_TMEM_FULL);
+            got = __shfl_sync(0xffffffffu, got, 0);
+            if (!got) return;
+            tc_fence_after();
+            float d[32];
+            tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + 32 * c), d);
+            tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + 32 * c + 16), d + 16);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) patch[lane * kPatchPitch + e] = d[e];
+            __syncwarp();
+          }
+#pragma unroll
+          for (int r = 0; r < kBatch; ++r) {
+            const float k_row = __shfl_sync(0xffffffffu, kr, r0 + r);
+            if (cok && r0 + r < rows) {
+              const int64_t at = (int64_t)(r0 + r) * I.cols;
+              const float d = patch[(r0 + r) * kPatchPitch + lane], g1 = gs * bf16_bits_to_float(g[r]);
+              const float mc = sc.cg * g1 + sc.c0 * d;
+              if (grouped) {
+                w[r] = w[r] - lr_s * (clamp_keep_nan(mc * k_row, sc.clip) + I.wd * w[r]);
+              } else {
+                v[r] = sc.beta2 * v[r] + (1.f - sc.beta2) * (g1 * g1);
+                adapm_param_update_n<1>(&w[r], &mc, &v[r], sc, lr_s, I.wd);
+                V[at] = v[r];
+              }
+              W[at] = w[r];
+              if (a.shadow) a.shadow_out[I.off + o + at] = (uint16_t)(pack_bf16x2(w[r], 0.f) & 0xffffu);
+            }
+          }
+        }
+        __syncwarp();                                        // the patch is free again
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.tempty[acc]);
+    }
+  }
+}
+
+template <bool kStream, bool kTma>
 __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a) {
+  constexpr int kStageBytes = kStream ? 4 * kBoxBytes : kBoxBytes;
+  constexpr int kQ = kApplyNT / kApplyQC;                    // quarters per tile
   extern __shared__ uint8_t dyn_smem[];
   __shared__ ApplyShared sh;
   __shared__ int skip_launch;
   if (threadIdx.x == 0) skip_launch = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   __syncthreads();
   if (skip_launch) return;   // an earlier launch of the step gave up: leave W and v untouched
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~(uintptr_t)1023);
-  uint8_t* smem_l = smem;
-  uint8_t* smem_r = smem + a.r_region_off;
-  uint8_t* smem_w = smem + a.w_region_off;
+  uint8_t* smem_r = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem_w = smem_r + a.w_region_off;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort = &sh.abort;
   const int n_sets = a.use_new ? 2 : 1;
 
   if (threadIdx.x == 0) {
-    mbar_init(&sh.lfull, 1); mbar_init(&sh.lempty, 1);
+    mbar_init(&sh.lfull, 4); mbar_init(&sh.lempty, 1);
     for (int i = 0; i < kApplyMaxStages; ++i) { mbar_init(&sh.rfull[i], 1); mbar_init(&sh.rempty[i], 1); }
-    for (int i = 0; i < kApplyAcc; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 8); }
-    for (int i = 0; i < kApplyMaxBufs; ++i) { mbar_init(&sh.wfull[i], 1); mbar_init(&sh.wdone[i], 8); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 8); }
+    for (int i = 0; i < kApplyMaxBufs; ++i) { mbar_init(&sh.wfull[i], 1); mbar_init(&sh.wdone[i], 4); }
     sh.abort = 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&sh.tmem_base, kApplyAcc * kApplyNT);
+    tmem_alloc(&sh.tmem_base, 512);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = sh.tmem_base;
+  const uint32_t tmem_base = sh.tmem_base;                   // A from column 0, accumulators at the end
+  const uint32_t tmem_acc = tmem_base + 512 - 2 * kApplyNT;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (all lanes run, one issues)
     const bool leader = elect_one();
-    uint32_t item_phase = 0, rphase = 0;
+    uint32_t rphase = 0;
     int rs = 0;
     bool ok = true;
-    int l_loads = 0, r_loads = 0;
+    int r_loads = 0;
     for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
       const ApplyItem& I = a.items[it];
       const CUtensorMap* const ml = a.maps + I.map_l;
       const CUtensorMap* const mr = a.maps + I.map_r;
-      const int n_tiles = I.n_tiles, row0 = I.row0;
+      const int n_tiles = I.n_tiles, row0 = I.row0, half = I.half, rp = I.rp;
+      // the columns of all parts in one run; with only the previous set in use, and that set in the right half, the
+      // run starts there
+      const int x0 = (n_sets == 1 && a.parity) ? 2 * half : 0;
+      const int nb = kStream ? (rp + 63) >> 6 : (n_sets * 2 * rp + 63) >> 6;
       int col0 = I.tile0 * kApplyNT;
-      if (kStream) {
-        // a stage = 64 columns of [L hi, L lo, R^T hi, R^T lo] of one set; previous set first
-        const int nbh = (I.rp + 63) >> 6, half = I.half;
-        for (int t = 0; t < n_tiles && ok; ++t, col0 += kApplyNT) {
-          for (int si = 0; si < n_sets && ok; ++si) {
-            const int xs = (si == 0 ? a.parity : 1 - a.parity) * 2 * half;
-            for (int jb = 0; jb < nbh; ++jb) {
-              if (!mbar_wait_warp(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-              uint8_t* st = smem_r + rs * (4 * kBoxBytes);
-              if (leader) {
-                mbar_arrive_expect_tx(&sh.rfull[rs], 4u * kBoxBytes);
-                tma_load_box(st, ml, xs + 64 * jb, row0, &sh.rfull[rs]);
-                tma_load_box(st + kBoxBytes, ml, xs + half + 64 * jb, row0, &sh.rfull[rs]);
-                tma_load_box(st + 2 * kBoxBytes, mr, xs + 64 * jb, col0, &sh.rfull[rs]);
-                tma_load_box(st + 3 * kBoxBytes, mr, xs + half + 64 * jb, col0, &sh.rfull[rs]);
-              }
-              __syncwarp();
-              ++r_loads;
-              if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
-            }
-          }
-        }
-        continue;
-      }
-      if (!mbar_wait_warp(&sh.lempty, item_phase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-      const int nb = n_sets == 2 ? I.nbc2 : I.nbc1;
-      // with only the previous set in use, and that set in the right half, the boxes start there
-      const int x0 = (n_sets == 1 && a.parity) ? 2 * I.rp : 0;
-      if (leader) {
-        mbar_arrive_expect_tx(&sh.lfull, (uint32_t)nb * kBoxBytes);
-        for (int bc = 0; bc < nb; ++bc) tma_load_box(smem_l + bc * kBoxBytes, ml, x0 + 64 * bc, row0, &sh.lfull);
-      }
-      __syncwarp();
-      ++l_loads;
       for (int t = 0; t < n_tiles && ok; ++t, col0 += kApplyNT) {
-        for (int bc = 0; bc < nb; ++bc) {
-          if (!mbar_wait_warp(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
-          if (leader) {
-            mbar_arrive_expect_tx(&sh.rfull[rs], (uint32_t)kBoxBytes);
-            tma_load_box(smem_r + rs * kBoxBytes, mr, x0 + 64 * bc, col0, &sh.rfull[rs]);
+        for (int si = 0; si < (kStream ? n_sets : 1) && ok; ++si) {
+          const int xs = (si == 0 ? a.parity : 1 - a.parity) * 2 * half;
+          for (int bc = 0; bc < nb; ++bc) {
+            if (!mbar_wait_warp(&sh.rempty[rs], rphase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) { ok = false; break; }
+            uint8_t* st = smem_r + rs * kStageBytes;
+            if (leader) {
+              mbar_arrive_expect_tx(&sh.rfull[rs], (uint32_t)kStageBytes);
+              if (kStream) {
+                tma_load_box(st, ml, xs + 64 * bc, row0, &sh.rfull[rs]);
+                tma_load_box(st + kBoxBytes, ml, xs + half + 64 * bc, row0, &sh.rfull[rs]);
+                tma_load_box(st + 2 * kBoxBytes, mr, xs + 64 * bc, col0, &sh.rfull[rs]);
+                tma_load_box(st + 3 * kBoxBytes, mr, xs + half + 64 * bc, col0, &sh.rfull[rs]);
+              } else {
+                tma_load_box(st, mr, x0 + 64 * bc, col0, &sh.rfull[rs]);
+              }
+            }
+            __syncwarp();
+            ++r_loads;
+            if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
           }
-          __syncwarp();
-          ++r_loads;
-          if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
         }
       }
-      item_phase ^= 1u;
     }
     if (!ok) {   // let the copies already issued land before the CTA exits
-      if (l_loads)
-        for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.lfull, (uint32_t)(l_loads - 1) & 1u); ++spin)
-          __nanosleep(64);
       const int back = r_loads < a.n_rstages ? r_loads : a.n_rstages;
       for (int q = 0; q < back; ++q) {
         int st = rs - 1 - q;
@@ -202,27 +278,27 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
     int rs = 0;
     int j = 0;   // running tile count of this CTA
     bool ok = true;
-    const uint32_t l_base = smem_u32(smem_l), r_base = smem_u32(smem_r);
+    const uint32_t r_base = uniform(smem_u32(smem_r)), a_base = uniform(tmem_base), acc_base = uniform(tmem_acc);
     const uint32_t dhi = desc_hi();
     const uint32_t idesc_pos = make_idesc(kApplyNT, false, false, false);
     const uint32_t idesc_neg = make_idesc(kApplyNT, false, false, true);
     for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
-      const int n_tiles = a.items[it].n_tiles;
-      const int ks = a.items[it].rp >> 4;     // 16-wide K steps per part (hi or lo of one set)
-      if (kStream) {
-        const int nbh = (ks + 3) >> 2;
-        for (int t = 0; t < n_tiles && ok; ++t, ++j) {
-          const int acc = j % kApplyAcc;
-          const uint32_t acc_phase = (uint32_t)(j / kApplyAcc) & 1u;
-          if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
+      const int n_tiles = uniform(a.items[it].n_tiles);
+      const int ks = uniform(a.items[it].rp >> 4);     // 16-wide K steps per part (hi or lo of one set)
+      if (!kStream && !mbar_wait_warp(&sh.lfull, item_phase, abort, a.status, ST_WAIT_FULL)) break;
+      for (int t = 0; t < n_tiles && ok; ++t, ++j) {
+        const int acc = j & 1;
+        if (!mbar_wait_warp(&sh.tempty[acc], ((uint32_t)(j >> 1) & 1u) ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d = acc_base + (uint32_t)(acc * kApplyNT);
+        if (kStream) {
+          const int nbh = (ks + 3) >> 2;
           for (int si = 0; si < n_sets && ok; ++si) {
             const uint32_t idesc = si ? idesc_neg : idesc_pos;      // the refitted set enters negated
             for (int jb = 0; jb < nbh; ++jb) {
               if (!mbar_wait_warp(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
               tc_fence_after();
-              const uint32_t st = r_base + (uint32_t)rs * (4u * kBoxBytes);
+              const uint32_t st = r_base + (uint32_t)(rs * kStageBytes);
               const uint32_t ahi = desc_lo(st, 16), alo = desc_lo(st + kBoxBytes, 16);
               const uint32_t bhi = desc_lo(st + 2 * kBoxBytes, 16), blo = desc_lo(st + 3 * kBoxBytes, 16);
               if (leader) {
@@ -241,64 +317,166 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
               if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
             }
           }
-          if (ok && leader) mma_commit(&sh.tfull[acc]);
-          __syncwarp();
-        }
-        continue;
-      }
-      const int nb = n_sets == 2 ? a.items[it].nbc2 : a.items[it].nbc1;
-      if (!mbar_wait_warp(&sh.lfull, item_phase, abort, a.status, ST_WAIT_FULL)) break;
-      for (int t = 0; t < n_tiles && ok; ++t, ++j) {
-        const int acc = j % kApplyAcc;
-        const uint32_t acc_phase = (uint32_t)(j / kApplyAcc) & 1u;
-        if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d = tmem_base + (uint32_t)(acc * kApplyNT);
-        const uint32_t la = desc_lo(l_base, 16);
-        // K step k of the [.., 4rp] operands: box k / 4 (16 KB apart), 32 bytes per step inside it
-        auto kstep = [](int k) { return (uint32_t)((k >> 2) * (kBoxBytes >> 4) + (k & 3) * 2); };
-        for (int bc = 0; bc < nb; ++bc) {
-          if (!mbar_wait_warp(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t rb = desc_lo(r_base + (uint32_t)rs * kBoxBytes, 16);
-          if (leader) {
+        } else {
+          int part = 0, w = 0;         // the box's first K step: part (hi, lo of one set, hi, lo of the other), step inside it
+          while (part < 2 * n_sets) {
+            if (!mbar_wait_warp(&sh.rfull[rs], rphase, abort, a.status, ST_WAIT_FULL)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t rb = desc_lo(r_base + (uint32_t)(rs * kStageBytes), 16);
+            if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const int kb = 4 * bc + kk;              // K step of [R0 hi | R0 lo | R hi | R lo] held by this box
-              if (kb < n_sets * 2 * ks) {
-                const int set = kb >= 2 * ks ? 1 : 0;
-                const int w = kb - set * 2 * ks;       // K step inside the set: hi part, then lo part
-                // the set that holds the refitted factors enters with a negated A operand
-                const uint32_t idesc = (n_sets == 2 && (set ^ a.parity)) ? idesc_neg : idesc_pos;
-                const uint64_t b = desc_join(rb + (uint32_t)(kk * 2), dhi);
-                // hi * hi and lo * hi, or hi * lo
-                mma_bf16(d, desc_join(la + kstep(w < ks ? kb : kb - ks), dhi), b, idesc, kb != 0);
-                if (w < ks) mma_bf16(d, desc_join(la + kstep(kb + ks), dhi), b, idesc, 1u);
+              for (int kk = 0; kk < 4; ++kk) {
+                int pp = part, ww = w + kk;
+                if (ww >= ks) { ww -= ks; ++pp; }
+                if (ww >= ks) { ww -= ks; ++pp; }
+                if (ww >= ks) { ww -= ks; ++pp; }
+                if (pp < 2 * n_sets) {
+                  const uint64_t b = desc_join(rb + (uint32_t)(kk * 2), dhi);
+                  const uint32_t at = a_base + (uint32_t)(8 * (pp * ks + ww));
+                  const uint32_t odd = (uint32_t)pp & 1u;
+                  // hi * hi and lo * hi, or hi * lo
+                  mma_bf16_ta(d, at - (odd ? (uint32_t)(8 * ks) : 0u), b, idesc_pos, (pp | ww) != 0);
+                  if (!odd) mma_bf16_ta(d, at + (uint32_t)(8 * ks), b, idesc_pos, 1u);
+                }
               }
+              mma_commit(&sh.rempty[rs]);
             }
-            mma_commit(&sh.rempty[rs]);
+            __syncwarp();
+            w += 4;
+            while (w >= ks) { w -= ks; ++part; }
+            if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
           }
-          __syncwarp();
-          if (++rs == a.n_rstages) { rs = 0; rphase ^= 1u; }
         }
         if (ok && leader) mma_commit(&sh.tfull[acc]);
         __syncwarp();
       }
-      if (ok && leader) mma_commit(&sh.lempty);
+      if (!kStream && ok && leader) mma_commit(&sh.lempty);
       __syncwarp();
       item_phase ^= 1u;
     }
+  } else if (warp < 10) {
+    // ------------------------------------------------------------------ epilogue
+    if constexpr (!kTma) {
+      apply_rows_epilogue(a, sh, reinterpret_cast<float*>(smem_w) + (warp - 2) * 32 * kPatchPitch, tmem_acc);
+    } else {
+      const int wq4 = warp & 3;                             // which 32 accumulator rows this warp may read
+      // The two groups of four warps take the quarters in turn.  With an even number of buffers a buffer belongs to one
+      // group: a group that waited on the other's buffers could be a whole phase ahead of a barrier, whose parity then
+      // reads as complete.
+      const int grp = (warp - 2) >> 2;
+      const uint32_t lane_addr = (uint32_t)(32 * wq4) << 16;
+      const int rloc = 32 * wq4 + lane;                     // this thread's row of the panel
+      StepScalars sc = a.sc;
+      const float gs = a.gscale ? *a.gscale : 1.f;
+      sc.cg *= gs;               // m^c = cg (gs g) + c0 D
+      // byte offsets of a 16-byte chunk of this thread's row inside a buffer: the 128-byte swizzle turns chunk c of
+      // row r into chunk c ^ (r % 8), the 64-byte swizzle chunk c of a 64-byte row into c ^ ((r / 2) % 4)
+      auto w_at = [&](int c) { return (uint32_t)(rloc * 128 + ((c ^ (rloc & 7)) << 4)); };
+      auto g_at = [&](int c) { return (uint32_t)(kWBoxBytes + rloc * 64 + ((c ^ ((rloc >> 1) & 3)) << 4)); };
+      int j = 0, b = grp;   // running tile count of this CTA, g / W buffer
+      uint32_t wphase = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
+        const ApplyItem I = a.items[it];
+        const bool grouped = I.v_mode == ADAPM_V_BLOCKMEAN;
+        const float lr_s = sc.lr * I.lr_scale;
+        const int row = I.row0 + rloc;
+        const bool rok = row < I.rows;
+        // one denominator per row when v is a group scalar: m^c / (sqrt(v) + eps) becomes a product
+        const float v_row = (rok && grouped) ? a.state[I.v_off + row / I.v_group_rows] : 0.f;
+        const float kr = sc.inv_bc1 / (sqrtf(v_row * sc.inv_bc2) + sc.eps);
+        const float kg = sc.cg * kr, kd = sc.c0 * kr;
+        for (int t = 0; t < I.n_tiles && ok; ++t, ++j) {
+          const int acc = j & 1;
+          // one lane per warp polls, then the warp agrees: the tensor-memory loads need all 32 lanes
+          bool got = true;
+          if (lane == 0) got = mbar_wait(&sh.tfull[acc], (uint32_t)(j >> 1) & 1u, abort, a.status, ST_WAIT_TMEM_FULL);
+          got = __shfl_sync(0xffffffffu, got, 0);
+          if (!got) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll 1
+          for (int q = grp; q < kQ; q += 2) {
+            if (!mbar_wait(&sh.wfull[b], wphase, abort, a.status, ST_WAIT_FULL)) ok = false;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            uint8_t* buf = smem_w + (size_t)b * a.buf_bytes;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              float d[16];
+              tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + q * kApplyQC + 16 * half), d);
+              float gf[16];
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const uint4 gg = *reinterpret_cast<const uint4*>(buf + g_at(2 * half + i));
+                const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                  gf[8 * i + 2 * x] = __uint_as_float(gw[x] << 16);
+                  gf[8 * i + 2 * x + 1] = __uint_as_float(gw[x] & 0xffff0000u);
+                }
+              }
+              tmem_ld_wait();
+              uint32_t shw[8];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                float4* wp = reinterpret_cast<float4*>(buf + w_at(4 * half + i));
+                const float4 wo = *wp;
+                float w[4] = {wo.x, wo.y, wo.z, wo.w};
+                if (grouped) {
+#pragma unroll
+                  for (int x = 0; x < 4; ++x) {
+                    const float ratio = clamp_keep_nan(gf[4 * i + x] * kg + d[4 * i + x] * kd, sc.clip);
+                    w[x] = w[x] - lr_s * (ratio + I.wd * w[x]);
+                  }
+                } else {
+                  float4* vp = reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at(4 * half + i));   // v lies like W
+                  const float4 vo = *vp;
+                  float vv[4] = {vo.x, vo.y, vo.z, vo.w}, mc[4];
+#pragma unroll
+                  for (int x = 0; x < 4; ++x) {
+                    const float g1 = gf[4 * i + x];
+                    vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
+                    mc[x] = sc.cg * g1 + sc.c0 * d[4 * i + x];
+                  }
+                  *vp = make_float4(vv[0], vv[1], vv[2], vv[3]);
+                  adapm_param_update_n<4>(w, mc, vv, sc, lr_s, I.wd);
+                }
+                *wp = make_float4(w[0], w[1], w[2], w[3]);
+                shw[2 * i] = pack_bf16x2(w[0], w[1]);
+                shw[2 * i + 1] = pack_bf16x2(w[2], w[3]);
+              }
+              if (a.shadow) {
+                // The bf16 copy of the new W takes the place of the gradient in the buffer (this thread's two 16-byte
+                // pieces, already read): it has g's box shape and swizzle, and is stored with the same kind of tensor
+                // map.
+                *reinterpret_cast<uint4*>(buf + g_at(2 * half)) = make_uint4(shw[0], shw[1], shw[2], shw[3]);
+                *reinterpret_cast<uint4*>(buf + g_at(2 * half + 1)) = make_uint4(shw[4], shw[5], shw[6], shw[7]);
+              }
+            }
+            fence_async_smem();   // every lane orders its own writes, the warp meets, one arrival per warp
+            if (q + 2 >= kQ) tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              mbar_arrive(&sh.wdone[b]);
+              if (q + 2 >= kQ) mbar_arrive(&sh.tempty[acc]);
+            }
+            b += 2;
+            if (b >= a.n_bufs) { b = grp; wphase ^= 1u; }
+          }
+        }
+      }
+    }
   } else if (warp == 10) {
     // ------------------------------------------------------------------ g / W mover
-    if (lane == 0) {
+    if (kTma && lane == 0) {
       // load cursor: runs n_bufs quarters ahead of the quarter being stored
       int ld_it = blockIdx.x, ld_q = 0, ld_nq = 0, n_loaded = 0;
       ApplyItem LI;
-      if (ld_it < a.n_items) { LI = a.items[ld_it]; ld_nq = 4 * LI.n_tiles; }
+      if (ld_it < a.n_items) { LI = a.items[ld_it]; ld_nq = kQ * LI.n_tiles; }
       auto load_next = [&]() {
         const int b = n_loaded % a.n_bufs;
         uint8_t* buf = smem_w + (size_t)b * a.buf_bytes;
-        const int col = (LI.tile0 + (ld_q >> 2)) * kApplyNT + (ld_q & 3) * kApplyQC;
+        const int col = LI.tile0 * kApplyNT + ld_q * kApplyQC;
         const bool with_v = LI.v_mode == ADAPM_V_ELEMENT;
         mbar_arrive_expect_tx(&sh.wfull[b], (uint32_t)(kApplyBufBytes + (with_v ? kWBoxBytes : 0)));
         tma_load_box(buf, a.maps + LI.map_w, col, LI.row0, &sh.wfull[b]);
@@ -307,7 +485,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
         ++n_loaded;
         if (++ld_q == ld_nq) {
           ld_it += gridDim.x; ld_q = 0; ld_nq = 0;
-          if (ld_it < a.n_items) { LI = a.items[ld_it]; ld_nq = 4 * LI.n_tiles; }
+          if (ld_it < a.n_items) { LI = a.items[ld_it]; ld_nq = kQ * LI.n_tiles; }
         }
       };
       for (int i = 0; i < a.n_bufs && ld_it < a.n_items; ++i) load_next();
@@ -315,10 +493,10 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
       bool ok = true;
       for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
         const ApplyItem I = a.items[it];
-        for (int q = 0; q < 4 * I.n_tiles; ++q, ++k) {
+        for (int q = 0; q < kQ * I.n_tiles; ++q, ++k) {
           const int b = k % a.n_bufs;
           if (!mbar_wait(&sh.wdone[b], (uint32_t)(k / a.n_bufs) & 1u, abort, a.status, ST_WAIT_DRAIN)) { ok = false; break; }
-          const int col = (I.tile0 + (q >> 2)) * kApplyNT + (q & 3) * kApplyQC;
+          const int col = I.tile0 * kApplyNT + q * kApplyQC;
           // (a quarter that lies past the last column is not stored)
           if (col < I.cols) {
             const uint8_t* buf = smem_w + (size_t)b * a.buf_bytes;
@@ -327,13 +505,14 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
             if (I.v_mode == ADAPM_V_ELEMENT) tma_store_box(a.maps + I.map_v, col, I.row0, buf + kApplyBufBytes);
           }
           bulk_commit_group();
-          if ((a.n_bufs < 2 || (k & 1)) && ld_it < a.n_items) {
+          if ((k & 1) && ld_it < a.n_items) {
             // two quarters at a time: their rows are neighbours in memory, and requests that reach DRAM
-            // together share its open pages.  They go into this buffer and the one stored before it,
-            // once both stores have read them.
+            // together share its open pages (one at a time, by a thread of its own: 8.2 instead of 6.8 ms on the 1.5B
+            // shapes with a per-element v).  They go into this buffer and the one stored before it, once both
+            // stores have read them.
             bulk_wait_group_read<0>();
             load_next();
-            if (a.n_bufs >= 2 && ld_it < a.n_items) load_next();
+            if (ld_it < a.n_items) load_next();
           }
         }
       }
@@ -346,112 +525,50 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
         }
       }
     }
-  } else {
-    // ------------------------------------------------------------------ epilogue
-    const int e = warp - 2;
-    const int wq4 = warp & 3;                             // which 32 accumulator rows this warp may read
-    const int half = e >> 2;                              // which 16 columns of a quarter
-    const uint32_t lane_addr = (uint32_t)(32 * wq4) << 16;
-    const int rloc = 32 * wq4 + lane;                     // this thread's row of the panel
-    StepScalars sc = a.sc;
-    const float gs = a.gscale ? *a.gscale : 1.f;
-    sc.cg *= gs;               // m^c = cg (gs g) + c0 D
-    // byte offsets of this thread's 16-byte chunks inside a buffer: the 128-byte swizzle turns chunk c of
-    // row r into chunk c ^ (r % 8), the 64-byte swizzle chunk c of a 64-byte row into c ^ ((r / 2) % 4)
-    uint32_t w_at[4], g_at[2];
+  } else if (!kStream) {
+    // ------------------------------------------------------------------ L panel -> tensor memory, one row per thread
+    // The loads of 64 columns are in flight together, and those of an item's first 64 before the tensor memory is free:
+    // the MMAs wait for this between two items.
+    const int sub = warp & 3;                                // which 32 lanes of tensor memory this warp may write
+    const uint32_t lane_addr = (uint32_t)(32 * sub) << 16;
+    uint32_t item_phase = 0;
+    for (int it = blockIdx.x; it < a.n_items; it += gridDim.x) {
+      const int rp = a.items[it].rp, row = a.items[it].row0 + 32 * sub + lane;
+      const bool rok = row < a.items[it].rows;
+      // [hi0 | lo0 | hi1 | lo1] without gaps (half = rp); with one set in use, that set alone
+      const int width = n_sets * 2 * rp;
+      const uint16_t* src = a.work + a.items[it].l_off + (int64_t)row * (4 * rp) + (n_sets == 2 ? 0 : a.parity * 2 * rp);
+      // the refitted set enters negated
+      const int neg0 = n_sets == 2 ? (1 - a.parity) * 2 * rp : width, neg1 = neg0 + 2 * rp;
+      uint4 x[8];
+      auto fetch = [&](int k0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w_at[i] = (uint32_t)(rloc * 128 + (((4 * half + i) ^ (rloc & 7)) << 4));
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      g_at[i] = (uint32_t)(kWBoxBytes + rloc * 64 + (((2 * half + i) ^ ((rloc >> 1) & 3)) << 4));
-    int j = 0, k = 0;   // running tile and quarter counts of this CTA
-    bool ok = true;
-    for (int it = blockIdx.x; it < a.n_items && ok; it += gridDim.x) {
-      const ApplyItem I = a.items[it];
-      const bool grouped = I.v_mode == ADAPM_V_BLOCKMEAN;
-      const float lr_s = sc.lr * I.lr_scale;
-      const int row = I.row0 + rloc;
-      const bool rok = row < I.rows;
-      // one denominator per row when v is a group scalar: m^c / (sqrt(v) + eps) becomes a product
-      const float v_row = (rok && grouped) ? a.state[I.v_off + row / I.v_group_rows] : 0.f;
-      const float kr = sc.inv_bc1 / (sqrtf(v_row * sc.inv_bc2) + sc.eps);
-      const int n_q = 4 * I.n_tiles;
-      for (int q = 0; q < n_q; ++q, ++k) {
-        const int jt = j + (q >> 2), sub = q & 3;
-        const int acc = jt % kApplyAcc;
-        const int b = k % a.n_bufs;
-        if (sub == 0) {
-          // one lane per warp polls, then the warp agrees: the tensor-memory loads need all 32 lanes
-          bool got = true;
-          if (lane == 0) got = mbar_wait(&sh.tfull[acc], (uint32_t)(jt / kApplyAcc) & 1u, abort, a.status, ST_WAIT_TMEM_FULL);
-          got = __shfl_sync(0xffffffffu, got, 0);
-          if (!got) { ok = false; break; }
-          tc_fence_after();
+        for (int i = 0; i < 8; ++i) {
+          x[i] = make_uint4(0, 0, 0, 0);
+          if (rok && k0 + 8 * i < width) x[i] = *reinterpret_cast<const uint4*>(src + k0 + 8 * i);
         }
-        float d[16];
-        tmem_ld16(tmem_base + lane_addr + (uint32_t)(acc * kApplyNT + sub * kApplyQC + 16 * half), d);
-        if (!mbar_wait(&sh.wfull[b], (uint32_t)(k / a.n_bufs) & 1u, abort, a.status, ST_WAIT_FULL)) ok = false;
-        ok = __all_sync(0xffffffffu, ok);
-        tmem_ld_wait();
-        if (!ok) break;
-        uint8_t* buf = smem_w + (size_t)b * a.buf_bytes;
-        float gf[16];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const uint4 gg = *reinterpret_cast<const uint4*>(buf + g_at[i]);
-          const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            gf[8 * i + 2 * x] = __uint_as_float(gw[x] << 16);
-            gf[8 * i + 2 * x + 1] = __uint_as_float(gw[x] & 0xffff0000u);
-          }
-        }
-        uint32_t shw[8];
+      };
+      fetch(0);
+      if (!mbar_wait_warp(&sh.lempty, item_phase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) break;
+      tc_fence_after();
+      for (int k0 = 0; k0 < width; k0 += 64) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          float4* wp = reinterpret_cast<float4*>(buf + w_at[i]);
-          const float4 wo = *wp;
-          float w[4] = {wo.x, wo.y, wo.z, wo.w};
-          if (grouped) {
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-              float ratio = (sc.cg * gf[4 * i + x] + sc.c0 * d[4 * i + x]) * kr;
-              ratio = ratio > sc.clip ? sc.clip : (ratio < -sc.clip ? -sc.clip : ratio);
-              w[x] = w[x] - lr_s * (ratio + I.wd * w[x]);
-            }
-          } else {
-            float4* vp = reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at[i]);   // v lies like W
-            const float4 vo = *vp;
-            float vv[4] = {vo.x, vo.y, vo.z, vo.w};
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-              const float g1 = gf[4 * i + x];
-              vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
-              w[x] = adapm_param_update(w[x], sc.cg * g1 + sc.c0 * d[4 * i + x], vv[x], sc, lr_s, I.wd);
-            }
-            *vp = make_float4(vv[0], vv[1], vv[2], vv[3]);
+          const int k = k0 + 16 * i;
+          if (k < width) {
+            const uint32_t flip = k >= neg0 && k < neg1 ? 0x80008000u : 0u;
+            const uint4 p = x[2 * i], q = x[2 * i + 1];
+            const uint32_t v[8] = {p.x ^ flip, p.y ^ flip, p.z ^ flip, p.w ^ flip, q.x ^ flip, q.y ^ flip, q.z ^ flip, q.w ^ flip};
+            tmem_st8(tmem_base + lane_addr + (uint32_t)(k >> 1), v);
           }
-          *wp = make_float4(w[0], w[1], w[2], w[3]);
-          shw[2 * i] = pack_bf16x2(w[0], w[1]);
-          shw[2 * i + 1] = pack_bf16x2(w[2], w[3]);
         }
-        if (a.shadow) {
-          // The bf16 copy of the new W takes the place of the gradient in the buffer (this thread's two 16-byte
-          // pieces, already read): it has g's box shape and swizzle, and the mover stores it with the same kind of
-          // tensor map.
-          *reinterpret_cast<uint4*>(buf + g_at[0]) = make_uint4(shw[0], shw[1], shw[2], shw[3]);
-          *reinterpret_cast<uint4*>(buf + g_at[1]) = make_uint4(shw[4], shw[5], shw[6], shw[7]);
-        }
-        // one arrival per warp: every lane orders its own writes (and tensor-memory reads), the warp meets
-        fence_async_smem();
-        if (sub == 3) tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(&sh.wdone[b]);
-          if (sub == 3) mbar_arrive(&sh.tempty[acc]);
-        }
+        if (k0 + 64 < width) fetch(k0 + 64);
       }
-      j += I.n_tiles;
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.lfull);
+      item_phase ^= 1u;
     }
   }
 
@@ -459,7 +576,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kApplyAcc * kApplyNT);
+    tmem_dealloc(tmem_base, 512);
   }
 }
 
