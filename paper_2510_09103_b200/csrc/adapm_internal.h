@@ -174,6 +174,7 @@ enum LaunchKind : int32_t {
   LK_TC_CONVERT, LK_TC_GRAM, LK_TC_PANEL, LK_TC_APPLY,
   LK_REDUCE_ROWS,       // reduce_final over the row sums of g^2 that the first refit pass left
   LK_GRADNORM,          // global gradient norm and the clip factor
+  LK_TC_PAD,            // gradients whose rows do not start on 16 bytes -> padded copies
   LK_TC_COPY,           // previous split copy of L -> final set (steps that hold L)
   LK_SPD_INVERSE,       // damped inverses of the r x r Gram matrices (preconditioned passes)
   LK_FP32_GRAM,         // the r x r matrices of an exact-fp32 refit pass

@@ -929,6 +929,7 @@ extern "C" const char* adapm_launch_kind_name(int32_t kind) {
     case LK_REDUCE_ROWS: return "reduce_rows";
     case LK_GRADNORM: return "grad_norm";
     case LK_TC_COPY: return "tc_copy";
+    case LK_TC_PAD: return "tc_pad";
     case LK_STREAM: return "stream_update";
     case LK_GEMM: return "gemm_simt";
     case LK_FP32_GRAM: return "fp32_gram";

@@ -1,6 +1,7 @@
 // Tensor-core (tcgen05) low-rank path: the per-step program of Algorithm 2's refit and of the
-// corrected update for every low-rank block whose layout the TMA engine can address
-// (bf16 gradients, cols a multiple of 8).
+// corrected update for the low-rank blocks with bf16 gradients and ranks up to 256.
+// The TMA engine wants rows that start on 16 bytes (cols a multiple of 8): gradients of other blocks are copied once
+// per step into a padded array of the workspace, from which the refit reads them.
 //
 // Per block the workspace holds three split-bf16 copies ("sets") of the factors, [L hi | L lo]
 // (rows x 2 half) and [R^T hi | R^T lo] (cols x 2 half): X and Y side by side in one array of row
@@ -97,6 +98,33 @@ __global__ void __launch_bounds__(256) tc_convert_kernel(const ConvertJob* __res
   }
 }
 
+struct PadJob {
+  int64_t src_off, dst_off;   // element offsets in the gradients and (bf16) in the workspace
+  int32_t rows, cols, ld;     // ld: row pitch of the copy, a multiple of 8
+  int32_t row_ctas;           // CTAs per row
+  int64_t first_cta;
+};
+constexpr int kPadChunk = 2048;   // columns per CTA
+
+// Rows of any alignment into rows that start on 16 bytes: 16 bytes out per thread, from eight 2-byte reads that neighbour
+// threads' reads complete to whole sectors.  Bound by memory: 4 bytes per element, 0.02 ms for 22 M elements.
+__global__ void __launch_bounds__(256) tc_pad_kernel(const PadJob* __restrict__ jobs, const int32_t* __restrict__ cta_job,
+                                                     const uint16_t* __restrict__ grads, uint16_t* __restrict__ work,
+                                                     const int32_t* __restrict__ status) {
+  if (*status != 0) return;
+  const PadJob J = jobs[cta_job[blockIdx.x]];
+  const int64_t q = (int64_t)blockIdx.x - J.first_cta;
+  const int64_t row = q / J.row_ctas;
+  const int col = (int)(q - row * J.row_ctas) * kPadChunk + 8 * (int)threadIdx.x;
+  if (col >= J.ld) return;
+  const uint16_t* src = grads + J.src_off + row * J.cols + col;
+  uint32_t h[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) h[e] = col + e < J.cols ? (uint32_t)src[e] : 0u;
+  *reinterpret_cast<uint4*>(work + J.dst_off + row * J.ld + col) =
+      make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+}
+
 struct CopyJob {
   int64_t src_off, dst_off;   // bf16 element offsets in the workspace
   int32_t rows, width;        // width in elements (a multiple of 8)
@@ -130,6 +158,8 @@ struct TcBlock {
   int32_t rp, half;
   int64_t lc[3], rtc[3], gs[4];    // bf16 element offsets in the workspace; sets 0 = X, 1 = Y, 2 = Z
   int32_t ld[3];                   // row pitch of set s of lc / rtc, in elements
+  int64_t gpad;                    // bf16 element offset of the padded copy of the gradient, or -1
+  int32_t ldg;                     // row pitch of the gradient the refit reads
   int64_t rowsum;                  // float offset of the row sums of g^2 in the workspace, or -1
   // preconditioned passes: split copies of L S_L and (S_R R)^T (pitch 2 half), and in floats the Gram matrices
   // R R^T, L^T L (gf, gf + r^2), their damped inverses (sf, sf + r^2) and the fp32 products L S_L, S_R R
@@ -189,7 +219,10 @@ bool tensor_path_block_ok(const adapm_hparams& hp, const adapm_block& b) {
   if (hp.lowrank_path == ADAPM_PATH_SIMT) return false;
   if (hp.grad_dtype != ADAPM_GRAD_BF16) return false;
   if (b.mom_mode != ADAPM_MOM_LOWRANK) return false;
-  if (b.cols % 8 != 0 || b.rank > 256) return false;   // 2 rp accumulator columns per panel, 512 in all
+  if (b.rank > 256) return false;                      // 2 rp accumulator columns per panel, 512 in all
+  // rows that do not start on 16 bytes: by way of a padded copy of the gradient, unless the caller asked for the tensor
+  // path as it is (its 2 bytes per element of workspace are not what that asks for) or for the preconditioned passes
+  if (b.cols % 8 != 0 && (hp.lowrank_path == ADAPM_PATH_TENSOR || hp.inner_precond)) return false;
   return tc::encode_tiled_fn() != nullptr;
 }
 
@@ -394,6 +427,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     t.ld[0] = t.ld[1] = 4 * t.half; t.ld[2] = 2 * t.half;
     for (int w = 0; w < 4; ++w) t.gs[w] = take((int64_t)2 * t.half * 2 * t.half);
     t.rowsum = -1;
+    t.gpad = -1;
+    t.ldg = (b.cols + 7) / 8 * 8;
     if (hp.inner_precond) {
       auto take_f = [&](int64_t floats) { const int64_t off = work_cursor; work_cursor += round_up(floats, kStateAlign); return off; };
       t.lct = take((int64_t)b.rows * 2 * t.half);
@@ -406,6 +441,10 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     P->blk.push_back(t);
   }
   P->work_end = work_cursor;
+  for (TcBlock& t : P->blk) {          // (rewritten every step: not part of what a rebuild of the split copies zeroes)
+    const adapm_block& b = c->blocks[t.id];
+    if (b.cols % 8 != 0 && K_eff > 0) t.gpad = take((int64_t)b.rows * t.ldg);
+  }
   // row sums of g^2 of the blocks with group scalars: written by the first refit pass, folded into v by a
   // reduction whose "partial sums" are the rows of a group
   for (TcBlock& t : P->blk) {
@@ -443,6 +482,24 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   P->smem_engine = std::max(P->engine_config(n_pan).smem, P->engine_config(gram_na).smem);
 
   auto& prog = c->program;
+
+  // ---- padded copies of the gradients whose rows do not start on 16 bytes --------------------------------
+  {
+    std::vector<PadJob> jobs;
+    std::vector<int32_t> cta_job;
+    for (const TcBlock& t : P->blk) {
+      if (t.gpad < 0) continue;
+      const adapm_block& b = c->blocks[t.id];
+      PadJob j{b.offset, t.gpad, b.rows, b.cols, t.ldg, (t.ldg + kPadChunk - 1) / kPadChunk, (int64_t)cta_job.size()};
+      cta_job.insert(cta_job.end(), (size_t)b.rows * j.row_ctas, (int32_t)jobs.size());
+      jobs.push_back(j);
+    }
+    if (!jobs.empty()) {
+      Launch L{LK_TC_PAD, append_items(c->h_tables, jobs), (int64_t)jobs.size(), (int64_t)cta_job.size()};
+      L.aux0 = append_items(c->h_tables, cta_job);
+      prog.push_back(L);
+    }
+  }
 
   // ---- convert -------------------------------------------------------------------------------------------
   // into the set that is "previous" at the step's parity; without refit passes the "final" factors are the
@@ -789,14 +846,18 @@ int tensor_prepare_step(adapm_ctx* c, const Bases& b, int64_t t, cudaStream_t s,
     CUtensorMap* m = slot->h_maps.data() + bi * kMapsPerBlock;
     const uint64_t rows = blk.rows, cols = blk.cols, half = t2.half;
     const uint32_t nb = (uint32_t)((2 * half + 63) / 64);
-    bool ok = tc::encode_bf16_matrix(&m[MAP_G], grads + blk.offset * 2, rows, cols, cols, 128);
-    ok = ok && tc::encode_bf16_matrix(&m[MAP_GT], grads + blk.offset * 2, rows, cols, cols, sk);
-    ok = ok && tc::encode_panel32(&m[MAP_W], params + blk.offset * 4, rows, cols, true);
-    ok = ok && tc::encode_panel32(&m[MAP_G32], grads + blk.offset * 2, rows, cols, false);
-    if (blk.v_mode == ADAPM_V_ELEMENT)
+    const bool aligned = cols % 8 == 0;           // else W, g, v and the bf16 copy are not reached by TMA
+    std::memset(m, 0, kMapsPerBlock * sizeof(CUtensorMap));
+    const char* g = t2.gpad >= 0 ? work + t2.gpad * 2 : grads + blk.offset * 2;
+    bool ok = true;
+    if (aligned || t2.gpad >= 0) {
+      ok = ok && tc::encode_bf16_matrix(&m[MAP_G], g, rows, cols, t2.ldg, 128);
+      ok = ok && tc::encode_bf16_matrix(&m[MAP_GT], g, rows, cols, t2.ldg, sk);
+    }
+    ok = ok && (!aligned || tc::encode_panel32(&m[MAP_W], params + blk.offset * 4, rows, cols, true));
+    ok = ok && (!aligned || tc::encode_panel32(&m[MAP_G32], grads + blk.offset * 2, rows, cols, false));
+    if (aligned && blk.v_mode == ADAPM_V_ELEMENT)
       ok = ok && tc::encode_panel32(&m[MAP_V], state + c->v_off[t2.id] * 4, rows, cols, true);
-    else
-      std::memset(&m[MAP_V], 0, sizeof(CUtensorMap));
     for (int q = 0; q < 3; ++q) {
       const uint64_t ld = (uint64_t)t2.ld[q];
       ok = ok && tc::encode_bf16_matrix(&m[MAP_LC + q], work + t2.lc[q] * 2, rows, 2 * half, ld, 128);
@@ -811,13 +872,9 @@ int tensor_prepare_step(adapm_ctx* c, const Bases& b, int64_t t, cudaStream_t s,
     if (c->hp.inner_precond) {
       ok = ok && tc::encode_bf16_chunked(&m[MAP_LCN_T], work + t2.lct * 2, rows, 2 * half, nb, sk);
       ok = ok && tc::encode_bf16_chunked(&m[MAP_RTCN_T], work + t2.rtct * 2, cols, 2 * half, nb, sk);
-    } else {
-      std::memset(&m[MAP_LCN_T], 0, 2 * sizeof(CUtensorMap));
     }
-    if (b.shadow)
+    if (aligned && b.shadow)
       ok = ok && tc::encode_panel32(&m[MAP_SH], reinterpret_cast<const char*>(b.shadow) + blk.offset * 2, rows, cols, false);
-    else
-      std::memset(&m[MAP_SH], 0, sizeof(CUtensorMap));
     for (int q = 0; q < 4; ++q)
       ok = ok && tc::encode_bf16_chunked(&m[MAP_GS + q], work + t2.gs[q] * 2, 2 * half, 2 * half, nb, sk);
     if (!ok) {
@@ -854,6 +911,10 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       tc_convert_kernel<<<(unsigned)L.grid, 256, 0, s>>>((const ConvertJob*)tab, (int)L.n_items, L.aux0,
                                                         (const float*)b.p[BASE_WORK], (uint16_t*)b.p[BASE_WORK],
                                                         c->d_status);
+      break;
+    case LK_TC_PAD:
+      tc_pad_kernel<<<(unsigned)L.grid, 256, 0, s>>>((const PadJob*)tab, (const int32_t*)(c->d_tables + L.aux0),
+                                                    (const uint16_t*)b.p[BASE_GRADS], (uint16_t*)b.p[BASE_WORK], c->d_status);
       break;
     case LK_TC_COPY:
       tc_copy_kernel<<<(unsigned)L.grid, 256, 0, s>>>((const CopyJob*)tab, (int)L.n_items, L.aux0,

@@ -52,3 +52,25 @@ def test_exact_fp32_refit_by_number_of_passes(iters, period):
     """K = 1 has no effective pass, K = 2 a single one that ends in the workspace, K = 3 two."""
     _follow([(150, 77, A.MOM_LOWRANK, 12, A.V_BLOCKMEAN, 1), (64, 264, A.MOM_LOWRANK, 5, A.V_BLOCKMEAN, 0)], dtype="f32",
             steps=5, inner_iters=iters, refresh_period=period)
+
+
+@pytest.mark.parametrize("vmode", [A.V_BLOCKMEAN, A.V_ELEMENT])
+@pytest.mark.parametrize("cols,rank", [(257, 12), (2049, 20), (1366, 128), (333, 160), (513, 209)])
+def test_bf16_gradients_whose_rows_do_not_start_on_16_bytes(cols, rank, vmode):
+    """The refit reads a padded copy, the apply kernel the gradient itself; beside an aligned block, with clipping and the
+    bf16 copy of the parameters."""
+    import torch
+    blocks = _blocks([(300, cols, A.MOM_LOWRANK, rank, vmode, 0 if vmode == A.V_ELEMENT else 1),
+                      (264, 264, A.MOM_LOWRANK, 16, vmode, 0 if vmode == A.V_ELEMENT else 8)])
+    run = ParityRun(WL.Workload("odd_rows", [], "bf16", "normal", steps=4), True, custom_blocks=blocks, shadow=True,
+                    hp_overrides=dict(max_grad_norm=0.5))
+    try:
+        for _ in range(4):
+            run.step()
+            run.compare()
+            for blk in run.blocks:
+                sl = slice(blk.offset, blk.offset + blk.rows * blk.cols)
+                assert torch.equal(run.shadow[sl], run.params[sl].to(torch.bfloat16))
+        assert run.ctx.adapm_get_status() == 0
+    finally:
+        run.close()
