@@ -413,7 +413,7 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
   }
   c->n_tensor_blocks = (int64_t)tc_ids.size();
 
-  // ---- state layout: [L,R of the CUDA-core low-rank blocks][L,R of the tensor-core ones]
+  // ---- state layout: [L,R of the low-rank blocks TMA cannot address in place][L,R of the others]
   //                    [m^f of every full block][v of every block] --------------------------------------
   c->m_off.assign(n, -1); c->l_off.assign(n, -1); c->r_off.assign(n, -1); c->v_off.assign(n, -1); c->v_cnt.assign(n, 0);
   int64_t cur = 0;
@@ -424,9 +424,16 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     c->bytes_L += (size_t)b.rows * b.rank * 4;
     c->bytes_R += (size_t)b.rank * b.cols * 4;
   };
-  for (int64_t i : lowrank_ids) place_factors(i);
-  c->lr_section_floats = cur;
-  for (int64_t i : tc_ids) place_factors(i);
+  // The layout does not depend on which kernels a block runs on today: blocks that TMA cannot address in place come
+  // first whether they take the CUDA-core path or a padded copy, so that checkpoints stay readable.
+  auto in_place = [&](const adapm_block& b) { return b.cols % 8 == 0 && tensor_path_block_ok(*hp, b); };
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i = 0; i < n; ++i) {
+      const adapm_block& b = c->blocks[i];
+      if (b.mom_mode == ADAPM_MOM_LOWRANK && in_place(b) == (pass == 1)) place_factors(i);
+    }
+    if (pass == 0) c->lr_section_floats = cur;
+  }
   for (int i = 0; i < n; ++i) {
     const adapm_block& b = c->blocks[i];
     if (b.mom_mode != ADAPM_MOM_FULL) continue;
