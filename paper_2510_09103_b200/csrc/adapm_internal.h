@@ -63,7 +63,7 @@ struct StreamBlk {
   int32_t units_per_group;  // SV_GROUP_READY: units a group is cut into (else 1)
   int64_t n_units;
   int32_t v_mode;        // StreamVMode
-  int32_t team;          // 32: one warp per unit (8 units per CTA); 256: one CTA per unit
+  int32_t team;          // threads per unit: 32, 64, 128 or 256 (256 / team units per CTA)
   int32_t vec_ok;        // units start on 16-byte boundaries
   int32_t pad_;
   float lr_scale, wd;
@@ -201,7 +201,7 @@ struct Launch {
 // kernel launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------------------------
 // `status` is the device status word: a kernel that finds it set writes nothing (an earlier launch gave up).
-int launch_stream(const StreamBlk* d_tab, const int32_t* d_cta_blk, int64_t grid, const Bases& b,
+int launch_stream(const StreamBlk* d_tab, const int32_t* d_cta_blk, int64_t grid, bool teams, const Bases& b,
                   const StepScalars& sc, int grad_dtype, cudaStream_t s);
 int launch_reduce_partial(const ReduceJob* d_tab, const int32_t* d_cta_job, int64_t n_jobs, int64_t n_units, const void* grads,
                           float* work, int grad_dtype, const int32_t* status, cudaStream_t s);

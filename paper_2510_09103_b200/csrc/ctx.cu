@@ -508,7 +508,8 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
       s.v_mode = SV_ELEMENT; s.team = 32; s.unit_elems = kWarpUnitMax;
       s.n_units = (numel + kWarpUnitMax - 1) / kWarpUnitMax; s.vec_ok = 1;
     } else if (group_elems <= kCtaUnitMax) {
-      s.v_mode = SV_GROUP_INLINE; s.team = group_elems <= kWarpUnitMax ? 32 : 256;
+      s.v_mode = SV_GROUP_INLINE;
+      s.team = group_elems <= kWarpUnitMax ? 32 : 256;
       s.unit_elems = (int32_t)group_elems; s.n_units = n_groups;
       s.vec_ok = (group_elems % kChunkElems == 0 || n_groups == 1) ? 1 : 0;
     } else {
@@ -518,9 +519,26 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
       s.vec_ok = (group_elems % kChunkElems == 0 || n_groups == 1) ? 1 : 0;
       add_reduce_job(rset_all, i, group_elems, n_groups);
     }
-    s.first_cta = cta_cursor;
-    cta_cursor += s.team == 32 ? (s.n_units + 7) / 8 : s.n_units;
     sblk.push_back(s);
+  }
+  // Groups of 2049 to 8192 elements (rows of wide models) in teams that just hold them, where they are a good part of the
+  // set: a CTA per row of 4096 left three quarters of its registers empty and ran at 3.4 TB/s, two warps per row 6.1.
+  bool stream_teams = false;
+  {
+    int64_t wide = 0, all = 0;
+    auto is_wide = [](const StreamBlk& s) { return s.v_mode == SV_GROUP_INLINE && s.team == 256 && s.group_elems <= kCtaUnitMax / 2; };
+    for (const StreamBlk& s : sblk) {
+      all += s.numel;
+      if (is_wide(s)) wide += s.numel;
+    }
+    stream_teams = wide > all / 16;
+    if (stream_teams)
+      for (StreamBlk& s : sblk)
+        if (is_wide(s)) s.team = s.group_elems <= kCtaUnitMax / 4 ? 64 : 128;
+  }
+  for (StreamBlk& s : sblk) {
+    s.first_cta = cta_cursor;
+    cta_cursor += (s.n_units + 256 / s.team - 1) / (256 / s.team);
   }
 
   // Group sums of g^2 of the low-rank blocks come from the reduction kernels, except on the tensor path when
@@ -587,6 +605,7 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     }
     Launch SL{LK_STREAM, off, (int64_t)sblk.size(), cta_cursor};
     SL.aux0 = append_table(c->h_tables, cta_blk);
+    SL.aux1 = stream_teams ? 1 : 0;
     prog.push_back(SL);
   }
 
@@ -867,7 +886,8 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
                                  c->d_gscale, s);
         break;
       case LK_STREAM:
-        rc = launch_stream((const StreamBlk*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, b, sc, hp.grad_dtype, s);
+        rc = launch_stream((const StreamBlk*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, L.aux1 != 0, b, sc,
+                           hp.grad_dtype, s);
         break;
       case LK_SPD_INVERSE:
         rc = launch_spd_inverse((const InverseJob*)tab, L.n_items, work, hp.precond_damping, c->d_status, s); break;

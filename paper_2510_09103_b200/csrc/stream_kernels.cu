@@ -5,9 +5,11 @@
 //   v  <- beta2 v + (1-beta2) g^2            (per element, or once per group with the group mean of g^2)
 //   m  <- beta1 m + (1-beta1) g              (full-momentum blocks only; m^c = m, else m^c = g)
 //   W  <- W - lr s_b ( clamp( m^c / (sqrt(v)+eps) ) + lambda_b W )
-// A work unit (one v group, or a 2048-element chunk) is owned by a team of 32 or 256 threads that
-// keeps the unit's gradient in registers, so g is read from memory exactly once even when the
+// A work unit (one v group, or a 2048-element chunk) is owned by a team of 32, 64, 128 or 256 threads (as
+// few as hold it, 64 elements each: a team's threads all wait for its slowest loads) that keeps the unit's gradient in registers, so g is read from memory exactly once even when the
 // group mean has to be known before any element can be updated.
+#include <type_traits>
+
 #include "adapm_internal.h"
 #include "device_math.cuh"
 
@@ -15,18 +17,24 @@ namespace adapm {
 
 namespace {
 
+// Barrier of the team this thread belongs to.
 template <int TEAM>
-__device__ __forceinline__ float team_sum(float x, float* smem8) {
+__device__ __forceinline__ void team_sync() {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / TEAM), "n"(TEAM) : "memory");
+}
+
+// smem: 12 floats of the team's own
+template <int TEAM>
+__device__ __forceinline__ float team_sum(float x, float* smem) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   if (TEAM == 32) return x;
-  const int w = threadIdx.x >> 5;
-  __syncthreads();                       // smem8 may still be read from a previous use
-  if ((threadIdx.x & 31) == 0) smem8[w] = x;
-  __syncthreads();
+  const int w = (threadIdx.x % TEAM) >> 5;
+  if ((threadIdx.x & 31) == 0) smem[w] = x;     // (a team works on one unit: the words are written once)
+  team_sync<TEAM>();
   float s = 0.f;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) s += smem8[i];   // same order in every thread
+  for (int i = 0; i < TEAM / 32; ++i) s += smem[i];   // same order in every thread
   return s;
 }
 
@@ -35,7 +43,7 @@ template <typename GT, int TEAM, bool HAS_M, bool HAS_V>
 __device__ __forceinline__ void run_unit(const StreamBlk& B, int64_t unit, float* __restrict__ params,
                                          const typename GT::elem* __restrict__ grads, float* __restrict__ state,
                                          const StepScalars& sc, float* smem8, float gs, uint16_t* __restrict__ shadow) {
-  const int lane = (TEAM == 32) ? (threadIdx.x & 31) : threadIdx.x;
+  const int lane = threadIdx.x % TEAM;
 
   int64_t ustart, group;
   int ulen;
@@ -123,14 +131,9 @@ __device__ __forceinline__ void run_unit(const StreamBlk& B, int64_t unit, float
     // one thread reads the old scalar and writes the new one; everyone else gets it by broadcast
     float v_old = 0.f;
     if (lane == 0) v_old = state[B.v_off + group];
+    if (TEAM > 32 && lane == 0) smem8[8] = v_old;
     const float tot = team_sum<TEAM>(ss, smem8);
-    if (TEAM == 32) {
-      v_old = __shfl_sync(0xffffffffu, v_old, 0);
-    } else {
-      if (threadIdx.x == 0) smem8[8] = v_old;
-      __syncthreads();
-      v_old = smem8[8];
-    }
+    v_old = TEAM == 32 ? __shfl_sync(0xffffffffu, v_old, 0) : smem8[8];
     v_group = sc.beta2 * v_old + (1.f - sc.beta2) * ((gs * gs) * (tot / (float)ulen));
     if (lane == 0) state[B.v_off + group] = v_group;
   } else if (B.v_mode == SV_GROUP_READY) {
@@ -222,7 +225,9 @@ __device__ __forceinline__ void run_unit_any(const StreamBlk& B, int64_t unit, f
   }
 }
 
-template <typename GT>
+// kTeams: the launch has units of 64 or 128 threads.  (Their code in the kernel costs the others some 5 %, so sets without
+// such units take the form that does not have it.)
+template <typename GT, bool kTeams>
 __global__ void __launch_bounds__(256, 2) stream_update_kernel(const StreamBlk* __restrict__ tab,
                                                                const int32_t* __restrict__ cta_blk,
                                                                float* __restrict__ params,
@@ -232,7 +237,7 @@ __global__ void __launch_bounds__(256, 2) stream_update_kernel(const StreamBlk* 
                                                                const float* __restrict__ gscale,
                                                                uint16_t* __restrict__ shadow) {
   __shared__ StreamBlk sB;
-  __shared__ float smem8[12];
+  __shared__ float team_smem[4][12];
   if (threadIdx.x == 0) {
     sB = tab[cta_blk[blockIdx.x]];                       // which block this CTA works on
     if (*status != 0) sB.team = 0;                       // an earlier launch gave up: write nothing
@@ -240,12 +245,16 @@ __global__ void __launch_bounds__(256, 2) stream_update_kernel(const StreamBlk* 
   __syncthreads();
   const int64_t cta_local = (int64_t)blockIdx.x - sB.first_cta;
   const float gs = gscale ? __ldg(gscale) : 1.f;
-  if (sB.team == 32) {
-    const int64_t unit = cta_local * 8 + (threadIdx.x >> 5);
-    if (unit < sB.n_units) run_unit_any<GT, 32>(sB, unit, params, grads, state, sc, smem8, gs, shadow);
-  } else if (sB.team == 256) {
-    run_unit_any<GT, 256>(sB, cta_local, params, grads, state, sc, smem8, gs, shadow);
-  }
+  auto run = [&](auto team_t) {
+    constexpr int kTeam = decltype(team_t)::value;
+    const int64_t unit = cta_local * (256 / kTeam) + (int)threadIdx.x / kTeam;
+    if (unit < sB.n_units)
+      run_unit_any<GT, kTeam>(sB, unit, params, grads, state, sc, team_smem[kTeam == 32 ? 0 : threadIdx.x / kTeam], gs, shadow);
+  };
+  if (sB.team == 32) run(std::integral_constant<int, 32>());
+  else if (kTeams && sB.team == 64) run(std::integral_constant<int, kTeams ? 64 : 32>());
+  else if (kTeams && sB.team == 128) run(std::integral_constant<int, kTeams ? 128 : 32>());
+  else if (sB.team == 256) run(std::integral_constant<int, 256>());
 }
 
 // ---- group sums of squares ---------------------------------------------------------------------
@@ -477,19 +486,17 @@ __global__ void __launch_bounds__(256) copy_ranges_kernel(const NormRange* __res
     }                                                \
   } while (0)
 
-int launch_stream(const StreamBlk* d_tab, const int32_t* d_cta_blk, int64_t grid, const Bases& b,
+int launch_stream(const StreamBlk* d_tab, const int32_t* d_cta_blk, int64_t grid, bool teams, const Bases& b,
                   const StepScalars& sc, int grad_dtype, cudaStream_t s) {
   if (grid <= 0) return ADAPM_OK;
+  auto launch = [&](auto kernel, auto* grads) {
+    kernel<<<(unsigned)grid, 256, 0, s>>>(d_tab, d_cta_blk, (float*)b.p[BASE_PARAMS], grads, (float*)b.p[BASE_STATE], sc,
+                                          b.status, b.gscale, b.shadow);
+  };
   if (grad_dtype == ADAPM_GRAD_BF16)
-    stream_update_kernel<GradBF16><<<(unsigned)grid, 256, 0, s>>>(d_tab, d_cta_blk, (float*)b.p[BASE_PARAMS],
-                                                                 (const uint16_t*)b.p[BASE_GRADS],
-                                                                 (float*)b.p[BASE_STATE], sc, b.status, b.gscale,
-                                                                 b.shadow);
+    launch(teams ? stream_update_kernel<GradBF16, true> : stream_update_kernel<GradBF16, false>, (const uint16_t*)b.p[BASE_GRADS]);
   else
-    stream_update_kernel<GradF32><<<(unsigned)grid, 256, 0, s>>>(d_tab, d_cta_blk, (float*)b.p[BASE_PARAMS],
-                                                                (const float*)b.p[BASE_GRADS],
-                                                                (float*)b.p[BASE_STATE], sc, b.status, b.gscale,
-                                                                b.shadow);
+    launch(teams ? stream_update_kernel<GradF32, true> : stream_update_kernel<GradF32, false>, (const float*)b.p[BASE_GRADS]);
   ADAPM_LAUNCH_CHECK();
   return ADAPM_OK;
 }

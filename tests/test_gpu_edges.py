@@ -74,3 +74,11 @@ def test_bf16_gradients_whose_rows_do_not_start_on_16_bytes(cols, rank, vmode):
         assert run.ctx.adapm_get_status() == 0
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_streaming_update_at_the_edges_of_its_teams(dtype):
+    """Groups that one, two, four and eight warps hold, and one element more and less."""
+    sizes = [2047, 2048, 2049, 4096, 4097, 4104, 8192, 8200, 16384, 16385]
+    _follow([(5 if n % 2 else 6, n, A.MOM_FULL if i % 3 else A.MOM_NONE, 0, A.V_BLOCKMEAN, 1)
+             for i, n in enumerate(sizes)], dtype=dtype)
