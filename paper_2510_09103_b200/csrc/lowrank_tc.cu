@@ -939,7 +939,7 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
         ADAPM_CUDA(cudaMemsetAsync(P->d_team_counters, 0, P->n_teams * sizeof(int32_t), s));
         a.team_counters = P->d_team_counters;
       }
-      tc::tc_items_kernel<<<(unsigned)L.grid, tc::kEngineThreads, e.smem, s>>>(a);
+      launch_chained(c->step_bytes < kChainedBytes, tc::tc_items_kernel, (unsigned)L.grid, tc::kEngineThreads, e.smem, s, a);
       break;
     }
     case LK_TC_APPLY: {
@@ -955,7 +955,7 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       a.buf_bytes = P->apply_buf_bytes;
       a.gscale = b.gscale;
       a.shadow = b.shadow != nullptr;
-      apply_kernel(L.aux0 != 0, L.aux1 != 0)<<<(unsigned)L.grid, tc::kApplyThreads, e.smem, s>>>(a);
+      launch_chained(c->step_bytes < kChainedBytes, apply_kernel(L.aux0 != 0, L.aux1 != 0), (unsigned)L.grid, tc::kApplyThreads, e.smem, s, a);
       break;
     }
     default:

@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(256) reduce_final_kernel(const ReduceJob* __re
                                                            const int32_t* __restrict__ status,
                                                            const float* __restrict__ gscale) {
   // groups are taken 32 at a time by a warp; inside the 32, jobs with small groups go lane by lane
+  wait_for_previous_kernel();
   const int64_t g0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
   if (g0 >= n_groups || *status != 0) return;
   const int lane = threadIdx.x & 31;
@@ -516,10 +517,10 @@ int launch_reduce_partial(const ReduceJob* d_tab, const int32_t* d_cta_job, int6
 }
 
 int launch_reduce_final(const ReduceJob* d_tab, int64_t n_jobs, int64_t n_groups, float* state, const float* work,
-                        float beta2, const int32_t* status, const float* gscale, cudaStream_t s) {
+                        float beta2, const int32_t* status, const float* gscale, bool chained, cudaStream_t s) {
   if (n_groups <= 0) return ADAPM_OK;
-  reduce_final_kernel<<<(unsigned)((n_groups + 255) / 256), 256, 0, s>>>(d_tab, (int)n_jobs, n_groups, state, work, beta2,
-                                                                        status, gscale);
+  launch_chained(chained, reduce_final_kernel, (unsigned)((n_groups + 255) / 256), 256, 0, s, d_tab, (int)n_jobs, n_groups, state, work,
+                 beta2, status, gscale);
   ADAPM_LAUNCH_CHECK();
   return ADAPM_OK;
 }

@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   extern __shared__ uint8_t dyn_smem[];
   __shared__ ApplyShared sh;
   __shared__ int skip_launch;
+  wait_for_previous_kernel();
   if (threadIdx.x == 0) skip_launch = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   __syncthreads();
   if (skip_launch) return;   // an earlier launch of the step gave up: leave W and v untouched

@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
   extern __shared__ uint8_t dyn_smem[];
   __shared__ EngineShared sh;
   __shared__ int skip_launch;
+  wait_for_previous_kernel();
   if (threadIdx.x == 0) skip_launch = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
   __syncthreads();
   if (skip_launch) return;   // an earlier launch gave up: write nothing (the whole CTA decides together)
