@@ -300,6 +300,10 @@ def kernel_algorithmic_work(kind: str, blocks, gsz: int, k_eff: int):
         # averaged over the 4 GEMM launches of one refit pass: (4 m n r + 8 r^2 (m + n)) / 4
         fl = sum(4.0 * nb(b) * b.rank + 8.0 * b.rank * b.rank * (b.rows + b.cols) for b in lowr) / 4.0
         return "alu", fl, "flops"
+    if kind == "fp32_refit":
+        # one refit pass on CUDA cores: both products with g and the two r x r products of each factor's update
+        fl = sum(4.0 * nb(b) * b.rank + 4.0 * b.rank * b.rank * (b.rows + b.cols) for b in lowr)
+        return "alu", fl, "flops"
     if kind == "tc_panel":
         # One refit pass is a contraction: g R^T and L^T g, 4 m n r flops per block (the doubling by the hi/lo
         # operand split and the small r x r products are the kernel's own and not counted).
