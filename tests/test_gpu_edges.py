@@ -1,4 +1,5 @@
 """Sizes where a kernel variant or a dispatch rule changes, against the oracle."""
+import numpy as np
 import pytest
 
 import workloads as WL
@@ -82,3 +83,77 @@ def test_streaming_update_at_the_edges_of_its_teams(dtype):
     sizes = [2047, 2048, 2049, 4096, 4097, 4104, 8192, 8200, 16384, 16385]
     _follow([(5 if n % 2 else 6, n, A.MOM_FULL if i % 3 else A.MOM_NONE, 0, A.V_BLOCKMEAN, 1)
              for i, n in enumerate(sizes)], dtype=dtype)
+
+
+# rows x cols of a block whose parameters move by TMA, of one whose rows start at any element, and the CUDA-core path
+UPDATE_FORMS = [(200, 264, A.PATH_TENSOR), (200, 267, A.PATH_AUTO), (200, 267, A.PATH_SIMT)]
+
+
+def _one_block(rows, cols, path, **hp):
+    """A low-rank block with a per-element v, frozen factors and a step that writes -lr * ratio over W = 0."""
+    import torch
+    blocks = [A.adapm_block(0, rows, cols, A.MOM_LOWRANK, 3, A.V_ELEMENT, 0, 1.0, 0.0)]
+    ctx = A.adapm_create(blocks, A.hparams(lr=1.0, grad_dtype=A.GRAD_BF16, inner_iters=0, lowrank_path=path, **hp))
+    state = torch.zeros(ctx.adapm_state_bytes() // 4, device="cuda")
+    work = torch.zeros(max(ctx.adapm_workspace_bytes() // 4, 1), device="cuda")
+    ctx.adapm_set_workspace(work)
+
+    def view(which):
+        at, n = ctx.adapm_state_layout(0, which)
+        return state[at:at + n]
+    return ctx, torch.zeros(-(-rows * cols // 8) * 8, device="cuda"), state, view
+
+
+@pytest.mark.parametrize("rows,cols,path", UPDATE_FORMS)
+def test_huge_quotients_are_clamped_and_not_turned_into_nan(rows, cols, path):
+    """m^c = beta1 L R of 1e15 to 1e29 over sqrt(v) + eps of 4e-15: the quotient overflows, the ratio is the clamp's."""
+    import torch
+    ctx, params, state, view = _one_block(rows, cols, path, beta1=0.9, beta2=0.0, eps=1e-20, clip=1.0, correction=0)
+    view(A.STATE_L).view(rows, 3)[:, 0] = 1.0
+    p = 10.0 ** torch.linspace(15, 29, cols, device="cuda")
+    p[1::2] *= -1
+    view(A.STATE_R).view(3, cols)[0] = p
+    grads = torch.full((params.numel(),), 4e-15, dtype=torch.bfloat16, device="cuda")
+    ctx.adapm_step(params, grads, state, 1)
+    got = params[:rows * cols].view(rows, cols).cpu()
+    assert torch.equal(got, -torch.sign(p).cpu().expand(rows, cols))
+    ctx.adapm_destroy()
+
+
+@pytest.mark.parametrize("rows,cols,path", UPDATE_FORMS)
+@pytest.mark.parametrize("t", [1, 2, 7])
+@pytest.mark.parametrize("eps", [0.0, 1e-8])
+@pytest.mark.parametrize("v_lo,v_hi,g_lo,g_hi", [(-14, -3, -8, 0), (-29.9, 29.9, -6, 6), (-31, -29, -20, -14),
+                                                 (29, 31, -3, 19), (-45, -36, -20, -18)])
+def test_root_and_quotient_of_the_update_against_the_functions(rows, cols, path, t, eps, v_lo, v_hi, g_lo, g_hi):
+    """W = 0, lr = 1, no decay, no clamp, frozen zero factors: the step writes -(g b1) / (sqrt(v b2) + eps) with b1, b2
+    the bias corrections of step t, and leaves v.  The same in numpy's fp32, whose root and quotient are rounded to
+    nearest as CUDA's sqrtf and / are, has to agree to the last bit but one; in 64 bits, to the roundings of g b1, v b2,
+    the root, the sum and the quotient, half an ulp each of them or of what they carry into the quotient (an ulp is up to
+    2^-23 of the value, the root halves what v b2 carries): 4.5 half ulps."""
+    import torch
+    ctx, params, state, view = _one_block(rows, cols, path, beta1=0.9, beta2=0.95, eps=eps, clip=float("inf"), adam_debias=1)
+    gen = torch.Generator(device="cuda").manual_seed(17 + t)
+    n = rows * cols
+
+    def log_uniform(lo, hi):
+        return 10.0 ** (torch.rand(n, generator=gen, device="cuda", dtype=torch.float64) * (hi - lo) + lo)
+    grads = torch.zeros(params.numel(), dtype=torch.bfloat16, device="cuda")
+    grads[:n] = (log_uniform(g_lo, g_hi) * (2.0 * torch.randint(0, 2, (n,), generator=gen, device="cuda") - 1)).to(torch.bfloat16)
+    view(A.STATE_V).copy_(log_uniform(v_lo, v_hi).float())
+    ctx.adapm_step(params, grads, state, t)
+    got = -params[:n].cpu().numpy()
+    v, g = view(A.STATE_V).cpu().numpy(), grads[:n].float().cpu().numpy()
+    ctx.adapm_destroy()
+    f = np.float32
+    bc1 = f(1.0 / (1.0 - float(f(0.9)) ** t))
+    bc2 = f(1.0 / (1.0 - float(f(0.95)) ** t))
+    with np.errstate(all="ignore"):
+        want = (g * bc1) / (np.sqrt(v * bc2) + f(eps))
+        exact = g.astype(np.float64) * float(bc1) / (np.sqrt(v.astype(np.float64) * float(bc2)) + float(f(eps)))
+        inside = np.isfinite(want) & (np.abs(want) >= np.finfo(f).tiny) & (v >= np.finfo(f).tiny)
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
+    ulps = np.abs(got[inside].astype(np.float64) - want[inside]) / np.spacing(np.abs(want[inside]))
+    assert ulps.max() <= 1.0
+    rel = np.abs(got[inside] - exact[inside]) / np.abs(exact[inside])
+    assert rel.max() <= 4.5 * 2.0 ** -24
