@@ -383,10 +383,10 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
         const float lr_s = sc.lr * I.lr_scale;
         const int row = I.row0 + rloc;
         const bool rok = row < I.rows;
-        // one denominator per row when v is a group scalar: m^c / (sqrt(v) + eps) becomes a product
+        // one denominator per row when v is a group scalar: m^c / (sqrt(v) + eps) becomes a product.  (m^c first: a group
+        // that never had a gradient has v = 0, and 0 * (1 / 0) + ... would be NaN with eps = 0 where m^c is not zero.)
         const float v_row = (rok && grouped) ? a.state[I.v_off + row / I.v_group_rows] : 0.f;
         const float kr = sc.inv_bc1 / (sqrtf(v_row * sc.inv_bc2) + sc.eps);
-        const float kg = sc.cg * kr, kd = sc.c0 * kr;
         for (int t = 0; t < I.n_tiles && ok; ++t, ++j) {
           const int acc = j & 1;
           // one lane per warp polls, then the warp agrees: the tensor-memory loads need all 32 lanes
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
                 if (grouped) {
 #pragma unroll
                   for (int x = 0; x < 4; ++x) {
-                    const float ratio = clamp_keep_nan(gf[4 * i + x] * kg + d[4 * i + x] * kd, sc.clip);
+                    const float ratio = clamp_keep_nan((sc.cg * gf[4 * i + x] + sc.c0 * d[4 * i + x]) * kr, sc.clip);
                     w[x] = w[x] - lr_s * (ratio + I.wd * w[x]);
                   }
                 } else {

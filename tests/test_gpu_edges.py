@@ -89,10 +89,10 @@ def test_streaming_update_at_the_edges_of_its_teams(dtype):
 UPDATE_FORMS = [(200, 264, A.PATH_TENSOR), (200, 267, A.PATH_AUTO), (200, 267, A.PATH_SIMT)]
 
 
-def _one_block(rows, cols, path, **hp):
-    """A low-rank block with a per-element v, frozen factors and a step that writes -lr * ratio over W = 0."""
+def _one_block(rows, cols, path, vmode=A.V_ELEMENT, **hp):
+    """A low-rank block with frozen factors and a step that writes -lr * ratio over W = 0."""
     import torch
-    blocks = [A.adapm_block(0, rows, cols, A.MOM_LOWRANK, 3, A.V_ELEMENT, 0, 1.0, 0.0)]
+    blocks = [A.adapm_block(0, rows, cols, A.MOM_LOWRANK, 3, vmode, 0 if vmode == A.V_ELEMENT else 1, 1.0, 0.0)]
     ctx = A.adapm_create(blocks, A.hparams(lr=1.0, grad_dtype=A.GRAD_BF16, inner_iters=0, lowrank_path=path, **hp))
     state = torch.zeros(ctx.adapm_state_bytes() // 4, device="cuda")
     work = torch.zeros(max(ctx.adapm_workspace_bytes() // 4, 1), device="cuda")
@@ -117,6 +117,24 @@ def test_huge_quotients_are_clamped_and_not_turned_into_nan(rows, cols, path):
     ctx.adapm_step(params, grads, state, 1)
     got = params[:rows * cols].view(rows, cols).cpu()
     assert torch.equal(got, -torch.sign(p).cpu().expand(rows, cols))
+    ctx.adapm_destroy()
+
+
+@pytest.mark.parametrize("rows,cols,path", UPDATE_FORMS)
+def test_rows_without_a_gradient_move_by_their_momentum_when_eps_is_zero(rows, cols, path):
+    """v = 0 and eps = 0: m^c = beta1 L R over zero is infinite and clamped, as long as m^c is not zero itself."""
+    import torch
+    ctx, params, state, view = _one_block(rows, cols, path, A.V_BLOCKMEAN, beta1=0.9, beta2=0.95, eps=0.0, clip=1.0,
+                                          correction=0)
+    view(A.STATE_L).view(rows, 3)[:, 0] = 1.0
+    p = torch.linspace(-1e-3, 1e-3, cols, device="cuda") + 1e-6
+    view(A.STATE_R).view(3, cols)[0] = p
+    grads = torch.zeros(params.numel(), dtype=torch.bfloat16, device="cuda")
+    grads[:rows // 2 * cols] = 1e-3
+    ctx.adapm_step(params, grads, state, 1)
+    got = params[:rows * cols].view(rows, cols).cpu()
+    assert torch.equal(got[rows // 2:], -torch.sign(p).cpu().expand(rows - rows // 2, cols))
+    assert bool(torch.isfinite(got).all())
     ctx.adapm_destroy()
 
 
