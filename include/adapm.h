@@ -24,7 +24,8 @@
  *   - adapm_step is asynchronous on `stream`, allocates nothing and never synchronises.  One context
  *     is used from one stream at a time.  Part of a step may run on a stream of the context's own; it starts
  *     after what `stream` holds when adapm_step is called and `stream` waits for it, so that the step is ordered
- *     on `stream` like a single kernel.  The first step that sees a new combination of params /
+ *     on `stream` like a single kernel, also when adapm_step returns an error after some of its launches (only where
+ *     the wait itself cannot be enqueued does the host wait instead).  The first step that sees a new combination of params /
  *     grads / state / workspace pointers describes the buffers to the TMA unit on the host (a few
  *     hundred microseconds) and copies that description from pageable memory: make that step
  *     outside any stream capture.  Four combinations are remembered.

@@ -368,6 +368,33 @@ void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std
   work_cursor = scratch_end;
 }
 
+// A step's branch on the context's own stream: however the step ends, the caller's stream waits for it.
+class SideBranch {
+ public:
+  SideBranch(adapm_ctx* c, cudaStream_t main) : c_(c), main_(main) {}
+  ~SideBranch() { (void)join(); }
+  cudaError_t fork() {
+    cudaError_t e = cudaEventRecord(c_->fork_event, main_);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c_->side_stream, c_->fork_event, 0);
+    open_ = e == cudaSuccess;
+    return e;
+  }
+  cudaError_t join() {
+    if (!open_) return cudaSuccess;
+    open_ = false;
+    cudaError_t e = cudaEventRecord(c_->join_event, c_->side_stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(main_, c_->join_event, 0);
+    // without the event the host waits: what the caller enqueues after the error must not overtake the branch
+    if (e != cudaSuccess) (void)cudaStreamSynchronize(c_->side_stream);
+    return e;
+  }
+
+ private:
+  adapm_ctx* c_;
+  cudaStream_t main_;
+  bool open_ = false;
+};
+
 }  // namespace
 
 // the tensor-core program of the low-rank blocks; defined in lowrank_tc.cu
@@ -878,8 +905,8 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
   // on a two-layer set of width 576, 1-2 % at 1 GB, nothing to be had above.  Per-launch profiling times the launches one
   // by one.
   const bool fork = c->side_stream && !prof && c->step_bytes < (size_t)4 << 30;
-  bool forked = false;
   cudaStream_t const main_stream = s;
+  SideBranch branch(c, main_stream);
   size_t li = 0;
   for (const Launch& L : c->program) {
     if ((L.only_convert && !convert) || (L.when == WHEN_EVEN && parity != 0) || (L.when == WHEN_ODD && parity != 1) ||
@@ -905,10 +932,8 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
         break;
       case LK_STREAM:
         if (fork) {
-          ADAPM_CUDA(cudaEventRecord(c->fork_event, main_stream));
-          ADAPM_CUDA(cudaStreamWaitEvent(c->side_stream, c->fork_event, 0));
+          ADAPM_CUDA(branch.fork());
           s = c->side_stream;
-          forked = true;
         }
         rc = launch_stream((const StreamBlk*)tab, (const int32_t*)(c->d_tables + L.aux0), L.grid, L.aux1 != 0, b, sc,
                            hp.grad_dtype, s);
@@ -942,10 +967,7 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
       ADAPM_CUDA(cudaEventRecord(c->prof_events[li], s));
     }
   }
-  if (forked) {
-    ADAPM_CUDA(cudaEventRecord(c->join_event, c->side_stream));
-    ADAPM_CUDA(cudaStreamWaitEvent(main_stream, c->join_event, 0));
-  }
+  ADAPM_CUDA(branch.join());
   c->last_step_launches = (int64_t)li;
   if (prof) c->prof_valid = 1;
   return ADAPM_OK;
