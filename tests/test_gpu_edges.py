@@ -175,3 +175,90 @@ def test_root_and_quotient_of_the_update_against_the_functions(rows, cols, path,
     assert ulps.max() <= 1.0
     rel = np.abs(got[inside] - exact[inside]) / np.abs(exact[inside])
     assert rel.max() <= 4.5 * 2.0 ** -24
+
+
+# a block whose update outlasts the low-rank launches many times over, beside low-rank blocks of both kinds of rows
+FORKED = [(32768, 4096, A.MOM_NONE, 0, A.V_BLOCKMEAN, 1), (264, 264, A.MOM_LOWRANK, 16, A.V_BLOCKMEAN, 8),
+          (300, 267, A.MOM_LOWRANK, 12, A.V_BLOCKMEAN, 1)]
+
+
+class _Copies:
+    """The same steps on one stream, launch after launch (the per-launch events switch the second stream off), and as a user
+    takes them."""
+
+    def __init__(self, dtype, stream, **hp):
+        import torch
+        gd, td = (A.GRAD_F32, torch.float32) if dtype == "f32" else (A.GRAD_BF16, torch.bfloat16)
+        blocks = _blocks(FORKED)
+        n = -(-(blocks[-1].offset + blocks[-1].rows * blocks[-1].cols) // 8) * 8
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        self.given = torch.randn(n, generator=gen, device="cuda").mul_(1e-3).to(td)
+        self.one, self.user = [], []
+        for kept in (self.one, self.user):
+            ctx = A.adapm_create(blocks, A.hparams(grad_dtype=gd, max_grad_norm=1.0, **hp))
+            state = torch.empty(ctx.adapm_state_bytes() // 4, device="cuda")
+            work = torch.zeros(ctx.adapm_workspace_bytes() // 4, device="cuda")
+            ctx.adapm_set_workspace(work)
+            ctx.adapm_state_init(state)
+            kept += [ctx, torch.full((n,), 0.02, device="cuda"), self.given.clone(), state]
+        self.one[0].adapm_set_profiling(True)
+        torch.cuda.synchronize()
+        self.stream, self.t = stream, 0
+
+    def expected(self):
+        import torch
+        ctx, params, grads, state = self.one
+        self.t += 1
+        ctx.adapm_step(params, grads, state, self.t)
+        torch.cuda.synchronize()
+        return params, state
+
+    def close(self):
+        for kept in (self.one, self.user):
+            assert kept[0].adapm_get_status() == 0
+            kept[0].adapm_destroy()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_work_behind_a_step_on_the_callers_stream_waits_for_all_of_it(dtype):
+    """The copies that follow a step see what it wrote, and what overwrites the gradients does not reach it."""
+    import torch
+    stream = torch.cuda.Stream()
+    c = _Copies(dtype, stream)
+    ctx, params, grads, state = c.user
+    for _ in range(3):
+        want_p, want_s = c.expected()
+        with torch.cuda.stream(stream):
+            ctx.adapm_step(params, grads, state, c.t)
+            got_p, got_s = params.clone(), state.clone()
+            grads.zero_()
+            grads.copy_(c.given)
+        stream.synchronize()
+        assert torch.equal(got_p, want_p) and torch.equal(got_s, want_s)
+        torch.cuda.synchronize()
+        assert torch.equal(params, got_p) and torch.equal(state, got_s)
+    c.close()
+
+
+@pytest.mark.parametrize("dtype,flags", [("f32", 0), ("bf16", 0), ("bf16", A.FLAG_FORCE_PANEL_TEAMS)])
+def test_a_step_captured_in_a_graph(dtype, flags):
+    """Two steps, a captured one that is replayed, and one more, against the same steps launch by launch."""
+    import torch
+    stream = torch.cuda.Stream()
+    c = _Copies(dtype, stream, flags=flags)
+    ctx, params, grads, state = c.user
+    for t in (1, 2, 3, 4):
+        want_p, want_s = c.expected()
+        if t == 3:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                ctx.adapm_step(params, grads, state, t)
+            with torch.cuda.stream(stream):
+                graph.replay()
+        else:
+            with torch.cuda.stream(stream):
+                ctx.adapm_step(params, grads, state, t)
+        torch.cuda.synchronize()
+        assert torch.equal(params, want_p) and torch.equal(state, want_s)
+    del graph
+    c.close()
