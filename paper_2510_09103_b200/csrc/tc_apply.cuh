@@ -528,8 +528,9 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
     }
   } else if (!kStream) {
     // ------------------------------------------------------------------ L panel -> tensor memory, one row per thread
-    // The loads of 160 columns are in flight together, and those of an item's first 160 before the tensor memory is
-    // free: the MMAs wait for this between two items (64 columns at a time cost 7 % of the kernel on the 1.5B shapes).
+    // The loads of 64 columns are in flight together, and those of an item's first 64 before the tensor memory is free:
+    // the MMAs wait for this between two items.  (160 columns at a time: 2.86 instead of 2.80 ms on the 1.5B shapes, 6.85
+    // instead of 6.58 with a per-element v, 1.39 instead of 1.36 on the 350M set at rank 128; 32: 2.89, 6.65 and 1.37.)
     const int sub = warp & 3;                                // which 32 lanes of tensor memory this warp may write
     const uint32_t lane_addr = (uint32_t)(32 * sub) << 16;
     uint32_t item_phase = 0;
@@ -541,10 +542,10 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
       const uint16_t* src = a.work + a.items[it].l_off + (int64_t)row * (4 * rp) + (n_sets == 2 ? 0 : a.parity * 2 * rp);
       // the refitted set enters negated
       const int neg0 = n_sets == 2 ? (1 - a.parity) * 2 * rp : width, neg1 = neg0 + 2 * rp;
-      uint4 x[20];
+      uint4 x[8];
       auto fetch = [&](int k0) {
 #pragma unroll
-        for (int i = 0; i < 20; ++i) {
+        for (int i = 0; i < 8; ++i) {
           x[i] = make_uint4(0, 0, 0, 0);
           if (rok && k0 + 8 * i < width) x[i] = *reinterpret_cast<const uint4*>(src + k0 + 8 * i);
         }
@@ -552,9 +553,9 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
       fetch(0);
       if (!mbar_wait_warp(&sh.lempty, item_phase ^ 1u, abort, a.status, ST_WAIT_EMPTY)) break;
       tc_fence_after();
-      for (int k0 = 0; k0 < width; k0 += 160) {
+      for (int k0 = 0; k0 < width; k0 += 64) {
 #pragma unroll
-        for (int i = 0; i < 10; ++i) {
+        for (int i = 0; i < 4; ++i) {
           const int k = k0 + 16 * i;
           if (k < width) {
             const uint32_t flip = k >= neg0 && k < neg1 ? 0x80008000u : 0u;
@@ -563,7 +564,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
             tmem_st8(tmem_base + lane_addr + (uint32_t)(k >> 1), v);
           }
         }
-        if (k0 + 160 < width) fetch(k0 + 160);
+        if (k0 + 64 < width) fetch(k0 + 64);
       }
       tmem_st_wait();
       tc_fence_before();
