@@ -323,7 +323,7 @@ void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std
           u.tn = tn_of(r); u.tiles_n = tiles_of(r);
           u.ga_off = gram(yc);
           u.gb_off = first ? -1 : (hold ? u.ga_off : gram(yp));
-          if (!first && !hold) grams.back().x_base = prev == 0 ? BASE_STATE : BASE_WORK;
+          if (!first && !hold) grams.back().x_base = BASE_WORK;
           const Cut q = cut(K, chunk_refit);
           u.k_chunk = q.k_chunk; u.splits = q.splits;
           const int tiles = u.tiles_n * ((owners + 127) / 128);
