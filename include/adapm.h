@@ -109,9 +109,10 @@ typedef struct {
   int32_t adam_debias;     /* 0 = Algorithm 1 as printed; 1 = divide by 1-beta^t (AdamW check)    */
   int32_t correction;      /* 1 = Eq. 3 on; 0 = ablation, m^c := m_t                               */
   int32_t lowrank_path;    /* ADAPM_PATH_*: which kernels run Algorithm 2's contractions.  AUTO: bf16
-                              gradients and ranks up to 256 on the tensor cores (factors as two bf16 parts),
-                              the rest in fp32; SIMT: all in fp32; TENSOR: refuses what AUTO would run in
-                              fp32 or could only reach through a padded copy (cols not a multiple of 8)  */
+                              gradients and ranks up to 256 on the tensor cores (factors as two bf16 parts,
+                              products good to about 2^-17), the rest in fp32; SIMT: all in fp32; TENSOR:
+                              refuses what AUTO would run in fp32 or could only reach through a padded
+                              copy (cols not a multiple of 8)                                           */
   uint64_t seed;           /* seeds L_0 in adapm_state_init                                        */
   uint32_t flags;          /* ADAPM_FLAG_*; 0 = defaults                                           */
   float   max_grad_norm;   /* global gradient clipping (Section 5.1: threshold 1.0): every gradient is

@@ -257,6 +257,12 @@ void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std
   auto tn_of = [&](int r) { return ((r + tiles_of(r) - 1) / tiles_of(r) + 7) / 8; };
   // K loops are cut so that a launch has about `waves` CTAs per SM and none is much longer than the rest; a chunk is
   // never below 128, where its partial products would cost as much as its share of the gradient.
+  // Measured (us per step of fp32 sets; tiny 176 with every setting: its chunks are 128 long either way):
+  //   waves of the refit launch    3     6     9     12    18       of the gram launch    1     2     4     8     16
+  //   gpt2_124m                    3757  3628  3627  3636  3594                            3712  3644  3629  3600  3616
+  //   12 layers of 768, rank 32    2780  2770  2771  2768  2782                            2916  2802  2770  2759  2774
+  //   6 layers of 512              890   842   838   839   853                             858   838   837   850   849
+  // Fewer leave the last wave uneven, more cost partial products; between 6 and 12, and 4 and 8, it hardly matters.
   struct Cut { int32_t k_chunk, splits; };
   auto cut = [](int K, int64_t chunk) {
     const int64_t n = std::max<int64_t>(1, (K + chunk / 2) / chunk);
@@ -265,7 +271,10 @@ void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std
     q.splits = (K + q.k_chunk - 1) / q.k_chunk;
     return q;
   };
-  constexpr int64_t kSms = 148, kWavesRefit = 9, kWavesGram = 4;
+  constexpr int64_t kWavesRefit = 9, kWavesGram = 4;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    sms = 148;
 
   for (int phase = (with_hold ? 1 : 0); phase <= (with_hold ? 2 : 0); ++phase) {
     const bool hold = phase == 2;
@@ -282,8 +291,8 @@ void build_fp32_program(adapm_ctx* c, const std::vector<int64_t>& ids, const std
         k_refit += tr * ((hold ? 0 : (int64_t)(b.rows + 127) / 128 * b.cols) + (int64_t)(b.cols + 127) / 128 * b.rows);
         k_gram += tg * ((hold ? 0 : (int64_t)b.cols) + b.rows);
       }
-      const int64_t chunk_refit = std::max<int64_t>(128, k_refit / (kSms * kWavesRefit));
-      const int64_t chunk_gram = std::max<int64_t>(128, k_gram / (kSms * kWavesGram));
+      const int64_t chunk_refit = std::max<int64_t>(128, k_refit / (sms * kWavesRefit));
+      const int64_t chunk_gram = std::max<int64_t>(128, k_gram / (sms * kWavesGram));
       std::vector<Fp32Gram> grams;
       std::vector<Fp32Refit> refits;
       int64_t at = scratch, counters = 0;
@@ -549,7 +558,10 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     sblk.push_back(s);
   }
   // Groups of 2049 to 8192 elements (rows of wide models) in teams that just hold them, where they are a good part of the
-  // set: a CTA per row of 4096 left three quarters of its registers empty and ran at 3.4 TB/s, two warps per row 6.1.
+  // set: a CTA per row of 4096 left three quarters of its registers empty and ran at 3.4 TB/s, two warps per row 6.1.  The
+  // kernel form with these teams runs the other units a little slower, so it takes a share of 1/16 of the elements to pay.
+  // Measured (us without | with, rows of 4096 among 300 M elements, bf16 gradients): rows of 768 at a share of 1 %
+  // 970|984, 3 % 976|989, 1/16 986|983, 1/8 1001|974, 1/4 1033|955; rows of 1600 892|900, 900|906, 913|905, 935|904, 980|898.
   bool stream_teams = false;
   {
     int64_t wide = 0, all = 0;

@@ -1,5 +1,5 @@
-// Exact-fp32 refit and apply of the low-rank path on CUDA cores: fp32 gradients, gradients whose rows
-// are not 16-byte aligned, ranks above what the tensor path takes.
+// Exact-fp32 refit and apply of the low-rank path on CUDA cores: fp32 gradients, ranks above what the
+// tensor path takes, and every block of a caller who asks for it (ADAPM_PATH_SIMT).
 //
 // One pass of Algorithm 2 is two launches.  `gram` makes the r x r matrices
 //   R R^T, R0 R^T, L^T L, L^T L0

@@ -107,7 +107,7 @@ struct PadJob {
 constexpr int kPadChunk = 2048;   // columns per CTA
 
 // Rows of any alignment into rows that start on 16 bytes: 16 bytes out per thread, from eight 2-byte reads that neighbour
-// threads' reads complete to whole sectors.  Bound by memory: 4 bytes per element, 0.02 ms for 22 M elements.
+// threads' reads complete to whole sectors.  4 bytes per element: 0.03 ms for 22 M elements (2.8 TB/s), beside a refit of 0.55 ms.
 __global__ void __launch_bounds__(256) tc_pad_kernel(const PadJob* __restrict__ jobs, const int32_t* __restrict__ cta_job,
                                                      const uint16_t* __restrict__ grads, uint16_t* __restrict__ work,
                                                      const int32_t* __restrict__ status) {
@@ -220,8 +220,11 @@ bool tensor_path_block_ok(const adapm_hparams& hp, const adapm_block& b) {
   if (hp.grad_dtype != ADAPM_GRAD_BF16) return false;
   if (b.mom_mode != ADAPM_MOM_LOWRANK) return false;
   if (b.rank > 256) return false;                      // 2 rp accumulator columns per panel, 512 in all
-  // rows that do not start on 16 bytes: by way of a padded copy of the gradient, unless the caller asked for the tensor
-  // path as it is (its 2 bytes per element of workspace are not what that asks for) or for the preconditioned passes
+  // Rows that do not start on 16 bytes: by way of a padded copy of the gradient, unless the caller asked for the tensor
+  // path as it is (its 2 bytes per element of workspace are not what that asks for) or for the preconditioned passes.
+  // (1024 x 2730 blocks of a 190 M model: 1.2 ms per step, 3.4 on the CUDA cores.  Such a block then has the precision of
+  // every other bf16 block under AUTO, products to 2^-17: largest errors of L, R and L R over ten steps of normal,
+  // t-distributed and heavy-rowed gradients 9.0e-6, 1.3e-5 and 6.2e-6, with ADAPM_PATH_SIMT 3.9e-7, 4.9e-7 and 3.4e-7.)
   if (b.cols % 8 != 0 && (hp.lowrank_path == ADAPM_PATH_TENSOR || hp.inner_precond)) return false;
   return tc::encode_tiled_fn() != nullptr;
 }

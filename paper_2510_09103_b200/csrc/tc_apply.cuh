@@ -13,8 +13,8 @@
 // so the accumulator ends up holding D = L0 R0 - L R.  Four warps load the L panel of the next item when
 // the last MMA of the present one is through.  With L in shared memory instead (4 rp columns x 128 rows: 80
 // KB at rank 80, 128 KB at rank 128) the operand reads of A share the shared memory's bandwidth and the ring
-// below has room for two or three buffers: 2.42 -> 1.4 ms at rank 128, 8.3 -> 6.8 ms on the 1.5B shapes with
-// a per-element v.
+// below has room for two or three buffers: 2.42 -> 1.36 ms at rank 128, 8.3 -> 6.6 ms on the 1.5B shapes with
+// a per-element v; with a group v, where the ring had four buffers, as fast as before.
 //
 // Ranks above 128 leave no room for L in tensor memory.  The kernel's second form (kStream) streams L as
 // well: a stage of its ring holds four boxes - 64 columns of L hi, L lo, R^T hi and R^T lo of one factor

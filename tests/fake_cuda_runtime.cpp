@@ -33,6 +33,7 @@ void fake_begin(long fail_at) { g_log.clear(); g_countdown = fail_at; }
 const char* fake_log() { g_countdown = -1; return g_log.c_str(); }
 
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char* cudaGetErrorName(cudaError_t) { return "fake"; }
 const char* cudaGetErrorString(cudaError_t) { return "fake"; }
