@@ -376,6 +376,11 @@ __global__ void __launch_bounds__(kThreads, 3) fp32_refit_kernel(const Fp32Refit
 // A 64 x 64 tile of D = c0 L0 R0 - c1 L R, put into shared memory (the stages' own room) so that the elementwise part
 // runs along the rows of W: a warp takes a row at a time, two adjacent columns per lane where the pitch allows it,
 // whatever the alignment of the rows.  What that part will read is asked into L2 before the products.
+// Against a 4 x 4 tile per thread of 256 threads that writes from registers (59 M elements in blocks of 1024 x 2730, fp32
+// gradients, us): rank 8 400|490 with row groups and 374|569 with a v per element, rank 51 842|785 and 828|846, rank 128
+// 1399|1220 and 1381|1275, rank 290 3034|2448: ahead where the memory sets the pace, behind on the products of larger
+// ranks (128 registers, issue slots half used, the FMA pipes busy 35 % of the time), and its sums, kept in two halves,
+// are a little closer to 64 bits.
 template <typename GT>
 __global__ void __launch_bounds__(kThreads, 4) fp32_apply_kernel(const ApplyBlk* __restrict__ tab,
                                                                  const int32_t* __restrict__ tile_blk, Bases b,

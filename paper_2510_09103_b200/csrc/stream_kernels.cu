@@ -5,9 +5,9 @@
 //   v  <- beta2 v + (1-beta2) g^2            (per element, or once per group with the group mean of g^2)
 //   m  <- beta1 m + (1-beta1) g              (full-momentum blocks only; m^c = m, else m^c = g)
 //   W  <- W - lr s_b ( clamp( m^c / (sqrt(v)+eps) ) + lambda_b W )
-// A work unit (one v group, or a 2048-element chunk) is owned by a team of 32, 64, 128 or 256 threads (as
-// few as hold it, 64 elements each: a team's threads all wait for its slowest loads) that keeps the unit's gradient in registers, so g is read from memory exactly once even when the
-// group mean has to be known before any element can be updated.
+// A work unit (one v group, or a 2048-element chunk) is owned by a team of 32, 64, 128 or 256 threads (as few as hold
+// it, 64 elements each: a team's threads all wait for its slowest loads) that keeps the unit's gradient in registers, so
+// g is read from memory exactly once even when the group mean has to be known before any element can be updated.
 #include <type_traits>
 
 #include "adapm_internal.h"
@@ -225,8 +225,8 @@ __device__ __forceinline__ void run_unit_any(const StreamBlk& B, int64_t unit, f
   }
 }
 
-// kTeams: the launch has units of 64 or 128 threads.  (Their code in the kernel costs the others some 5 %, so sets without
-// such units take the form that does not have it.)
+// kTeams: the launch has units of 64 or 128 threads.  (Their code in the kernel costs the others 1 to 2 %, so sets without
+// many such units take the form that does not have it: see the rule in adapm_create.)
 template <typename GT, bool kTeams>
 __global__ void __launch_bounds__(256, 2) stream_update_kernel(const StreamBlk* __restrict__ tab,
                                                                const int32_t* __restrict__ cta_blk,
