@@ -102,30 +102,30 @@ __device__ __forceinline__ float clamp_keep_nan(float x, float c) {
 // Compared with sqrtf and / on 2^26 pairs each of v in [1e-14, 1e-3] and in [1e-28, 1e28]: the same largest and the same
 // rms error against 64 bits, the root the nearest float every time.
 // What lies outside the range where the iteration holds takes the functions themselves: zero and near-zero v, NaN, and
-// what could overflow on the way.  With |m| <= 1e20 and d >= 1e-15 neither q nor q d - m leaves the range of a float,
-// and only quotients below 1e-20 lose bits of the residual to underflow.
+// what could overflow on the way.  With |m^c| <= 1e14, a bias correction of at most 1e6 and d >= 1e-15 neither q nor
+// q d - m leaves the range of a float, and only quotients below 1e-20 lose bits of the residual to underflow.
 template <int N>
 __device__ __forceinline__ void adapm_param_update_n(float* w, const float* mc, const float* v, const StepScalars& sc,
                                                      float lr_s, float wd) {
-  float vs[N], m[N], lo = 1.f, hi = 1.f;
-  bool usual = sc.eps <= 1e30f;
+  float vs[N], lo = 1.f, hi = 1.f;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     vs[e] = v[e] * sc.inv_bc2;
-    m[e] = mc[e] * sc.inv_bc1;
     lo = fminf(lo, vs[e]);
     hi = fmaxf(hi, vs[e]);
-    usual = usual && fabsf(m[e]) <= 1e20f && vs[e] == vs[e];      // (false for a NaN)
   }
-  if (usual && lo >= 1e-30f && hi <= 1e30f) {
+  bool usual = lo >= 1e-30f && hi <= 1e30f && sc.eps <= 1e30f && sc.inv_bc1 <= 1e6f;
+#pragma unroll
+  for (int e = 0; e < N; ++e) usual = usual && fabsf(mc[e]) <= 1e14f && vs[e] == vs[e];      // (false for a NaN)
+  if (usual) {
 #pragma unroll
     for (int e = 0; e < N; ++e) {
       const float y = rsqrtf(vs[e]);
       float s = vs[e] * y;
       s = fmaf(fmaf(-s, s, vs[e]), 0.5f * y, s);
-      const float d = s + sc.eps, r = __fdividef(1.f, d);
-      float q = m[e] * r;
-      q = fmaf(fmaf(-q, d, m[e]), r, q);
+      const float d = s + sc.eps, r = __fdividef(1.f, d), m = mc[e] * sc.inv_bc1;
+      float q = m * r;
+      q = fmaf(fmaf(-q, d, m), r, q);
       w[e] = w[e] - lr_s * (clamp_keep_nan(q, sc.clip) + wd * w[e]);
     }
   } else {
