@@ -254,6 +254,20 @@ ApplyKernel apply_kernel(bool stream, bool tma) {
   return tma ? tc::tc_apply_kernel<false, true> : tc::tc_apply_kernel<false, false>;
 }
 
+// Lets a kernel be launched with `need` bytes of dynamic shared memory.  The limit belongs to the kernel, not to the context
+// that asks: it is set to the most the device has, so that contexts of other shapes, made before or after, keep theirs.
+template <typename Kernel>
+cudaError_t allow_dynamic_smem(Kernel kernel, int need) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  most -= (int)fa.sharedSizeBytes;
+  return need <= most ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) : cudaErrorInvalidValue;
+}
+
 int round16(int x) { return (x + 15) / 16 * 16; }
 int round64(int x) { return (x + 63) / 64 * 64; }
 
@@ -540,7 +554,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     // one CTA per SM) can be resident at once: ask the runtime whether an SM takes a CTA of this size at all (a
     // device or an MPS share with less shared memory or fewer registers does not), else hand items out longest-first.
     int resident = 0;
-    cudaFuncSetAttribute(tc::tc_items_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P->smem_engine);
+    (void)allow_dynamic_smem(tc::tc_items_kernel, P->smem_engine);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tc::tc_items_kernel, tc::kEngineThreads,
                                                       (size_t)P->smem_engine) != cudaSuccess || resident < 1)
       team_mode = 1;
@@ -790,12 +804,10 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     m.h_maps.resize(P->blk.size() * kMapsPerBlock);
   }
   if (e == cudaSuccess && P->n_teams > 0) e = cudaMalloc((void**)&P->d_team_counters, P->n_teams * sizeof(int32_t));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::tc_items_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P->smem_engine);
+  if (e == cudaSuccess) e = allow_dynamic_smem(tc::tc_items_kernel, P->smem_engine);
   for (int form = 0; form < 4; ++form)
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(apply_kernel(form >> 1, form & 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               P->apply_config(form >> 1, form & 1).smem);
+      e = allow_dynamic_smem(apply_kernel(form >> 1, form & 1), P->apply_config(form >> 1, form & 1).smem);
   if (e != cudaSuccess) {
     set_cuda_error(e, "build_tensor_program");
     return ADAPM_ECUDA;

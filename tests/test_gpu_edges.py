@@ -262,3 +262,19 @@ def test_a_step_captured_in_a_graph(dtype, flags):
         assert torch.equal(params, want_p) and torch.equal(state, want_s)
     del graph
     c.close()
+
+
+def test_contexts_of_different_shapes_side_by_side():
+    """Shared-memory needs differ by rank, by kind of v and by form of the apply kernel: contexts made later, larger or
+    smaller, leave the earlier ones working."""
+    runs = [ParityRun(WL.Workload(f"c{i}", [], "bf16", "normal", steps=2), True, custom_blocks=_blocks([spec]))
+            for i, spec in enumerate([(264, 328, A.MOM_LOWRANK, 128, A.V_ELEMENT, 0), (264, 264, A.MOM_LOWRANK, 200, A.V_BLOCKMEAN, 1),
+                                      (300, 333, A.MOM_LOWRANK, 40, A.V_BLOCKMEAN, 1), (264, 264, A.MOM_LOWRANK, 8, A.V_BLOCKMEAN, 1)])]
+    try:
+        for _ in range(2):
+            for run in runs:
+                run.step()
+                run.compare()
+    finally:
+        for run in runs:
+            run.close()
