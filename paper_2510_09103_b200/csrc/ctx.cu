@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <new>
 
 #include <nvtx3/nvToolsExt.h>
@@ -424,14 +425,9 @@ using namespace adapm;
 
 extern "C" const char* adapm_last_cuda_error(void) { return g_cuda_error.c_str(); }
 
-extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const adapm_hparams* hp, adapm_ctx** out) {
-  if (!blocks || n_blocks <= 0 || !hp || !out) return ADAPM_EINVAL;
-  *out = nullptr;
-  int rc = validate(blocks, n_blocks, *hp);
-  if (rc != ADAPM_OK) return rc;
-
-  adapm_ctx* c = new (std::nothrow) adapm_ctx();
-  if (!c) return ADAPM_EINVAL;
+// Fills in the context, or leaves it as far as it came for adapm_destroy.
+static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blocks, const adapm_hparams* hp) {
+  int rc = ADAPM_OK;
   c->blocks.assign(blocks, blocks + n_blocks);
   c->hp = *hp;
   const int n = (int)n_blocks;
@@ -443,8 +439,8 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     const adapm_block& b = c->blocks[i];
     if (b.mom_mode != ADAPM_MOM_LOWRANK) continue;
     if (tensor_path_block_ok(*hp, b)) tc_ids.push_back(i);
-    else if (hp->lowrank_path == ADAPM_PATH_TENSOR) { delete c; return ADAPM_EUNSUPPORTED; }
-    else if (hp->inner_precond && b.rank > 4096) { delete c; return ADAPM_EUNSUPPORTED; }
+    else if (hp->lowrank_path == ADAPM_PATH_TENSOR) return ADAPM_EUNSUPPORTED;
+    else if (hp->inner_precond && b.rank > 4096) return ADAPM_EUNSUPPORTED;
     else lowrank_ids.push_back(i);
   }
   c->n_tensor_blocks = (int64_t)tc_ids.size();
@@ -685,7 +681,7 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
     std::vector<ReduceJob> row_jobs;
     int64_t row_groups = 0;
     rc = build_tensor_program(c, tc_ids, etas, work_cursor, row_jobs, row_groups);
-    if (rc != ADAPM_OK) { adapm_destroy(c); return rc; }
+    if (rc != ADAPM_OK) return rc;
     if (!row_jobs.empty()) {
       const int64_t off = append_table(c->h_tables, row_jobs);
       for (Launch& L : prog)
@@ -731,11 +727,28 @@ extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const a
   }
   if (e != cudaSuccess) {
     set_cuda_error(e, "adapm_create upload");
-    adapm_destroy(c);
     return ADAPM_ECUDA;
   }
-  *out = c;
   return ADAPM_OK;
+}
+
+extern "C" int adapm_create(const adapm_block* blocks, int64_t n_blocks, const adapm_hparams* hp, adapm_ctx** out) {
+  if (!blocks || n_blocks <= 0 || !hp || !out) return ADAPM_EINVAL;
+  *out = nullptr;
+  adapm_ctx* c = nullptr;
+  int rc;
+  try {
+    rc = validate(blocks, n_blocks, *hp);
+    if (rc != ADAPM_OK) return rc;
+    c = new adapm_ctx();
+    rc = create_context(c, blocks, n_blocks, hp);
+  } catch (const std::exception&) {       // tables too large for the host's memory: a size no device holds either
+    set_error_text("adapm_create: out of host memory");
+    rc = ADAPM_EINVAL;
+  }
+  if (rc != ADAPM_OK) adapm_destroy(c);
+  else *out = c;
+  return rc;
 }
 
 extern "C" void adapm_destroy(adapm_ctx* c) {

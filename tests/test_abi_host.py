@@ -3,6 +3,8 @@ planner equals the oracle's planner bit for bit, and bad descriptors are rejecte
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -81,6 +83,18 @@ def test_create_rejects_bad_descriptors_on_the_host():
     assert _create_code([ok], inner_precond=2) == -1
     assert _create_code([ok], inner_precond=1, precond_damping=-1.0) == -3
     assert _create_code([ok], inner_precond=1, precond_damping=float("nan")) == -3
+
+
+def test_create_returns_an_error_where_the_tables_do_not_fit_the_host():
+    """2^62 elements ask for launch tables of 2^50 bytes.  In a process of its own: an exception that leaves the C entry
+    would end it."""
+    code = ("import paper_2510_09103_b200 as A, ctypes\n"
+            "n = 2**31 - 1\n"
+            "arr = (A.adapm_block * 1)(A.adapm_block(0, n, n, A.MOM_NONE, 0, A.V_ELEMENT, 0, 1.0, 0.1))\n"
+            "h, hp = ctypes.c_void_p(), A.hparams()\n"
+            "print(A.load().adapm_create(arr, 1, ctypes.byref(hp), ctypes.byref(h)), h.value)\n")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0 and res.stdout.split() == ["-1", "None"], res.stderr
 
 
 def test_hparams_struct_matches_the_header():
