@@ -206,8 +206,8 @@ int adapm_set_lr(adapm_ctx* ctx, float lr);
  * One optimizer step over all blocks (Algorithm 1, loop body); t is the 1-based step count.
  * The tensor-core path keeps bf16 copies of the factors L, R in the workspace from one step to the
  * next.  It rebuilds them from the state buffer when t is not the successor of the previous call's
- * t, when the state or workspace pointer changed, after adapm_state_init and after
- * adapm_state_changed; a caller who writes L or R in the state buffer between two consecutive steps
+ * t, when the state or workspace pointer changed, after adapm_state_init, after a step that returned an
+ * error and after adapm_state_changed; a caller who writes L or R in the state buffer between two consecutive steps
  * (importing a checkpoint into the same buffer) must call adapm_state_changed.
  */
 int adapm_step(adapm_ctx* ctx, void* params, const void* grads, void* state, int64_t t, adapm_stream stream);

@@ -884,11 +884,7 @@ extern "C" int adapm_selftest_expired_wait(adapm_ctx* c, adapm_stream stream) {
   return run_expired_wait_probe(c, (cudaStream_t)stream);
 }
 
-extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* state, int64_t t, adapm_stream stream) {
-  if (!c || !params || !grads || !state || t < 1) return ADAPM_EINVAL;
-  if ((uintptr_t)params % 256 || (uintptr_t)grads % 256 || (uintptr_t)state % 256) return ADAPM_EALIGN;
-  if (c->work_floats > 0 && (!c->workspace || c->workspace_bytes < (size_t)c->work_floats * 4)) return ADAPM_ENOWORKSPACE;
-  cudaStream_t s = (cudaStream_t)stream;
+static int enqueue_step(adapm_ctx* c, void* params, const void* grads, void* state, int64_t t, cudaStream_t s) {
   const adapm_hparams& hp = c->hp;
 
   StepScalars sc;
@@ -996,6 +992,16 @@ extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* s
   c->last_step_launches = (int64_t)li;
   if (prof) c->prof_valid = 1;
   return ADAPM_OK;
+}
+
+extern "C" int adapm_step(adapm_ctx* c, void* params, const void* grads, void* state, int64_t t, adapm_stream stream) {
+  if (!c || !params || !grads || !state || t < 1) return ADAPM_EINVAL;
+  if ((uintptr_t)params % 256 || (uintptr_t)grads % 256 || (uintptr_t)state % 256) return ADAPM_EALIGN;
+  if (c->work_floats > 0 && (!c->workspace || c->workspace_bytes < (size_t)c->work_floats * 4)) return ADAPM_ENOWORKSPACE;
+  const int rc = enqueue_step(c, params, grads, state, t, (cudaStream_t)stream);
+  // some launches may be missing: the bf16 copies of the factors no longer follow the step number, whatever comes next
+  if (rc != ADAPM_OK) tensor_state_changed(c);
+  return rc;
 }
 
 extern "C" int adapm_set_profiling(adapm_ctx* c, int32_t on) {

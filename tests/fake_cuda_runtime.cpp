@@ -77,7 +77,7 @@ int build_tensor_program(adapm_ctx*, const std::vector<int64_t>&, const std::vec
 int tensor_prepare_step(adapm_ctx*, const Bases&, int64_t, cudaStream_t, int*, int*) { return ADAPM_EUNSUPPORTED; }
 int run_tensor_launch(adapm_ctx*, const Launch&, const Bases&, const StepScalars&, int, cudaStream_t) { return ADAPM_EUNSUPPORTED; }
 void destroy_tensor_program(adapm_ctx*) {}
-void tensor_state_changed(adapm_ctx*) {}
+void tensor_state_changed(adapm_ctx*) { note("rebuild", nullptr, nullptr); }
 int run_expired_wait_probe(adapm_ctx*, cudaStream_t) { return ADAPM_EUNSUPPORTED; }
 size_t probe_table(std::vector<unsigned char>& out) { out.resize(16); return 16; }
 }  // namespace adapm

@@ -70,11 +70,12 @@ def test_every_way_a_step_can_end_leaves_the_callers_stream_behind_all_of_it(dri
     rc, log, loose, early = _step(driver, h, -1)
     assert rc == 0 and not loose and not early
     assert len({a for op, a, _ in log if op == "launch"}) == 2, "the set is one that forks"
-    assert "sync" not in {op for op, _, _ in log}
+    assert not {"sync", "rebuild"} & {op for op, _, _ in log}
     for n in range(len(log)):
         rc, log_n, loose, early = _step(driver, h, n)
         assert ("failed", 0, 0) in log_n and rc == -4      # ADAPM_ECUDA
         assert not loose and not early, f"call {n} failed: {log_n}"
+        assert ("rebuild", 0, 0) in log_n, "the next step must not trust the factors' bf16 copies"
     driver.adapm_destroy(h)
 
 
