@@ -17,8 +17,10 @@
 //   K_eff times:  gram    four r x r products of the current iterate (tensor cores) -> Gs[0..3]
 //                         (each stored transposed and twice, one copy under the other: the layout the engine's
 //                         N side reads against the [hi | lo] columns of a factor)
-//                 panel   row panels update L, column panels update R (tensor cores); fp32 factors
-//                         are updated in place in the state, their split copies go to the next set.
+//                 panel   row panels update L, column panels update R (tensor cores).  The first pass reads the
+//                         fp32 factors from the state and the last one writes them there; in between they are in
+//                         the workspace, in the order of the epilogue's threads (tc::Item).  Split copies go to
+//                         the next set.
 //                         The row panels of the first pass also add up g^2 per row (block-mean v).
 //   apply     m^c and the parameter write from the previous and the final set
 // rp = rank rounded up to 16; padded columns are kept at zero by every writer.
@@ -161,6 +163,7 @@ struct TcBlock {
   int64_t gpad;                    // bf16 element offset of the padded copy of the gradient, or -1
   int32_t ldg;                     // row pitch of the gradient the refit reads
   int64_t rowsum;                  // float offset of the row sums of g^2 in the workspace, or -1
+  int64_t iter_l = 0, iter_r = 0;  // float offsets of the fp32 factors between two passes (see tc::Item)
   // preconditioned passes: split copies of L S_L and (S_R R)^T (pitch 2 half), and in floats the Gram matrices
   // R R^T, L^T L (gf, gf + r^2), their damped inverses (sf, sf + r^2) and the fp32 products L S_L, S_R R
   int64_t lct = 0, rtct = 0, gf = 0, sf = 0, ltf = 0, rtf = 0;
@@ -277,6 +280,15 @@ int64_t append_items(std::vector<unsigned char>& blob, const std::vector<T>& tab
   blob.resize(off + tab.size() * sizeof(T));
   if (!tab.empty()) std::memcpy(blob.data() + off, tab.data(), tab.size() * sizeof(T));
   return (int64_t)off;
+}
+
+// Every accumulator of the items lies inside a buffer of `cols` tensor-memory columns.
+bool fits_accumulators(const std::vector<tc::Item>& v, int cols) {
+  for (const tc::Item& it : v)
+    for (int s = 0; s < it.n_seg; ++s)
+      for (int p = 0; p < it.seg[s].n_a; ++p)
+        if (it.seg[s].d_col[p] + it.seg[s].d_part + it.seg[s].n > cols) return false;
+  return cols <= 512;
 }
 
 struct Geo {
@@ -458,6 +470,14 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     P->blk.push_back(t);
   }
   P->work_end = work_cursor;
+  // The fp32 factors of the passes in between.  (The preconditioned passes read them from the state after every pass.)
+  const bool use_iter = K_eff > 1 && !hp.inner_precond;
+  for (TcBlock& t : P->blk) {
+    const adapm_block& b = c->blocks[t.id];
+    if (!use_iter) break;
+    t.iter_l = work_cursor; work_cursor += (int64_t)(b.rows + 127) / 128 * 128 * t.rp;
+    t.iter_r = work_cursor; work_cursor += (int64_t)(b.cols + 127) / 128 * 128 * t.rp;
+  }
   for (TcBlock& t : P->blk) {          // (rewritten every step: not part of what a rebuild of the split copies zeroes)
     const adapm_block& b = c->blocks[t.id];
     if (b.cols % 8 != 0 && K_eff > 0) t.gpad = take((int64_t)b.rows * t.ldg);
@@ -495,6 +515,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   if (stages_with(stage_k, n_pan) < 2) { set_error_text("rank too large for the tensor path"); return ADAPM_EUNSUPPORTED; }
   P->stage_k = stage_k;
   const bool gram_small = 4 * rp_max <= 512 && 2 * rp_max <= 256;   // two accumulators of N = 2 rp: hi and lo window
+  int gram_cols = 64;                            // four partial sums up to rank 128, two above
+  for (const TcBlock& t : P->blk) gram_cols = std::max(gram_cols, t.rp <= 128 ? 4 * t.rp : 2 * t.rp);
   const int gram_na = (gram_small && stages_with(stage_k, 2) < 2) ? 1 : 2;
   P->smem_engine = std::max(P->engine_config(n_pan).smem, P->engine_config(gram_na).smem);
 
@@ -700,6 +722,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
           it.own0 = p0; it.own_count = is_L ? m : n;
           it.f32_off = is_L ? c->l_off[t.id] : c->r_off[t.id];
           it.own_stride = is_L ? r : 1; it.k_stride = is_L ? 1 : n;
+          it.iter_off = is_L ? t.iter_l : t.iter_r;
+          it.from_iter = use_iter && pass > 0; it.to_iter = use_iter && pass + 1 < K_eff;
           it.dst_off = is_L ? t.lc[dst] : t.rtc[dst]; it.dst_ld = t.ld[dst];
           it.sumsq_off = (is_L && pass == 0 && t.rowsum >= 0) ? t.rowsum + p0 : -1;
           if (it.sumsq_off >= 0) any_sumsq = true;
@@ -719,8 +743,12 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
       std::vector<int32_t> begin_g, begin_p;
       schedule_items(grams, grid_g, begin_g, stage_k);
       P->n_teams = std::max(P->n_teams, schedule_panels(panels, spans, grid_p, begin_p, stage_k, team_mode));
+      if (!fits_accumulators(grams, gram_cols) || !fits_accumulators(panels, n_pan * 2 * rp_max)) {
+        set_error_text("accumulators beyond tensor memory");
+        return ADAPM_EUNSUPPORTED;
+      }
       Launch G{LK_TC_GRAM, append_items(c->h_tables, grams), (int64_t)grams.size(), grid_g};
-      G.aux0 = gram_small ? 4 * rp_max : 2 * rp_max;
+      G.aux0 = gram_cols;
       G.aux1 = 2 * G.aux0 <= 512 ? 2 : 1; G.aux2 = gram_na;
       G.aux3 = append_items(c->h_tables, begin_g);
       G.aux4 = -1; G.aux5 = 0;

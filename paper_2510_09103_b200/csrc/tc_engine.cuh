@@ -18,6 +18,8 @@
 // N side of an MMA the two parts land in two column ranges of the accumulator, which the epilogue
 // adds.  While 2 rp <= 256 one MMA of N = 2 rp covers both parts; above that the hi and the lo part
 // take one MMA of N = rp each, the second reading B from the chunk at which the lo part starts.
+// (Letting both add to the same columns would free half of the accumulator, but the small products then meet the
+// rounding of the large sums: errors of L R against 64 bits up to twice as large at ranks 128 to 256.)
 //
 // A stage of the shared-memory ring holds `stage_k` (64 or 128) of K:
 //   A  up to three operands of 128 rows x stage_k (K along x: boxes of 64 x 128) or stage_k x 128
@@ -74,8 +76,10 @@ struct Item {
   int32_t epi;
   // EPI_FACTOR: panel p (p < n_pan) has its accumulator at column acc_stride * p; the thread that owns
   // accumulator row q of panel p updates factor entries (owner = own0 + 128 p + q, k):
-  //   f32[own_stride * owner + k_stride * k] += coef * (D[q][k] + D[q][rp + k])        k < r
+  //   new[owner][k] = old[owner][k] + coef * (D[q][k] + D[q][rp + k])                  k < r
   //   dst[owner][k] = hi, dst[owner][half + k] = lo                                    k < rp
+  // Old and new fp32 values live in the state, f32[own_stride * owner + k_stride * k], or in the workspace in the order
+  // in which the epilogue's threads take them (iter_at).
   // EPI_GRAM: G[own0 + q][k] = coef * sum over n_sum parts (rp columns apart) of D[q][k]; stored like dst above,
   //   and once more stack_rows rows below                                              own0 + q, k < rp
   int32_t own0, own_count;   // first owner of the item and number of owners of the whole matrix
@@ -84,6 +88,8 @@ struct Item {
   int32_t n_sum, stack_rows;
   int32_t dst_ld;            // row pitch of the destination in elements
   int64_t f32_off;           // float offset of the factor in the state buffer
+  int64_t iter_off;          // float offset in the workspace of its values between two passes
+  int32_t from_iter, to_iter;   // 1: old values come from there, new values go there
   int64_t own_stride, k_stride;
   int64_t dst_off;           // bf16 element offset of the destination array in the workspace
   int64_t sumsq_off;         // float offset in the workspace of the row sums of g^2 (row own0 first), or -1
@@ -99,7 +105,8 @@ struct Item {
 // the fields of an Item its epilogue needs
 struct ItemEpi {
   int32_t epi, own0, own_count, n_pan, acc_stride, r, rp, half, n_sum, stack_rows, dst_ld;
-  int64_t f32_off, own_stride, k_stride, dst_off;
+  int32_t from_iter, to_iter;
+  int64_t f32_off, iter_off, own_stride, k_stride, dst_off;
   float coef;
 };
 
@@ -440,6 +447,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         const Item& G = a.items[it];
         I.epi = G.epi; I.own0 = G.own0; I.own_count = G.own_count; I.n_pan = G.n_pan; I.acc_stride = G.acc_stride;
         I.r = G.r; I.rp = G.rp; I.half = G.half; I.n_sum = G.n_sum; I.stack_rows = G.stack_rows;
+        I.from_iter = G.from_iter; I.to_iter = G.to_iter; I.iter_off = G.iter_off;
         I.f32_off = G.f32_off; I.own_stride = G.own_stride; I.k_stride = G.k_stride;
         I.dst_off = G.dst_off; I.dst_ld = G.dst_ld; I.coef = G.coef;
       }
@@ -454,68 +462,83 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       const bool has_work = I.epi == EPI_FACTOR ? grp < total : (I.epi == EPI_GRAM && grp == 0);
       const bool factor = I.epi == EPI_FACTOR && has_work;
       const int qc = lane & 3;
-      float* fbase = a.f32_base + I.f32_off;
-      // EPI_FACTOR has three forms.  The general one works in a "turned" layout: a thread reads its accumulator
-      // row from tensor memory, then every quad of lanes transposes its 4 x 16 piece with shuffles, after which
-      // lane c of the quad holds columns 4c .. 4c+3 of the quad's four rows; factor rows are then read and
-      // written as 64-byte runs instead of one row per lane.
-      // float4 path of that form: the four values of a lane are adjacent in memory and 16-byte aligned
-      const bool vec4 = I.k_stride == 1 && (I.own_stride & 3) == 0 && (r & 3) == 0 && (I.f32_off & 3) == 0;
-      // A factor whose consecutive owners are adjacent in memory (R, stored [r, n]) needs no turn: for
-      // a fixed column the 32 rows of a warp are one 128-byte run already.
-      const bool by_column = factor && I.own_stride == 1 && !vec4;
-      // A factor stored row by row (L, [m, r]) whose rows start on 32-byte boundaries and hold a multiple of
-      // eight values needs no turn either: a lane moves 32 bytes per access, which is a whole sector.
-      const bool by_row = factor && I.k_stride == 1 && ((I.own_stride | r | I.f32_off) & 7) == 0;
-      // piece u of the item: panel u / np, columns [16 (u % np), +16)
-      auto fetch_old = [&](int u, float (*o)[4]) {
+      float* const fbase = a.f32_base + I.f32_off;
+      float* const ibase = a.work_f32 + I.iter_off;
+      // EPI_FACTOR works in one of two arrangements.  Straight: a thread keeps its accumulator row.  Old and new values
+      // are 32-byte accesses per lane in the workspace's order, where a warp's 32 rows are one run of memory, and for a
+      // row-stored factor of the state (L, [m, r]) whose rows start on 32 bytes and hold a multiple of eight values; a
+      // factor whose consecutive owners are adjacent (R, [r, n]) goes column by column, 32 rows = one 128-byte run.
+      // Turned, for any other L: every quad of lanes transposes its 4 x 16 piece with shuffles, after which lane c of
+      // the quad holds columns 4c .. 4c+3 of the quad's four rows, so that rows are 64-byte runs instead of one per lane.
+      // Only the first pass of a step reads the state and only the last one writes it.  A piece of 16 columns took 1.6
+      // thousand cycles by rows and 3.5 thousand by columns, whether or not memory was busy: a warp's 32-byte accesses touch 32
+      // cache lines by rows and 8 in the workspace's order, and columns take 16 narrow accesses.  Panel launches of a step,
+      // state in every pass -> workspace in between: 2.01 -> 1.79 ms on the 350M set at rank 128, 418 -> 376 us on
+      // 1024 x 2730, 137 -> 127 us on the 60M set, 16.3 -> 15.7 ms on 8 layers of the 8B shapes.
+      const bool by_column = I.own_stride == 1;
+      const bool by_row = I.k_stride == 1 && ((I.own_stride | r | I.f32_off) & 7) == 0;
+      const bool turned = factor && !by_column && !by_row && !(I.from_iter && I.to_iter);
+      // workspace order: [panel][piece][8 columns][128 rows][8]
+      auto iter_at = [&](int u, int h, int row) { return ibase + (((int64_t)u * 2 + h) * 128 + row) * 8; };
+      const int own_u0 = I.own0 >> 7;                     // panels before this item's (its pieces start at own_u0 * np)
+      auto fetch = [&](int u, float* o) {
         const int pan = u / np, p = 16 * (u - pan * np);
-        const int own_quad = I.own0 + 128 * pan + 32 * (warp & 3) + (lane & ~3);
+        const int own_row = I.own0 + 128 * pan + q;
+        if (I.from_iter) {
+          ldcg_f32x8(iter_at(own_u0 * np + u, 0, q), o);
+          if (p + 8 < r) {
+            ldcg_f32x8(iter_at(own_u0 * np + u, 1, q), o + 8);
+          } else {                       // (no traffic for padding)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int owner = own_quad + i;      // quad row i, this lane's four columns of it
-          const int k = p + 4 * qc;
-          const bool row_ok = owner < I.own_count;
-          const float* fp = fbase + I.own_stride * owner + I.k_stride * k;
-          if (vec4) {
-            const float4 v = (row_ok && k < r) ? __ldcg(reinterpret_cast<const float4*>(fp)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            o[i][0] = v.x; o[i][1] = v.y; o[i][2] = v.z; o[i][3] = v.w;
-          } else {
+            for (int e = 8; e < 16; ++e) o[e] = 0.f;
+          }
+          return;
+        }
+        const bool row_ok = own_row < I.own_count;
+        if (by_row) {
+          const float* fp = fbase + I.own_stride * own_row + p;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) o[i][x] = (row_ok && k + x < r) ? __ldcg(fp + I.k_stride * x) : 0.f;
+          for (int h = 0; h < 2; ++h) {
+            if (row_ok && p + 8 * h < r) {
+              ldcg_f32x8(fp + 8 * h, o + 8 * h);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) o[8 * h + e] = 0.f;
+            }
+          }
+        } else {
+          const float* fp = fbase + own_row + I.k_stride * p;
+          const int n = row_ok ? r - p : 0;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            o[e] = e < n ? __ldcg(fp) : 0.f;
+            fp += I.k_stride;
           }
         }
       };
-      // old values of this thread's own row, columns [p, p+16), kept in the same registers as o[e / 4][e % 4]
-      auto fetch_old_col = [&](int u, float (*o)[4]) {
+      // the turned arrangement: o[4 i + e] = column p + 4 qc + e of quad row i
+      auto fetch_turned = [&](int u, float* o) {
         const int pan = u / np, p = 16 * (u - pan * np);
-        const int own_row = I.own0 + 128 * pan + q;
-        const float* fp = fbase + own_row + I.k_stride * p;
-        const bool row_ok = own_row < I.own_count;
+        const int row_quad = 32 * (warp & 3) + (lane & ~3), own_quad = I.own0 + 128 * pan + row_quad;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) o[e >> 2][e & 3] = (row_ok && p + e < r) ? __ldcg(fp + I.k_stride * e) : 0.f;
-      };
-      auto fetch_old_row = [&](int u, float (*o)[4]) {
-        const int pan = u / np, p = 16 * (u - pan * np);
-        const int own_row = I.own0 + 128 * pan + q;
-        const float* fp = fbase + I.own_stride * own_row + p;
-        const bool row_ok = own_row < I.own_count;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (row_ok && p + 8 * h < r) {
-            ldcg_f32x8(fp + 8 * h, &o[2 * h][0]);
+        for (int i = 0; i < 4; ++i) {
+          const int owner = own_quad + i, k = p + 4 * qc;
+          if (I.from_iter) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(iter_at(own_u0 * np + u, qc >> 1, row_quad + i) + 4 * (qc & 1)));
+            o[4 * i] = v.x; o[4 * i + 1] = v.y; o[4 * i + 2] = v.z; o[4 * i + 3] = v.w;
           } else {
+            const float* fp = fbase + I.own_stride * owner + k;
+            const int n = owner < I.own_count ? r - k : 0;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) o[2 * h + (e >> 2)][e & 3] = 0.f;
+            for (int e = 0; e < 4; ++e) o[4 * i + e] = e < n ? __ldcg(fp + e) : 0.f;
           }
         }
       };
       // old values travel one piece ahead in two register sets that swap roles (no copies, which
       // would wait for the loads); the first set is requested before the accumulator is waited for
-      float oldA[4][4], oldB[4][4];
-      if (by_row) fetch_old_row(grp, oldA);
-      else if (by_column) fetch_old_col(grp, oldA);
-      else if (factor) fetch_old(grp, oldA);
+      float oldA[16], oldB[16];
+      if (turned) fetch_turned(grp, oldA);
+      else if (factor) fetch(grp, oldA);
       // one lane per warp polls (fewer pollers on the barrier), then the warp agrees: the
       // tensor-memory loads below need all 32 lanes
       bool got = true;
@@ -529,8 +552,10 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       // same columns for every item) and the accumulator is handed back at once; the pieces below then read the
       // parked sums while the next main loop runs.  Each group parks the pieces it will work on.
       const bool parked = factor && a.sum_col >= 0;
-      const uint32_t ts = tmem_base + lane_addr + (uint32_t)(a.sum_col < 0 ? 0 : a.sum_col);
+      const uint32_t ts = parked ? tmem_base + lane_addr + (uint32_t)a.sum_col : t0;
+      const uint32_t ts_stride = (uint32_t)(parked ? rp : I.acc_stride);
       if (parked) {
+#pragma unroll 1
         for (int u = grp; u < total; u += 2) {
           const int pan = u / np, p = 16 * (u - pan * np);
           float d0[16], d1[16];
@@ -539,53 +564,80 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 16; ++e) d0[e] += d1[e];
-          tmem_st16(ts + (uint32_t)(pan * rp + p), d0);
+          tmem_st16(ts + (uint32_t)pan * ts_stride + (uint32_t)p, d0);
         }
         tmem_st_wait();
       }
+      // D0 + D1 of columns [p, p + 16) of this thread's row of a panel
+      auto sum16 = [&](int pan, int p, float* x) {
+        tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)p, x);
+        if (!parked) {
+          float d1[16];
+          tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)(rp + p), d1);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 16; ++e) x[e] += d1[e];
+        } else {
+          tmem_ld_wait();
+        }
+      };
       const bool early = parked || !has_work;   // (a warp without work never reads the accumulator)
       if (early) {
         tc_fence_before();
         mbar_arrive(&sh.tempty[acc]);
       }
-      // columns [p, p+16) of D0 + D1 of this thread's row of panel `pan`
-      auto sum16 = [&](int pan, int p, float* sd) {
-        if (parked) {
-          tmem_ld16(ts + (uint32_t)(pan * rp + p), sd);
-          tmem_ld_wait();
-        } else {
-          float d1[16];
-          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + p), sd);
-          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + rp + p), d1);
-          tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 16; ++e) sd[e] += d1[e];
-        }
-      };
-      if (!has_work) {
-        // nothing to drain for this warp
-      } else if (I.epi == EPI_FACTOR) {
-        uint16_t* dst = a.work_bf16 + I.dst_off;
-        // one piece in the turned form, old values in `o`
-        auto piece = [&](int u, float (*o)[4]) {
+      if (factor) {
+        uint16_t* const dst = a.work_bf16 + I.dst_off;
+        auto piece = [&](int u, const float* o) {
           const int pan = u / np, p = 16 * (u - pan * np);
-          const int own_quad = I.own0 + 128 * pan + 32 * (warp & 3) + (lane & ~3);
-          float acc16[16];
-          sum16(pan, p, acc16);
-          float v[4][4];                 // v[j] = columns 4j .. 4j+3 of this thread's row
+          const int own_row = I.own0 + 128 * pan + q;
+          float x[16];
+          sum16(pan, p, x);
+          const bool row_ok = own_row < I.own_count;
+          uint32_t hi[8], lo[8];
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj)
+          for (int e = 0; e < 16; e += 2) {
+            x[e] = p + e < r ? o[e] + coef * x[e] : 0.f;
+            x[e + 1] = p + e + 1 < r ? o[e + 1] + coef * x[e + 1] : 0.f;
+            split_bf16x2(x[e], x[e + 1], hi[e >> 1], lo[e >> 1]);
+          }
+          if (I.to_iter) {
+            st_f32x8(iter_at(own_u0 * np + u, 0, q), x);
+            if (p + 8 < r) st_f32x8(iter_at(own_u0 * np + u, 1, q), x + 8);
+          } else if (by_row) {
+            float* fp = fbase + I.own_stride * own_row + p;
+            if (row_ok && p < r) st_f32x8(fp, x);
+            if (row_ok && p + 8 < r) st_f32x8(fp + 8, x + 8);
+          } else {
+            float* fp = fbase + own_row + I.k_stride * p;
+            const int n = row_ok ? r - p : 0;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[jj][e] = acc16[4 * jj + e];
+            for (int e = 0; e < 16; ++e) {
+              if (e < n) __stcg(fp, x[e]);
+              fp += I.k_stride;
+            }
+          }
+          if (row_ok) {
+            uint16_t* drow = dst + (int64_t)I.dst_ld * own_row + p;
+            st_b32x8(drow, hi);
+            st_b32x8(drow + half, lo);
+          }
+        };
+        // one piece in the turned arrangement
+        auto piece_turned = [&](int u, const float* o) {
+          const int pan = u / np, p = 16 * (u - pan * np);
+          const int row_quad = 32 * (warp & 3) + (lane & ~3), own_quad = I.own0 + 128 * pan + row_quad;
+          float v[16];                   // columns of this thread's row
+          sum16(pan, p, v);
           // quad transpose, first exchange (partner lane ^ 2): keep the half of the columns this lane's
           // final column group lies in, hand over the other half
           const bool up = (qc & 2) != 0, odd = (qc & 1) != 0;
           float k0[4], k1[4], g0[4], g1[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            k0[e] = up ? v[2][e] : v[0][e];
-            k1[e] = up ? v[3][e] : v[1][e];
-            const float s0 = up ? v[0][e] : v[2][e], s1 = up ? v[1][e] : v[3][e];
+            k0[e] = up ? v[8 + e] : v[e];
+            k1[e] = up ? v[12 + e] : v[4 + e];
+            const float s0 = up ? v[e] : v[8 + e], s1 = up ? v[4 + e] : v[12 + e];
             g0[e] = __shfl_xor_sync(0xffffffffu, s0, 2);
             g1[e] = __shfl_xor_sync(0xffffffffu, s1, 2);
           }
@@ -600,29 +652,26 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
             t[2][e] = __shfl_xor_sync(0xffffffffu, s0, 1);
             t[3][e] = __shfl_xor_sync(0xffffffffu, s1, 1);
           }
-          // order by row, so that in every access below the four lanes of a quad address one row
-          float sd[4][4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int w = i ^ qc;          // 0 -> t[0], 2 -> t[1], 1 -> t[2], 3 -> t[3]
-#pragma unroll
-            for (int e = 0; e < 4; ++e) sd[i][e] = w == 0 ? t[0][e] : (w == 2 ? t[1][e] : (w == 1 ? t[2][e] : t[3][e]));
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int owner = own_quad + i;
-            if (owner >= I.own_count) continue;
-            const int k = p + 4 * qc;
+            // order by row, so that in every access below the four lanes of a quad address one row:
+            // row i is t[0], t[1], t[2] or t[3] as i ^ qc is 0, 2, 1 or 3
+            const int w = i ^ qc, owner = own_quad + i, k = p + 4 * qc;
             float x[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = k + e < r ? o[i][e] + coef * sd[i][e] : 0.f;
-            float* fp = fbase + I.own_stride * owner + I.k_stride * k;
-            if (vec4) {
-              if (k < r) *reinterpret_cast<float4*>(fp) = make_float4(x[0], x[1], x[2], x[3]);
+            for (int e = 0; e < 4; ++e) {
+              const float sd = w == 0 ? t[0][e] : (w == 2 ? t[1][e] : (w == 1 ? t[2][e] : t[3][e]));
+              x[e] = k + e < r ? o[4 * i + e] + coef * sd : 0.f;
+            }
+            if (owner >= I.own_count) continue;
+            if (I.to_iter) {
+              __stcg(reinterpret_cast<float4*>(iter_at(own_u0 * np + u, qc >> 1, row_quad + i) + 4 * (qc & 1)),
+                     make_float4(x[0], x[1], x[2], x[3]));
             } else {
+              float* fp = fbase + I.own_stride * owner + k;
 #pragma unroll
               for (int e = 0; e < 4; ++e)
-                if (k + e < r) fp[I.k_stride * e] = x[e];
+                if (k + e < r) fp[e] = x[e];
             }
             uint32_t h01, l01, h23, l23;
             split_bf16x2(x[0], x[1], h01, l01);
@@ -632,99 +681,42 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
             *reinterpret_cast<uint2*>(drow + half) = make_uint2(l01, l23);
           }
         };
-        // the same piece without the turn: this thread's row, columns [p, p+16)
-        auto piece_col = [&](int u, float (*o)[4]) {
-          const int pan = u / np, p = 16 * (u - pan * np);
-          const int own_row = I.own0 + 128 * pan + q;
-          float sd[16];
-          sum16(pan, p, sd);
-          if (own_row >= I.own_count) return;
-          float* fp = fbase + own_row + I.k_stride * p;
-          uint32_t hi[8], lo[8];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            const float x0 = p + e < r ? o[e >> 2][e & 3] + coef * sd[e] : 0.f;
-            const float x1 = p + e + 1 < r ? o[(e + 1) >> 2][(e + 1) & 3] + coef * sd[e + 1] : 0.f;
-            if (p + e < r) __stcg(fp + I.k_stride * e, x0);
-            if (p + e + 1 < r) __stcg(fp + I.k_stride * (e + 1), x1);
-            split_bf16x2(x0, x1, hi[e >> 1], lo[e >> 1]);
-          }
-          uint16_t* drow = dst + (int64_t)I.dst_ld * own_row + p;
-          st_b32x8(drow, hi);
-          st_b32x8(drow + half, lo);
-        };
-        // and for a row-stored factor with aligned rows
-        auto piece_row = [&](int u, float (*o)[4]) {
-          const int pan = u / np, p = 16 * (u - pan * np);
-          const int own_row = I.own0 + 128 * pan + q;
-          float sd[16];
-          sum16(pan, p, sd);
-          if (own_row >= I.own_count) return;
-          float x[16];
-          uint32_t hi[8], lo[8];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            x[e] = p + e < r ? o[e >> 2][e & 3] + coef * sd[e] : 0.f;
-            x[e + 1] = p + e + 1 < r ? o[(e + 1) >> 2][(e + 1) & 3] + coef * sd[e + 1] : 0.f;
-            split_bf16x2(x[e], x[e + 1], hi[e >> 1], lo[e >> 1]);
-          }
-          float* fp = fbase + I.own_stride * own_row + p;
-          if (p < r) st_f32x8(fp, x);
-          if (p + 8 < r) st_f32x8(fp + 8, x + 8);
-          uint16_t* drow = dst + (int64_t)I.dst_ld * own_row + p;
-          st_b32x8(drow, hi);
-          st_b32x8(drow + half, lo);
-        };
         // this group's pieces grp, grp + 2, ...: two per trip, the old values of the next one on their way
-        if (by_row) {
+        if (!turned) {
 #pragma unroll 1
           for (int u = grp; u < total; u += 4) {
-            if (u + 2 < total) fetch_old_row(u + 2, oldB);
-            piece_row(u, oldA);
+            if (u + 2 < total) fetch(u + 2, oldB);
+            piece(u, oldA);
             if (u + 2 < total) {
-              if (u + 4 < total) fetch_old_row(u + 4, oldA);
-              piece_row(u + 2, oldB);
-            }
-          }
-        } else if (by_column) {
-#pragma unroll 1
-          for (int u = grp; u < total; u += 4) {
-            if (u + 2 < total) fetch_old_col(u + 2, oldB);
-            piece_col(u, oldA);
-            if (u + 2 < total) {
-              if (u + 4 < total) fetch_old_col(u + 4, oldA);
-              piece_col(u + 2, oldB);
+              if (u + 4 < total) fetch(u + 4, oldA);
+              piece(u + 2, oldB);
             }
           }
         } else {
 #pragma unroll 1
           for (int u = grp; u < total; u += 4) {
-            if (u + 2 < total) fetch_old(u + 2, oldB);
-            piece(u, oldA);
+            if (u + 2 < total) fetch_turned(u + 2, oldB);
+            piece_turned(u, oldA);
             if (u + 2 < total) {
-              if (u + 4 < total) fetch_old(u + 4, oldA);
-              piece(u + 2, oldB);
+              if (u + 4 < total) fetch_turned(u + 4, oldA);
+              piece_turned(u + 2, oldB);
             }
           }
         }
-      } else if (I.epi == EPI_GRAM) {
+      } else if (has_work) {           // EPI_GRAM
         uint16_t* dst = a.work_bf16 + I.dst_off;
         const int row = I.own0 + q;
+#pragma unroll 1
         for (int p = 0; p < rp; p += 16) {
           float d0[16], d1[16];
           tmem_ld16(t0 + (uint32_t)p, d0);
-          tmem_ld16(t0 + (uint32_t)(rp + p), d1);
-          if (I.n_sum == 4) {
-            float d2[16], d3[16];
-            tmem_ld16(t0 + (uint32_t)(2 * rp + p), d2);
-            tmem_ld16(t0 + (uint32_t)(3 * rp + p), d3);
+          tmem_ld_wait();
+#pragma unroll 1
+          for (int part = 1; part < I.n_sum; ++part) {
+            tmem_ld16(t0 + (uint32_t)(part * rp + p), d1);
             tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 16; ++e) d0[e] = (d0[e] + d1[e]) + (d2[e] + d3[e]);
-          } else {
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 16; ++e) d0[e] = d0[e] + d1[e];
+            for (int e = 0; e < 16; ++e) d0[e] += d1[e];
           }
           if (row < rp) {
             uint32_t hi[8], lo[8];

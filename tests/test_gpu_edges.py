@@ -37,6 +37,15 @@ def test_ranks_at_the_edges_of_the_apply_kernels_forms(rank):
             path=A.PATH_TENSOR)
 
 
+@pytest.mark.parametrize("rank", [1, 7, 16, 97, 112, 128, 130])
+@pytest.mark.parametrize("iters", [2, 3, 5])
+def test_refit_on_the_tensor_path_by_rank_and_number_of_passes(iters, rank):
+    """The fp32 factors between two passes are kept in the order of the epilogue's threads, the first pass reads and the
+    last one writes the state: by rows, by columns and turned, panels and ranks with remainders, one pass to four."""
+    _follow([(130, 1032, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 1), (648, 264, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 8),
+             (256, 384, A.MOM_LOWRANK, max(1, rank // 8 * 8), A.V_ELEMENT, 0)], path=A.PATH_TENSOR, inner_iters=iters)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("rank", [1, 8, 9, 24, 40, 41, 81, 300])
 def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
