@@ -32,15 +32,28 @@ void set_cuda_error(cudaError_t e, const char* where);
 // lost 4 %, so those are launched plainly.
 constexpr size_t kChainedBytes = (size_t)3 << 29;      // 1.6 GB
 template <typename... Params, typename... Args>
-inline cudaError_t launch_chained(bool chained, void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
-                                  Args... args) {
+inline cudaError_t launch_clusters(bool chained, unsigned cluster, void (*kernel)(Params...), unsigned grid, unsigned threads,
+                                   size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at; cfg.numAttrs = chained ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  cfg.attrs = at; cfg.numAttrs = 0;
+  if (chained) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = cluster;
+    at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(bool chained, void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                                  Args... args) {
+  return launch_clusters(chained, 1, kernel, grid, threads, smem, s, args...);
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void wait_for_previous_kernel() {

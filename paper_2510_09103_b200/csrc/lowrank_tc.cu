@@ -47,12 +47,13 @@ enum {
   MAP_LCT = 5,      // + set: the same, boxes of 64 x stage_k
   MAP_LCN = 8,      // + set: the same as 64-column chunks (N side)
   MAP_RTC = 11, MAP_RTCT = 14, MAP_RTCN = 17,   // the same three views of [R^T hi | R^T lo]
-  MAP_GS = 20,      // + which: Gram operands as chunks
+  MAP_GS = 20,      // + which: Gram operands, boxes of 64 x stage_k
   MAP_W = 24, MAP_G32 = 25, MAP_V = 26,          // W, g, v in quarter-tile boxes (apply)
   MAP_LCAT = 27, MAP_RCAT = 28,                  // X and Y side by side as one matrix (apply)
   MAP_SH = 29,                                   // the bf16 copy of W, boxes like g's (apply; zero without a shadow)
   MAP_LCN_T = 30, MAP_RTCN_T = 31,               // N side of the transformed factors L S_L and (S_R R)^T (preconditioned passes)
-  kMapsPerBlock = 32
+  MAP_LCT_T = 32, MAP_RTCT_T = 33,               // the same in boxes of 64 x stage_k
+  kMapsPerBlock = 34
 };
 
 struct ConvertJob {
@@ -179,15 +180,14 @@ struct MapSet {                     // tensor maps for one combination of caller
 struct TcProgram {
   std::vector<TcBlock> blk;
   int64_t n_convert_owners = 0;
-  int smem_engine = 0;
   int nb_max = 1, stage_k = 128, rp_max = 16, half_max = 16;
   int64_t work_begin = 0, work_end = 0;   // the tensor path's part of the workspace, in floats
-  // shared-memory plan of an engine launch whose segments have up to n_a A operands
+  // shared-memory plan of an engine launch whose segments have up to n_a A operands in a CTA; pair: panel launches
   struct EngineConfig { int a_bytes, stage_bytes, n_stages, smem; };
-  EngineConfig engine_config(int n_a) const {
+  EngineConfig engine_config(bool pair, int n_a) const {
     EngineConfig e;
     e.a_bytes = n_a * 256 * stage_k;
-    e.stage_bytes = e.a_bytes + stage_k * 128 * nb_max;
+    e.stage_bytes = e.a_bytes + stage_k * 128 * (pair ? (rp_max + 63) / 64 : nb_max);
     e.n_stages = std::min(8, (224 * 1024) / e.stage_bytes);
     e.smem = std::max(e.n_stages, 1) * e.stage_bytes + 1024;
     return e;
@@ -287,7 +287,7 @@ bool fits_accumulators(const std::vector<tc::Item>& v, int cols) {
   for (const tc::Item& it : v)
     for (int s = 0; s < it.n_seg; ++s)
       for (int p = 0; p < it.seg[s].n_a; ++p)
-        if (it.seg[s].d_col[p] + it.seg[s].d_part + it.seg[s].n > cols) return false;
+        if (it.seg[s].d_col[p] + it.seg[s].d_part + (it.seg[s].n2 ? it.seg[s].n2 : it.seg[s].n) > cols) return false;
   return cols <= 512;
 }
 
@@ -296,18 +296,22 @@ struct Geo {
 };
 
 // One segment.  A: 2-D map `map_a`, operand p at (ax + dax p, ay + day p), K along x (a_mode 0) or along y
-// (a_mode 1).  B: chunked map `map_b`, K rows from 0.  rp2 = 2 rp decides between one MMA of N = 2 rp and two
-// of N = rp (the second from the chunk where the lo part starts).
-tc::Seg make_seg(const Geo& g, int map_a, int ax, int ay, int a_mode, int n_a, int dax, int day, int map_b, int rp,
+// (a_mode 1).  B: K rows from 0 of `map_b`.  A Gram item (one CTA) has its [hi | lo] columns by chunks, up to rank 128 as one
+// MMA of N = 2 rp, above as two of N = rp (the second from the chunk where the lo part starts).  A panel item (a pair of CTAs)
+// has the hi columns in the CTA of rank 0 and the lo columns in the other, as one MMA of N = 2 rp up to rank 128; above, the
+// first takes the columns below 128 of both parts and the second the rest.
+tc::Seg make_seg(const Geo& g, bool pair, int map_a, int ax, int ay, int a_mode, int n_a, int dax, int day, int map_b, int rp,
                  int half, int k, int d0, int d_step, int first) {
   tc::Seg s;
   std::memset(&s, 0, sizeof(s));
   s.map_a = map_a; s.map_b = map_b;
   for (int p = 0; p < n_a; ++p) { s.ax[p] = ax + dax * p; s.ay[p] = ay + day * p; s.d_col[p] = (int16_t)(d0 + d_step * p); }
   s.a_mode = (int16_t)a_mode; s.n_a = (int16_t)n_a; s.k = round16(k); s.first = (int16_t)first;
-  if (2 * rp <= 256) { s.n = (int16_t)(2 * rp); s.n_mma = 1; }
-  else { s.n = (int16_t)rp; s.n_mma = 2; s.b2_chunk = (int16_t)(half / 64); s.d_part = (int16_t)rp; }
-  s.tx_bytes = (uint32_t)(n_a * 256 * g.stage_k + g.stage_k * 128 * g.nb);
+  if (2 * rp <= 256) s.n = (int16_t)(2 * rp);
+  else if (pair) { s.n = 256; s.n2 = (int16_t)(2 * rp - 256); s.b2_chunk = 2; s.d_part = 256; }
+  else { s.n = s.n2 = (int16_t)rp; s.b2_chunk = (int16_t)(half / 64); s.d_part = (int16_t)rp; }
+  s.n_b = (int16_t)((rp + 63) / 64); s.b_x = (int16_t)half;
+  s.tx_bytes = (uint32_t)(n_a * 256 * g.stage_k + g.stage_k * 128 * (pair ? s.n_b : g.nb));
   return s;
 }
 
@@ -502,23 +506,37 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   const int nb_max = (2 * half_max + 63) / 64;
   P->nb_max = nb_max;
 
-  // ---- stage depth and panels per item ---------------------------------------------------------------------------
-  // As many panels share a B box as tensor memory has room for accumulators (2 rp columns each) and shared
-  // memory for at least two stages; K = 128 stages while two of them fit, else K = 64.
-  auto stages_with = [&](int stage_k, int n_a) { return (224 * 1024) / (n_a * 256 * stage_k + stage_k * 128 * nb_max); };
-  int n_pan = hp.tune_panels > 0 ? hp.tune_panels : 2;
+  // ---- stage depth and panels per CTA ---------------------------------------------------------------------------
+  // Panels of a CTA share B; two of them while their sums find room beside their accumulators (parked, see the engine's
+  // epilogue), else one with two accumulator buffers: the four panel launches of a step with one | two panels, us: 350M set
+  // rank 8 968 | 669, 1.5B set (rank 80) 7267 | 5164, 350M set at rank 128 1522 | 1985.
+  // K = 64 stages: a ring of many small ones rides out the latency of DRAM and of the way through the barriers of the pair
+  // better than two of K = 128 (rank 8 801 | 669, rank 80 5480 | 5164).
+  // Sets with few items per pair take one panel and K = 128: the last round of items is shorter, and of the short K loops
+  // every stage costs a trip through the barriers.  us per step, two panels and K = 64 | one and K = 128, by items (of two
+  // panels) per pair: 0.4 (tiny set) 113 | 106, 2.2 (60M) 375 | 371, 4.3 (1024 x 2730) 1190 | 1164, 5.2 (124M) 796 | 821,
+  // 13 (350M rank 8) 1645 | 1733.
+  auto stages_with = [&](int stage_k, int n_a, bool pair) {
+    return (224 * 1024) / (n_a * 256 * stage_k + stage_k * 128 * (pair ? (rp_max + 63) / 64 : nb_max));
+  };
+  int64_t panel_items = 0;                       // with two panels per CTA
+  for (const TcBlock& t : P->blk) panel_items += (c->blocks[t.id].rows + 511) / 512 + (c->blocks[t.id].cols + 511) / 512;
+  const bool few_items = panel_items < (int64_t)P->n_sms * 9 / 4;      // 4.5 per pair
+  int n_pan = hp.tune_panels > 0 ? hp.tune_panels : (few_items || 6 * rp_max > 512 ? 1 : 2);
   n_pan = std::max(1, std::min({n_pan, tc::kMaxA, 512 / (2 * rp_max)}));
-  int stage_k = hp.tune_stage_k == 64 || hp.tune_stage_k == 128 ? hp.tune_stage_k : 128;
-  if (hp.tune_stage_k == 0 && stages_with(128, std::min(n_pan, 2)) < 2) stage_k = 64;
-  while (n_pan > 1 && stages_with(stage_k, n_pan) < 2) --n_pan;
-  if (stages_with(stage_k, n_pan) < 2) stage_k = 64;
-  if (stages_with(stage_k, n_pan) < 2) { set_error_text("rank too large for the tensor path"); return ADAPM_EUNSUPPORTED; }
+  int stage_k = hp.tune_stage_k == 64 || hp.tune_stage_k == 128 ? hp.tune_stage_k : (few_items ? 128 : 64);
+  const bool gram_small = 2 * rp_max <= 256;     // two accumulators of N = 2 rp: hi and lo window
+  if (hp.tune_stage_k == 0 && stages_with(stage_k, n_pan, true) < 2) stage_k = 64;
+  if (stages_with(stage_k, gram_small ? 1 : 2, false) < 2) stage_k = 64;
+  while (n_pan > 1 && stages_with(stage_k, n_pan, true) < 2) --n_pan;
+  if (stages_with(stage_k, gram_small ? 1 : 2, false) < 2 || stages_with(stage_k, n_pan, true) < 2) {
+    set_error_text("rank too large for the tensor path");
+    return ADAPM_EUNSUPPORTED;
+  }
   P->stage_k = stage_k;
-  const bool gram_small = 4 * rp_max <= 512 && 2 * rp_max <= 256;   // two accumulators of N = 2 rp: hi and lo window
   int gram_cols = 64;                            // four partial sums up to rank 128, two above
   for (const TcBlock& t : P->blk) gram_cols = std::max(gram_cols, t.rp <= 128 ? 4 * t.rp : 2 * t.rp);
-  const int gram_na = (gram_small && stages_with(stage_k, 2) < 2) ? 1 : 2;
-  P->smem_engine = std::max(P->engine_config(n_pan).smem, P->engine_config(gram_na).smem);
+  const int gram_na = (gram_small && stages_with(stage_k, 2, false) < 2) ? 1 : 2;
 
   auto& prog = c->program;
 
@@ -571,15 +589,22 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   // With a refresh period T > 1 a step either refits both factors (phase 1) or holds L and refits R (phase 2:
   // Gram matrices of L only, column panels only, and the split copy of L carried over to the final set).
   int team_mode = (hp.flags & ADAPM_FLAG_NO_PANEL_TEAMS) ? 1 : ((hp.flags & ADAPM_FLAG_FORCE_PANEL_TEAMS) ? 2 : 0);
+  int n_pairs = std::max(1, P->n_sms / 2);
   {
-    // The team pacing lets CTAs of a launch wait for one another, which is only sound when the whole grid (at most
-    // one CTA per SM) can be resident at once: ask the runtime whether an SM takes a CTA of this size at all (a
-    // device or an MPS share with less shared memory or fewer registers does not), else hand items out longest-first.
+    // The team pacing lets pairs of a launch wait for one another, which is only sound when the whole grid (at most
+    // one CTA per SM) can be resident at once: ask the runtime how many pairs of this size the device (or an MPS share of
+    // it) takes, and hand items out longest-first if it cannot say.
+    const int smem = P->engine_config(true, n_pan).smem;
+    (void)allow_dynamic_smem(tc::tc_items_kernel<true>, smem);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * n_pairs); cfg.blockDim = dim3(tc::kEngineThreads); cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.attrs = &at; cfg.numAttrs = 1;
     int resident = 0;
-    (void)allow_dynamic_smem(tc::tc_items_kernel, P->smem_engine);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tc::tc_items_kernel, tc::kEngineThreads,
-                                                      (size_t)P->smem_engine) != cudaSuccess || resident < 1)
-      team_mode = 1;
+    if (cudaOccupancyMaxActiveClusters(&resident, tc::tc_items_kernel<true>, &cfg) != cudaSuccess || resident < 1) team_mode = 1;
+    else n_pairs = std::min(n_pairs, resident);
     (void)cudaGetLastError();
   }
   const bool with_hold = hp.refresh_period > 1 && K_eff > 0;
@@ -678,14 +703,14 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
             tc::Item it;
             std::memset(&it, 0, sizeof(it));
             if (small && gram_na == 2) {
-              it.seg[0] = make_seg(geo, map_y_t, 0, 0, 1, 2, half, 0, map_x_n, rp, half, kext, 0, 2 * rp, 1);
+              it.seg[0] = make_seg(geo, false, map_y_t, 0, 0, 1, 2, half, 0, map_x_n, rp, half, kext, 0, 2 * rp, 1);
               it.n_seg = 1; it.n_sum = 4;
             } else if (small) {
-              it.seg[0] = make_seg(geo, map_y_t, 0, 0, 1, 1, 0, 0, map_x_n, rp, half, kext, 0, 0, 1);
-              it.seg[1] = make_seg(geo, map_y_t, half, 0, 1, 1, 0, 0, map_x_n, rp, half, kext, 2 * rp, 0, 1);
+              it.seg[0] = make_seg(geo, false, map_y_t, 0, 0, 1, 1, 0, 0, map_x_n, rp, half, kext, 0, 0, 1);
+              it.seg[1] = make_seg(geo, false, map_y_t, half, 0, 1, 1, 0, 0, map_x_n, rp, half, kext, 2 * rp, 0, 1);
               it.n_seg = 2; it.n_sum = 4;
             } else {
-              it.seg[0] = make_seg(geo, map_y_t, w0, 0, 1, 2, half, 0, map_x_n, rp, half, kext, 0, 0, 1);
+              it.seg[0] = make_seg(geo, false, map_y_t, w0, 0, 1, 2, half, 0, map_x_n, rp, half, kext, 0, 0, 1);
               it.seg[0].same_acc = 1;
               it.n_seg = 1; it.n_sum = 2;
             }
@@ -698,6 +723,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
         // the factor on the N side of every product: itself, or its transformed copy in a preconditioned pass
         const int nR = precond ? mb + MAP_RTCN_T : mb + MAP_RTCN + src;
         const int nL = precond ? mb + MAP_LCN_T : mb + MAP_LCN + srcL;
+        const int pR = precond ? mb + MAP_RTCT_T : mb + MAP_RTCT + src;      // (the same in the boxes of panel items)
+        const int pL = precond ? mb + MAP_LCT_T : mb + MAP_LCT + srcL;
         if (!hold) {
           gram(mb + MAP_RTCT + src, nR, n, 0, -1.f / a1);  // Bop1[j][k] = -(R R^T)[j][k] / (1-b1), stored as [k][j]
           gram(mb + MAP_RTCT + prev, nR, n, 1, b1 / a1);   // Bop2[j][k] = b1 (R R0^T)[j][k] / (1-b1)
@@ -705,17 +732,17 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
         gram(mb + MAP_LCT + srcL, nL, m, 2, -1.f / a1);    // Bop3[j][k] = -(L^T L)[j][k] / (1-b1)
         gram(mb + MAP_LCT + prev, nL, m, 3, b1 / a1);      // Bop4[j][k] = b1 (L^T L0)[j][k] / (1-b1)
 
-        // one item = up to n_pan adjacent panels of 128 owners that share every B box
+        // one item = adjacent panels of 128 owners, np for each CTA of a pair, that share B
         auto panel = [&](bool is_L, int p0, int np) {
           tc::Item it;
           std::memset(&it, 0, sizeof(it));
           const int mS = (is_L ? mb + MAP_LC : mb + MAP_RTC) + src, m0 = (is_L ? mb + MAP_LC : mb + MAP_RTC) + prev;
           const int g1 = mb + MAP_GS + (is_L ? 0 : 2), g2 = g1 + 1;
-          if (is_L) it.seg[0] = make_seg(geo, mb + MAP_G, 0, p0, 0, np, 0, 128, nR, rp, half, n, 0, 2 * rp, 1);  // g R^T
-          else it.seg[0] = make_seg(geo, mb + MAP_GT, p0, 0, 1, np, 128, 0, nL, rp, half, m, 0, 2 * rp, 1);      // g^T L
+          if (is_L) it.seg[0] = make_seg(geo, true, mb + MAP_G, 0, p0, 0, np, 0, 128, pR, rp, half, n, 0, 2 * rp, 1);  // g R^T
+          else it.seg[0] = make_seg(geo, true, mb + MAP_GT, p0, 0, 1, np, 128, 0, pL, rp, half, m, 0, 2 * rp, 1);      // g^T L
           // [hi | lo] of the current and of the previous factor against the stacked Gram operands
-          it.seg[1] = make_seg(geo, mS, 0, p0, 0, np, 0, 128, g1, rp, half, half + rp, 0, 2 * rp, 0);
-          it.seg[2] = make_seg(geo, m0, 0, p0, 0, np, 0, 128, g2, rp, half, half + rp, 0, 2 * rp, 0);
+          it.seg[1] = make_seg(geo, true, mS, 0, p0, 0, np, 0, 128, g1, rp, half, half + rp, 0, 2 * rp, 0);
+          it.seg[2] = make_seg(geo, true, m0, 0, p0, 0, np, 0, 128, g2, rp, half, half + rp, 0, 2 * rp, 0);
           it.n_seg = 3;
           it.n_pan = np; it.acc_stride = 2 * rp;
           it.epi = tc::EPI_FACTOR; it.r = r; it.rp = rp; it.half = half; it.coef = coef;
@@ -732,14 +759,14 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
         BlockSpan sp;
         sp.first = panels.size();
         if (!hold)
-          for (int p0 = 0; p0 < m; p0 += 128 * n_pan) panel(true, p0, std::min(n_pan, (m - p0 + 127) / 128));
+          for (int p0 = 0; p0 < m; p0 += 256 * n_pan) panel(true, p0, std::min(n_pan, (m - p0 + 255) / 256));
         sp.n_row = panels.size() - sp.first;
-        for (int p0 = 0; p0 < n; p0 += 128 * n_pan) panel(false, p0, std::min(n_pan, (n - p0 + 127) / 128));
+        for (int p0 = 0; p0 < n; p0 += 256 * n_pan) panel(false, p0, std::min(n_pan, (n - p0 + 255) / 256));
         sp.n_col = panels.size() - sp.first - sp.n_row;
         spans.push_back(sp);
       }
       const int grid_g = (int)std::min<int64_t>((int64_t)grams.size(), P->n_sms);
-      const int grid_p = (int)std::min<int64_t>((int64_t)panels.size(), P->n_sms);
+      const int grid_p = (int)std::min<int64_t>((int64_t)panels.size(), n_pairs);       // pairs
       std::vector<int32_t> begin_g, begin_p;
       schedule_items(grams, grid_g, begin_g, stage_k);
       P->n_teams = std::max(P->n_teams, schedule_panels(panels, spans, grid_p, begin_p, stage_k, team_mode));
@@ -832,7 +859,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     m.h_maps.resize(P->blk.size() * kMapsPerBlock);
   }
   if (e == cudaSuccess && P->n_teams > 0) e = cudaMalloc((void**)&P->d_team_counters, P->n_teams * sizeof(int32_t));
-  if (e == cudaSuccess) e = allow_dynamic_smem(tc::tc_items_kernel, P->smem_engine);
+  if (e == cudaSuccess) e = allow_dynamic_smem(tc::tc_items_kernel<true>, P->engine_config(true, n_pan).smem);
+  if (e == cudaSuccess) e = allow_dynamic_smem(tc::tc_items_kernel<false>, P->engine_config(false, gram_na).smem);
   for (int form = 0; form < 4; ++form)
     if (e == cudaSuccess)
       e = allow_dynamic_smem(apply_kernel(form >> 1, form & 1), P->apply_config(form >> 1, form & 1).smem);
@@ -915,11 +943,13 @@ int tensor_prepare_step(adapm_ctx* c, const Bases& b, int64_t t, cudaStream_t s,
     if (c->hp.inner_precond) {
       ok = ok && tc::encode_bf16_chunked(&m[MAP_LCN_T], work + t2.lct * 2, rows, 2 * half, nb, sk);
       ok = ok && tc::encode_bf16_chunked(&m[MAP_RTCN_T], work + t2.rtct * 2, cols, 2 * half, nb, sk);
+      ok = ok && tc::encode_bf16_matrix(&m[MAP_LCT_T], work + t2.lct * 2, rows, 2 * half, 2 * half, sk);
+      ok = ok && tc::encode_bf16_matrix(&m[MAP_RTCT_T], work + t2.rtct * 2, cols, 2 * half, 2 * half, sk);
     }
     if (aligned && b.shadow)
       ok = ok && tc::encode_panel32(&m[MAP_SH], reinterpret_cast<const char*>(b.shadow) + blk.offset * 2, rows, cols, false);
     for (int q = 0; q < 4; ++q)
-      ok = ok && tc::encode_bf16_chunked(&m[MAP_GS + q], work + t2.gs[q] * 2, 2 * half, 2 * half, nb, sk);
+      ok = ok && tc::encode_bf16_matrix(&m[MAP_GS + q], work + t2.gs[q] * 2, 2 * half, 2 * half, 2 * half, sk);
     if (!ok) {
       set_error_text("cuTensorMapEncodeTiled failed for a low-rank block");
       return ADAPM_ECUDA;
@@ -970,7 +1000,8 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       a.items = (const tc::Item*)tab; a.n_items = (int32_t)L.n_items; a.maps = P->cur_maps;
       a.f32_base = (float*)b.p[BASE_STATE]; a.work_bf16 = (uint16_t*)b.p[BASE_WORK]; a.work_f32 = (float*)b.p[BASE_WORK];
       a.status = c->d_status;
-      const TcProgram::EngineConfig e = P->engine_config((int)L.aux2);
+      const bool pair = L.kind == LK_TC_PANEL;
+      const TcProgram::EngineConfig e = P->engine_config(pair, (int)L.aux2);
       a.stage_k = P->stage_k; a.stage_bytes = e.stage_bytes; a.n_stages = e.n_stages; a.a_bytes = e.a_bytes;
       a.acc_cols = (int32_t)L.aux0; a.n_acc = (int32_t)L.aux1;
       a.cta_begin = (const int32_t*)(c->d_tables + L.aux3);
@@ -982,7 +1013,8 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
         ADAPM_CUDA(cudaMemsetAsync(P->d_team_counters, 0, P->n_teams * sizeof(int32_t), s));
         a.team_counters = P->d_team_counters;
       }
-      launch_chained(c->step_bytes < kChainedBytes, tc::tc_items_kernel, (unsigned)L.grid, tc::kEngineThreads, e.smem, s, a);
+      if (pair) launch_clusters(c->step_bytes < kChainedBytes, 2, tc::tc_items_kernel<true>, 2 * (unsigned)L.grid, tc::kEngineThreads, e.smem, s, a);
+      else launch_chained(c->step_bytes < kChainedBytes, tc::tc_items_kernel<false>, (unsigned)L.grid, tc::kEngineThreads, e.smem, s, a);
       break;
     }
     case LK_TC_APPLY: {
@@ -1012,7 +1044,7 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
   return ADAPM_OK;
 }
 
-// Diagnostic: one CTA of the engine whose only item waits for a team counter that nothing advances, with a wait
+// Diagnostic: one pair of CTAs of the engine whose only item waits for a team counter that nothing advances, with a wait
 // limit of about a millisecond.  The kernel must return, leave ST_WAIT_TEAM in the status word and free its
 // tensor memory; the context stays usable.
 int run_expired_wait_probe(adapm_ctx* c, cudaStream_t s) {
@@ -1028,7 +1060,7 @@ int run_expired_wait_probe(adapm_ctx* c, cudaStream_t s) {
   a.sum_col = -1; a.sumsq_on = 0;
   a.team_counters = c->d_status + 16;       // a zeroed word beside the status word that nothing adds to
   a.team_spin_limit = 1u << 12; a.wait_spin_limit = tc::kWaitSpinDefault;
-  tc::tc_items_kernel<<<1, tc::kEngineThreads, 4096, s>>>(a);
+  launch_clusters(false, 2, tc::tc_items_kernel<true>, 2, tc::kEngineThreads, 4096, s, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_cuda_error(e, "run_expired_wait_probe");

@@ -52,6 +52,46 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Arrives at the same barrier of CTA `rank` of the cluster.  (With .release.cluster an arrival takes a thousand cycles, which
+// set the pace of the whole pair; the threads that arrive here have written nothing the other CTA reads: what they report is
+// shared memory that TMA has filled and tensor memory that has been read, ordered by the barrier and tcgen05.fence.)
+__device__ __forceinline__ void mbar_arrive_at(uint64_t* bar, uint32_t rank) {
+  asm volatile(
+      "{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, %1;\n"
+      "mbarrier.arrive.shared::cluster.b64 _, [ra];\n}" ::"r"(smem_u32(bar)),
+      "r"(rank)
+      : "memory");
+}
+
+// ---- pairs of CTAs -----------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A word of shared memory of CTA `rank`, at the address it has in this CTA.
+__device__ __forceinline__ int load_shared_of(const int* p, uint32_t rank) {
+  int v;
+  asm volatile("{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %1, %2;\nld.shared::cluster.s32 %0, [ra];\n}"
+               : "=r"(v)
+               : "r"(smem_u32(p)), "r"(rank)
+               : "memory");
+  return v;
+}
+
+// Whether the phase with the given parity is complete; does not suspend.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Waits for the phase with the given parity to complete.  Gives up after `limit` polls or as
 // soon as another thread of the CTA has given up (*abort != 0); then sets *abort, records `code` in
 // the device status word and returns false.  Callers leave their loops on false.
@@ -89,6 +129,8 @@ __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xf
 // shapes: 2.1 -> 1.4 ms).
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* status,
                                                int32_t code, uint32_t limit = kSpinLimit) {
+  for (int it = 0; it < 8; ++it)
+    if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
   for (uint32_t it = 0; it < limit; ++it) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     if (it > 32) {
@@ -161,23 +203,45 @@ __device__ __forceinline__ void bulk_wait_group() {
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- tcgen05 -------------------------------------------------------------------------------------
+// PAIR: the cta_group::2 forms, which one kernel may not mix with the others.  Both CTAs of the pair allocate and free
+// together; the CTA of rank 0 issues the MMAs and the commits for both.
+template <bool PAIR = false>
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_result, uint32_t cols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)),
-               "r"(cols)
-               : "memory");
+  if (PAIR)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)),
+                 "r"(cols)
+                 : "memory");
+  else
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)),
+                 "r"(cols)
+                 : "memory");
 }
+template <bool PAIR = false>
 __device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  if (PAIR) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  else asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+template <bool PAIR = false>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+  if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+  else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
+// D[tmem] (+)= A[smem] * B[smem]; issued by one thread.  PAIR: M = 256, each CTA holds 128 rows of A and D and half of
+// the columns of B (the lower half in the CTA of rank 0), at the same addresses.
+template <bool PAIR = false>
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          uint32_t accumulate) {
+  if (PAIR) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+    return;
+  }
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
@@ -193,8 +257,17 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// The mbarrier gets one arrival when every MMA this thread issued before has completed.
+// The mbarrier gets one arrival when every MMA this thread issued before has completed.  PAIR: in both CTAs.
+template <bool PAIR = false>
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  if (PAIR) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+    return;
+  }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
@@ -232,8 +305,8 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---- descriptors -----------------------------------------------------------------------------------
-// Instruction descriptor of kind::f16 with bf16 operands and fp32 accumulation, M = 128.
-__device__ __host__ __forceinline__ uint32_t make_idesc(int n, bool a_mn_major, bool b_mn_major, bool negate_a) {
+// Instruction descriptor of kind::f16 with bf16 operands and fp32 accumulation.
+__device__ __host__ __forceinline__ uint32_t make_idesc(int n, bool a_mn_major, bool b_mn_major, bool negate_a, int m = 128) {
   uint32_t d = 0;
   d |= 1u << 4;                          // accumulator format: fp32
   d |= 1u << 7;                          // A format: bf16
@@ -242,7 +315,7 @@ __device__ __host__ __forceinline__ uint32_t make_idesc(int n, bool a_mn_major, 
   d |= (a_mn_major ? 1u : 0u) << 15;
   d |= (b_mn_major ? 1u : 0u) << 16;
   d |= (uint32_t)(n >> 3) << 17;
-  d |= (uint32_t)(128 >> 4) << 24;
+  d |= (uint32_t)(m >> 4) << 24;
   return d;
 }
 

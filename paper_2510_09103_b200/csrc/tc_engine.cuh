@@ -1,6 +1,7 @@
 // A persistent, warp-specialised tcgen05 engine that runs a table of "items".  An item is a short
 // list of K-loops ("segments") that accumulate into 128-row accumulators in tensor memory,
-// followed by an epilogue that turns the accumulators into the result of one step of Algorithm 2:
+// followed by an epilogue that turns the accumulators into the result of one step of Algorithm 2.
+// It has two forms: panel items run on pairs of CTAs (cta_group::2, M = 256), Gram items on single ones.
 //
 //   refit of L (row panels of 128 rows of a block, Algorithm 2's L update):
 //       D = g R^T + [L hi | L lo] X + [L0 hi | L0 lo] Y     X = [Bop1; Bop1], Bop1 = -(R R^T)/(1-b1)
@@ -16,8 +17,9 @@
 // lo parts are stored side by side ([rows, 2 half]: hi columns from 0, lo columns from `half`;
 // half = rp = r rounded up to 16 while 2 rp <= 256, else rp rounded up to 64), so that used as the
 // N side of an MMA the two parts land in two column ranges of the accumulator, which the epilogue
-// adds.  While 2 rp <= 256 one MMA of N = 2 rp covers both parts; above that the hi and the lo part
-// take one MMA of N = rp each, the second reading B from the chunk at which the lo part starts.
+// adds.  In a pair the CTA of rank 0 holds the hi columns of B and the other one the lo columns; one MMA of N = 2 rp takes
+// both up to rank 128, above that the first takes N = 256 (128 columns of each part) and a second one the rest.  A Gram item
+// above rank 128 takes one MMA of N = rp for the hi and one for the lo part, which starts at a chunk of its own.
 // (Letting both add to the same columns would free half of the accumulator, but the small products then meet the
 // rounding of the large sums: errors of L R against 64 bits up to twice as large at ranks 128 to 256.)
 //
@@ -25,15 +27,21 @@
 //   A  up to three operands of 128 rows x stage_k (K along x: boxes of 64 x 128) or stage_k x 128
 //      columns (K along y: two boxes of 64 x stage_k).  All are multiplied with the same B and fill
 //      one accumulator each: the more operands share a B, the fewer bytes a flop brings in
-//   B  one 3-D box: stage_k rows x (64 x chunks) columns of a [rows, 2 half] array, i.e. the N side
-//      read MN-major with its 64-column chunks one box apart
-// Warp roles (512 threads, 128 registers each): warp 0 issues the TMA loads of a stage, warp 1 issues
-// its MMAs, warps 4-7 add up g^2 per row from the gradient tiles of the first segment when the
-// launch asks for it (the second-moment statistic of the block-mean form then needs no pass of its
-// own over g), warps 8-15 drain the accumulators (two groups of four warps that take the 16-column
-// pieces of an item alternately); warps 2 and 3 have no work.  The two issuing warps run dependent
-// scalar code, so their per-stage instruction count is what bounds the rate; both loops are kept
-// short, and all lanes run them so that their operands stay in uniform registers (mbar_wait_warp).  With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
+//   B  stage_k rows of 64-column chunks of a [rows, 2 half] array, i.e. the N side read MN-major with its chunks one box
+//      apart; in a pair each CTA's own part
+// Why pairs: with M = 128 every MMA reads A and all of B from the shared memory of its SM and every CTA brings in all of
+// B, 115 of the 128 bytes a cycle an SM's shared memory delivers at rank 80 before the fills; at rank 204, where tensor
+// memory has room for one panel, four fifths of the fills are B.  A pair reads and fills half of B per SM.  A panel launch,
+// one CTA -> pair: 3.65 -> 2.5 ms on eight layers of the 8B shapes, 1.20 -> 1.11 ms on the 1.5B set, 437 -> 370 us on the
+// 350M set at rank 128, 172 -> 147 at rank 8.  What is left there: the power cap (SM clocks of 1.3 to 1.5 GHz while these
+// launches run) and, per stage, the serial path of the warp that issues the MMAs.
+// Warp roles (512 threads, 128 registers each): warp 0 loads A, warp 3 loads B, warp 1 issues the MMAs (in a pair that of
+// rank 0, for both), warp 2 of rank 1 tells rank 0 which of its stages are full, warps 4-7 add up g^2 per row from the
+// gradient tiles of the first segment when the launch asks for it (the second-moment statistic of the block-mean form then
+// needs no pass of its own over g), warps 8-15 drain the accumulators (two groups of four warps that take the 16-column
+// pieces of an item alternately).  The issuing warps run dependent scalar code, so their per-stage instruction count bounds
+// the rate; all lanes run the loops on values that the compiler knows to be uniform (mbar_wait_warp, uniform).
+// With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
 // Every wait is bounded; when one runs out the CTA records a status bit, stops taking work and
 // leaves through the common exit (which frees its tensor memory).  A launch that finds the status
 // word set on entry does nothing.
@@ -50,33 +58,36 @@ constexpr int kMaxSegs = 4;
 constexpr int kMaxA = 3;
 constexpr int kEngineThreads = 512;
 constexpr uint32_t kTeamSpinDefault = 1u << 22;   // polls of 256 ns each: about a second
+constexpr uint32_t kDrainSpins = 1u << 16;         // of a copy in flight when a CTA gives up: tens of milliseconds
 constexpr uint32_t kWaitSpinDefault = 1u << 23;   // mbarrier polls: at least as long as a team wait
 
 enum : int32_t { EPI_FACTOR = 0, EPI_GRAM = 1, EPI_NONE = 2 };   // EPI_NONE: a filler that only keeps a CTA in step
 
 struct Seg {
   int32_t map_a;             // 2-D tensor map: boxes of 64 x 128 (a_mode 0) or 64 x stage_k (a_mode 1)
-  int32_t map_b;             // 3-D tensor map (64, rows, chunks), box 64 x stage_k x chunks
+  int32_t map_b;             // one CTA: 3-D tensor map (64, rows, chunks), box 64 x stage_k x chunks; pair: 2-D, boxes of 64 x stage_k
   int32_t ax[kMaxA], ay[kMaxA];   // element coordinates of the first box of each A operand
   int32_t k;                 // K extent, multiple of 16
-  uint32_t tx_bytes;         // bytes one stage of this segment brings in
+  uint32_t tx_bytes;         // bytes one stage of this segment brings into a CTA
   int16_t a_mode;            // 0: K runs along x (K-major A), 1: K runs along y (MN-major A)
   int16_t n;                 // N of one MMA (multiple of 16, <= 256)
-  int16_t n_a;               // A operands (1..kMaxA)
-  int16_t n_mma;             // 1, or 2: a second MMA per K step reads B from chunk b2_chunk and adds at +d_part
+  int16_t n_a;               // A operands of a CTA (1..kMaxA)
+  int16_t n2;                // N of a second MMA per K step that reads B from chunk b2_chunk and adds at +d_part, or 0
   int16_t d_col[kMaxA];      // accumulator column of each A operand
   int16_t first;             // 1: its first MMA overwrites the accumulators
   int16_t b2_chunk, d_part;
   int16_t same_acc;          // 1: the A operands share one accumulator (all but the first always accumulate)
+  int16_t n_b, b_x;          // pair: boxes of B per CTA, and the column of B at which the part of the CTA of rank 1 starts
 };
 
 struct Item {
   Seg seg[kMaxSegs];
   int32_t n_seg;
   int32_t epi;
-  // EPI_FACTOR: panel p (p < n_pan) has its accumulator at column acc_stride * p; the thread that owns
-  // accumulator row q of panel p updates factor entries (owner = own0 + 128 p + q, k):
-  //   new[owner][k] = old[owner][k] + coef * (D[q][k] + D[q][rp + k])                  k < r
+  // EPI_FACTOR: a CTA has n_pan panels, those of the CTA of rank 1 (and its A operands) follow on those of rank 0, and
+  // panels beyond own_count do not exist.  Panel p has its accumulator at column acc_stride * p; the thread that owns
+  // accumulator row q of panel p updates factor entries (owner = first + 128 p + q, k):
+  //   new[owner][k] = old[owner][k] + coef * (D hi[q][k] + D lo[q][k])                 k < r
   //   dst[owner][k] = hi, dst[owner][half + k] = lo                                    k < rp
   // Old and new fp32 values live in the state, f32[own_stride * owner + k_stride * k], or in the workspace in the order
   // in which the epilogue's threads take them (iter_at).
@@ -135,76 +146,142 @@ struct EngineArgs {
 struct __align__(8) EngineShared {
   uint64_t full[8], empty[8], tfull[2], tempty[2];
   uint32_t tmem_base;
-  int abort;
+  int abort, skip;
 };
 
-// The loads of one stage: NA operands of NBOX boxes each, then the B box.  Compile-time counts keep the issuing
-// thread's instruction stream short (it runs dependent scalar code; its rate bounds the pipeline).
+// The A operands of one stage, NBOX boxes each.  Compile-time counts keep the issuing thread's instruction stream short (it
+// runs dependent scalar code; its rate bounds the pipeline).
 template <int NA, int NBOX>
-__device__ __forceinline__ void load_stage(uint8_t* sa, int a_tile, int box_bytes, int a_bytes, const CUtensorMap* ma,
-                                           const CUtensorMap* mb, const int* x, const int* y, int yb, uint64_t* bar) {
+__device__ __forceinline__ void load_operands(uint8_t* sa, int a_tile, int box_bytes, const CUtensorMap* ma, const int* x,
+                                              const int* y, uint64_t* bar) {
 #pragma unroll
   for (int p = 0; p < NA; ++p)
 #pragma unroll
     for (int j = 0; j < NBOX; ++j) tma_load_box(sa + p * a_tile + j * box_bytes, ma, x[p] + 64 * j, y[p], bar);
-  tma_load_box3(sa + a_bytes, mb, 0, yb, 0, bar);
 }
 
-// The MMAs of one stage: nk K steps, NA operands, NM MMAs per operand and step.
-template <int NA, int NM, bool MN_MAJOR_A>
-__device__ __forceinline__ void mma_stage(const uint32_t* dcol, uint32_t d_part, uint32_t same, uint32_t sa, int a_tile,
-                                          uint32_t a_lbo, uint32_t blo, uint32_t b2, uint32_t dhi, uint32_t idesc, int nk,
-                                          uint32_t accumulate) {
-  uint32_t alo[NA];
-#pragma unroll
-  for (int p = 0; p < NA; ++p) alo[p] = desc_lo(sa + (uint32_t)(p * a_tile), a_lbo);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    if (q < nk) {
-      const uint32_t astep = MN_MAJOR_A ? (uint32_t)(q * 128) : (uint32_t)((q >> 2) * (kBoxBytes >> 4) + (q & 3) * 2);
-      const uint64_t bd = desc_join(blo + (uint32_t)(q * 128), dhi);
-#pragma unroll
-      for (int p = 0; p < NA; ++p) {
-        const uint64_t ad = desc_join(alo[p] + astep, dhi);
-        const uint32_t acc_p = q > 0 ? 1u : ((p > 0 && same) ? 1u : accumulate);
-        mma_bf16(dcol[p], ad, bd, idesc, acc_p);
-        if (NM == 2) mma_bf16(dcol[p] + d_part, ad, desc_join(blo + b2 + (uint32_t)(q * 128), dhi), idesc, acc_p);
-      }
-    }
+// Lets the copies already issued into a ring of `n_stages` land before the CTA exits.  (stage, phase): where the next would go.
+__device__ __forceinline__ void drain_ring(uint64_t* full, int stage, uint32_t phase, uint32_t issued, int n_stages) {
+  const int back = issued < (uint32_t)n_stages ? (int)issued : n_stages;
+  for (int q = 0; q < back; ++q) {
+    int st = stage - 1 - q;
+    uint32_t ph = phase;
+    if (st < 0) { st += n_stages; ph ^= 1u; }
+    for (uint32_t spin = 0; spin < kDrainSpins && !mbar_try_wait(&full[st], ph); ++spin) __nanosleep(64);
   }
 }
 
+// What the warp that issues the MMAs carries from stage to stage (the same in all lanes).
+struct MmaCursor {
+  int stage;
+  uint32_t phase;
+};
+struct MmaSeg {
+  uint32_t dcol[kMaxA], d_part, same, accumulate, idesc, idesc2, b2, b_lbo;
+  int k;
+};
+
+// The stages of one segment: KS K steps each (less in the last one), NA operands, NM MMAs per operand and step.  The loop is
+// instantiated for the counts and all lanes run it on uniform values: the warp issues in program order, and what it does
+// beside the MMAs of a stage (300 to 800 cycles of tensor work) has to fit in the same time.
+template <bool PAIR, int NA, int NM, bool MN_MAJOR_A, int KS>
+__device__ __forceinline__ bool mma_segment(const EngineArgs& a, EngineShared& sh, MmaCursor& cur, const MmaSeg& S, uint32_t ring,
+                                            bool leader) {
+  constexpr int kStageK = 16 * KS;
+  const uint32_t dhi = desc_hi();
+  const uint32_t a_lbo = MN_MAJOR_A ? S.b_lbo : 16u;
+  uint32_t accumulate = S.accumulate;
+  for (int k_left = S.k; k_left > 0; k_left -= kStageK) {
+    if (!mbar_wait_warp(&sh.full[cur.stage], cur.phase, &sh.abort, a.status, ST_WAIT_FULL, a.wait_spin_limit)) return false;
+    tc_fence_after();
+    // per K step of 16, in 16-byte units: K along x walks 32 B inside a box and 16 KB to the next box; K along y walks 16
+    // rows of 128 B
+    const uint32_t slot = ring + (uint32_t)(cur.stage * a.stage_bytes);
+    const uint32_t alo = desc_lo(slot, a_lbo);
+    const uint32_t blo = desc_lo(slot + (uint32_t)a.a_bytes, S.b_lbo);
+    if (leader) {
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        if (16 * q < k_left) {
+          const uint32_t astep = MN_MAJOR_A ? (uint32_t)(q * 128) : (uint32_t)((q >> 2) * (kBoxBytes >> 4) + (q & 3) * 2);
+          const uint64_t bd = desc_join(blo + (uint32_t)(q * 128), dhi);
+#pragma unroll
+          for (int p = 0; p < NA; ++p) {
+            const uint64_t ad = desc_join(alo + (uint32_t)(p * (256 * kStageK >> 4)) + astep, dhi);
+            const uint32_t acc_p = q > 0 ? 1u : ((p > 0 && S.same) ? 1u : accumulate);
+            mma_bf16<PAIR>(S.dcol[p], ad, bd, S.idesc, acc_p);
+            if (NM == 2) mma_bf16<PAIR>(S.dcol[p] + S.d_part, ad, desc_join(blo + S.b2 + (uint32_t)(q * 128), dhi), S.idesc2, acc_p);
+          }
+        }
+      }
+      mma_commit<PAIR>(&sh.empty[cur.stage]);
+    }
+    __syncwarp();
+    accumulate = 1u;
+    if (++cur.stage == a.n_stages) { cur.stage = 0; cur.phase ^= 1u; }
+  }
+  return true;
+}
+
+// The form of a segment: the operand counts that the items of a launch have (one panel per CTA where two MMAs are needed; A of
+// a Gram item always has K along y).
+template <bool PAIR, int KS>
+__device__ __forceinline__ bool mma_segment_any(const EngineArgs& a, EngineShared& sh, MmaCursor& cur, const MmaSeg& S, int n_a,
+                                                bool two, bool mn_major, uint32_t ring, bool leader) {
+#define ADAPM_MMA(NA, NM, MN) return mma_segment<PAIR, NA, NM, MN, KS>(a, sh, cur, S, ring, leader)
+  if (!PAIR) {
+    if (two) { if (n_a == 2) ADAPM_MMA(2, 2, true); ADAPM_MMA(1, 2, true); }
+    if (n_a == 2) ADAPM_MMA(2, 1, true);
+    ADAPM_MMA(1, 1, true);
+  }
+  if (two) { if (mn_major) ADAPM_MMA(1, 2, true); ADAPM_MMA(1, 2, false); }
+  if (mn_major) {
+    if (n_a == 2) ADAPM_MMA(2, 1, true);
+    if (n_a == 3) ADAPM_MMA(3, 1, true);
+    ADAPM_MMA(1, 1, true);
+  }
+  if (n_a == 2) ADAPM_MMA(2, 1, false);
+  if (n_a == 3) ADAPM_MMA(3, 1, false);
+  ADAPM_MMA(1, 1, false);
+#undef ADAPM_MMA
+}
+
+template <bool PAIR>
 __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs a) {
   extern __shared__ uint8_t dyn_smem[];
   __shared__ EngineShared sh;
-  __shared__ int skip_launch;
   wait_for_previous_kernel();
-  if (threadIdx.x == 0) skip_launch = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
-  __syncthreads();
-  if (skip_launch) return;   // an earlier launch gave up: write nothing (the whole CTA decides together)
+  const uint32_t rank = PAIR ? cluster_rank() : 0u;
+  const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort = &sh.abort;
   const uint32_t wlim = a.wait_spin_limit;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 8; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], a.sumsq_on ? 5 : 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 256); }
+    for (int i = 0; i < 8; ++i) {
+      mbar_init(&sh.full[i], PAIR && rank == 0 ? 3 : 2);      // A, B, and for rank 0 the other CTA's stage
+      mbar_init(&sh.empty[i], PAIR && a.sumsq_on ? 5 : 1);
+    }
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], PAIR ? 16 : 8); }
     sh.abort = 0;
+    sh.skip = *reinterpret_cast<volatile int32_t*>(a.status) != 0;
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&sh.tmem_base, 512);
-    tmem_relinquish();
+    tmem_alloc<PAIR>(&sh.tmem_base, 512);
+    tmem_relinquish<PAIR>();
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = sh.tmem_base;
-  const int it_begin = a.cta_begin[blockIdx.x], it_end = a.cta_begin[blockIdx.x + 1];
+  // an earlier launch gave up: write nothing (the CTAs that work together decide together)
+  const bool skip = (PAIR ? load_shared_of(&sh.skip, 0) : sh.skip) != 0;
+  const int it_begin = uniform(skip ? 0 : a.cta_begin[unit]), it_end = uniform(skip ? 0 : a.cta_begin[unit + 1]);
   const int stage_k = a.stage_k;
   const int a_tile = 256 * stage_k;                 // bytes of one A operand of a stage
-  const int ksteps = stage_k >> 4;                  // MMA K steps per full stage
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (all lanes run, one issues)
@@ -215,8 +292,8 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
     bool ok = true;
     for (int it = it_begin; it < it_end && ok; ++it) {
       const Item& I = a.items[it];
-      const int wait_count = I.wait_count, signal = I.signal, n_seg = I.n_seg;
-      int32_t* const team = a.team_counters + I.team;
+      const int wait_count = uniform(I.wait_count), signal = uniform((int)I.signal), n_seg = uniform(I.n_seg);
+      int32_t* const team = a.team_counters + uniform((int)I.team);
       if (wait_count > 0) {
         // Bounded like every wait here: a team member that never arrives ends this CTA with a status, not a
         // hang.  The bound is generous (about a second), because a member may start late when other work
@@ -235,14 +312,13 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       }
       for (int s = 0; s < n_seg && ok; ++s) {
         const Seg& S = I.seg[s];
-        const CUtensorMap* ma = a.maps + S.map_a;
-        const CUtensorMap* mb = a.maps + S.map_b;
-        const int nst = (S.k + stage_k - 1) / stage_k, a_mode = S.a_mode, n_a = S.n_a;
-        const uint32_t tx_bytes = S.tx_bytes;
+        const CUtensorMap* ma = a.maps + uniform(S.map_a);
+        const int nst = (uniform(S.k) + stage_k - 1) / stage_k, a_mode = uniform((int)S.a_mode), n_a = uniform((int)S.n_a);
+        const uint32_t tx_bytes = (uint32_t)(n_a * a_tile);
+        const int after = (int)rank * 128 * n_a;      // rank 1's operands follow on those of rank 0
         int x[kMaxA], y[kMaxA];
 #pragma unroll
-        for (int p = 0; p < kMaxA; ++p) { x[p] = S.ax[p]; y[p] = S.ay[p]; }
-        int yb = 0;
+        for (int p = 0; p < kMaxA; ++p) { x[p] = uniform(S.ax[p]) + (a_mode ? after : 0); y[p] = uniform(S.ay[p]) + (a_mode ? 0 : after); }
         const int dx = a_mode ? 0 : stage_k, dy = a_mode ? stage_k : 0;
         // K along x: stage_k / 64 boxes of 64 x 128, 16 KB apart; K along y: two boxes of 64 x stage_k
         const int n_box = a_mode ? 2 : (stage_k >> 6);
@@ -253,102 +329,116 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           uint64_t* bar = &sh.full[stage];
           if (leader) {
             mbar_arrive_expect_tx(bar, tx_bytes);
-            if (n_box == 2) {
-              if (n_a == 2) load_stage<2, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else if (n_a == 3) load_stage<3, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else load_stage<1, 2>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+#define ADAPM_LOAD(NA, NBOX) load_operands<NA, NBOX>(sa, a_tile, box_bytes, ma, x, y, bar)
+            if (!PAIR) {
+              if (n_a == 2) ADAPM_LOAD(2, 2); else ADAPM_LOAD(1, 2);
+            } else if (n_box == 2) {
+              if (n_a == 2) ADAPM_LOAD(2, 2); else if (n_a == 3) ADAPM_LOAD(3, 2); else ADAPM_LOAD(1, 2);
             } else {
-              if (n_a == 2) load_stage<2, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else if (n_a == 3) load_stage<3, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
-              else load_stage<1, 1>(sa, a_tile, box_bytes, a.a_bytes, ma, mb, x, y, yb, bar);
+              if (n_a == 2) ADAPM_LOAD(2, 1); else if (n_a == 3) ADAPM_LOAD(3, 1); else ADAPM_LOAD(1, 1);
             }
+#undef ADAPM_LOAD
           }
           __syncwarp();
 #pragma unroll
           for (int p = 0; p < kMaxA; ++p) { x[p] += dx; y[p] += dy; }
-          yb += stage_k;
           ++issued;
           if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
         }
       }
-      if (ok && signal && leader) atomicAdd(team, signal);
+      if (ok && signal && leader && rank == 0) atomicAdd(team, signal);
     }
-    if (!ok) {
-      // leave no copy in flight: every stage that was filled must have landed before the CTA exits
-      const int back = issued < (uint32_t)a.n_stages ? (int)issued : a.n_stages;
-      for (int q = 0; q < back; ++q) {
-        int st = stage - 1 - q;
-        uint32_t ph = phase;
-        if (st < 0) { st += a.n_stages; ph ^= 1u; }
-        for (uint32_t spin = 0; spin < kSpinLimit && !mbar_try_wait(&sh.full[st], ph); ++spin) __nanosleep(64);
-      }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (all lanes run, one issues)
+    if (!ok) drain_ring(sh.full, stage, phase, issued, a.n_stages);
+  } else if (warp == 3) {
+    // ------------------------------------------------------------------ producer of B (a warp of its own: an expected
+    // count and a box take 100 cycles each to issue, and a stage of 64 K is multiplied in 300 to 800)
     const bool leader = elect_one();
     int stage = 0;
     uint32_t phase = 0;
+    uint32_t issued = 0;
+    bool ok = true;
+    const int b_box = stage_k * 128;
+    for (int it = it_begin; it < it_end && ok; ++it) {
+      const Item& I = a.items[it];
+      const int n_seg = uniform(I.n_seg);
+      for (int s = 0; s < n_seg && ok; ++s) {
+        const Seg& S = I.seg[s];
+        const CUtensorMap* mb = a.maps + uniform(S.map_b);
+        const int nst = (uniform(S.k) + stage_k - 1) / stage_k, n_b = uniform((int)S.n_b), xb = rank ? uniform((int)S.b_x) : 0;
+        const uint32_t tx_bytes = uniform(S.tx_bytes) - (uint32_t)(uniform((int)S.n_a) * a_tile);
+        for (int c = 0; c < nst; ++c) {
+          if (!mbar_wait_warp(&sh.empty[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
+          uint8_t* sb = stages + stage * a.stage_bytes + a.a_bytes;
+          uint64_t* bar = &sh.full[stage];
+          if (leader) {
+            mbar_arrive_expect_tx(bar, tx_bytes);
+            if (PAIR) {
+              tma_load_box(sb, mb, xb, c * stage_k, bar);
+              if (n_b > 1) tma_load_box(sb + b_box, mb, xb + 64, c * stage_k, bar);
+              if (n_b > 2) tma_load_box(sb + 2 * b_box, mb, xb + 128, c * stage_k, bar);
+              if (n_b > 3) tma_load_box(sb + 3 * b_box, mb, xb + 192, c * stage_k, bar);
+            } else {
+              tma_load_box3(sb, mb, 0, c * stage_k, 0, bar);
+            }
+          }
+          __syncwarp();
+          ++issued;
+          if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
+    if (!ok) drain_ring(sh.full, stage, phase, issued, a.n_stages);
+  } else if (warp == 1 && rank == 0) {
+    // ------------------------------------------------------------------ MMA issuer (all lanes run, one issues)
+    const bool leader = elect_one();
+    MmaCursor cur = {0, 0u};
     bool ok = true;
     int j = 0;
-    const uint32_t stages_u32 = smem_u32(stages);
-    const uint32_t dhi = desc_hi();
-    const uint32_t b_lbo = (uint32_t)stage_k * 128u;      // bytes between the 64-column chunks of B
+    const uint32_t ring = uniform(smem_u32(stages)), d0 = uniform(tmem_base);
     for (int it = it_begin; it < it_end && ok; ++it, ++j) {
       const Item& I = a.items[it];
       const int acc = j % a.n_acc;
       const uint32_t acc_phase = (uint32_t)(j / a.n_acc) & 1u;
       if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY, wlim)) break;
       tc_fence_after();
-      const uint32_t d_base = tmem_base + (uint32_t)(acc * a.acc_cols);
-      const int n_seg = I.n_seg;
+      const uint32_t d_base = d0 + (uint32_t)(acc * a.acc_cols);
+      const int n_seg = uniform(I.n_seg);
       for (int s = 0; s < n_seg && ok; ++s) {
-        const Seg& S = I.seg[s];
-        const int k = S.k, n_a = S.n_a, n_mma = S.n_mma, a_mode = S.a_mode;
-        const uint32_t idesc = make_idesc(S.n, a_mode != 0, true, false);
-        const int nst = (k + stage_k - 1) / stage_k;
-        // per K step of 16, in 16-byte units: K along x walks 32 B inside a box and 16 KB to the
-        // next box; K along y walks 16 rows of 128 B
-        const uint32_t a_lbo = a_mode ? b_lbo : 16u;
-        const uint32_t b2 = ((uint32_t)S.b2_chunk * b_lbo) >> 4;
-        uint32_t accumulate = S.first ? 0u : 1u;
-        const uint32_t d_part = (uint32_t)S.d_part, same = (uint32_t)S.same_acc;
-        uint32_t dcol[kMaxA];
+        const Seg& G = I.seg[s];
+        const int n_a = uniform((int)G.n_a), n2 = uniform((int)G.n2), a_mode = uniform((int)G.a_mode);
+        MmaSeg S;
+        S.k = uniform(G.k);
+        S.idesc = uniform(make_idesc(G.n, a_mode != 0, true, false, PAIR ? 256 : 128));
+        S.idesc2 = make_idesc(n2, a_mode != 0, true, false, PAIR ? 256 : 128);
+        S.b_lbo = (uint32_t)stage_k * 128u;               // bytes between the 64-column chunks of B
+        S.b2 = (uniform((uint32_t)G.b2_chunk) * S.b_lbo) >> 4;
+        S.accumulate = uniform((uint32_t)G.first) ? 0u : 1u;
+        S.d_part = uniform((uint32_t)G.d_part); S.same = uniform((uint32_t)G.same_acc);
 #pragma unroll
-        for (int p = 0; p < kMaxA; ++p) dcol[p] = d_base + (uint32_t)S.d_col[p];
-        int k_left = k;
-        for (int c = 0; c < nst; ++c, k_left -= stage_k) {
+        for (int p = 0; p < kMaxA; ++p) S.dcol[p] = d_base + uniform((uint32_t)G.d_col[p]);
+        ok = stage_k == 64 ? mma_segment_any<PAIR, 4>(a, sh, cur, S, n_a, n2 != 0, a_mode != 0, ring, leader)
+                           : mma_segment_any<PAIR, 8>(a, sh, cur, S, n_a, n2 != 0, a_mode != 0, ring, leader);
+      }
+      if (ok && leader) mma_commit<PAIR>(&sh.tfull[acc]);
+      __syncwarp();
+    }
+  } else if (PAIR && warp == 2 && rank == 1) {
+    // ------------------------------------------------------------------ tells rank 0 of every stage that is full here
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int it = it_begin; it < it_end && ok; ++it) {
+      const Item& I = a.items[it];
+      const int n_seg = uniform(I.n_seg);
+      for (int s = 0; s < n_seg && ok; ++s) {
+        const int nst = (uniform(I.seg[s].k) + stage_k - 1) / stage_k;
+        for (int c = 0; c < nst; ++c) {
           if (!mbar_wait_warp(&sh.full[stage], phase, abort, a.status, ST_WAIT_FULL, wlim)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = stages_u32 + (uint32_t)(stage * a.stage_bytes);
-          const uint32_t blo = desc_lo(sa + (uint32_t)a.a_bytes, b_lbo);
-          const int nk = k_left >= stage_k ? ksteps : (k_left + 15) >> 4;
-          if (leader) {
-            if (n_mma == 2) {
-              if (a_mode) {
-                if (n_a == 2) mma_stage<2, 2, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-                else mma_stage<1, 2, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              } else {
-                if (n_a == 2) mma_stage<2, 2, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-                else mma_stage<1, 2, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              }
-            } else if (a_mode) {
-              if (n_a == 2) mma_stage<2, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else if (n_a == 3) mma_stage<3, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else mma_stage<1, 1, true>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-            } else {
-              if (n_a == 2) mma_stage<2, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else if (n_a == 3) mma_stage<3, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-              else mma_stage<1, 1, false>(dcol, d_part, same, sa, a_tile, a_lbo, blo, b2, dhi, idesc, nk, accumulate);
-            }
-            mma_commit(&sh.empty[stage]);
-          }
+          if (lane == 0) mbar_arrive_at(&sh.full[stage], 0);
           __syncwarp();
-          accumulate = 1u;
           if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
         }
       }
-      if (ok && leader) mma_commit(&sh.tfull[acc]);
-      __syncwarp();
     }
   } else if (warp < 4) {
     // no work
@@ -360,7 +450,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
     // whatever order the swizzle put them in), so a warp reads four rows per access without bank conflicts; a
     // lane keeps one partial sum per row it visits, and the eight partial sums of a row are added in a fixed
     // order at the end of the item.
-    if (a.sumsq_on) {
+    if (PAIR && a.sumsq_on) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -414,7 +504,8 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           }
         }
         if (mine && ok) {
-          float* out = a.work_f32 + I.sumsq_off;
+          const int after = (int)rank * 128 * n_a0;
+          float* out = a.work_f32 + I.sumsq_off + after;
 #pragma unroll
           for (int p = 0; p < kMaxA; ++p) {
             if (p < n_a0) {
@@ -425,7 +516,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
                 s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
                 s2 += __shfl_xor_sync(0xffffffffu, s2, 4);
                 const int row = 128 * p + 4 * i + rsub;
-                if (piece == 0 && I.own0 + row < I.own_count) out[row] = s2;
+                if (piece == 0 && I.own0 + after + row < I.own_count) out[row] = s2;
               }
             }
           }
@@ -450,17 +541,21 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         I.from_iter = G.from_iter; I.to_iter = G.to_iter; I.iter_off = G.iter_off;
         I.f32_off = G.f32_off; I.own_stride = G.own_stride; I.k_stride = G.k_stride;
         I.dst_off = G.dst_off; I.dst_ld = G.dst_ld; I.coef = G.coef;
+        if (PAIR) {                                     // rank 1's panels follow on those of rank 0; some may not exist
+          I.own0 += (int)rank * 128 * I.n_pan;
+          I.n_pan = max(0, min(I.n_pan, (I.own_count - I.own0 + 127) >> 7));
+        }
       }
       const int acc = j % a.n_acc;
       const uint32_t acc_phase = (uint32_t)(j / a.n_acc) & 1u;
       const int rp = I.rp, r = I.r, half = I.half;
       const int np = rp >> 4;                             // 16-column pieces per panel
-      const int total = I.epi == EPI_FACTOR ? I.n_pan * np : 0;
+      const int total = PAIR && I.epi == EPI_FACTOR ? I.n_pan * np : 0;
       // Gradients scaled by gs (global norm clipping): the factor update is linear in g, so the Gram operands
       // are divided by gs where they are made and the whole accumulator is multiplied by it here.
-      const float coef = I.epi == EPI_FACTOR ? I.coef * gs : I.coef / gs;
-      const bool has_work = I.epi == EPI_FACTOR ? grp < total : (I.epi == EPI_GRAM && grp == 0);
-      const bool factor = I.epi == EPI_FACTOR && has_work;
+      const float coef = PAIR ? I.coef * gs : I.coef / gs;
+      const bool factor = PAIR && grp < total;
+      const bool has_work = PAIR ? factor : (I.epi == EPI_GRAM && grp == 0);
       const int qc = lane & 3;
       float* const fbase = a.f32_base + I.f32_off;
       float* const ibase = a.work_f32 + I.iter_off;
@@ -537,8 +632,8 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       // old values travel one piece ahead in two register sets that swap roles (no copies, which
       // would wait for the loads); the first set is requested before the accumulator is waited for
       float oldA[16], oldB[16];
-      if (turned) fetch_turned(grp, oldA);
-      else if (factor) fetch(grp, oldA);
+      if (PAIR && turned) fetch_turned(grp, oldA);
+      else if (PAIR && factor) fetch(grp, oldA);
       // one lane per warp polls (fewer pollers on the barrier), then the warp agrees: the
       // tensor-memory loads below need all 32 lanes
       bool got = true;
@@ -554,13 +649,17 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       const bool parked = factor && a.sum_col >= 0;
       const uint32_t ts = parked ? tmem_base + lane_addr + (uint32_t)a.sum_col : t0;
       const uint32_t ts_stride = (uint32_t)(parked ? rp : I.acc_stride);
+      // Where column p of a panel and its lo part are: the first MMA of a K step makes [hi | lo] of columns below 128, the
+      // second one (ranks above 128) the same of the others, from column 256.
+      auto hi_col = [&](int p) { return p < 128 ? p : p + 128; };
+      auto lo_col = [&](int p) { return p < 128 ? p + min(rp, 128) : p + rp; };
       if (parked) {
 #pragma unroll 1
         for (int u = grp; u < total; u += 2) {
           const int pan = u / np, p = 16 * (u - pan * np);
           float d0[16], d1[16];
-          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + p), d0);
-          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + rp + p), d1);
+          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + hi_col(p)), d0);
+          tmem_ld16(t0 + (uint32_t)(pan * I.acc_stride + lo_col(p)), d1);
           tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 16; ++e) d0[e] += d1[e];
@@ -570,10 +669,10 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       }
       // D0 + D1 of columns [p, p + 16) of this thread's row of a panel
       auto sum16 = [&](int pan, int p, float* x) {
-        tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)p, x);
+        tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)(parked ? p : hi_col(p)), x);
         if (!parked) {
           float d1[16];
-          tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)(rp + p), d1);
+          tmem_ld16(ts + (uint32_t)pan * ts_stride + (uint32_t)lo_col(p), d1);
           tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 16; ++e) x[e] += d1[e];
@@ -581,12 +680,18 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           tmem_ld_wait();
         }
       };
-      const bool early = parked || !has_work;   // (a warp without work never reads the accumulator)
-      if (early) {
+      // the accumulator goes back to the warp that issues the MMAs: one arrival per warp, at rank 0
+      auto hand_back = [&]() {
         tc_fence_before();
-        mbar_arrive(&sh.tempty[acc]);
-      }
-      if (factor) {
+        __syncwarp();
+        if (lane == 0) {
+          if (PAIR) mbar_arrive_at(&sh.tempty[acc], 0);
+          else mbar_arrive(&sh.tempty[acc]);
+        }
+      };
+      const bool early = parked || !has_work;   // (a warp without work never reads the accumulator)
+      if (early) hand_back();
+      if (PAIR && factor) {
         uint16_t* const dst = a.work_bf16 + I.dst_off;
         auto piece = [&](int u, const float* o) {
           const int pan = u / np, p = 16 * (u - pan * np);
@@ -703,7 +808,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
             }
           }
         }
-      } else if (has_work) {           // EPI_GRAM
+      } else if (!PAIR && has_work) {  // EPI_GRAM
         uint16_t* dst = a.work_bf16 + I.dst_off;
         const int row = I.own0 + q;
 #pragma unroll 1
@@ -734,18 +839,16 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           }
         }
       }
-      if (!early) {
-        tc_fence_before();
-        mbar_arrive(&sh.tempty[acc]);
-      }
+      if (!early) hand_back();
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();      // neither CTA leaves while the other may still reach into it
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 512);
+    tmem_dealloc<PAIR>(tmem_base, 512);
   }
 }
 

@@ -46,6 +46,16 @@ def test_refit_on_the_tensor_path_by_rank_and_number_of_passes(iters, rank):
              (256, 384, A.MOM_LOWRANK, max(1, rank // 8 * 8), A.V_ELEMENT, 0)], path=A.PATH_TENSOR, inner_iters=iters)
 
 
+@pytest.mark.parametrize("panels,stage_k", [(0, 0), (1, 64), (2, 128), (3, 64)])
+@pytest.mark.parametrize("rank", [5, 33, 80, 128, 144, 256])
+def test_panels_at_the_edges_of_a_pair_of_ctas(rank, panels, stage_k):
+    """A pair has up to six panels of 128 rows or columns, three for each CTA: sides where the second CTA has none, one row of
+    one, or fewer panels than the first; ranks that a CTA's half of the factor's columns fills partly, whole and with a second MMA."""
+    _follow([(n, m, A.MOM_LOWRANK, min(rank, n, m), A.V_BLOCKMEAN, 1)
+             for n, m in [(100, 264), (128, 129 * 8), (257, 384), (385, 520), (640, 776)]], path=A.PATH_TENSOR, steps=3,
+            tune_panels=panels, tune_stage_k=stage_k)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("rank", [1, 8, 9, 24, 40, 41, 81, 300])
 def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
