@@ -246,8 +246,24 @@ int launch_reduce_partial(const ReduceJob* d_tab, const int32_t* d_cta_job, int6
 int launch_reduce_final(const ReduceJob* d_tab, int64_t n_jobs, int64_t n_groups, float* state, const float* work,
                         float beta2, const int32_t* status, const float* gscale, bool chained, cudaStream_t s);
 // global gradient norm: per-chunk sums of g^2 over every block, then {s, s^2} = clip factor into gscale
-struct NormRange { int64_t off, numel, first_cta; };
+// A range of elements that the CTAs from first_cta take kNormChunk at a time.  In the norm pass, a range with group_elems > 0
+// is taken kNormUnits warp units per CTA instead, a group as `chunks` units of up to kWarpUnitMax elements, and the sum of each
+// unit is left rows_off + its number floats after the sums of the CTAs.
+struct NormRange {
+  int64_t off, numel, first_cta;
+  int64_t group_elems = 0, rows_off = 0;
+  int32_t chunks = 0, pad_ = 0;
+};
 constexpr int kNormChunk = 16384;
+constexpr int kNormUnits = 16;
+// Global clipping and the finite check read every gradient once before anything uses one.  That pass also leaves the group
+// sums of the low-rank blocks whose rows start on 16 bytes.
+inline bool norm_pass_on(const adapm_hparams& hp) {
+  return (hp.max_grad_norm > 0.f && hp.max_grad_norm <= 3.4028235e38f) || (hp.flags & ADAPM_FLAG_CHECK_FINITE);
+}
+inline bool norm_pass_sums_groups(const adapm_hparams& hp, const adapm_block& b) {
+  return norm_pass_on(hp) && b.mom_mode == ADAPM_MOM_LOWRANK && b.v_mode == ADAPM_V_BLOCKMEAN && b.cols % kChunkElems == 0;
+}
 int launch_gradnorm(const NormRange* d_tab, const int32_t* d_cta_range, int64_t n_ctas, const void* grads, int grad_dtype,
                     float* partials, float max_norm, int check_finite, float* gscale, int32_t* status, cudaStream_t s);
 int launch_gemm(const GemmProb* d_tab, int64_t n_prob, int64_t n_tiles, const Bases& b, int grad_dtype,

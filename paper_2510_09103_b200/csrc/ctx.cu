@@ -506,7 +506,7 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
   // two-stage group sums of g^2: `rjobs` run every step, `rjobs_hold` only in steps that hold L (there the
   // tensor path has no row panels to take the row sums from)
   struct ReduceSet { std::vector<ReduceJob> jobs; int64_t units = 0, groups = 0; };
-  ReduceSet rset_all, rset_hold;
+  ReduceSet rset_all, rset_hold, rset_norm;      // of every step; of steps that hold L; of sums that the norm pass leaves
   int64_t cta_cursor = 0, work_cursor = 0;
   auto add_reduce_job = [&](ReduceSet& rs, int i, int64_t group_elems, int64_t n_groups) {
     std::vector<ReduceJob>& rjobs = rs.jobs;
@@ -576,8 +576,9 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
     cta_cursor += (s.n_units + 256 / s.team - 1) / (256 / s.team);
   }
 
-  // Group sums of g^2 of the low-rank blocks come from the reduction kernels, except on the tensor path when
-  // there is a refit pass: its row panels read every row of g anyway and leave the row sums behind.
+  // Group sums of g^2 of the low-rank blocks come from the norm pass where there is one (see norm_pass_sums_groups), else on
+  // the tensor path with a refit pass from that: its row panels read every row of g anyway and leave the row sums behind.
+  // Else, and on steps that hold L, from the reduction kernels.
   const bool fold_sumsq = K_eff > 0 && !(hp->flags & ADAPM_FLAG_NO_SUMSQ_FOLD);
   const bool with_hold = hp->refresh_period > 1 && K_eff > 0;
   for (int pass = 0; pass < 2; ++pass) {
@@ -587,6 +588,7 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
       if (b.v_mode != ADAPM_V_BLOCKMEAN) continue;
       const int64_t numel = (int64_t)b.rows * b.cols;
       const int64_t group_elems = b.v_group_rows == 0 ? numel : (int64_t)b.v_group_rows * b.cols;
+      if (norm_pass_sums_groups(*hp, b)) continue;
       add_reduce_job((pass == 1 && fold_sumsq) ? rset_hold : rset_all, (int)i, group_elems, numel / group_elems);
     }
   }
@@ -594,16 +596,24 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
   auto& prog = c->program;
   // Global gradient-norm clipping (and the finite check, which rides on the same reduction) needs the norm of
   // every gradient before anything uses one: a pass of its own over g.
-  const bool clip_on = hp->max_grad_norm > 0.f && std::isfinite(hp->max_grad_norm);
-  if (clip_on || (hp->flags & ADAPM_FLAG_CHECK_FINITE)) {
+  if (norm_pass_on(*hp)) {
     std::vector<NormRange> ranges;
     std::vector<int32_t> cta_range;
     for (int i = 0; i < n; ++i) {
       const adapm_block& b = c->blocks[i];
       NormRange r{b.offset, (int64_t)b.rows * b.cols, (int64_t)cta_range.size()};
-      for (int64_t q = 0; q < (r.numel + kNormChunk - 1) / kNormChunk; ++q) cta_range.push_back((int32_t)ranges.size());
+      int64_t ctas = (r.numel + kNormChunk - 1) / kNormChunk;
+      if (norm_pass_sums_groups(*hp, b)) {
+        r.group_elems = b.v_group_rows == 0 ? r.numel : (int64_t)b.v_group_rows * b.cols;
+        add_reduce_job(rset_norm, i, r.group_elems, r.numel / r.group_elems);
+        const ReduceJob& j = rset_norm.jobs.back();
+        r.chunks = j.chunks_per_group; r.rows_off = j.part_off;          // (counted from the sums of the CTAs below)
+        ctas = (j.n_groups * r.chunks + kNormUnits - 1) / kNormUnits;
+      }
+      cta_range.insert(cta_range.end(), (size_t)ctas, (int32_t)ranges.size());
       ranges.push_back(r);
     }
+    for (NormRange& r : ranges) r.rows_off -= work_cursor;
     Launch GN{LK_GRADNORM, append_table(c->h_tables, ranges), (int64_t)ranges.size(), (int64_t)cta_range.size()};
     GN.aux0 = append_table(c->h_tables, cta_range);
     GN.aux1 = work_cursor;                                   // per-chunk sums
@@ -611,8 +621,8 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
     prog.push_back(GN);
     c->use_gscale = 1;
   }
-  for (int which = 0; which < 2; ++which) {
-    const ReduceSet& rs = which ? rset_hold : rset_all;
+  for (int which = 0; which < 3; ++which) {
+    const ReduceSet& rs = which == 0 ? rset_all : which == 1 ? rset_hold : rset_norm;
     const std::vector<ReduceJob>& rjobs = rs.jobs;
     if (rjobs.empty()) continue;
     const int64_t off = append_table(c->h_tables, rjobs);
@@ -625,8 +635,8 @@ static int create_context(adapm_ctx* c, const adapm_block* blocks, int64_t n_blo
     }
     Launch RP{LK_REDUCE_PARTIAL, off, (int64_t)rjobs.size(), (rs.units + 7) / 8, rs.units};
     RP.aux1 = append_table(c->h_tables, cta_job);
-    RP.phase = which ? 2 : 0;
-    prog.push_back(RP);
+    RP.phase = which == 1 ? 2 : 0;
+    if (which < 2) prog.push_back(RP);
     Launch RF{LK_REDUCE_FINAL, off, (int64_t)rjobs.size(), (rs.groups + 7) / 8, rs.groups};
     RF.phase = RP.phase;
     prog.push_back(RF);

@@ -490,7 +490,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   // reduction whose "partial sums" are the rows of a group
   for (TcBlock& t : P->blk) {
     const adapm_block& b = c->blocks[t.id];
-    if (!fold_sumsq || b.v_mode != ADAPM_V_BLOCKMEAN) continue;
+    if (!fold_sumsq || b.v_mode != ADAPM_V_BLOCKMEAN || norm_pass_sums_groups(hp, b)) continue;
     t.rowsum = work_cursor;
     work_cursor += round_up(b.rows, kStateAlign);
     const int group_rows = b.v_group_rows == 0 ? b.rows : b.v_group_rows;
@@ -729,8 +729,11 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
           gram(mb + MAP_RTCT + src, nR, n, 0, -1.f / a1);  // Bop1[j][k] = -(R R^T)[j][k] / (1-b1), stored as [k][j]
           gram(mb + MAP_RTCT + prev, nR, n, 1, b1 / a1);   // Bop2[j][k] = b1 (R R0^T)[j][k] / (1-b1)
         }
-        gram(mb + MAP_LCT + srcL, nL, m, 2, -1.f / a1);    // Bop3[j][k] = -(L^T L)[j][k] / (1-b1)
-        gram(mb + MAP_LCT + prev, nL, m, 3, b1 / a1);      // Bop4[j][k] = b1 (L^T L0)[j][k] / (1-b1)
+        // (with L held the first pass's serve them all: L^T L0 and L^T L do not change, nor does the scale of the gradient)
+        if (!hold || precond || pass == 0) {
+          gram(mb + MAP_LCT + srcL, nL, m, 2, -1.f / a1);    // Bop3[j][k] = -(L^T L)[j][k] / (1-b1)
+          gram(mb + MAP_LCT + prev, nL, m, 3, b1 / a1);      // Bop4[j][k] = b1 (L^T L0)[j][k] / (1-b1)
+        }
 
         // one item = adjacent panels of 128 owners, np for each CTA of a pair, that share B
         auto panel = [&](bool is_L, int p0, int np) {
@@ -780,7 +783,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
       G.aux3 = append_items(c->h_tables, begin_g);
       G.aux4 = -1; G.aux5 = 0;
       G.when = when; G.phase = phase;
-      prog.push_back(G);
+      if (!grams.empty()) prog.push_back(G);
       Launch Q{LK_TC_PANEL, append_items(c->h_tables, panels), (int64_t)panels.size(), grid_p};
       Q.aux0 = n_pan * 2 * rp_max; Q.aux1 = 2 * Q.aux0 <= 512 ? 2 : 1;
       Q.aux2 = n_pan;

@@ -403,22 +403,38 @@ __global__ void __launch_bounds__(256) gradnorm_partial_kernel(const NormRange* 
   __shared__ float warp_sums[8];
   if (*status != 0) return;
   const NormRange R = tab[cta_range[blockIdx.x]];
-  const int64_t start = ((int64_t)blockIdx.x - R.first_cta) * kNormChunk;
-  const int64_t rem = R.numel - start;
-  const int len = rem < kNormChunk ? (int)rem : kNormChunk;
-  const typename GT::elem* g = grads + R.off + start;
-  const int nchunks = (len + kChunkElems - 1) / kChunkElems;
   float ss = 0.f;
-  for (int idx = threadIdx.x; idx < nchunks; idx += 256) {
-    const int e0 = idx * kChunkElems;
-    typename GT::raw8 r = (e0 + kChunkElems <= len) ? GT::load8(g + e0) : GT::load8_guarded(g + e0, len - e0);
-    float f[8];
-    GT::unpack(r, f);
+  if (R.group_elems > 0) {
+    const int64_t u0 = ((int64_t)blockIdx.x - R.first_cta) * kNormUnits, n_units = R.numel / R.group_elems * R.chunks;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) ss = fmaf(f[i], f[i], ss);
+    for (int q = 0; q < kNormUnits / 8; ++q) {
+      const int64_t u = u0 + 8 * q + (threadIdx.x >> 5);
+      if (u < n_units) {
+        const int64_t group = u / R.chunks, in_group = (u - group * R.chunks) * kWarpUnitMax;
+        const int64_t rem = R.group_elems - in_group;
+        const float t = warp_chunk_sumsq<GT>(grads + R.off + group * R.group_elems + in_group,
+                                             rem < kWarpUnitMax ? (int)rem : kWarpUnitMax, true);
+        if ((threadIdx.x & 31) == 0) partials[R.rows_off + u] = t;
+        ss += t;
+      }
+    }
+  } else {
+    const int64_t start = ((int64_t)blockIdx.x - R.first_cta) * kNormChunk;
+    const int64_t rem = R.numel - start;
+    const int len = rem < kNormChunk ? (int)rem : kNormChunk;
+    const typename GT::elem* g = grads + R.off + start;
+    const int nchunks = (len + kChunkElems - 1) / kChunkElems;
+    for (int idx = threadIdx.x; idx < nchunks; idx += 256) {
+      const int e0 = idx * kChunkElems;
+      typename GT::raw8 r = (e0 + kChunkElems <= len) ? GT::load8(g + e0) : GT::load8_guarded(g + e0, len - e0);
+      float f[8];
+      GT::unpack(r, f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) ss = fmaf(f[i], f[i], ss);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = ss;
   __syncthreads();
   if (threadIdx.x == 0) {

@@ -96,6 +96,16 @@ def test_bf16_gradients_whose_rows_do_not_start_on_16_bytes(cols, rank, vmode):
         run.close()
 
 
+@pytest.mark.parametrize("dtype,period", [("bf16", 0), ("bf16", 3), ("f32", 0)])
+def test_group_sums_left_by_the_norm_pass(dtype, period):
+    """Clipped steps: rows of less than a warp unit of 2048, of exactly one, of one and a piece, groups of several rows, the
+    whole block as one group, more and fewer units than a CTA takes, and a row length that the pass leaves to others."""
+    _follow([(33, 2040, A.MOM_LOWRANK, 5, A.V_BLOCKMEAN, 1), (16, 2048, A.MOM_LOWRANK, 6, A.V_BLOCKMEAN, 1),
+             (18, 2056, A.MOM_LOWRANK, 7, A.V_BLOCKMEAN, 3), (200, 136, A.MOM_LOWRANK, 8, A.V_BLOCKMEAN, 0),
+             (30, 77, A.MOM_LOWRANK, 4, A.V_BLOCKMEAN, 1), (64, 80, A.MOM_LOWRANK, 4, A.V_ELEMENT, 0),
+             (5, 264, A.MOM_FULL, 0, A.V_BLOCKMEAN, 1)], dtype=dtype, steps=5, max_grad_norm=0.2, refresh_period=period)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_streaming_update_at_the_edges_of_its_teams(dtype):
     """Groups that one, two, four and eight warps hold, and one element more and less."""
