@@ -514,14 +514,14 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   // better than two of K = 128 (rank 8 801 | 669, rank 80 5480 | 5164).
   // Sets with few items per pair take one panel and K = 128: the last round of items is shorter, and of the short K loops
   // every stage costs a trip through the barriers.  us per step, two panels and K = 64 | one and K = 128, by items (of two
-  // panels) per pair: 0.4 (tiny set) 113 | 106, 2.2 (60M) 375 | 371, 4.3 (1024 x 2730) 1190 | 1164, 5.2 (124M) 796 | 821,
-  // 13 (350M rank 8) 1645 | 1733.
+  // panels) per pair: 0.3 (tiny set) 113 | 106, 1.7 (60M) 375 | 371, 3.5 (1024 x 2730) 1190 | 1164, 3.9 (124M) 796 | 821,
+  // 10 (350M rank 8) 1645 | 1733.
   auto stages_with = [&](int stage_k, int n_a, bool pair) {
     return (224 * 1024) / (n_a * 256 * stage_k + stage_k * 128 * (pair ? (rp_max + 63) / 64 : nb_max));
   };
   int64_t panel_items = 0;                       // with two panels per CTA
   for (const TcBlock& t : P->blk) panel_items += (c->blocks[t.id].rows + 511) / 512 + (c->blocks[t.id].cols + 511) / 512;
-  const bool few_items = panel_items < (int64_t)P->n_sms * 9 / 4;      // 4.5 per pair
+  const bool few_items = 4 * panel_items < (int64_t)15 * (P->n_sms / 2);      // 3.75 per pair
   int n_pan = hp.tune_panels > 0 ? hp.tune_panels : (few_items || 6 * rp_max > 512 ? 1 : 2);
   n_pan = std::max(1, std::min({n_pan, tc::kMaxA, 512 / (2 * rp_max)}));
   int stage_k = hp.tune_stage_k == 64 || hp.tune_stage_k == 128 ? hp.tune_stage_k : (few_items ? 128 : 64);
