@@ -94,6 +94,15 @@ __device__ __forceinline__ float clamp_keep_nan(float x, float c) {
   return y;
 }
 
+// The same with the values it needs by themselves, for the rare elements of the function below (out of line: its root and
+// quotient would be unrolled with that one's loops, and a loop of its own would keep the values in local memory).
+static __device__ __noinline__ float adapm_param_update_rare(float w, float mc, float v, float inv_bc1, float inv_bc2, float eps,
+                                                             float clip, float lr_s, float wd) {
+  float ratio = (mc * inv_bc1) / (sqrtf(v * inv_bc2) + eps);
+  ratio = ratio > clip ? clip : (ratio < -clip ? -clip : ratio);
+  return w - lr_s * (ratio + wd * w);
+}
+
 // The update of N elements with a second moment of their own.  The root and the quotient start from the hardware's
 // approximations (an ulp or two off) and take one step of Newton's iteration each, with the residual in a fused
 // multiply-add (Markstein, IBM J. Res. Dev. 34, 1990): s += (v - s^2) y / 2 with y ~ 1/sqrt(v), q += (m - q d) r with
@@ -129,8 +138,9 @@ __device__ __forceinline__ void adapm_param_update_n(float* w, const float* mc, 
       w[e] = w[e] - lr_s * (clamp_keep_nan(q, sc.clip) + wd * w[e]);
     }
   } else {
-#pragma unroll 1
-    for (int e = 0; e < N; ++e) w[e] = adapm_param_update(w[e], mc[e], v[e], sc, lr_s, wd);
+#pragma unroll
+    for (int e = 0; e < N; ++e)
+      w[e] = adapm_param_update_rare(w[e], mc[e], v[e], sc.inv_bc1, sc.inv_bc2, sc.eps, sc.clip, lr_s, wd);
   }
 }
 

@@ -418,33 +418,49 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
               }
               tmem_ld_wait();
               uint32_t shw[8];
+              if (grouped) {
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float4* wp = reinterpret_cast<float4*>(buf + w_at(4 * half + i));
-                const float4 wo = *wp;
-                float w[4] = {wo.x, wo.y, wo.z, wo.w};
-                if (grouped) {
+                for (int i = 0; i < 4; ++i) {
+                  float4* wp = reinterpret_cast<float4*>(buf + w_at(4 * half + i));
+                  const float4 wo = *wp;
+                  float w[4] = {wo.x, wo.y, wo.z, wo.w};
 #pragma unroll
                   for (int x = 0; x < 4; ++x) {
                     const float ratio = clamp_keep_nan((sc.cg * gf[4 * i + x] + sc.c0 * d[4 * i + x]) * kr, sc.clip);
                     w[x] = w[x] - lr_s * (ratio + I.wd * w[x]);
                   }
-                } else {
-                  float4* vp = reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at(4 * half + i));   // v lies like W
-                  const float4 vo = *vp;
-                  float vv[4] = {vo.x, vo.y, vo.z, vo.w}, mc[4];
-#pragma unroll
-                  for (int x = 0; x < 4; ++x) {
-                    const float g1 = gf[4 * i + x];
-                    vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
-                    mc[x] = sc.cg * g1 + sc.c0 * d[4 * i + x];
-                  }
-                  *vp = make_float4(vv[0], vv[1], vv[2], vv[3]);
-                  adapm_param_update_n<4>(w, mc, vv, sc, lr_s, I.wd);
+                  *wp = make_float4(w[0], w[1], w[2], w[3]);
+                  shw[2 * i] = pack_bf16x2(w[0], w[1]);
+                  shw[2 * i + 1] = pack_bf16x2(w[2], w[3]);
                 }
-                *wp = make_float4(w[0], w[1], w[2], w[3]);
-                shw[2 * i] = pack_bf16x2(w[0], w[1]);
-                shw[2 * i + 1] = pack_bf16x2(w[2], w[3]);
+              } else {
+                // Sixteen elements at a time: their chains of a root and a quotient each run side by side.  Four at a time, with
+                // the rare elements in a loop that kept them in local memory, a quarter took 8.1 thousand cycles of its group:
+                // 7.5 -> 5.7 ms on the 1.5B shapes, 1.65 -> 1.25 on the 350M set at rank 128; group scalars 3.0 -> 2.5 ms.
+                float w[16], vv[16];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const float4 wo = *reinterpret_cast<const float4*>(buf + w_at(4 * half + i));
+                  const float4 vo = *reinterpret_cast<const float4*>(buf + kApplyBufBytes + w_at(4 * half + i));   // v lies like W
+                  w[4 * i] = wo.x; w[4 * i + 1] = wo.y; w[4 * i + 2] = wo.z; w[4 * i + 3] = wo.w;
+                  vv[4 * i] = vo.x; vv[4 * i + 1] = vo.y; vv[4 * i + 2] = vo.z; vv[4 * i + 3] = vo.w;
+                }
+#pragma unroll
+                for (int x = 0; x < 16; ++x) {
+                  const float g1 = gf[x];
+                  vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
+                  d[x] = sc.cg * g1 + sc.c0 * d[x];                          // m^c
+                }
+                adapm_param_update_n<16>(w, d, vv, sc, lr_s, I.wd);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  *reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at(4 * half + i)) =
+                      make_float4(vv[4 * i], vv[4 * i + 1], vv[4 * i + 2], vv[4 * i + 3]);
+                  *reinterpret_cast<float4*>(buf + w_at(4 * half + i)) =
+                      make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                  shw[2 * i] = pack_bf16x2(w[4 * i], w[4 * i + 1]);
+                  shw[2 * i + 1] = pack_bf16x2(w[4 * i + 2], w[4 * i + 3]);
+                }
               }
               if (a.shadow) {
                 // The bf16 copy of the new W takes the place of the gradient in the buffer (this thread's two 16-byte
