@@ -193,15 +193,17 @@ struct TcProgram {
     return e;
   }
   int apply_buf_bytes = 0;
+  bool any_element_v = false;
   // shared-memory plan of an apply launch
-  struct ApplyConfig { int n_rstages, w_region, n_bufs, smem; };
+  struct ApplyConfig { int groups, n_rstages, w_region, n_bufs, smem; };
   ApplyConfig apply_config(bool stream, bool tma) const {
     ApplyConfig e;
+    e.groups = !tma || (any_element_v && !stream) ? 4 : 2;
     e.n_rstages = stream ? 2 : 4;
     e.w_region = e.n_rstages * (stream ? 4 : 1) * tc::kBoxBytes;
-    // (an even number: see the kernel's epilogue)
-    e.n_bufs = tma ? std::min(tc::kApplyMaxBufs, (226 * 1024 - e.w_region) / apply_buf_bytes) & ~1 : 0;
-    e.smem = e.w_region + (tma ? e.n_bufs * apply_buf_bytes : tc::kPatchesBytes) + 1024;
+    // (a multiple of the groups: see the kernel's epilogue)
+    e.n_bufs = tma ? std::min(tc::kApplyMaxBufs, (226 * 1024 - e.w_region) / apply_buf_bytes) / e.groups * e.groups : 0;
+    e.smem = e.w_region + (tma ? e.n_bufs * apply_buf_bytes : 4 * e.groups * tc::kPatchBytes) + 1024;
     return e;
   }
   int n_sms = 148;
@@ -252,9 +254,10 @@ void tensor_state_changed(adapm_ctx* c) {
 namespace {
 
 using ApplyKernel = void (*)(tc::ApplyArgs);
-ApplyKernel apply_kernel(bool stream, bool tma) {
-  if (stream) return tma ? tc::tc_apply_kernel<true, true> : tc::tc_apply_kernel<true, false>;
-  return tma ? tc::tc_apply_kernel<false, true> : tc::tc_apply_kernel<false, false>;
+ApplyKernel apply_kernel(bool stream, bool tma, int groups) {
+  if (!tma) return stream ? tc::tc_apply_kernel<true, false, 4> : tc::tc_apply_kernel<false, false, 4>;
+  if (stream) return tc::tc_apply_kernel<true, true, 2>;
+  return groups == 4 ? tc::tc_apply_kernel<false, true, 4> : tc::tc_apply_kernel<false, true, 2>;
 }
 
 // Lets a kernel be launched with `need` bytes of dynamic shared memory.  The limit belongs to the kernel, not to the context
@@ -807,20 +810,22 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   {
     std::vector<tc::ApplyItem> lists[2][2];      // [L streamed][rows of the parameters start on 16 bytes]
     bool any_element_v = false;
-    int64_t all_tiles = 0;
+    int64_t form_tiles[2][2] = {};
     for (const TcBlock& t : P->blk) {
       const adapm_block& b = c->blocks[t.id];
-      all_tiles += (int64_t)((b.rows + 127) / 128) * ((b.cols + tc::kApplyNT - 1) / tc::kApplyNT);
+      form_tiles[2 * t.rp > 256 ? 1 : 0][b.cols % 8 == 0 ? 1 : 0] += (int64_t)((b.rows + 127) / 128) * ((b.cols + tc::kApplyNT - 1) / tc::kApplyNT);
     }
-    // Column tiles per item: 16 where the set is large (the L panel is loaded once per item), fewer where that would
-    // leave CTAs without work.
-    const int run_len = (int)std::min<int64_t>(16, std::max<int64_t>(1, all_tiles / (4 * P->n_sms)));
     for (size_t bi = 0; bi < P->blk.size(); ++bi) {
       const TcBlock& t = P->blk[bi];
       const adapm_block& b = c->blocks[t.id];
       const int mb = (int)bi * kMapsPerBlock;
       if (b.v_mode == ADAPM_V_ELEMENT) any_element_v = true;
       const int tiles = (b.cols + tc::kApplyNT - 1) / tc::kApplyNT;
+      // Column tiles per item: 16 where the launch is large (the L panel is loaded once per item), fewer where that would
+      // leave CTAs without work.  By the launch's own tiles: by those of all forms 8 blocks of 1024 x 2730 beside aligned ones
+      // made 192 items for 148 CTAs, 253 -> 186 us.
+      const int64_t of_launch = form_tiles[2 * t.rp > 256 ? 1 : 0][b.cols % 8 == 0 ? 1 : 0];
+      const int run_len = (int)std::min<int64_t>(16, std::max<int64_t>(1, of_launch / (4 * P->n_sms)));
       const int runs = (tiles + run_len - 1) / run_len;
       for (int p0 = 0; p0 < b.rows; p0 += 128) {
         for (int q = 0; q < runs; ++q) {
@@ -840,6 +845,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
         }
       }
     }
+    P->any_element_v = any_element_v;
     P->apply_buf_bytes = tc::kApplyBufBytes + (any_element_v ? tc::kWBoxBytes : 0);
     for (int form = 0; form < 4; ++form) {
       std::vector<tc::ApplyItem>& items = lists[form >> 1][form & 1];
@@ -866,7 +872,8 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   if (e == cudaSuccess) e = allow_dynamic_smem(tc::tc_items_kernel<false>, P->engine_config(false, gram_na).smem);
   for (int form = 0; form < 4; ++form)
     if (e == cudaSuccess)
-      e = allow_dynamic_smem(apply_kernel(form >> 1, form & 1), P->apply_config(form >> 1, form & 1).smem);
+      e = allow_dynamic_smem(apply_kernel(form >> 1, form & 1, P->apply_config(form >> 1, form & 1).groups),
+                             P->apply_config(form >> 1, form & 1).smem);
   if (e != cudaSuccess) {
     set_cuda_error(e, "build_tensor_program");
     return ADAPM_ECUDA;
@@ -1033,7 +1040,8 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       a.buf_bytes = P->apply_buf_bytes;
       a.gscale = b.gscale;
       a.shadow = b.shadow != nullptr;
-      launch_chained(c->step_bytes < kChainedBytes, apply_kernel(L.aux0 != 0, L.aux1 != 0), (unsigned)L.grid, tc::kApplyThreads, e.smem, s, a);
+      launch_chained(c->step_bytes < kChainedBytes, apply_kernel(L.aux0 != 0, L.aux1 != 0, e.groups), (unsigned)L.grid,
+                     tc::apply_threads(e.groups), e.smem, s, a);
       break;
     }
     default:

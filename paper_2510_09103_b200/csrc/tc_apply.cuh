@@ -25,13 +25,16 @@
 // kTma (parameter rows start on 16 bytes: cols a multiple of 8): g and W never pass through registers on
 // their way in or out.  A mover thread brings them in quarters (128 rows x 32 columns: 16 KB of W, 8 KB of
 // g) by TMA into a ring of shared-memory buffers, several quarters ahead of their use, and writes the
-// updated W back from the same buffer by TMA.  The two groups of 128 epilogue threads take the quarters in
+// updated W back from the same buffer by TMA.  The groups of 128 epilogue threads take the quarters in
 // turn; a thread owns one row of the panel: it reads its accumulator row from tensor memory, its columns of g
 // and W from the (swizzled) buffer, and puts the new W back in place.  A per-element v, where a block has
 // one, travels like W.
 // (Quarters of 32 rows x 128 columns take four times as many boxes: 4.4 ms instead of 3.0 on the 1.5B shapes.)
 // Otherwise an epilogue warp turns a 32 x 32 chunk of the accumulator through a patch of shared memory and
 // works along the rows of the parameters, one column per lane, whatever the alignment of the rows.
+// Four groups where the arithmetic or the latency of that form sets the pace, two where the ring of buffers does (with four it
+// has to be four deep instead of six, or the ring of R half as deep): per-element v 5.30 -> 4.90 ms on the 1.5B shapes and 1.18
+// -> 1.05 on the 350M set at rank 128, rows of 2730 184 -> 140 us; group scalars 2.50 -> 2.71 or 3.15 ms, kept at two.
 // The m x n matrices m_t, r_t and m^c are never stored.
 #pragma once
 
@@ -44,7 +47,8 @@
 namespace adapm {
 namespace tc {
 
-constexpr int kApplyThreads = 480;         // producer, MMA, eight epilogue warps, mover, four warps that load L
+// producer, MMA, epilogue warps in groups of four, mover, four warps that load L
+constexpr int apply_threads(int groups) { return 32 * (2 + 4 * groups + 1 + 4); }
 constexpr int kApplyNT = 128;              // columns per tile
 constexpr int kApplyQC = 32;               // columns per quarter tile
 constexpr int kApplyMaxStages = 8;         // R ring depth limit
@@ -53,7 +57,7 @@ constexpr int kWBoxBytes = 128 * kApplyQC * 4;   // a quarter tile of W: 128 row
 constexpr int kGBoxBytes = 128 * kApplyQC * 2;   // and of g: 128 rows of 64 bytes
 constexpr int kApplyBufBytes = kWBoxBytes + kGBoxBytes;    // + kWBoxBytes where a block has a per-element v
 constexpr int kPatchPitch = 33;            // floats per row of an epilogue warp's patch
-constexpr int kPatchesBytes = 8 * 32 * kPatchPitch * 4;
+constexpr int kPatchBytes = 32 * kPatchPitch * 4;
 
 struct ApplyItem {
   int64_t off;               // element offset of the block in params / grads
@@ -89,7 +93,7 @@ struct ApplyArgs {
   int32_t shadow;            // 1: the bf16 copy of the parameters is written with W
   int32_t n_rstages;         // R ring depth (1..kApplyMaxStages); a stage is one 64 x 128 box of R^T (kStream: four boxes)
   int32_t w_region_off;      // byte offset of the g / W ring (kTma) or of the patches inside the dynamic shared memory
-  int32_t n_bufs;            // g / W ring depth (2..kApplyMaxBufs, even: see the epilogue)
+  int32_t n_bufs;            // g / W ring depth (up to kApplyMaxBufs, a multiple of the groups: see the epilogue)
   int32_t buf_bytes;         // one buffer: W, g and, if any block of the launch has a per-element v, v
 };
 
@@ -102,10 +106,11 @@ struct __align__(8) ApplyShared {
 };
 
 // The epilogue of one warp without TMA: 32 x 32 chunks of the accumulator, one column per lane.
+template <int kGroups>
 __device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplyShared& sh, float* patch, uint32_t tmem_acc) {
-  constexpr int kChunks = kApplyNT / 32, kBatch = 16;
+  constexpr int kChunks = kApplyNT / 32, kBatch = kGroups == 4 ? 8 : 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = warp & 3, grp = (warp - 2) >> 2;           // which 32 accumulator rows; chunks grp, grp + 2, ...
+  const int sub = warp & 3, grp = (warp - 2) >> 2;           // which 32 accumulator rows; chunks grp, grp + kGroups, ...
   const uint32_t lane_addr = (uint32_t)(32 * sub) << 16;
   const StepScalars& sc = a.sc;
   const float gs = a.gscale ? *a.gscale : 1.f;
@@ -123,7 +128,7 @@ __device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplySha
     }
     for (int t = 0; t < I.n_tiles; ++t, ++j) {
       const int acc = j & 1;
-      for (int c = grp; c < kChunks; c += 2) {
+      for (int c = grp; c < kChunks; c += kGroups) {
         const int col = (I.tile0 + t) * kApplyNT + 32 * c + lane;
         const bool cok = col < I.cols;
         const int64_t o = (int64_t)row0 * I.cols + col;
@@ -151,12 +156,14 @@ __device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplySha
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) return;
             tc_fence_after();
-            float d[32];
-            tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + 32 * c), d);
-            tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + 32 * c + 16), d + 16);
-            tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) patch[lane * kPatchPitch + e] = d[e];
+            for (int x = 0; x < 32; x += 16) {
+              float d[16];
+              tmem_ld16(tmem_acc + lane_addr + (uint32_t)(acc * kApplyNT + 32 * c + x), d);
+              tmem_ld_wait();
+#pragma unroll
+              for (int e = 0; e < 16; ++e) patch[lane * kPatchPitch + x + e] = d[e];
+            }
             __syncwarp();
           }
 #pragma unroll
@@ -187,8 +194,8 @@ __device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplySha
   }
 }
 
-template <bool kStream, bool kTma>
-__global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a) {
+template <bool kStream, bool kTma, int kGroups>
+__global__ void __launch_bounds__(apply_threads(kGroups), 1) tc_apply_kernel(ApplyArgs a) {
   constexpr int kStageBytes = kStream ? 4 * kBoxBytes : kBoxBytes;
   constexpr int kQ = kApplyNT / kApplyQC;                    // quarters per tile
   extern __shared__ uint8_t dyn_smem[];
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
   if (threadIdx.x == 0) {
     mbar_init(&sh.lfull, 4); mbar_init(&sh.lempty, 1);
     for (int i = 0; i < kApplyMaxStages; ++i) { mbar_init(&sh.rfull[i], 1); mbar_init(&sh.rempty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 8); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], 4 * kGroups); }
     for (int i = 0; i < kApplyMaxBufs; ++i) { mbar_init(&sh.wfull[i], 1); mbar_init(&sh.wdone[i], 4); }
     sh.abort = 0;
     mbar_fence_init();
@@ -355,13 +362,13 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
       __syncwarp();
       item_phase ^= 1u;
     }
-  } else if (warp < 10) {
+  } else if (warp < 2 + 4 * kGroups) {
     // ------------------------------------------------------------------ epilogue
     if constexpr (!kTma) {
-      apply_rows_epilogue(a, sh, reinterpret_cast<float*>(smem_w) + (warp - 2) * 32 * kPatchPitch, tmem_acc);
+      apply_rows_epilogue<kGroups>(a, sh, reinterpret_cast<float*>(smem_w) + (warp - 2) * 32 * kPatchPitch, tmem_acc);
     } else {
       const int wq4 = warp & 3;                             // which 32 accumulator rows this warp may read
-      // The two groups of four warps take the quarters in turn.  With an even number of buffers a buffer belongs to one
+      // The groups of four warps take the quarters in turn.  With a multiple of kGroups of buffers a buffer belongs to one
       // group: a group that waited on the other's buffers could be a whole phase ahead of a barrier, whose parity then
       // reads as complete.
       const int grp = (warp - 2) >> 2;
@@ -396,11 +403,12 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
           if (!got) { ok = false; break; }
           tc_fence_after();
 #pragma unroll 1
-          for (int q = grp; q < kQ; q += 2) {
+          for (int q = grp; q < kQ; q += kGroups) {
             if (!mbar_wait(&sh.wfull[b], wphase, abort, a.status, ST_WAIT_FULL)) ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             uint8_t* buf = smem_w + (size_t)b * a.buf_bytes;
+            const int col = (I.tile0 + t) * kApplyNT + q * kApplyQC;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
               float d[16];
@@ -434,32 +442,38 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
                   shw[2 * i + 1] = pack_bf16x2(w[2], w[3]);
                 }
               } else {
-                // Sixteen elements at a time: their chains of a root and a quotient each run side by side.  Four at a time, with
+                // kBatch elements at a time: their chains of a root and a quotient each run side by side.  Four at a time, with
                 // the rare elements in a loop that kept them in local memory, a quarter took 8.1 thousand cycles of its group:
                 // 7.5 -> 5.7 ms on the 1.5B shapes, 1.65 -> 1.25 on the 350M set at rank 128; group scalars 3.0 -> 2.5 ms.
-                float w[16], vv[16];
+                constexpr int kBatch = kGroups == 4 ? 8 : 16;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const float4 wo = *reinterpret_cast<const float4*>(buf + w_at(4 * half + i));
-                  const float4 vo = *reinterpret_cast<const float4*>(buf + kApplyBufBytes + w_at(4 * half + i));   // v lies like W
-                  w[4 * i] = wo.x; w[4 * i + 1] = wo.y; w[4 * i + 2] = wo.z; w[4 * i + 3] = wo.w;
-                  vv[4 * i] = vo.x; vv[4 * i + 1] = vo.y; vv[4 * i + 2] = vo.z; vv[4 * i + 3] = vo.w;
-                }
+                for (int i0 = 0; i0 < 4; i0 += kBatch / 4) {
+                  float w[kBatch], vv[kBatch], mc[kBatch];
 #pragma unroll
-                for (int x = 0; x < 16; ++x) {
-                  const float g1 = gf[x];
-                  vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
-                  d[x] = sc.cg * g1 + sc.c0 * d[x];                          // m^c
-                }
-                adapm_param_update_n<16>(w, d, vv, sc, lr_s, I.wd);
+                  for (int i = 0; i < kBatch / 4; ++i) {
+                    const float4 wo = *reinterpret_cast<const float4*>(buf + w_at(4 * half + i0 + i));
+                    const float4 vo = *reinterpret_cast<const float4*>(buf + kApplyBufBytes + w_at(4 * half + i0 + i));   // v lies like W
+                    w[4 * i] = wo.x; w[4 * i + 1] = wo.y; w[4 * i + 2] = wo.z; w[4 * i + 3] = wo.w;
+                    vv[4 * i] = vo.x; vv[4 * i + 1] = vo.y; vv[4 * i + 2] = vo.z; vv[4 * i + 3] = vo.w;
+                  }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  *reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at(4 * half + i)) =
-                      make_float4(vv[4 * i], vv[4 * i + 1], vv[4 * i + 2], vv[4 * i + 3]);
-                  *reinterpret_cast<float4*>(buf + w_at(4 * half + i)) =
-                      make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-                  shw[2 * i] = pack_bf16x2(w[4 * i], w[4 * i + 1]);
-                  shw[2 * i + 1] = pack_bf16x2(w[4 * i + 2], w[4 * i + 3]);
+                  for (int x = 0; x < kBatch; ++x) {
+                    const float g1 = gf[4 * i0 + x];
+                    vv[x] = sc.beta2 * vv[x] + (1.f - sc.beta2) * ((gs * g1) * (gs * g1));
+                    mc[x] = sc.cg * g1 + sc.c0 * d[4 * i0 + x];
+                    // (rows and columns out of range hold zeros, are not stored, and would all take the rare path)
+                    if (!rok || col + 16 * half + 4 * i0 + (x & 8) >= I.cols) vv[x] = 1.f;
+                  }
+                  adapm_param_update_n<kBatch>(w, mc, vv, sc, lr_s, I.wd);
+#pragma unroll
+                  for (int i = 0; i < kBatch / 4; ++i) {
+                    *reinterpret_cast<float4*>(buf + kApplyBufBytes + w_at(4 * half + i0 + i)) =
+                        make_float4(vv[4 * i], vv[4 * i + 1], vv[4 * i + 2], vv[4 * i + 3]);
+                    *reinterpret_cast<float4*>(buf + w_at(4 * half + i0 + i)) =
+                        make_float4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                    shw[2 * (i0 + i)] = pack_bf16x2(w[4 * i], w[4 * i + 1]);
+                    shw[2 * (i0 + i) + 1] = pack_bf16x2(w[4 * i + 2], w[4 * i + 3]);
+                  }
                 }
               }
               if (a.shadow) {
@@ -471,19 +485,19 @@ __global__ void __launch_bounds__(kApplyThreads, 1) tc_apply_kernel(ApplyArgs a)
               }
             }
             fence_async_smem();   // every lane orders its own writes, the warp meets, one arrival per warp
-            if (q + 2 >= kQ) tc_fence_before();
+            if (q + kGroups >= kQ) tc_fence_before();
             __syncwarp();
             if (lane == 0) {
               mbar_arrive(&sh.wdone[b]);
-              if (q + 2 >= kQ) mbar_arrive(&sh.tempty[acc]);
+              if (q + kGroups >= kQ) mbar_arrive(&sh.tempty[acc]);
             }
-            b += 2;
+            b += kGroups;
             if (b >= a.n_bufs) { b = grp; wphase ^= 1u; }
           }
         }
       }
     }
-  } else if (warp == 10) {
+  } else if (warp == 2 + 4 * kGroups) {
     // ------------------------------------------------------------------ g / W mover
     if (kTma && lane == 0) {
       // load cursor: runs n_bufs quarters ahead of the quarter being stored
