@@ -49,6 +49,7 @@ __device__ __forceinline__ float load1(const float* p) { return *p; }
 __device__ __forceinline__ float load1(const uint16_t* p) { return bf16_bits_to_float(*p); }
 
 constexpr int kThreads = 128;            // 2 x 2 warps
+constexpr int kAsyncStages = 3;          // of the loops that copy straight into shared memory
 template <int RI_, int TN_, int BK_>
 struct Tile {
   static constexpr int RI = RI_, TN = TN_, BK = BK_;
@@ -56,6 +57,7 @@ struct Tile {
   // Row pitch in shared memory: BK + 4 makes the eight rows a warp reads at once start 4 banks apart, all different.
   static constexpr int P = BK + 4;
   static constexpr int kFloats = 2 * (kRows + kCols) * P;     // two stages, so that a stage costs one barrier
+  static constexpr int kAsyncFloats = kAsyncStages * (kRows + kCols) * P;
 };
 
 // An operand: `n` rows (owners or columns of the tile, from i0) of K elements.  along_k: stored [n, K] with K
@@ -129,6 +131,62 @@ struct Operand {
   }
 };
 
+// 4 or 16 bytes from global into shared memory without a register in between; zeros if not `ok`.
+__device__ __forceinline__ void copy4_async(float* dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copy16_async(float* dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
+}
+
+// The same operand, fp32 and unscaled, copied into the stages without registers in between.  A thread's elements of a stage
+// are a fixed step apart, so that a stage costs it one address and one comparison each.
+template <int ROWS, int BK>
+struct AsyncOperand {
+  static_assert(BK == 16 && kThreads == 128 && ROWS % 8 == 0, "places below");
+  static constexpr int P = BK + 4;
+  const float* p;             // of this thread's first element of the operand
+  int64_t ld;
+  int rows, k, dst;           // rows left from its first one, its first k of a stage, its place in a stage
+  bool along_k, vec;
+
+  __device__ __forceinline__ void set(const float* p_, int64_t ld_, int i0, int n, bool along_k_, int K) {
+    const int tid = threadIdx.x;
+    ld = ld_; along_k = along_k_; vec = along_k_ && (ld_ & 3) == 0;
+    int row;
+    if (vec) { row = tid / 4; k = tid % 4 * 4; }                     // whole vectors: rows 32 apart
+    else if (along_k) { row = tid / 16; k = tid % 16; }              // rows 8 apart
+    // across K, a warp takes eight rows, whole sectors, of four K (its words then lie in 32 banks); rows 8 apart
+    else { row = tid % 8; k = tid / 8; }
+    p = p_ + (along_k ? (int64_t)(i0 + row) * ld + k : (int64_t)k * ld + i0 + row);
+    rows = n - i0 - row;
+    if (rows <= 0 || k >= K) p = p_;            // (nothing is read, but the address stays inside the operand)
+    dst = row * P + k;
+  }
+  __device__ __forceinline__ void copy(float* s, int k0, int k_end) const {
+    const bool in = k0 + k < k_end;
+    const float* const src = p + (along_k ? (int64_t)k0 : (int64_t)k0 * ld);
+    if (vec) {
+#pragma unroll
+      for (int q = 0; q < (ROWS + 31) / 32; ++q) {
+        if (ROWS % 32 != 0 && 32 * q + (int)threadIdx.x / 4 >= ROWS) continue;
+        const bool ok = in && 32 * q < rows;
+        copy16_async(s + dst + 32 * q * P, ok ? src + 32 * q * ld : p, ok);
+      }
+    } else {
+      const int64_t step = along_k ? 8 * ld : 8;
+#pragma unroll
+      for (int q = 0; q < ROWS / 8; ++q) {
+        const bool ok = in && 8 * q < rows;
+        copy4_async(s + dst + 8 * q * P, ok ? src + q * step : p, ok);
+      }
+    }
+  }
+};
+
 // Which elements of a tile this thread holds: rows row(i), columns col(c).
 template <typename S>
 struct Lane {
@@ -153,6 +211,60 @@ __device__ __forceinline__ void zero_acc(Acc<S>& acc) {
     for (int c = 0; c < S::TN; ++c) acc[i][c] = 0ull;
 }
 
+// acc += X Y^T over one stage of K
+template <typename S>
+__device__ __forceinline__ void tile_stage(Acc<S>& acc, const float* xr, const float* yr) {
+#pragma unroll
+  for (int k = 0; k < S::BK; k += 4) {
+    ulonglong2 y[S::TN];
+#pragma unroll
+    for (int c = 0; c < S::TN; ++c) y[c] = *reinterpret_cast<const ulonglong2*>(&yr[4 * c * S::P + k]);
+#pragma unroll
+    for (int i = 0; i < S::RI; ++i) {
+      const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&xr[8 * i * S::P + k]);
+#pragma unroll
+      for (int c = 0; c < S::TN; ++c) acc[i][c] = fma_f32x2(x.x, y[c].x, acc[i][c]);
+#pragma unroll
+      for (int c = 0; c < S::TN; ++c) acc[i][c] = fma_f32x2(x.y, y[c].y, acc[i][c]);
+    }
+  }
+}
+
+// acc += X Y^T over k in [k_begin, k_end), with kAsyncStages - 1 stages of copies in flight.
+// Through registers, one stage ahead, the warps waited for their loads between bursts of FMAs (a third of their stalls) and held
+// 21 to 24 registers for them.  Four refit launches of a step, us, registers -> copies: 6 layers of 768 x 3072 rank 8 769 -> 533,
+// rank 38 1286 -> 977, rank 128 3581 -> 2884; rows of 2130 rank 38 1107 -> 834; the tiny set (rank 12) 107 -> 90.  Two CTAs of
+// 248 registers per SM instead of three of 168: 569, 960, 3140.
+template <typename S, typename X, typename Y>
+__device__ __forceinline__ void tile_loop_async(Acc<S>& acc, const X& xop, const Y& yop, int k_begin, int k_end, float* sm) {
+  const Lane<S> at;
+  constexpr int kStage = (S::kRows + S::kCols) * S::P;
+  const float* const xr = sm + at.r0 * S::P;
+  const float* const yr = sm + (S::kRows + at.c0) * S::P;
+  __syncthreads();                              // an earlier loop may still be reading the stages
+  int fill = 0, use = 0, k_fill = k_begin;
+  auto next = [&]() {
+    if (k_fill < k_end) {
+      xop.copy(sm + fill, k_fill, k_end);
+      yop.copy(sm + fill + S::kRows * S::P, k_fill, k_end);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    k_fill += S::BK;
+    fill = fill == (kAsyncStages - 1) * kStage ? 0 : fill + kStage;
+  };
+#pragma unroll
+  for (int i = 0; i < kAsyncStages - 1; ++i) next();
+#pragma unroll 1
+  for (int k0 = k_begin; k0 < k_end; k0 += S::BK) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAsyncStages - 2) : "memory");
+    __syncthreads();                            // everyone's copies of this stage are here, and the one before it is free
+    next();
+    tile_stage<S>(acc, xr + use, yr + use);
+    use = use == (kAsyncStages - 1) * kStage ? 0 : use + kStage;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 // acc += X Y^T over k in [k_begin, k_end).
 template <typename S, typename X, typename Y>
 __device__ __forceinline__ void tile_loop(Acc<S>& acc, X& xop, Y& yop, int k_begin, int k_end, float* sm) {
@@ -173,20 +285,7 @@ __device__ __forceinline__ void tile_loop(Acc<S>& acc, X& xop, Y& yop, int k_beg
       xop.fetch(k0 + S::BK, k_end);
       yop.fetch(k0 + S::BK, k_end);
     }
-#pragma unroll
-    for (int k = 0; k < S::BK; k += 4) {
-      ulonglong2 y[S::TN];
-#pragma unroll
-      for (int c = 0; c < S::TN; ++c) y[c] = *reinterpret_cast<const ulonglong2*>(&yr[buf + 4 * c * S::P + k]);
-#pragma unroll
-      for (int i = 0; i < S::RI; ++i) {
-        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(&xr[buf + 8 * i * S::P + k]);
-#pragma unroll
-        for (int c = 0; c < S::TN; ++c) acc[i][c] = fma_f32x2(x.x, y[c].x, acc[i][c]);
-#pragma unroll
-        for (int c = 0; c < S::TN; ++c) acc[i][c] = fma_f32x2(x.y, y[c].y, acc[i][c]);
-      }
-    }
+    tile_stage<S>(acc, xr + buf, yr + buf);
   }
 }
 
@@ -299,7 +398,13 @@ __device__ __forceinline__ void refit_tile(const Fp32Refit& U, int unit, const B
   Acc<S> acc;
   zero_acc<S>(acc);
   Operand<S::kCols, S::BK, float> yop;
-  {
+  if constexpr (sizeof(GT) == 4) {
+    AsyncOperand<S::kRows, S::BK> xa;
+    AsyncOperand<S::kCols, S::BK> ya;
+    xa.set(static_cast<const float*>(b.p[BASE_GRADS]) + U.g_off, U.ldg, mt * S::kRows, U.owners, U.along_k, U.K);
+    ya.set(static_cast<const float*>(b.p[U.y_base]) + U.y_off, U.along_k ? U.K : r, nt * S::kCols, r, U.along_k, U.K);
+    tile_loop_async<S>(acc, xa, ya, k_begin, k_end, sm);
+  } else {
     Operand<S::kRows, S::BK, GT> xop;
     xop.set(static_cast<const GT*>(b.p[BASE_GRADS]) + U.g_off, U.ldg, mt * S::kRows, U.owners, U.along_k, 1.f);
     yop.set(static_cast<const float*>(b.p[U.y_base]) + U.y_off, U.along_k ? U.K : r, nt * S::kCols, r, U.along_k, 1.f);
@@ -353,7 +458,7 @@ template <typename GT>
 __global__ void __launch_bounds__(kThreads, 3) fp32_refit_kernel(const Fp32Refit* __restrict__ tab,
                                                                  const int32_t* __restrict__ unit_job, Bases b,
                                                                  int32_t* __restrict__ counters) {
-  __shared__ __align__(16) float sm[Tile<8, 5, 16>::kFloats];
+  __shared__ __align__(16) float sm[sizeof(GT) == 4 ? Tile<8, 5, 16>::kAsyncFloats : Tile<8, 5, 16>::kFloats];
   __shared__ Fp32Refit sU;
   if (threadIdx.x == 0) {
     sU = tab[unit_job[blockIdx.x]];

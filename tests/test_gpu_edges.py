@@ -67,6 +67,15 @@ def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
              (304, 304, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 0)], dtype=dtype, path=A.PATH_SIMT)
 
 
+@pytest.mark.parametrize("rank", [3, 12, 38])
+def test_exact_fp32_refit_at_the_ends_of_its_stages(rank):
+    """K of less than the stages in flight, of whole stages and one more; rows and columns that are not a multiple of four, or
+    of eight."""
+    _follow([(m, n, A.MOM_LOWRANK, min(rank, m, n), A.V_BLOCKMEAN, 1)
+             for m, n in [(5, 4), (16, 17), (33, 31), (47, 48), (49, 132), (129, 130), (136, 64)]], dtype="f32",
+            path=A.PATH_SIMT)
+
+
 @pytest.mark.parametrize("iters,period", [(1, 0), (2, 0), (3, 0), (2, 3), (3, 3), (5, 3)])
 def test_exact_fp32_refit_by_number_of_passes(iters, period):
     """K = 1 has no effective pass, K = 2 a single one that ends in the workspace, K = 3 two."""
