@@ -121,7 +121,7 @@ typedef struct {
                               it).  Reading: both factors are refitted by Algorithm 2 at steps 1, T+1,
                               2T+1, ...; in between L is held and only R moves (the R half of Algorithm 2).
                               0 or 1 = Algorithm 1 as printed, every step                          */
-  int32_t tune_panels;     /* tensor path: 128-row panels per refit item (1..3); 0 = automatic     */
+  int32_t tune_panels;     /* tensor path: 128-row panels per CTA of a refit item (1..3); 0 = auto  */
   int32_t tune_stage_k;    /* tensor path: K per shared-memory stage (64 or 128); 0 = automatic    */
   int32_t inner_precond;   /* 0 = Algorithm 2 as printed.  1 = preconditioned passes (a variant, not in
                               the paper: scaled gradient descent): dl/dL is multiplied from the right
