@@ -42,25 +42,35 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                "r"(bytes)
                : "memory");
 }
+// What a wait makes of the arrivals it saw.
+enum Wait : int {
+  WAIT_CTA,          // threads and copies of this CTA: acquire
+  WAIT_PAIR,         // threads, copies and commits of either CTA of a pair: acquire at cluster scope
+  WAIT_PAIR_TC       // the same where only tensor memory is at stake, which the tcgen05 fences on both sides order: relaxed
+};
+// Whether the phase with the given parity is complete; may suspend the thread for a while first.
+template <Wait W = WAIT_CTA>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendHintNs)
-      : "memory");
+#define ADAPM_TRY_WAIT(SEM)                                                                                                       \
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity" SEM ".shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}" \
+               : "=r"(ok)                                                                                                         \
+               : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendHintNs)                                                             \
+               : "memory")
+  if (W == WAIT_CTA) ADAPM_TRY_WAIT("");
+  else if (W == WAIT_PAIR) ADAPM_TRY_WAIT(".acquire.cluster");
+  else ADAPM_TRY_WAIT(".relaxed.cluster");
+#undef ADAPM_TRY_WAIT
   return ok != 0;
 }
 
-// Arrives at the same barrier of CTA `rank` of the cluster.  (With .release.cluster an arrival takes a thousand cycles, which
-// set the pace of the whole pair; the threads that arrive here have written nothing the other CTA reads: what they report is
-// shared memory that TMA has filled and tensor memory that has been read, ordered by the barrier and tcgen05.fence.)
-__device__ __forceinline__ void mbar_arrive_at(uint64_t* bar, uint32_t rank) {
-  asm volatile(
-      "{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, %1;\n"
-      "mbarrier.arrive.shared::cluster.b64 _, [ra];\n}" ::"r"(smem_u32(bar)),
-      "r"(rank)
-      : "memory");
+// Arrives at the barrier of another CTA of the cluster (address from shared_of) to say that this thread has read what it
+// wanted from tensor memory.  The order is the one the instruction set documents for tcgen05 across threads:
+// tcgen05.fence::before_thread_sync, an arrival that is relaxed at cluster scope, a wait at that scope and
+// tcgen05.fence::after_thread_sync.  It orders nothing else: memory that this thread wrote is not made visible.
+// (A releasing arrival at that scope takes a thousand cycles, between two items of every pair.)
+__device__ __forceinline__ void mbar_arrive_relaxed_at(uint32_t bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // ---- pairs of CTAs -----------------------------------------------------------------------------------
@@ -72,33 +82,42 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The address in the cluster's window of what lies at `p` in the shared memory of CTA `rank`.
+__device__ __forceinline__ uint32_t shared_of(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
 // A word of shared memory of CTA `rank`, at the address it has in this CTA.
 __device__ __forceinline__ int load_shared_of(const int* p, uint32_t rank) {
   int v;
-  asm volatile("{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %1, %2;\nld.shared::cluster.s32 %0, [ra];\n}"
-               : "=r"(v)
-               : "r"(smem_u32(p)), "r"(rank)
-               : "memory");
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(shared_of(p, rank)) : "memory");
   return v;
 }
 
 // Whether the phase with the given parity is complete; does not suspend.
+template <Wait W = WAIT_CTA>
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
+#define ADAPM_TEST_WAIT(SEM)                                                                                                   \
+  asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity" SEM ".shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}" \
+               : "=r"(ok)                                                                                                      \
+               : "r"(smem_u32(bar)), "r"(parity)                                                                               \
+               : "memory")
+  if (W == WAIT_CTA) ADAPM_TEST_WAIT("");
+  else if (W == WAIT_PAIR) ADAPM_TEST_WAIT(".acquire.cluster");
+  else ADAPM_TEST_WAIT(".relaxed.cluster");
+#undef ADAPM_TEST_WAIT
   return ok != 0;
 }
 // Waits for the phase with the given parity to complete.  Gives up after `limit` polls or as
 // soon as another thread of the CTA has given up (*abort != 0); then sets *abort, records `code` in
 // the device status word and returns false.  Callers leave their loops on false.
+template <Wait W = WAIT_CTA>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* status,
                                           int32_t code, uint32_t limit = kSpinLimit) {
   for (uint32_t it = 0; it < limit; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<W>(bar, parity)) return true;
     if (it > 32) {
       __nanosleep(it > 4096 ? 256 : 32);
       if ((it & 255u) == 0 && *abort) return false;
@@ -127,12 +146,13 @@ __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xf
 // first, and those moves, not the MMAs, set the pace (measured on the refit engine, four panel launches of a step:
 // 858 -> 752 us at rank 8, 159 -> 140 us on the 60M shapes; on the apply kernel without its memory traffic, 1.5B
 // shapes: 2.1 -> 1.4 ms).
+template <Wait W = WAIT_CTA>
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* status,
                                                int32_t code, uint32_t limit = kSpinLimit) {
   for (int it = 0; it < 8; ++it)
-    if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_test_wait<W>(bar, parity))) return true;
   for (uint32_t it = 0; it < limit; ++it) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_try_wait<W>(bar, parity))) return true;
     if (it > 32) {
       __nanosleep(it > 4096 ? 256 : 32);
       if ((it & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0)) return false;
@@ -168,6 +188,16 @@ __device__ __forceinline__ void tma_load_box(void* smem_dst, const void* tmap, i
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
           smem_u32(smem_dst)),
       "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// The same in a pair of CTAs: into the shared memory of this CTA, its bytes counted at a barrier of either of them (address
+// from shared_of).
+__device__ __forceinline__ void tma_load_box_pair(void* smem_dst, const void* tmap, int x, int y, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_u32(smem_dst)),
+      "l"(tmap), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
 

@@ -36,11 +36,15 @@
 // 350M set at rank 128, 172 -> 147 at rank 8.  What is left there: the power cap (SM clocks of 1.3 to 1.5 GHz while these
 // launches run) and, per stage, the serial path of the warp that issues the MMAs.
 // Warp roles (512 threads, 128 registers each): warp 0 loads A, warp 3 loads B, warp 1 issues the MMAs (in a pair that of
-// rank 0, for both), warp 2 of rank 1 tells rank 0 which of its stages are full, warps 4-7 add up g^2 per row from the
-// gradient tiles of the first segment when the launch asks for it (the second-moment statistic of the block-mean form then
-// needs no pass of its own over g), warps 8-15 drain the accumulators (two groups of four warps that take the 16-column
-// pieces of an item alternately).  The issuing warps run dependent scalar code, so their per-stage instruction count bounds
-// the rate; all lanes run the loops on values that the compiler knows to be uniform (mbar_wait_warp, uniform).
+// rank 0, for both), warps 4-7 add up g^2 per row from the gradient tiles of the first segment when the launch asks for it
+// (the second-moment statistic of the block-mean form then needs no pass of its own over g), warps 8-15 drain the
+// accumulators (two groups of four warps that take the 16-column pieces of an item alternately).  The issuing warps run
+// dependent scalar code, so their per-stage instruction count bounds the rate; all lanes run the loops on values that the
+// compiler knows to be uniform (mbar_wait_warp, uniform).
+// The copies of both CTAs of a pair are counted at the barriers of rank 0, whose MMAs read them; rank 1 learns from the commit
+// of those MMAs that a stage of its own has been filled and multiplied.  The row sums of rank 1 are therefore made between the
+// MMAs of a stage and its next fill, those of rank 0 beside the MMAs.  (A commit ahead of the MMAs, to let rank 1 start with
+// them: 871 -> 862 us per step where the ring has three stages, 9.11 -> 9.16 ms on the 1.5B set.)
 // With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
 // Every wait is bounded; when one runs out the CTA records a status bit, stops taking work and
 // leaves through the common exit (which frees its tensor memory).  A launch that finds the status
@@ -144,30 +148,39 @@ struct EngineArgs {
 };
 
 struct __align__(8) EngineShared {
-  uint64_t full[8], empty[8], tfull[2], tempty[2];
+  uint64_t full[8], empty[8], summed[8], tfull[2], tempty[2];
   uint32_t tmem_base;
   int abort, skip;
 };
 
 // The A operands of one stage, NBOX boxes each.  Compile-time counts keep the issuing thread's instruction stream short (it
 // runs dependent scalar code; its rate bounds the pipeline).
-template <int NA, int NBOX>
+template <bool PAIR, int NA, int NBOX>
 __device__ __forceinline__ void load_operands(uint8_t* sa, int a_tile, int box_bytes, const CUtensorMap* ma, const int* x,
-                                              const int* y, uint64_t* bar) {
+                                              const int* y, uint64_t* bar, uint32_t pair_bar) {
 #pragma unroll
   for (int p = 0; p < NA; ++p)
 #pragma unroll
-    for (int j = 0; j < NBOX; ++j) tma_load_box(sa + p * a_tile + j * box_bytes, ma, x[p] + 64 * j, y[p], bar);
+    for (int j = 0; j < NBOX; ++j) {
+      if (PAIR) tma_load_box_pair(sa + p * a_tile + j * box_bytes, ma, x[p] + 64 * j, y[p], pair_bar);
+      else tma_load_box(sa + p * a_tile + j * box_bytes, ma, x[p] + 64 * j, y[p], bar);
+    }
 }
 
 // Lets the copies already issued into a ring of `n_stages` land before the CTA exits.  (stage, phase): where the next would go.
-__device__ __forceinline__ void drain_ring(uint64_t* full, int stage, uint32_t phase, uint32_t issued, int n_stages) {
+// (Rank 1 of a pair has no barrier that counts its own: it allows them a few milliseconds, a thousand times what a copy takes.)
+template <bool PAIR>
+__device__ __forceinline__ void drain_ring(uint64_t* full, int stage, uint32_t phase, uint32_t issued, int n_stages, uint32_t rank) {
+  if (PAIR && rank != 0) {
+    for (uint32_t spin = 0; issued > 0 && spin < kDrainSpins; ++spin) __nanosleep(64);
+    return;
+  }
   const int back = issued < (uint32_t)n_stages ? (int)issued : n_stages;
   for (int q = 0; q < back; ++q) {
     int st = stage - 1 - q;
     uint32_t ph = phase;
     if (st < 0) { st += n_stages; ph ^= 1u; }
-    for (uint32_t spin = 0; spin < kDrainSpins && !mbar_try_wait(&full[st], ph); ++spin) __nanosleep(64);
+    for (uint32_t spin = 0; spin < kDrainSpins && !mbar_try_wait<PAIR ? WAIT_PAIR : WAIT_CTA>(&full[st], ph); ++spin) __nanosleep(64);
   }
 }
 
@@ -192,7 +205,8 @@ __device__ __forceinline__ bool mma_segment(const EngineArgs& a, EngineShared& s
   const uint32_t a_lbo = MN_MAJOR_A ? S.b_lbo : 16u;
   uint32_t accumulate = S.accumulate;
   for (int k_left = S.k; k_left > 0; k_left -= kStageK) {
-    if (!mbar_wait_warp(&sh.full[cur.stage], cur.phase, &sh.abort, a.status, ST_WAIT_FULL, a.wait_spin_limit)) return false;
+    if (!mbar_wait_warp<PAIR ? WAIT_PAIR : WAIT_CTA>(&sh.full[cur.stage], cur.phase, &sh.abort, a.status, ST_WAIT_FULL,
+                                                     a.wait_spin_limit)) return false;
     tc_fence_after();
     // per K step of 16, in 16-byte units: K along x walks 32 B inside a box and 16 KB to the next box; K along y walks 16
     // rows of 128 B
@@ -260,8 +274,9 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 8; ++i) {
-      mbar_init(&sh.full[i], PAIR && rank == 0 ? 3 : 2);      // A, B, and for rank 0 the other CTA's stage
-      mbar_init(&sh.empty[i], PAIR && a.sumsq_on ? 5 : 1);
+      mbar_init(&sh.full[i], 2);                              // A and B (of a pair: those of rank 0, for both CTAs)
+      mbar_init(&sh.empty[i], PAIR && a.sumsq_on && rank == 0 ? 5 : 1);
+      mbar_init(&sh.summed[i], 4);
     }
     for (int i = 0; i < 2; ++i) { mbar_init(&sh.tfull[i], 1); mbar_init(&sh.tempty[i], PAIR ? 16 : 8); }
     sh.abort = 0;
@@ -282,6 +297,10 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
   const int it_begin = uniform(skip ? 0 : a.cta_begin[unit]), it_end = uniform(skip ? 0 : a.cta_begin[unit + 1]);
   const int stage_k = a.stage_k;
   const int a_tile = 256 * stage_k;                 // bytes of one A operand of a stage
+  constexpr Wait kWait = PAIR ? WAIT_PAIR : WAIT_CTA, kTensorWait = PAIR ? WAIT_PAIR_TC : WAIT_CTA;
+  // what a producer waits for: in rank 1 the row sums come after the MMAs, in rank 0 they arrive at the same barrier
+  uint64_t* const free_bar = PAIR && rank != 0 && a.sumsq_on ? sh.summed : sh.empty;
+  const uint32_t pair_full = PAIR ? uniform(shared_of(sh.full, 0)) : 0u;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (all lanes run, one issues)
@@ -324,12 +343,13 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         const int n_box = a_mode ? 2 : (stage_k >> 6);
         const int box_bytes = a_mode ? stage_k * 128 : kBoxBytes;
         for (int c = 0; c < nst; ++c) {
-          if (!mbar_wait_warp(&sh.empty[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
+          if (!mbar_wait_warp<kWait>(&free_bar[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
           uint8_t* sa = stages + stage * a.stage_bytes;
           uint64_t* bar = &sh.full[stage];
           if (leader) {
-            mbar_arrive_expect_tx(bar, tx_bytes);
-#define ADAPM_LOAD(NA, NBOX) load_operands<NA, NBOX>(sa, a_tile, box_bytes, ma, x, y, bar)
+            if (!PAIR || rank == 0) mbar_arrive_expect_tx(bar, PAIR ? 2 * tx_bytes : tx_bytes);
+            const uint32_t pair_bar = pair_full + 8u * (uint32_t)stage;
+#define ADAPM_LOAD(NA, NBOX) load_operands<PAIR, NA, NBOX>(sa, a_tile, box_bytes, ma, x, y, bar, pair_bar)
             if (!PAIR) {
               if (n_a == 2) ADAPM_LOAD(2, 2); else ADAPM_LOAD(1, 2);
             } else if (n_box == 2) {
@@ -348,7 +368,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       }
       if (ok && signal && leader && rank == 0) atomicAdd(team, signal);
     }
-    if (!ok) drain_ring(sh.full, stage, phase, issued, a.n_stages);
+    if (!ok) drain_ring<PAIR>(sh.full, stage, phase, issued, a.n_stages, rank);
   } else if (warp == 3) {
     // ------------------------------------------------------------------ producer of B (a warp of its own: an expected
     // count and a box take 100 cycles each to issue, and a stage of 64 K is multiplied in 300 to 800)
@@ -367,16 +387,17 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         const int nst = (uniform(S.k) + stage_k - 1) / stage_k, n_b = uniform((int)S.n_b), xb = rank ? uniform((int)S.b_x) : 0;
         const uint32_t tx_bytes = uniform(S.tx_bytes) - (uint32_t)(uniform((int)S.n_a) * a_tile);
         for (int c = 0; c < nst; ++c) {
-          if (!mbar_wait_warp(&sh.empty[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
+          if (!mbar_wait_warp<kWait>(&free_bar[stage], phase ^ 1u, abort, a.status, ST_WAIT_EMPTY, wlim)) { ok = false; break; }
           uint8_t* sb = stages + stage * a.stage_bytes + a.a_bytes;
           uint64_t* bar = &sh.full[stage];
           if (leader) {
-            mbar_arrive_expect_tx(bar, tx_bytes);
+            if (!PAIR || rank == 0) mbar_arrive_expect_tx(bar, PAIR ? 2 * tx_bytes : tx_bytes);
             if (PAIR) {
-              tma_load_box(sb, mb, xb, c * stage_k, bar);
-              if (n_b > 1) tma_load_box(sb + b_box, mb, xb + 64, c * stage_k, bar);
-              if (n_b > 2) tma_load_box(sb + 2 * b_box, mb, xb + 128, c * stage_k, bar);
-              if (n_b > 3) tma_load_box(sb + 3 * b_box, mb, xb + 192, c * stage_k, bar);
+              const uint32_t pair_bar = pair_full + 8u * (uint32_t)stage;
+              tma_load_box_pair(sb, mb, xb, c * stage_k, pair_bar);
+              if (n_b > 1) tma_load_box_pair(sb + b_box, mb, xb + 64, c * stage_k, pair_bar);
+              if (n_b > 2) tma_load_box_pair(sb + 2 * b_box, mb, xb + 128, c * stage_k, pair_bar);
+              if (n_b > 3) tma_load_box_pair(sb + 3 * b_box, mb, xb + 192, c * stage_k, pair_bar);
             } else {
               tma_load_box3(sb, mb, 0, c * stage_k, 0, bar);
             }
@@ -387,7 +408,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         }
       }
     }
-    if (!ok) drain_ring(sh.full, stage, phase, issued, a.n_stages);
+    if (!ok) drain_ring<PAIR>(sh.full, stage, phase, issued, a.n_stages, rank);
   } else if (warp == 1 && rank == 0) {
     // ------------------------------------------------------------------ MMA issuer (all lanes run, one issues)
     const bool leader = elect_one();
@@ -399,7 +420,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       const Item& I = a.items[it];
       const int acc = j % a.n_acc;
       const uint32_t acc_phase = (uint32_t)(j / a.n_acc) & 1u;
-      if (!mbar_wait_warp(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY, wlim)) break;
+      if (!mbar_wait_warp<kTensorWait>(&sh.tempty[acc], acc_phase ^ 1u, abort, a.status, ST_WAIT_TMEM_EMPTY, wlim)) break;
       tc_fence_after();
       const uint32_t d_base = d0 + (uint32_t)(acc * a.acc_cols);
       const int n_seg = uniform(I.n_seg);
@@ -422,24 +443,6 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       if (ok && leader) mma_commit<PAIR>(&sh.tfull[acc]);
       __syncwarp();
     }
-  } else if (PAIR && warp == 2 && rank == 1) {
-    // ------------------------------------------------------------------ tells rank 0 of every stage that is full here
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int it = it_begin; it < it_end && ok; ++it) {
-      const Item& I = a.items[it];
-      const int n_seg = uniform(I.n_seg);
-      for (int s = 0; s < n_seg && ok; ++s) {
-        const int nst = (uniform(I.seg[s].k) + stage_k - 1) / stage_k;
-        for (int c = 0; c < nst; ++c) {
-          if (!mbar_wait_warp(&sh.full[stage], phase, abort, a.status, ST_WAIT_FULL, wlim)) { ok = false; break; }
-          if (lane == 0) mbar_arrive_at(&sh.full[stage], 0);
-          __syncwarp();
-          if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
-        }
-      }
-    }
   } else if (warp < 4) {
     // no work
   } else if (warp < 8) {
@@ -451,6 +454,8 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
     // lane keeps one partial sum per row it visits, and the eight partial sums of a row are added in a fixed
     // order at the end of the item.
     if (PAIR && a.sumsq_on) {
+      uint64_t* const ready = rank == 0 ? sh.full : sh.empty;      // (empty: filled, and multiplied as well)
+      uint64_t* const done = rank == 0 ? sh.empty : sh.summed;
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -471,7 +476,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
           const int n_box = stage_k >> 6;
           for (int c = 0; c < nst; ++c) {
             bool got = true;
-            if (lane == 0) got = mbar_wait(&sh.full[stage], phase, abort, a.status, ST_WAIT_FULL, wlim);
+            if (lane == 0) got = mbar_wait<WAIT_PAIR>(&ready[stage], phase, abort, a.status, ST_WAIT_FULL, wlim);
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) { ok = false; break; }
             if (mine && s == 0) {
@@ -499,7 +504,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
               }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.empty[stage]);
+            if (lane == 0) mbar_arrive(&done[stage]);
             if (++stage == a.n_stages) { stage = 0; phase ^= 1u; }
           }
         }
@@ -637,7 +642,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
       // one lane per warp polls (fewer pollers on the barrier), then the warp agrees: the
       // tensor-memory loads below need all 32 lanes
       bool got = true;
-      if (lane == 0) got = mbar_wait(&sh.tfull[acc], acc_phase, abort, a.status, ST_WAIT_TMEM_FULL, wlim);
+      if (lane == 0) got = mbar_wait<kTensorWait>(&sh.tfull[acc], acc_phase, abort, a.status, ST_WAIT_TMEM_FULL, wlim);
       got = __shfl_sync(0xffffffffu, got, 0);
       if (!got) break;
       tc_fence_after();
@@ -685,7 +690,7 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (PAIR) mbar_arrive_at(&sh.tempty[acc], 0);
+          if (PAIR) mbar_arrive_relaxed_at(shared_of(&sh.tempty[acc], 0));
           else mbar_arrive(&sh.tempty[acc]);
         }
       };

@@ -56,6 +56,43 @@ def test_panels_at_the_edges_of_a_pair_of_ctas(rank, panels, stage_k):
             tune_panels=panels, tune_stage_k=stage_k)
 
 
+@pytest.mark.parametrize("rank", [12, 80, 144])
+def test_a_step_repeats_bit_for_bit_beside_other_work(rank):
+    """The order between the two CTAs of a pair (stages filled by one and multiplied by the other, tensor memory read by one
+    and overwritten by the other, row sums of the second CTA) does not depend on timing: the same step again and again, while
+    copies on another stream come and go."""
+    import torch
+    blocks = _blocks([(n, m, A.MOM_LOWRANK, rank, A.V_BLOCKMEAN, 1) for n, m in [(640, 776), (1000, 520), (384, 2048), (2050, 264)]])
+    total = blocks[-1].offset + blocks[-1].rows * blocks[-1].cols
+    ctx = A.adapm_create(blocks, A.hparams(grad_dtype=A.GRAD_BF16, lowrank_path=A.PATH_TENSOR))
+    gen = torch.Generator(device="cuda").manual_seed(rank)
+    params0 = torch.randn(total, generator=gen, device="cuda")
+    grads = torch.randn(total, generator=gen, device="cuda").mul_(1e-3).bfloat16()
+    state = torch.zeros(ctx.adapm_state_bytes() // 4, device="cuda")
+    work = torch.zeros(ctx.adapm_workspace_bytes() // 4, device="cuda")
+    ctx.adapm_set_workspace(work)
+    ctx.adapm_state_init(state)
+    ctx.adapm_step(params0, grads, state, 1)
+    state0, params = state.clone(), params0.clone()
+    noise, side = torch.zeros(1 << 24, device="cuda"), torch.cuda.Stream()
+    first = None
+    for i in range(24):
+        params.copy_(params0)
+        state.copy_(state0)
+        ctx.adapm_state_changed()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            for _ in range(i % 4):
+                noise.add_(1.0)
+        ctx.adapm_step(params, grads, state, 2)
+        torch.cuda.synchronize()
+        if first is None:
+            first = params.clone(), state.clone()
+        assert torch.equal(first[0], params) and torch.equal(first[1], state), f"repeat {i}"
+    assert ctx.adapm_get_status() == 0
+    ctx.adapm_destroy()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("rank", [1, 8, 9, 24, 40, 41, 81, 300])
 def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
