@@ -1017,7 +1017,7 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
       a.cta_begin = (const int32_t*)(c->d_tables + L.aux3);
       a.sum_col = (int32_t)L.aux4; a.sumsq_on = (int32_t)L.aux5;
       a.team_counters = nullptr;
-      a.team_spin_limit = tc::kTeamSpinDefault; a.wait_spin_limit = tc::kWaitSpinDefault;
+      a.team_spin_limit[0] = a.team_spin_limit[1] = tc::kTeamSpinDefault; a.wait_spin_limit = tc::kWaitSpinDefault;
       a.gscale = b.gscale;
       if (L.kind == LK_TC_PANEL && P->d_team_counters) {
         ADAPM_CUDA(cudaMemsetAsync(P->d_team_counters, 0, P->n_teams * sizeof(int32_t), s));
@@ -1056,8 +1056,8 @@ int run_tensor_launch(adapm_ctx* c, const Launch& L, const Bases& b, const StepS
 }
 
 // Diagnostic: one pair of CTAs of the engine whose only item waits for a team counter that nothing advances, with a wait
-// limit of about a millisecond.  The kernel must return, leave ST_WAIT_TEAM in the status word and free its
-// tensor memory; the context stays usable.
+// limit of about a millisecond in rank 0 and the usual one in rank 1, which has to hear of it from the other.  The kernel must
+// return, leave ST_WAIT_TEAM in the status word and free its tensor memory; the context stays usable.
 int run_expired_wait_probe(adapm_ctx* c, cudaStream_t s) {
   struct Probe { tc::Item item; int32_t begin[4]; };
   static_assert(sizeof(Probe) % 4 == 0, "probe table");
@@ -1070,7 +1070,8 @@ int run_expired_wait_probe(adapm_ctx* c, cudaStream_t s) {
   a.cta_begin = (const int32_t*)(c->d_probe + sizeof(tc::Item));
   a.sum_col = -1; a.sumsq_on = 0;
   a.team_counters = c->d_status + 16;       // a zeroed word beside the status word that nothing adds to
-  a.team_spin_limit = 1u << 12; a.wait_spin_limit = tc::kWaitSpinDefault;
+  a.team_spin_limit[0] = 1u << 12; a.team_spin_limit[1] = tc::kTeamSpinDefault;
+  a.wait_spin_limit = tc::kWaitSpinDefault;
   launch_clusters(false, 2, tc::tc_items_kernel<true>, 2, tc::kEngineThreads, 4096, s, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

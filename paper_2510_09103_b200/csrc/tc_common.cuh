@@ -20,8 +20,8 @@ namespace tc {
 constexpr int kBoxRows = 128;
 constexpr int kBoxCols = 64;                       // bf16 elements: 128 bytes
 constexpr int kBoxBytes = kBoxRows * kBoxCols * 2; // 16384
-constexpr uint32_t kSpinLimit = 1u << 20;          // bounded waits: about a second of polling in all
 constexpr uint32_t kSuspendHintNs = 1000;          // a poll may park the thread this long before it reports failure
+constexpr uint32_t kSpinLimit = 1u << 20;          // bounded waits, in polls of 0.3 to 1.3 us: about a second
 
 // status bits a kernel may set when a bounded wait runs out
 enum : int32_t { ST_WAIT_FULL = 1, ST_WAIT_EMPTY = 2, ST_WAIT_TMEM_FULL = 4, ST_WAIT_TMEM_EMPTY = 8, ST_WAIT_DRAIN = 16,
@@ -110,8 +110,17 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 #undef ADAPM_TEST_WAIT
   return ok != 0;
 }
+// Tells the other waiting threads that this one has given up; PAIR: those of the other CTA of the pair too, which would
+// otherwise find out by their own limits, one after the other.  (Its shared memory is there until the closing cluster barrier.)
+template <bool PAIR>
+__device__ __forceinline__ void give_up(volatile int* abort) {
+  *abort = 1;
+  if (PAIR)
+    asm volatile("st.relaxed.cluster.shared::cluster.s32 [%0], 1;" ::"r"(shared_of(const_cast<const int*>(abort), cluster_rank() ^ 1u))
+                 : "memory");
+}
 // Waits for the phase with the given parity to complete.  Gives up after `limit` polls or as
-// soon as another thread of the CTA has given up (*abort != 0); then sets *abort, records `code` in
+// soon as another thread of the CTA, or of the pair, has given up (*abort != 0); then sets *abort, records `code` in
 // the device status word and returns false.  Callers leave their loops on false.
 template <Wait W = WAIT_CTA>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* status,
@@ -123,7 +132,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
       if ((it & 255u) == 0 && *abort) return false;
     }
   }
-  *abort = 1;
+  give_up<W != WAIT_CTA>(abort);
   atomicOr(status, code);
   return false;
 }
@@ -158,7 +167,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
       if ((it & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0)) return false;
     }
   }
-  *abort = 1;
+  give_up<W != WAIT_CTA>(abort);
   atomicOr(status, code);
   return false;
 }

@@ -46,8 +46,8 @@
 // MMAs of a stage and its next fill, those of rank 0 beside the MMAs.  (A commit ahead of the MMAs, to let rank 1 start with
 // them: 871 -> 862 us per step where the ring has three stages, 9.11 -> 9.16 ms on the 1.5B set.)
 // With two accumulator buffers the epilogue of one item overlaps the K-loops of the next.
-// Every wait is bounded; when one runs out the CTA records a status bit, stops taking work and
-// leaves through the common exit (which frees its tensor memory).  A launch that finds the status
+// Every wait is bounded; when one runs out the CTA records a status bit, stops taking work, tells the other CTA of its
+// pair to do the same and leaves through the common exit (which frees its tensor memory).  A launch that finds the status
 // word set on entry does nothing.
 #pragma once
 
@@ -62,8 +62,8 @@ constexpr int kMaxSegs = 4;
 constexpr int kMaxA = 3;
 constexpr int kEngineThreads = 512;
 constexpr uint32_t kTeamSpinDefault = 1u << 22;   // polls of 256 ns each: about a second
-constexpr uint32_t kDrainSpins = 1u << 16;         // of a copy in flight when a CTA gives up: tens of milliseconds
-constexpr uint32_t kWaitSpinDefault = 1u << 23;   // mbarrier polls: at least as long as a team wait
+constexpr uint32_t kDrainSpins = 1u << 16;         // for the copies in flight when a CTA gives up: 4 to 70 milliseconds in all
+constexpr uint32_t kWaitSpinDefault = 1u << 23;   // mbarrier polls of 0.3 to 1.3 us: 2 to 10 seconds, longer than a team wait
 
 enum : int32_t { EPI_FACTOR = 0, EPI_GRAM = 1, EPI_NONE = 2 };   // EPI_NONE: a filler that only keeps a CTA in step
 
@@ -143,7 +143,8 @@ struct EngineArgs {
   int32_t sum_col;           // EPI_FACTOR: first of the tensor-memory columns the epilogue parks D0 + D1 in, or -1
   int32_t sumsq_on;          // 1: warps 4-7 follow the stages and sum g^2 for items that have sumsq_off >= 0
   int32_t* team_counters;    // one counter per team, zero at launch (nullptr when no item waits)
-  uint32_t team_spin_limit, wait_spin_limit;
+  uint32_t team_spin_limit[2];   // of the CTAs of a pair
+  uint32_t wait_spin_limit;
   const float* gscale;       // device scalar: every gradient counts as gscale[0] * g (nullptr: 1)
 };
 
@@ -176,11 +177,12 @@ __device__ __forceinline__ void drain_ring(uint64_t* full, int stage, uint32_t p
     return;
   }
   const int back = issued < (uint32_t)n_stages ? (int)issued : n_stages;
+  uint32_t spin = 0;       // (a stage that the other CTA of a pair has not loaded never completes)
   for (int q = 0; q < back; ++q) {
     int st = stage - 1 - q;
     uint32_t ph = phase;
     if (st < 0) { st += n_stages; ph ^= 1u; }
-    for (uint32_t spin = 0; spin < kDrainSpins && !mbar_try_wait<PAIR ? WAIT_PAIR : WAIT_CTA>(&full[st], ph); ++spin) __nanosleep(64);
+    for (; spin < kDrainSpins && !mbar_try_wait<PAIR ? WAIT_PAIR : WAIT_CTA>(&full[st], ph); ++spin) __nanosleep(64);
   }
 }
 
@@ -320,14 +322,16 @@ __global__ void __launch_bounds__(kEngineThreads, 1) tc_items_kernel(EngineArgs 
         volatile int32_t* cnt = team;
         uint32_t spin = 0;
         while (__any_sync(0xffffffffu, *cnt < wait_count)) {
-          if (++spin >= a.team_spin_limit || ((spin & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0))) { ok = false; break; }
+          if (++spin >= (rank == 0 ? a.team_spin_limit[0] : a.team_spin_limit[1])) {
+            give_up<PAIR>(abort);
+            if (leader) atomicOr(a.status, ST_WAIT_TEAM);
+            ok = false;
+            break;
+          }
+          if ((spin & 255u) == 0 && __any_sync(0xffffffffu, *abort != 0)) { ok = false; break; }
           __nanosleep(256);
         }
-        if (!ok) {
-          *abort = 1;
-          if (leader) atomicOr(a.status, ST_WAIT_TEAM);
-          break;
-        }
+        if (!ok) break;
       }
       for (int s = 0; s < n_seg && ok; ++s) {
         const Seg& S = I.seg[s];

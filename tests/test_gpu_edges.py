@@ -93,6 +93,21 @@ def test_a_step_repeats_bit_for_bit_beside_other_work(rank):
     ctx.adapm_destroy()
 
 
+def test_a_cta_that_gives_up_takes_the_other_one_of_its_pair_along():
+    """One CTA's wait runs out after a millisecond; the other one, in a wait of its own of more than a second (2^22 polls of at
+    least 256 ns), leaves with it."""
+    import time
+    ctx = A.adapm_create(_blocks([(256, 256, A.MOM_LOWRANK, 12, A.V_BLOCKMEAN, 1)]), A.hparams(grad_dtype=A.GRAD_BF16))
+    took = []
+    for _ in range(3):                  # (the first one also loads the kernel)
+        t0 = time.perf_counter()
+        ctx.adapm_selftest_expired_wait()
+        assert ctx.adapm_get_status() == A.ST_WAIT_TEAM
+        took.append(time.perf_counter() - t0)
+    assert min(took) < 0.5, took
+    ctx.adapm_destroy()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("rank", [1, 8, 9, 24, 40, 41, 81, 300])
 def test_exact_fp32_refit_at_the_edges_of_its_tiles(rank, dtype):
