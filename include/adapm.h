@@ -30,7 +30,7 @@
  *     hundred microseconds) and copies that description from pageable memory: make that step
  *     outside any stream capture.  Four combinations are remembered.
  *   - Every wait inside a kernel is bounded.  If one runs out (a GPU shared with other work that
- *     keeps this library's CTAs from running together for about a second), the kernel stops, sets a
+ *     keeps this library's CTAs from running together for one to ten seconds), the kernel stops, sets a
  *     bit in the device status word, and every later kernel of this context returns without writing
  *     until adapm_get_status has been called.  adapm_get_status then returns ADAPM_EDEVICE: the
  *     factors of some low-rank blocks are a mix of two iterates and the step is incomplete, so
@@ -60,7 +60,9 @@ enum {
   ADAPM_FLAG_NO_PANEL_TEAMS = 1,     /* hand the refit's panel items out longest-first: no CTA waits for another
                                         (for callers who share the GPU with long-running kernels)            */
   ADAPM_FLAG_FORCE_PANEL_TEAMS = 2,  /* team schedule even for sets with few blocks (small profiling cases)  */
-  ADAPM_FLAG_NO_SUMSQ_FOLD = 4,      /* block-mean v of tensor-path blocks from a pass of its own over g     */
+  ADAPM_FLAG_NO_SUMSQ_FOLD = 4,      /* block-mean v of tensor-path blocks from a pass of its own over g; no
+                                        effect on blocks with cols a multiple of 8 when clipping or the finite
+                                        check is on: that pass over g makes their sums                     */
   ADAPM_FLAG_CHECK_FINITE = 8        /* a NaN or Inf anywhere in the gradients: the step writes nothing and
                                         adapm_get_status reports bit 64 (costs one more pass over g)        */
 };
@@ -171,7 +173,9 @@ int adapm_state_breakdown(const adapm_ctx* ctx, size_t* full_m, size_t* L, size_
  * L is [rows, rank] and R is [rank, cols], both row-major and dense. */
 int adapm_state_layout(const adapm_ctx* ctx, int64_t block, int which, int64_t* offset, int64_t* count);
 
-/* Transient device memory one step needs (factor iterates, A = g R^T, B = L^T g, partial sums). */
+/* Transient device memory one step needs: split bf16 copies of the factors (12 (rows + cols) x rank bytes per tensor-path
+ * block, ranks rounded up to 16), their fp32 values between two refit passes (4 (rows + cols) x rank), padded copies of
+ * unaligned gradients, r x r matrices, partial sums. */
 size_t adapm_workspace_bytes(const adapm_ctx* ctx);
 int adapm_set_workspace(adapm_ctx* ctx, void* dev_ptr, size_t bytes);
 

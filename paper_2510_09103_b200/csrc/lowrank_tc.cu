@@ -180,7 +180,7 @@ struct MapSet {                     // tensor maps for one combination of caller
 struct TcProgram {
   std::vector<TcBlock> blk;
   int64_t n_convert_owners = 0;
-  int nb_max = 1, stage_k = 128, rp_max = 16, half_max = 16;
+  int nb_max = 1, stage_k = 128, rp_max = 16;
   int64_t work_begin = 0, work_end = 0;   // the tensor path's part of the workspace, in floats
   // shared-memory plan of an engine launch whose segments have up to n_a A operands in a CTA; pair: panel launches
   struct EngineConfig { int a_bytes, stage_bytes, n_stages, smem; };
@@ -505,7 +505,7 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
     row_groups += j.n_groups;
     row_jobs.push_back(j);
   }
-  P->rp_max = rp_max; P->half_max = half_max;
+  P->rp_max = rp_max;
   const int nb_max = (2 * half_max + 63) / 64;
   P->nb_max = nb_max;
 

@@ -391,9 +391,14 @@ __global__ void __launch_bounds__(256) meansq_final_kernel(const float* __restri
 }
 
 // ---- global gradient norm ---------------------------------------------------------------------------
-// Stage 1: one CTA per chunk of up to 16384 elements of one block; every thread adds its elements in a fixed
-// order, the warps and the CTA reduce in a fixed order.  Stage 2: one CTA adds the per-chunk sums in double,
-// again in a fixed order, and writes s = min(1, c / norm) and s^2.
+// Stage 1: one CTA per chunk of up to 16384 elements of one block, or, where the group sums are wanted too, per 16 warp units:
+// a unit is a group or a piece of one of up to 2048 elements, summed by one warp and left for the group's reduction.  Every
+// thread adds its elements in a fixed order, the warps and the CTA reduce in a fixed order.  Stage 2: one CTA adds the sums of
+// the CTAs in double, again in a fixed order, and writes s = min(1, c / norm) and s^2.
+// A short row leaves lanes of its unit idle, as it does in reduce_partial, whose pass over g this one saves.  32 M elements, rank
+// 8, clipped, us per step with a pass for each | one for both: rows of 8 13570 | 11062, 64 1710 | 1476, 128 904 | 791, 256
+// 564 | 441, 264 622 | 509, 384 421 | 381, 512 356 | 326, 768 303 | 288; fp32 rows of 256 1145 | 873.  (The panels' pairs and
+// the fp32 copies are in these figures too; no row length lost.)
 template <typename GT>
 __global__ void __launch_bounds__(256) gradnorm_partial_kernel(const NormRange* __restrict__ tab,
                                                                const int32_t* __restrict__ cta_range,

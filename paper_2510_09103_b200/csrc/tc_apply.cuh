@@ -34,7 +34,8 @@
 // works along the rows of the parameters, one column per lane, whatever the alignment of the rows.
 // Four groups where the arithmetic or the latency of that form sets the pace, two where the ring of buffers does (with four it
 // has to be four deep instead of six, or the ring of R half as deep): per-element v 5.30 -> 4.90 ms on the 1.5B shapes and 1.18
-// -> 1.05 on the 350M set at rank 128, rows of 2730 184 -> 140 us; group scalars 2.50 -> 2.71 or 3.15 ms, kept at two.
+// -> 1.05 on the 350M set at rank 128, rows of 2730 184 -> 140 us; group scalars 2.50 -> 2.71 or 3.15 ms, kept at two.  The form
+// with TMA is chosen for the set: one low-rank block with a per-element v makes its launch take four groups for all blocks.
 // The m x n matrices m_t, r_t and m^c are never stored.
 #pragma once
 
@@ -105,10 +106,11 @@ struct __align__(8) ApplyShared {
   int abort;
 };
 
-// The epilogue of one warp without TMA: 32 x 32 chunks of the accumulator, one column per lane.
+// The epilogue of one warp without TMA: 32 x 32 chunks of the accumulator, one column per lane.  (Rows in flight: a warp has 80
+// registers in this form.)
 template <int kGroups>
 __device__ __forceinline__ void apply_rows_epilogue(const ApplyArgs& a, ApplyShared& sh, float* patch, uint32_t tmem_acc) {
-  constexpr int kChunks = kApplyNT / 32, kBatch = kGroups == 4 ? 8 : 16;
+  constexpr int kChunks = kApplyNT / 32, kBatch = 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = warp & 3, grp = (warp - 2) >> 2;           // which 32 accumulator rows; chunks grp, grp + kGroups, ...
   const uint32_t lane_addr = (uint32_t)(32 * sub) << 16;

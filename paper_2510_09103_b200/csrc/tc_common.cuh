@@ -358,31 +358,13 @@ __device__ __host__ __forceinline__ uint32_t make_idesc(int n, bool a_mn_major, 
   return d;
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle (addresses and offsets in 16-byte units).
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;                // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;                // layout: 128-byte swizzle
-  return d;
-}
-// The same descriptor as two 32-bit halves, so that stepping through K only adds to the low half.
-// low: start address and leading byte offset; high: stride byte offset, version, swizzle mode.
+// Shared-memory matrix descriptor, 128-byte swizzle, as two 32-bit halves, so that stepping through K only adds to the low
+// half.  Addresses and offsets in 16-byte units.  low: start address and leading byte offset; high: stride byte offset, version, swizzle mode.
 __device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
   return ((smem_addr >> 4) & 0x3FFFu) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }
 __device__ __forceinline__ uint32_t desc_hi() { return (1024u >> 4) | (1u << 14) | (2u << 29); }
 __device__ __forceinline__ uint64_t desc_join(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
-// K-major operand (8-row groups 1024 B apart); k16 = which 16-wide K step inside the 64-wide box.
-__device__ __forceinline__ uint64_t desc_k_major(uint32_t smem_addr, int k16) {
-  return desc_join(desc_lo(smem_addr + 32u * (uint32_t)k16, 16), desc_hi());
-}
-// MN-major operand made of boxes `lbo_bytes` apart; k16 = which 16-row K step inside the box.
-__device__ __forceinline__ uint64_t desc_mn_major(uint32_t smem_addr, int k16, uint32_t lbo_bytes) {
-  return desc_join(desc_lo(smem_addr + 2048u * (uint32_t)k16, lbo_bytes), desc_hi());
-}
 
 // ---- split bf16 --------------------------------------------------------------------------------------
 // x ~ hi + lo with both parts bf16 (round to nearest even): the pair carries about 16 significant bits.
@@ -395,12 +377,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2_rn(float x0, float x1) {
 __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   hi = pack_bf16x2_rn(x0, x1);
   lo = pack_bf16x2_rn(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
-}
-__device__ __forceinline__ void split_bf16(float x, uint16_t& hi, uint16_t& lo) {
-  uint32_t h, l;
-  split_bf16x2(x, 0.f, h, l);
-  hi = (uint16_t)(h & 0xffffu);
-  lo = (uint16_t)(l & 0xffffu);
 }
 
 }  // namespace tc

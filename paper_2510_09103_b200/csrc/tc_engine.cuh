@@ -246,7 +246,7 @@ __device__ __forceinline__ bool mma_segment_any(const EngineArgs& a, EngineShare
                                                 bool two, bool mn_major, uint32_t ring, bool leader) {
 #define ADAPM_MMA(NA, NM, MN) return mma_segment<PAIR, NA, NM, MN, KS>(a, sh, cur, S, ring, leader)
   if (!PAIR) {
-    if (two) { if (n_a == 2) ADAPM_MMA(2, 2, true); ADAPM_MMA(1, 2, true); }
+    if (two) ADAPM_MMA(2, 2, true);          // (above rank 128 always both parts of A)
     if (n_a == 2) ADAPM_MMA(2, 1, true);
     ADAPM_MMA(1, 1, true);
   }
