@@ -516,23 +516,29 @@ int build_tensor_program(adapm_ctx* c, const std::vector<int64_t>& tc_ids, const
   // K = 64 stages: a ring of many small ones rides out the latency of DRAM and of the way through the barriers of the pair
   // better than two of K = 128 (rank 8 801 | 669, rank 80 5480 | 5164).
   // Sets with few items per pair take one panel: the last round of items is shorter.  Up to rank 64, where the ring then still
-  // has four stages, they take K = 128 with it: of the short K loops every stage costs a trip through the barriers.  Above,
-  // with three stages of K = 128 (two above rank 128), K = 64 is better: layers of width 1024, us per step, 64 | 128, rank 80:
-  // 2 layers 361 | 373, 4 478 | 506; rank 96: 4 510 | 537, 8 848 | 873; rank 128: 2 455 | 528, 4 599 | 677, 8 988 | 1053.
+  // has four stages, they take K = 128 with it: of the short K loops every stage costs a trip through the barriers.
   // us per step, two panels and K = 64 | one and K = 128, by items (of two panels) per pair: 0.3 (tiny set) 114 | 106, 1.5
   // (width 1024, 4 layers, rank 51) 447 | 432, 1.7 (60M) 376 | 375, 2.3 (6 layers) 546 | 549, 3.0 (8 layers) 668 | 692, 3.5
   // (1024 x 2730) 1042 | 1027, 3.9 (124M) 741 | 762, 10 (350M rank 8) 1615 | 1727.  Between two and four the better one
   // depends on how the items' lengths fall; the line keeps the last set that gains from it.
+  // Above rank 64 a ring of K = 128 has three stages, and one panel with K = 64 is better where items are few.  us per step, two
+  // panels K = 64 | one K = 64 | one K = 128: rank 80, 0.7 (width 1600, 1 layer) 544 | 472 | 493, 1.3 (768, 4 layers, rank
+  // 76) 394 | 379 | 396, 1.5 (1024, 4) 497 | 478 | 506, 2.0 (1600, 3) 713 | 710 | 769, 2.3 (1024, 6) 584 | 612 | 645, 2.7 (1600, 4)
+  // 858 | 998 | 957, 3.0 (1024, 8) 720 | 804 | 826.  With one panel in any case, K = 64 | 128: rank 96, 1.5 (1024, 4) 510 | 537,
+  // 2.0 (1600, 3) 746 | 805, 2.7 (1600, 4) 1046 | 1001, 3.0 (1024, 8) 848 | 873, 3.4 (1600, 5) 1266 | 1184; rank 102, 2048,
+  // 1 to 5 layers 722 | 913 to 1952 | 2157; rank 128, 1.5 (1024, 4) 599 | 677, 2.7 (1600, 4) 1098 | 1219.
   auto stages_with = [&](int stage_k, int n_a, bool pair) {
     return (224 * 1024) / (n_a * 256 * stage_k + stage_k * 128 * (pair ? (rp_max + 63) / 64 : nb_max));
   };
   int64_t panel_items = 0;                       // with two panels per CTA
   for (const TcBlock& t : P->blk) panel_items += (c->blocks[t.id].rows + 511) / 512 + (c->blocks[t.id].cols + 511) / 512;
-  const bool few_items = 4 * panel_items < (int64_t)15 * (P->n_sms / 2);      // 3.75 per pair
-  int n_pan = hp.tune_panels > 0 ? hp.tune_panels : (few_items || 6 * rp_max > 512 ? 1 : 2);
+  auto fewer_than = [&](int quarters) { return 4 * panel_items < (int64_t)quarters * (P->n_sms / 2); };     // per pair
+  const bool two_fit = 6 * rp_max <= 512, deep = stages_with(128, 1, true) >= 4;
+  const bool few_items = fewer_than(!deep && two_fit ? 9 : 15);
+  int n_pan = hp.tune_panels > 0 ? hp.tune_panels : (few_items || !two_fit ? 1 : 2);
   n_pan = std::max(1, std::min({n_pan, tc::kMaxA, 512 / (2 * rp_max)}));
   int stage_k = hp.tune_stage_k;
-  if (stage_k == 0) stage_k = few_items && stages_with(128, n_pan, true) >= 4 ? 128 : 64;
+  if (stage_k == 0) stage_k = few_items && (deep || (rp_max <= 96 && !fewer_than(9))) ? 128 : 64;
   const bool gram_small = 2 * rp_max <= 256;     // two accumulators of N = 2 rp: hi and lo window
   if (hp.tune_stage_k == 0 && stages_with(stage_k, n_pan, true) < 2) stage_k = 64;
   if (stages_with(stage_k, gram_small ? 1 : 2, false) < 2) stage_k = 64;
